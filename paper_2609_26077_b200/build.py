@@ -8,7 +8,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfmm_b200.so")
 SOURCES = ["fmm_api.cu", "fmm_encode.cu", "fmm_gemm.cu", "fmm_stats.cu"]
-HEADERS = [os.path.join(CSRC, "fmm_internal.h"), os.path.join(HERE, "..", "include", "fmm.h")]
+HEADERS = [os.path.join(CSRC, h) for h in sorted(os.listdir(CSRC)) if h.endswith((".h", ".cuh"))] + [
+    os.path.join(HERE, "..", "include", "fmm.h")]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-cudart", "static"]
@@ -21,7 +22,7 @@ def _stale(out):
     if not os.path.exists(out):
         return True
     t = os.path.getmtime(out)
-    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS + [os.path.join(CSRC, "fmm_ptx.cuh")]
+    deps = [os.path.join(CSRC, s) for s in SOURCES] + HEADERS
     return any(os.path.getmtime(d) > t for d in deps)
 
 

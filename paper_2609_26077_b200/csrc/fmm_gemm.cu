@@ -59,6 +59,11 @@ struct Cfg {
     // its producer and issuer, which also handle the scale tiles, spilled at 56.
     static constexpr int REGS_CTRL = (MX || MODE == MODE_FP32_OUT_WARP) ? 72 : 56, REGS_EPI = (MX || MODE == MODE_FP32_OUT_WARP) ? 208 : 224;
     static_assert(EPI_WARP0 * 32 * REGS_CTRL + EPI_WARPS * 32 * REGS_EPI <= NUM_THREADS * REGS_AT_LAUNCH, "register pool");
+    // Warp index, CTA rank and TMEM base as values the compiler knows to be warp-uniform (see warp_uniform): 3 % of the
+    // block-32 kernel at n = 8192 and 4096, 7 % of the single-CTA UE8M0 kernel at 1280 x 2816 x 3328.  Not for the UE8M0
+    // pair kernel, whose 256-column instructions hide their issue (2 % slower), nor for the weight-tile kernel, which
+    // then spills in the promotion loop (10 % slower at n = 4096).
+    static constexpr bool UNIFORM = !(MX && NCTA == 2) && MODE != MODE_FP32_SB_TILE;
     static constexpr int BROWS = BN / NCTA;                  // T_r rows this CTA loads per stage
     static constexpr int A_BYTES = BM * BK;
     static constexpr int B_BYTES = BROWS * BK;
@@ -210,8 +215,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const Ctl ctl{abort_flag, p.status};
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int cta_rank = (NCTA == 2) ? (int)cluster_ctarank() : 0;
+    auto uniform = [](uint32_t v) { return C::UNIFORM ? warp_uniform(v) : v; };
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int cta_rank = (NCTA == 2) ? (int)uniform(cluster_ctarank()) : 0;
     const bool leader = (cta_rank == 0);
     const int unit = blockIdx.x / NCTA;            // CTA or CTA pair index
     const int units = gridDim.x / NCTA;
@@ -232,7 +238,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     __syncthreads();
     if (NCTA == 2) cluster_sync();                 // the peer's barriers are initialised before anyone signals them
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = uniform(*tmem_slot);
 
     const int tiles_n = p.n / BN;
     const int kstages = p.k / BK;

@@ -19,6 +19,12 @@ __device__ __forceinline__ void cluster_sync()
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// A value that is the same in all lanes, in a form the compiler knows to be warp-uniform.  Warp indices and TMEM
+// addresses pass through here: tcgen05 instructions take their addresses and descriptors from uniform registers, and a
+// value not known to be uniform is moved there again before every instruction (four MMAs and a commit of a 128 x 128
+// tile issue in 256 cycles with uniform operands and in 378 without; one MMA and a commit in 171 and 288).
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 // true in exactly one lane of a converged warp (the same lane on every call)
 __device__ __forceinline__ bool elect_one()
 {
