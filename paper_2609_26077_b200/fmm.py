@@ -57,6 +57,18 @@ def lib():
         L.fmm_debug_build.restype = C.c_int
         for name in EXPORTS:
             getattr(L, name)
+        # the calls of the hot path take plain integers for pointers and sizes (one conversion each instead of an object)
+        ptr, i64, size = C.c_void_p, C.c_int64, C.c_size_t
+        L.fmm_workspace_bytes.argtypes = [ptr, i64, i64, i64, ptr]
+        L.fmm_host_workspace_bytes.argtypes = [ptr, i64, i64, i64, ptr]
+        L.fmm_quantized_view.argtypes = [ptr, i64, i64, i64, C.c_int, C.c_char] + [ptr] * 6
+        L.fmm_matmul.argtypes = [ptr, ptr, ptr, ptr, i64, i64, i64, ptr, size, ptr]
+        L.fmm_matmul_host.argtypes = [ptr, ptr, ptr, ptr, i64, i64, i64, ptr, size, ptr]
+        L.fmm_encode_only.argtypes = [ptr, ptr, ptr, i64, i64, i64, ptr, size, ptr]
+        L.fmm_multiply_only.argtypes = [ptr, ptr, i64, i64, i64, ptr, size, ptr]
+        L.fmm_ref_gemm_fp64.argtypes = [ptr, ptr, ptr, i64, i64, i64, ptr]
+        L.fmm_error_stats.argtypes = [ptr, ptr, i64, i64, ptr, ptr, size, ptr]
+        L.fmm_error_stats_noalloc.argtypes = [ptr, ptr, i64, i64, ptr, ptr]
         _lib = L
     return _lib
 
@@ -91,14 +103,32 @@ def fmm_brent_residual(U, V, W):
     return r.value
 
 
+_raw_stream = None
+
+
 def _stream_ptr(stream):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    """cudaStream_t of `stream`, or of the current stream of the current device, as an integer."""
+    global _raw_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None:
+        import torch
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        # torch.cuda.current_stream() builds a Stream object on every call (3 us); the raw handle is what is needed
+        _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+        torch.cuda.current_stream()          # initialises CUDA
+    return _raw_stream()
 
 
-def _dev_ptr(t):
-    return C.c_void_p(t.data_ptr())
+_f32 = None
+
+
+def _float32():
+    global _f32
+    if _f32 is None:
+        import torch
+        _f32 = torch.float32
+    return _f32
 
 
 class Plan:
@@ -116,7 +146,8 @@ class Plan:
         _check(lib().fmm_plan_create(C.byref(h), C.c_int(self.rank), _fptr(self.U), _fptr(self.V), _fptr(self.W),
                                      C.c_int(self.levels), C.byref(qp)), "fmm_plan_create")
         self._h = h
-        self._ws = None
+        self._ws = None              # (tensor, aligned address) of the cached workspace
+        self._need = {}              # workspace bytes by (M, N, K)
 
     def close(self):
         if getattr(self, "_h", None):
@@ -134,39 +165,60 @@ class Plan:
         return (self.rank ** self.levels) if self.levels > 0 else 1
 
     def workspace_bytes(self, M, N, K):
-        b = C.c_size_t()
-        _check(lib().fmm_workspace_bytes(self._h, C.c_int64(M), C.c_int64(N), C.c_int64(K), C.byref(b)),
-               "fmm_workspace_bytes")
-        return b.value
+        key = (M, N, K)
+        need = self._need.get(key)
+        if need is None:
+            b = C.c_size_t()
+            _check(lib().fmm_workspace_bytes(self._h, M, N, K, C.byref(b)), "fmm_workspace_bytes")
+            if len(self._need) >= 256:
+                self._need.clear()
+            need = self._need[key] = b.value
+        return need
+
+    def _own_workspace(self, need, device):
+        """The cached buffer, made anew when it is too small or on another device; (tensor, aligned address)."""
+        ws = self._ws
+        if ws is None or ws[0].numel() < need + 1024 or ws[0].device != device:
+            import torch
+            buf = torch.empty(need + 1024, dtype=torch.uint8, device=device)
+            ws = self._ws = (buf, buf.data_ptr() + (-buf.data_ptr()) % 1024)
+        return ws
 
     def workspace(self, M, N, K, device="cuda"):
         """A torch byte tensor large enough for this size (cached; 1024-byte aligned)."""
         import torch
+        device = torch.device(device)
+        if device.type == "cuda" and device.index is None:
+            device = torch.device("cuda", torch.cuda.current_device())
         need = self.workspace_bytes(M, N, K)
-        if self._ws is None or self._ws.numel() < need + 1024 or str(self._ws.device) != str(torch.device(device)):
-            self._ws = torch.empty(need + 1024, dtype=torch.uint8, device=device)
-        off = (-self._ws.data_ptr()) % 1024
-        return self._ws[off:off + need]
+        buf, addr = self._own_workspace(need, device)
+        off = addr - buf.data_ptr()
+        return buf[off:off + need]
 
     def matmul(self, A, B, out=None, workspace=None, stream=None):
         """fmm_matmul: C = A @ B through the realization, all steps on the device."""
-        import torch
         M, K = A.shape
         K2, N = B.shape
-        assert K == K2 and A.dtype == torch.float32 and B.dtype == torch.float32
+        f32 = _float32()
+        assert K == K2 and A.dtype is f32 and B.dtype is f32
         assert A.is_contiguous() and B.is_contiguous() and A.is_cuda and B.is_cuda
         if out is None:
-            out = torch.empty((M, N), dtype=torch.float32, device=A.device)
-        ws = workspace if workspace is not None else self.workspace(M, N, K, A.device)
-        _check(lib().fmm_matmul(self._h, _dev_ptr(A), _dev_ptr(B), _dev_ptr(out), C.c_int64(M), C.c_int64(N),
-                                C.c_int64(K), _dev_ptr(ws), C.c_size_t(ws.numel()), _stream_ptr(stream)), "fmm_matmul")
+            out = A.new_empty((M, N))
+        if workspace is not None:
+            ws, nbytes = workspace.data_ptr(), workspace.numel()
+        else:
+            nbytes = self.workspace_bytes(M, N, K)
+            ws = self._own_workspace(nbytes, A.device)[1]
+        status = _lib.fmm_matmul(self._h, A.data_ptr(), B.data_ptr(), out.data_ptr(), M, N, K, ws, nbytes, _stream_ptr(stream))
+        if status:
+            _check(status, "fmm_matmul")
         return out
 
     def host_workspace(self, M, N, K, device="cuda"):
         """Device buffer for matmul_host: fmm_host_workspace_bytes, 1024-byte aligned (a fresh tensor per call)."""
         import torch
         need = C.c_size_t()
-        _check(lib().fmm_host_workspace_bytes(self._h, C.c_int64(M), C.c_int64(N), C.c_int64(K), C.byref(need)),
+        _check(lib().fmm_host_workspace_bytes(self._h, M, N, K, C.byref(need)),
                "fmm_host_workspace_bytes")
         buf = torch.empty(need.value + 1024, dtype=torch.uint8, device=device)
         off = (-buf.data_ptr()) % 1024
@@ -180,29 +232,27 @@ class Plan:
         assert K == K2 and tuple(out.shape) == (M, N)
         for t in (A, B, out):
             assert t.dtype == torch.float32 and t.is_contiguous() and not t.is_cuda
-        _check(lib().fmm_matmul_host(self._h, C.c_void_p(A.data_ptr()), C.c_void_p(B.data_ptr()), C.c_void_p(out.data_ptr()),
-                                     C.c_int64(M), C.c_int64(N), C.c_int64(K), _dev_ptr(workspace),
-                                     C.c_size_t(workspace.numel()), _stream_ptr(stream)), "fmm_matmul_host")
+        _check(lib().fmm_matmul_host(self._h, A.data_ptr(), B.data_ptr(), out.data_ptr(), M, N, K, workspace.data_ptr(),
+                                     workspace.numel(), _stream_ptr(stream)), "fmm_matmul_host")
         return out
 
     def encode_only(self, A, B, workspace=None, stream=None):
         M, K = A.shape
         _, N = B.shape
         ws = workspace if workspace is not None else self.workspace(M, N, K, A.device)
-        _check(lib().fmm_encode_only(self._h, _dev_ptr(A), _dev_ptr(B), C.c_int64(M), C.c_int64(N), C.c_int64(K),
-                                     _dev_ptr(ws), C.c_size_t(ws.numel()), _stream_ptr(stream)), "fmm_encode_only")
+        _check(lib().fmm_encode_only(self._h, A.data_ptr(), B.data_ptr(), M, N, K,
+                                     ws.data_ptr(), ws.numel(), _stream_ptr(stream)), "fmm_encode_only")
         return ws
 
     def multiply_only(self, M, N, K, out, workspace=None, stream=None):
         ws = workspace if workspace is not None else self.workspace(M, N, K, out.device)
-        _check(lib().fmm_multiply_only(self._h, _dev_ptr(out), C.c_int64(M), C.c_int64(N), C.c_int64(K),
-                                       _dev_ptr(ws), C.c_size_t(ws.numel()), _stream_ptr(stream)), "fmm_multiply_only")
+        _check(lib().fmm_multiply_only(self._h, out.data_ptr(), M, N, K,
+                                       ws.data_ptr(), ws.numel(), _stream_ptr(stream)), "fmm_multiply_only")
         return out
 
     def quantized_view(self, M, N, K, term, side):
         vals = [C.c_size_t(), C.c_int64(), C.c_int64(), C.c_size_t(), C.c_int64(), C.c_int64()]
-        _check(lib().fmm_quantized_view(self._h, C.c_int64(M), C.c_int64(N), C.c_int64(K), C.c_int(term),
-                                        C.c_char(side.encode()), *[C.byref(v) for v in vals]), "fmm_quantized_view")
+        _check(lib().fmm_quantized_view(self._h, M, N, K, int(term), side.encode(), *[C.byref(v) for v in vals]), "fmm_quantized_view")
         return tuple(v.value for v in vals)
 
     def quantized_operand(self, ws, M, N, K, term, side):
@@ -248,12 +298,12 @@ class Plan:
 
 
 def fmm_ref_gemm_fp64(A, B, out=None, stream=None):
-    import torch
     M, K = A.shape
     _, N = B.shape
     if out is None:
+        import torch
         out = torch.empty((M, N), dtype=torch.float64, device=A.device)
-    _check(lib().fmm_ref_gemm_fp64(_dev_ptr(A), _dev_ptr(B), _dev_ptr(out), C.c_int64(M), C.c_int64(N), C.c_int64(K),
+    _check(lib().fmm_ref_gemm_fp64(A.data_ptr(), B.data_ptr(), out.data_ptr(), M, N, K,
                                    _stream_ptr(stream)), "fmm_ref_gemm_fp64")
     return out
 
@@ -263,16 +313,16 @@ _scratch = {}
 
 def fmm_error_stats(Cm, Cref, out3=None, stream=None):
     """Device tensor [sum (C-Cref)^2, sum Cref^2, max |C-Cref|] (fp64)."""
-    import torch
     M, N = Cm.shape
+    dev = Cm.device
     if out3 is None:
-        out3 = torch.empty(3, dtype=torch.float64, device=Cm.device)
-    key = str(Cm.device)
-    if key not in _scratch:
-        _scratch[key] = torch.empty(lib().fmm_error_stats_scratch_bytes(), dtype=torch.uint8, device=Cm.device)
-    sc = _scratch[key]
-    _check(lib().fmm_error_stats(_dev_ptr(Cm), _dev_ptr(Cref), C.c_int64(M), C.c_int64(N), _dev_ptr(out3),
-                                 _dev_ptr(sc), C.c_size_t(sc.numel()), _stream_ptr(stream)), "fmm_error_stats")
+        import torch
+        out3 = torch.empty(3, dtype=torch.float64, device=dev)
+    sc = _scratch.get(dev)
+    if sc is None:
+        sc = _scratch[dev] = Cm.new_empty(lib().fmm_error_stats_scratch_bytes() // 4)       # fp32 elements
+    _check(lib().fmm_error_stats(Cm.data_ptr(), Cref.data_ptr(), M, N, out3.data_ptr(), sc.data_ptr(), 4 * sc.numel(),
+                                 _stream_ptr(stream)), "fmm_error_stats")
     return out3
 
 
@@ -280,7 +330,7 @@ def fmm_error_stats_noalloc(Cm, Cref, out3, stream=None):
     """fmm_error_stats_noalloc: same statistics, block partials in the library's built-in scratch.
     Nothing is allocated here either: the caller supplies out3 (3 doubles on the device)."""
     M, N = Cm.shape
-    _check(lib().fmm_error_stats_noalloc(_dev_ptr(Cm), _dev_ptr(Cref), C.c_int64(M), C.c_int64(N), _dev_ptr(out3),
+    _check(lib().fmm_error_stats_noalloc(Cm.data_ptr(), Cref.data_ptr(), M, N, out3.data_ptr(),
                                          _stream_ptr(stream)), "fmm_error_stats_noalloc")
     return out3
 
