@@ -221,6 +221,8 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     // the pair-fused walk order belongs to the UE8M0 kernel; the fp32-scale kernels keep the products in term order
     for (int r = 0; r < FMM_MAX_RANK; ++r)
         g.order[r] = (plan->qp.scale_mode == FMM_SCALE_UE8M0_CEIL && plan->levels >= 1) ? plan->order[r] : r;
+    g.device = plan->device; g.sms = plan->sms;
+    g.R = lv >= 1 ? plan->rank : 1; g.nq = lv >= 1 ? 4 : 1; g.W = plan->W;
     g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0;
     g.guard = fmm_make_guard(dest, (size_t)g.Mfull * (size_t)g.Nfull * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
     fmm_status_t s = fmm_launch_gemm(g, plan->qp.block_k, (int)plan->qp.scale_mode, st, launches);
@@ -315,11 +317,14 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
     if (major != 10) return FMM_ERR_ARCH;
 
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) { cudaGetLastError(); return FMM_ERR_CUDA; }
+
     fmm_plan* p = new (std::nothrow) fmm_plan;
     if (!p) return FMM_ERR_ALLOC;
     memset(static_cast<void*>(p), 0, sizeof(*p));
     p->last_launches.store(0, std::memory_order_relaxed);
-    p->rank = rank; p->levels = levels; p->qp = *qp; p->device = dev;
+    p->rank = rank; p->levels = levels; p->qp = *qp; p->device = dev; p->sms = sms;
     if (levels > 0)
         for (int r = 0; r < rank; ++r)
             for (int j = 0; j < 4; ++j) { p->U[r][j] = U[r * 4 + j]; p->V[r][j] = V[r * 4 + j]; p->W[r][j] = W[r * 4 + j]; }

@@ -22,18 +22,10 @@
 //               two columns per instruction (fp32x2), overlapped with the next TMEM load.
 //
 // Every wait is bounded: on time-out a status word is set and all roles leave the kernel.
-#include <string.h>
-#include <atomic>
-#include "fmm_internal.h"
-#include "fmm_ptx.cuh"
+#include "fmm_gemm_common.cuh"
 
 namespace {
-using namespace fmmptx;
 
-// Internal third mode of the product kernel: FP32 scales whose B-side value is constant over each
-// 128-column tile (the 128 x 128 weight tiles of App. E.5).  The promotion then needs one multiply per row
-// and K block (s = sA * sB_tile) and one FMA per element, instead of a multiply and an FMA per element.
-constexpr int MODE_FP32_SB_TILE = 2;
 // Internal fourth mode: FP32 scales (per column, as mode 0) with a dedicated output warp.  The promoting warps hand
 // a finished product to it through a shared-memory copy of the (unweighted) accumulators and go straight on with
 // the next term; the W-weighted stores / add-reductions then overlap the next term's promotion instead of stalling
@@ -41,8 +33,6 @@ constexpr int MODE_FP32_SB_TILE = 2;
 // cross-over near 16 stages of 128 k); the dispatcher picks the mode per launch.
 constexpr int MODE_FP32_OUT_WARP = 3;
 
-constexpr int BM = 128;                 // rows per CTA
-constexpr int BK = 128;                 // K elements (= bytes) per pipeline stage: one swizzle row
 constexpr int EPI_WARPS = 8;               // two per TMEM lane quadrant, each half of the tile's columns
 constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, scale producer (FP32 modes), idle
 constexpr int NUM_THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
@@ -125,40 +115,6 @@ struct Cfg {
     static_assert(!MX || (SF_COLS <= 16 && OFF_HOLD + 2 * HOLD_T <= 512), "TMEM budget");
     static_assert(!MX || HOLD_T == 112 || HOLD_T == 48, "hold area is parked with 32- and 16-column stores");
 };
-
-constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;   // 2 s: far beyond any legitimate wait
-
-struct Ctl {
-    volatile int* abort_flag;   // shared memory
-    int* status;                // global status words
-    unsigned long long limit_ns = WAIT_LIMIT_NS;
-};
-
-// Bounded mbarrier wait.  Returns false after WAIT_LIMIT_NS or when another role has given up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const Ctl& ctl, int where)
-{
-    uint32_t spins = 0;
-    uint64_t t0 = 0;
-    while (!mbar_try_wait(bar, parity)) {
-        if ((++spins & 0x3FFu) == 0) {
-            if (*ctl.abort_flag) return false;
-            const uint64_t now = global_timer();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > ctl.limit_ns) {
-                *ctl.abort_flag = 1;
-                atomicCAS(ctl.status, 0, where);
-                return false;
-            }
-        }
-    }
-    return true;
-}
-// Same, with a warp-uniform verdict (the epilogue warps execute .sync.aligned instructions afterwards).
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const Ctl& ctl, int where)
-{
-    const bool ok = mbar_wait(bar, parity, ctl, where);
-    return __all_sync(0xffffffffu, ok);
-}
 
 // Self-test of the bounded wait: one warp waits on a barrier that nothing ever signals; the wait must
 // give up after limit_ns, record `where` in the status word and let the kernel end normally.
@@ -806,37 +762,6 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 }
 
 // --------------------------------------------------------------------------------- host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) != cudaSuccess ||
-            qres != cudaDriverEntryPointSuccess)
-            return nullptr;
-        fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
-}
-
-bool make_map_2d(CUtensorMap* tm, CUtensorMapDataType dt, int elt_bytes, const void* ptr, uint64_t inner, uint64_t outer,
-                 uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {inner, outer};
-    cuuint64_t strides[1] = {inner * (uint64_t)elt_bytes};
-    cuuint32_t box[2] = {box_inner, box_outer};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(tm, dt, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-              swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 template <int BN, int MODE, int BLK, int NCTA>
 fmm_status_t launch(const GemmParams& g, cudaStream_t st)
 {
@@ -855,9 +780,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     } else {
         tmSFA = tmA; tmSFB = tmB;       // unused in this mode
     }
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int dev = g.device, sms = g.sms;
     // the dynamic shared memory limit is a per-device attribute of the function: set once per device
     static std::atomic<bool> attr_set[64];
     if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
@@ -954,7 +877,9 @@ fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long li
 fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_t st, int* launches)
 {
     fmm_status_t s;
-    if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, st);
+    const int ksplit = fmm_split_choice(g, blk, mode);
+    if (ksplit > 0) s = fmm_launch_split(g, blk, mode, ksplit, st);
+    else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, st);
     else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, st);
     else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, st);
     else s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 128>(g, st);

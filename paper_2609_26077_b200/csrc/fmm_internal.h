@@ -77,7 +77,7 @@ struct fmm_plan {
     fmm_quant_params_t qp;
     float U[FMM_MAX_RANK][4], V[FMM_MAX_RANK][4], W[FMM_MAX_RANK][4];
     int terms;
-    int device;
+    int device, sms;
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
     int* d_out_start;         // [terms + 1]
@@ -153,6 +153,9 @@ struct GemmParams {
     const int* out_start; const FmmOutEntry* out;
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder tables (UE8M0 kernel)
     int order[FMM_MAX_RANK]; int steps;
+    int device, sms;                        // the plan's device and its SM count
+    int R, nq;                              // products per parent; blocks of a parent's matrix (4, or 1 for the cubic product)
+    const float (*W)[4];                    // innermost decoder, R x 4 (host pointer; unused when nq == 1)
     int* status;
     int terms_per_group;                    // consecutive terms that feed the same output blocks (R at levels >= 2, else all)
     int sb_tile;                            // fp32 scales, blk 128: the B-side scale is constant over each 128-column tile
@@ -164,6 +167,9 @@ struct GemmParams {
 fmm_status_t fmm_stats_guard_read(int* code);
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st);
 fmm_status_t fmm_launch_guard_selftest(int* status, cudaStream_t st);
+// K shares per term with which the cluster kernel (fmm_split.cu) takes this product; 0: the persistent kernel is faster
+int fmm_split_choice(const GemmParams& p, int blk, int mode);
+fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, int ksplit, cudaStream_t st);
 fmm_status_t fmm_launch_gemm(const GemmParams& p, int blk, int mode, cudaStream_t st, int* launches);
 
 static inline int64_t fmm_ipow(int64_t b, int e) { int64_t r = 1; while (e-- > 0) r *= b; return r; }

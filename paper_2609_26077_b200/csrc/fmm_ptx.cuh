@@ -18,6 +18,11 @@ __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// the same without ordering memory: nothing written before it needs to be seen by the other CTAs
+__device__ __forceinline__ void cluster_sync_relaxed()
+{
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
 
 // A value that is the same in all lanes, in a form the compiler knows to be warp-uniform.  Warp indices and TMEM
 // addresses pass through here: tcgen05 instructions take their addresses and descriptors from uniform registers, and a
