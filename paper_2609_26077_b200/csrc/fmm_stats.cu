@@ -93,56 +93,106 @@ __global__ void __launch_bounds__(STAT_THREADS) error_final_kernel(const double*
     if (threadIdx.x == 0 && FMM_GUARD(guard, out3, 24, 1602)) { out3[0] = sd; out3[1] = sr; out3[2] = mx; }
 }
 
-// 64x64 output tile per block of 16x16 threads, 4x4 outputs per thread, K step 16.
-__global__ void __launch_bounds__(256) ref_gemm_fp64_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                           double* __restrict__ C, int64_t M, int64_t N, int64_t K,
-                                                           const FmmGuard guard)
+// fp64 product of fp32 operands on the fp64 tensor path: T x T outputs per block of four warps (each T/2 x T/2, as
+// m16n8k4 fragments), K in steps of 16 through a ring of shared-memory stages filled by cp.async.  Operands stay fp32 in
+// shared memory and are widened (exactly) when a fragment is read: half the shared-memory bytes of a double copy, and the
+// conversions run beside the multiply-adds.  Rows are padded to 20 and T + 8 words so that a fragment read touches all 32
+// banks.  Bound: the fp64 pipe, 37 TFLOP/s measured with DFMA and with mma alike; fragments feed it with a fourth of the
+// operand reads of a 4 x 4 register tile (which took 1.12 ms at n = 2048).  T = 64 keeps the last wave full at the usual
+// sizes (7 tiles per SM at n = 2048); T = 32 spreads problems of fewer 64 x 64 tiles than SMs.  ALIGNED: both operands
+// 16-byte aligned (16-byte copies; 4-byte ones otherwise).
+constexpr int REF_BK = 16, REF_STAGES = 4;
+
+__device__ __forceinline__ void ref_mma(double (&c)[4], double a0, double a1, double b)
 {
-    __shared__ float As[16][64 + 1];   // [k][m]
-    __shared__ float Bs[16][64];       // [k][n]
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int64_t m0 = (int64_t)blockIdx.y * 64, n0 = (int64_t)blockIdx.x * 64;
-    double acc[4][4];
+    asm volatile("mma.sync.aligned.m16n8k4.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
+                 : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3]) : "d"(a0), "d"(a1), "d"(b));
+}
+template <bool ALIGNED>
+__device__ __forceinline__ void ref_copy16(float* dst, const float* src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (ALIGNED) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + 4 * i), "l"(src + i) : "memory");
+}
+
+template <int T, bool ALIGNED>
+__global__ void __launch_bounds__(128, T == 64 ? 4 : 8)
+ref_gemm_fp64_kernel(const float* __restrict__ A, const float* __restrict__ B, double* __restrict__ C, int64_t M, int64_t N, int64_t K,
+                     const FmmGuard guard)
+{
+    constexpr int LDA = REF_BK + 4, LDB = T + 8;
+    constexpr int MF = T / 32, NF = T / 16;               // m16 and n8 fragments of a warp's T/2 x T/2 outputs
+    __shared__ __align__(16) float As[REF_STAGES][T][LDA];          // [m][k]
+    __shared__ __align__(16) float Bs[REF_STAGES][REF_BK][LDB];     // [k][n]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int wm = (warp >> 1) * (T / 2), wn = (warp & 1) * (T / 2);
+    const int64_t m0 = (int64_t)blockIdx.y * T, n0 = (int64_t)blockIdx.x * T;
+    auto load = [&](int stage, int64_t k0) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    for (int64_t k0 = 0; k0 < K; k0 += 16) {
-        // A tile: 64 rows x 16 k = 1024 floats, 4 per thread
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = threadIdx.x + e * 256;
-            const int r = idx >> 4, kk = idx & 15;
-            As[kk][r] = A[(m0 + r) * K + k0 + kk];
+        for (int i = threadIdx.x; i < T * (REF_BK / 4); i += 128) {
+            const int r = i / (REF_BK / 4), c = i % (REF_BK / 4) * 4;
+            ref_copy16<ALIGNED>(&As[stage][r][c], A + (m0 + r) * K + k0 + c);
         }
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int idx = threadIdx.x + e * 256;
-            const int kk = idx >> 6, c = idx & 63;
-            Bs[kk][c] = B[(k0 + kk) * N + n0 + c];
+        for (int i = threadIdx.x; i < REF_BK * (T / 4); i += 128) {
+            const int r = i / (T / 4), c = i % (T / 4) * 4;
+            ref_copy16<ALIGNED>(&Bs[stage][r][c], B + (k0 + r) * N + n0 + c);
         }
-        __syncthreads();
+    };
+    double acc[MF][NF][4];
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double a[4], b[4];
+    for (int i = 0; i < MF; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = (double)As[kk][ty * 4 + i];
+        for (int j = 0; j < NF; ++j)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = (double)Bs[kk][tx * 4 + j];
+            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
+    const int steps = (int)(K / REF_BK);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+    for (int s = 0; s < REF_STAGES - 1; ++s) {
+        if (s < steps) load(s, (int64_t)s * REF_BK);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    for (int s = 0; s < steps; ++s) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(REF_STAGES - 2) : "memory");
+        __syncthreads();                                   // stage s has landed, stage s - 1 has been read by every warp
+        if (s + REF_STAGES - 1 < steps) load((s + REF_STAGES - 1) % REF_STAGES, (int64_t)(s + REF_STAGES - 1) * REF_BK);
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        const int st = s % REF_STAGES;
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+        for (int kk = 0; kk < REF_BK; kk += 4) {
+            double a[MF][2], b[NF];
+#pragma unroll
+            for (int i = 0; i < MF; ++i)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) a[i][h] = (double)As[st][wm + 16 * i + 8 * h + (lane >> 2)][kk + (lane & 3)];
+#pragma unroll
+            for (int j = 0; j < NF; ++j) b[j] = (double)Bs[st][kk + (lane & 3)][wn + 8 * j + (lane >> 2)];
+#pragma unroll
+            for (int i = 0; i < MF; ++i)
+#pragma unroll
+                for (int j = 0; j < NF; ++j) ref_mma(acc[i][j], a[i][0], a[i][1], b[j]);
         }
-        __syncthreads();
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        double* c = C + (m0 + ty * 4 + i) * N + n0 + tx * 4;
-        if (!FMM_GUARD(guard, c, 32, 1603)) continue;
-        reinterpret_cast<double2*>(c)[0] = make_double2(acc[i][0], acc[i][1]);
-        reinterpret_cast<double2*>(c)[1] = make_double2(acc[i][2], acc[i][3]);
-    }
+    for (int i = 0; i < MF; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int j = 0; j < NF; ++j) {
+                double* c = C + (m0 + wm + 16 * i + 8 * h + (lane >> 2)) * N + n0 + wn + 8 * j + 2 * (lane & 3);
+                if (FMM_GUARD(guard, c, 16, 1603)) *reinterpret_cast<double2*>(c) = make_double2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+            }
+}
+
+template <int T>
+void launch_ref(const float* A, const float* B, double* C, int64_t M, int64_t N, int64_t K, const FmmGuard& guard, cudaStream_t st)
+{
+    const dim3 grid((unsigned)(N / T), (unsigned)(M / T));
+    if ((((uintptr_t)A | (uintptr_t)B) & 15) == 0) ref_gemm_fp64_kernel<T, true><<<grid, 128, 0, st>>>(A, B, C, M, N, K, guard);
+    else ref_gemm_fp64_kernel<T, false><<<grid, 128, 0, st>>>(A, B, C, M, N, K, guard);
 }
 
 // Device address of g_stats_guard_code on the current device (FMM_DEBUG build; the release build passes no word and
@@ -212,9 +262,10 @@ fmm_status_t fmm_ref_gemm_fp64(const float* A, const float* B, double* Cref, int
     if (!A || !B || !Cref) return FMM_ERR_INVALID_ARG;
     if (M <= 0 || N <= 0 || K <= 0 || (M % 64) || (N % 64) || (K % 16)) return FMM_ERR_SHAPE;
     if ((uintptr_t)Cref & 15) return FMM_ERR_INVALID_ARG;
-    dim3 grid((unsigned)(N / 64), (unsigned)(M / 64));
     const FmmGuard guard = fmm_make_guard(Cref, sizeof(double) * (size_t)M * (size_t)N, nullptr, 0, stats_guard_word());
-    ref_gemm_fp64_kernel<<<grid, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(A, B, Cref, M, N, K, guard);
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if ((M / 64) * (N / 64) < 148) launch_ref<32>(A, B, Cref, M, N, K, guard, st);
+    else launch_ref<64>(A, B, Cref, M, N, K, guard, st);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
