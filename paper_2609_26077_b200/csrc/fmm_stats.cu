@@ -66,15 +66,16 @@ __global__ void __launch_bounds__(STAT_THREADS) error_partial_kernel(const float
         sr = fma(r.x, r.x, sr); sr = fma(r.y, r.y, sr);
         mx = fmax(mx, fmax(fabs(d0), fabs(d1)));
     };
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i + 3 * stride < pairs; i += 4 * stride) {
+    // (the last trip is predicated, not a loop of single loads: at n = 4096 a thread makes 7 trips)
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += 4 * stride) {
         float2 c[4]; double2 r[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { c[u] = __ldcs(C2 + i + u * stride); r[u] = __ldcs(R2 + i + u * stride); }
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < pairs) { c[u] = __ldcs(C2 + i + u * stride); r[u] = __ldcs(R2 + i + u * stride); }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) add(c[u], r[u]);
+        for (int u = 0; u < 4; ++u)
+            if (i + u * stride < pairs) add(c[u], r[u]);
     }
-    for (; i < pairs; i += stride) add(__ldcs(C2 + i), __ldcs(R2 + i));
     block_reduce3(sd, sr, mx, sm);
     if (threadIdx.x == 0 && FMM_GUARD(guard, partial + blockIdx.x * 3, 24, 1601)) {
         partial[blockIdx.x * 3] = sd; partial[blockIdx.x * 3 + 1] = sr; partial[blockIdx.x * 3 + 2] = mx;
@@ -86,11 +87,27 @@ __global__ void __launch_bounds__(STAT_THREADS) error_final_kernel(const double*
 {
     __shared__ double sm[3 * (STAT_THREADS / 32)];
     double sd = 0.0, sr = 0.0, mx = 0.0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");       // launched under the first kernel's tail: its partials are complete now
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         sd += partial[i * 3]; sr += partial[i * 3 + 1]; mx = fmax(mx, partial[i * 3 + 2]);
     }
     block_reduce3(sd, sr, mx, sm);
     if (threadIdx.x == 0 && FMM_GUARD(guard, out3, 24, 1602)) { out3[0] = sd; out3[1] = sr; out3[2] = mx; }
+}
+
+// Both stages.  The second is launched with the programmatic-serialization attribute, so that its launch latency falls
+// under the first (2 us of 38 at n = 4096).
+fmm_status_t launch_stats(const float* C, const double* Cref, int64_t count, double* partial, double* out3, const FmmGuard& guard, cudaStream_t st)
+{
+    error_partial_kernel<<<STAT_BLOCKS, STAT_THREADS, 0, st>>>(C, Cref, count, partial, guard);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1); cfg.blockDim = dim3(STAT_THREADS); cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, error_final_kernel, static_cast<const double*>(partial), STAT_BLOCKS, out3, guard);
+    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
 // fp64 product of fp32 operands on the fp64 tensor path: T x T outputs per block of four warps (each T/2 x T/2, as
@@ -251,9 +268,7 @@ fmm_status_t fmm_error_stats(const float* C, const double* Cref, int64_t M, int6
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     double* partial = static_cast<double*>(scratch);
     const FmmGuard guard = fmm_make_guard(partial, sizeof(double) * 3 * STAT_BLOCKS, out3, sizeof(double) * 3, stats_guard_word());
-    error_partial_kernel<<<STAT_BLOCKS, STAT_THREADS, 0, st>>>(C, Cref, M * N, partial, guard);
-    error_final_kernel<<<1, STAT_THREADS, 0, st>>>(partial, STAT_BLOCKS, out3, guard);
-    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+    return launch_stats(C, Cref, M * N, partial, out3, guard, st);
 }
 
 fmm_status_t fmm_ref_gemm_fp64(const float* A, const float* B, double* Cref, int64_t M, int64_t N, int64_t K,
@@ -310,9 +325,7 @@ fmm_status_t fmm_error_stats_noalloc(const float* C, const double* Cref, int64_t
     // every one of the STAT_BLOCKS slots is rewritten by the first kernel, so nothing left behind by
     // an earlier call is ever read and no clearing is needed
     const FmmGuard guard = fmm_make_guard(partial, sizeof(double) * 3 * STAT_BLOCKS, out3, sizeof(double) * 3, stats_guard_word());
-    error_partial_kernel<<<STAT_BLOCKS, STAT_THREADS, 0, st>>>(C, Cref, M * N, partial, guard);
-    error_final_kernel<<<1, STAT_THREADS, 0, st>>>(partial, STAT_BLOCKS, out3, guard);
-    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+    return launch_stats(C, Cref, M * N, partial, out3, guard, st);
 }
 
 int64_t fmm_error_stats_noalloc_max_elements(void) { return NOALLOC_MAX_ELEMS; }
