@@ -123,10 +123,12 @@ fmm_status_t fmm_matmul(const fmm_plan_t* plan, const float* A, const float* B, 
  *   memory makes the three copies asynchronous; pageable memory works but the copies then block the caller.
  *   workspace dev, 1024-byte aligned, at least fmm_host_workspace_bytes() bytes, caller-owned: the product's
  *   workspace followed by device staging for A, B and C.
- * Everything is enqueued on cuda_stream in order (upload A, upload B, product, download C) and nothing is
- * synchronised: C is valid once the stream has drained.  Calls on different streams with different workspaces
- * overlap one call's uploads with another's product and download (the links are full duplex); that is the
- * intended use for a sequence of products.  Errors as fmm_matmul, except that the host pointers need no
+ * Nothing is synchronised: C is valid once cuda_stream has drained, and work enqueued on it before and after the call is
+ * ordered with the whole call.  Inside a call with pinned operands of 8 MB or more and at most one level, the larger
+ * operand goes up in strips that are encoded, multiplied and downloaded on side streams of the plan while later strips are
+ * on their way (same results to the bit; up to four calls of a plan at a time have side streams of their own).  Calls on
+ * different streams with different workspaces overlap one call's uploads with another's product and download (the links
+ * are full duplex); that is the intended use for a sequence of products.  Errors as fmm_matmul, except that the host pointers need no
  * particular alignment; fmm_host_workspace_bytes returns FMM_ERR_INVALID_ARG for a null plan or bytes. */
 fmm_status_t fmm_host_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K,
                                       size_t* bytes);

@@ -3,9 +3,73 @@
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
+#include <mutex>
 #include <new>
 #include <vector>
 #include "fmm_internal.h"
+
+constexpr int HOST_STRIPS = 8;
+
+// Side streams and events of one fmm_matmul_host call in flight.
+struct HostLane {
+    cudaStream_t comp = nullptr, down = nullptr;
+    cudaEvent_t up[HOST_STRIPS + 1] = {}, mul[HOST_STRIPS] = {}, done[2] = {};
+    bool taken = false;           // a host thread is enqueuing on it
+    bool create()
+    {
+        bool ok = cudaStreamCreateWithFlags(&comp, cudaStreamNonBlocking) == cudaSuccess && cudaStreamCreateWithFlags(&down, cudaStreamNonBlocking) == cudaSuccess;
+        auto make = [&](cudaEvent_t& e) { ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess; };
+        for (auto& e : up) make(e);
+        for (auto& e : mul) make(e);
+        for (auto& e : done) make(e);
+        if (!ok) cudaGetLastError();
+        return ok;
+    }
+    ~HostLane()
+    {
+        for (auto& e : up) if (e) cudaEventDestroy(e);
+        for (auto& e : mul) if (e) cudaEventDestroy(e);
+        for (auto& e : done) if (e) cudaEventDestroy(e);
+        if (comp) cudaStreamDestroy(comp);
+        if (down) cudaStreamDestroy(down);
+    }
+    bool idle() const
+    {
+        for (auto& e : done) if (cudaEventQuery(e) != cudaSuccess) { cudaGetLastError(); return false; }
+        return true;
+    }
+};
+
+// A plan's lanes, made when first needed, at most MAX of them, destroyed with the plan.  A lane serves one call at a time: one
+// whose last call has drained if there is one, else a new one, else the longest unused (its streams keep the order then).
+// nullptr when every lane is being enqueued on by another thread: the caller then does without.
+struct FmmHostLanes {
+    static constexpr int MAX = 4;
+    std::mutex mutex;
+    std::vector<HostLane*> lanes;          // least recently used first
+    HostLane* acquire()
+    {
+        std::lock_guard<std::mutex> lock(mutex);
+        HostLane* pick = nullptr;
+        for (HostLane* l : lanes) if (!l->taken && l->idle()) { pick = l; break; }
+        if (!pick && (int)lanes.size() < MAX) {
+            pick = new (std::nothrow) HostLane;
+            if (!pick || !pick->create()) { delete pick; return nullptr; }
+            lanes.push_back(pick);
+        }
+        if (!pick) for (HostLane* l : lanes) if (!l->taken) { pick = l; break; }
+        if (!pick) return nullptr;
+        pick->taken = true;
+        for (size_t i = 0; i + 1 < lanes.size(); ++i) if (lanes[i] == pick) std::swap(lanes[i], lanes[i + 1]);
+        return pick;
+    }
+    void release(HostLane* l)
+    {
+        std::lock_guard<std::mutex> lock(mutex);
+        l->taken = false;
+    }
+    ~FmmHostLanes() { for (HostLane* l : lanes) delete l; }
+};
 
 namespace {
 
@@ -106,9 +170,13 @@ void fill_coef(float dst[FMM_MAX_RANK][4], const float src[FMM_MAX_RANK][4], int
         for (int j = 0; j < 4; ++j) dst[r][j] = src[r][j];
 }
 
-// One side of steps 1-2: outer levels as fp32 combinations, last level fused with the quantizer.
+// A strip of the leaf rows of A and C (m0 .. m1) or of the leaf columns of B and C (n0 .. n1), in every block.
+struct Strip { int64_t m0, m1, n0, n1; };
+
+// One side of steps 1-2: outer levels as fp32 combinations, last level fused with the quantizer.  [lo, hi) is the strip of
+// leaf rows (A) or columns (B) to encode: everything, or with at most one level a part of it (multiples of 128).
 fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* X,
-                         int64_t rows, int64_t cols, bool b_side, cudaStream_t st, int* launches)
+                         int64_t rows, int64_t cols, bool b_side, int64_t lo, int64_t hi, bool overlap, cudaStream_t st, int* launches)
 {
     const int R = plan->rank, lv = plan->levels;
     const int blk = plan->qp.block_k, mode = (int)plan->qp.scale_mode;
@@ -123,34 +191,40 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     e.preround_bf16 = (b_side && plan->qp.b_preround_bf16) ? 1 : 0;
     e.guard = fmm_make_guard(e.q_out, (size_t)L.terms * (size_t)((b_side ? L.n : L.m) * L.k),
                              e.s_out, (size_t)L.terms * (b_side ? L.sb_term : L.sa_term), plan->d_status + FMM_GUARD_WORD);
+    // first element of the strip in every array
+    const int64_t strip_in = b_side ? lo : lo * cols;
+    e.q_out += lo * L.k;
+    e.s_out = static_cast<char*>(e.s_out) + (mode == FMM_SCALE_UE8M0_CEIL ? lo / 128 * 512 : lo * 4 * (b_side ? 1 : 128 / blk));
     fmm_status_t s;
     if (lv == 0) {
         // Plain quantization of the matrix itself.  The matrix is cut into four panels (row panels of A,
         // column panels of B) that are handled like four "combinations" with identity coefficients, so
         // each thread keeps four independent loads in flight; the outputs land where the unsplit
         // matrix would put them.
-        const bool panels = b_side ? (cols % (e.b_tile ? 512 : 256) == 0) : (rows % 4 == 0);
-        e.in = X; e.in_batch_stride = 0; e.ld = cols; e.batch = 1;
-        e.overlap_prev = b_side ? 1 : 0;
+        const int64_t ext = hi - lo;               // rows of A / columns of B in this launch
+        const bool panels = b_side ? (ext % (e.b_tile ? 512 : 256) == 0) : (ext % 4 == 0);
+        e.in = X + strip_in; e.in_batch_stride = 0; e.ld = cols; e.batch = 1;
+        e.overlap_prev = b_side && overlap ? 1 : 0;
+        e.s_ld = (int)(b_side ? cols : rows); e.sf_blocks = (int)((b_side ? cols : rows) / 128);
         if (panels) {
             e.nq = 4; e.R = 4;
             for (int r = 0; r < 4; ++r) e.coef[r][r] = 1.0f;
             if (b_side) {
-                e.rows = (int)rows; e.cols = (int)(cols / 4);
-                for (int j = 0; j < 4; ++j) e.qoff[j] = (int64_t)j * (cols / 4);
-                e.s_step = (int)(cols / 4); e.s_ld = (int)cols; e.sf_blocks = (int)(cols / 128);
+                e.rows = (int)rows; e.cols = (int)(ext / 4);
+                for (int j = 0; j < 4; ++j) e.qoff[j] = (int64_t)j * (ext / 4);
             } else {
-                e.rows = (int)(rows / 4); e.cols = (int)cols;
-                for (int j = 0; j < 4; ++j) e.qoff[j] = (int64_t)j * (rows / 4) * cols;
-                e.s_step = (int)(rows / 4); e.s_ld = (int)rows; e.sf_blocks = (int)(rows / 128);
+                e.rows = (int)(ext / 4); e.cols = (int)cols;
+                for (int j = 0; j < 4; ++j) e.qoff[j] = (int64_t)j * (ext / 4) * cols;
             }
+            e.s_step = (int)(ext / 4);
             // the four panels share one scale array (panel r is shifted by r * s_step rows / columns inside it)
             e.s_term_stride = 0;
         } else {
-            e.rows = (int)rows; e.cols = (int)cols; e.nq = 1; e.R = 1;
+            e.rows = (int)(b_side ? rows : ext); e.cols = (int)(b_side ? ext : cols); e.nq = 1; e.R = 1;
             e.coef[0][0] = 1.0f;
-            e.s_step = 0; e.s_ld = (int)(b_side ? cols : rows); e.sf_blocks = (int)((b_side ? cols : rows) / 128);
+            e.s_step = 0;
         }
+        e.q_term = (int64_t)e.rows * e.cols;
     } else {
         const float* cur = X;
         int64_t cur_rows = rows, cur_cols = cols, cur_ld = cols, cur_stride = 0;
@@ -173,16 +247,18 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
             cur = c.out; cur_rows /= 2; cur_cols /= 2; cur_ld = cur_cols; cur_stride = cur_rows * cur_cols;
             batch *= R;
         }
-        e.in = cur; e.in_batch_stride = cur_stride; e.ld = cur_ld; e.batch = batch;
+        e.in = cur + strip_in; e.in_batch_stride = cur_stride; e.ld = cur_ld; e.batch = batch;
         // the B-side leaf encoder may start under the tail of the A-side one (launched just before it by fmm_matmul /
         // fmm_encode_only) when it reads the caller's matrix itself, i.e. nothing a kernel of this call has written
-        e.overlap_prev = (b_side && cur == X) ? 1 : 0;
+        e.overlap_prev = (b_side && overlap && cur == X) ? 1 : 0;
         const int div = fused2 ? 4 : 2;
         e.rows = (int)(cur_rows / div); e.cols = (int)(cur_cols / div); e.nq = 4; e.R = R;
         e.qoff[0] = 0; e.qoff[1] = e.cols; e.qoff[2] = (int64_t)e.rows * e.ld; e.qoff[3] = (int64_t)e.rows * e.ld + e.cols;
         for (int j = 0; j < 4; ++j) e.qoff_outer[j] = 2 * e.qoff[j];
         fill_coef(e.coef, coef, R);
         e.s_step = 0; e.s_ld = b_side ? e.cols : e.rows; e.sf_blocks = (b_side ? e.cols : e.rows) / 128;
+        e.q_term = (int64_t)e.rows * e.cols;
+        if (b_side) e.cols = (int)(hi - lo); else e.rows = (int)(hi - lo);
         if (fused2) {
             s = b_side ? fmm_launch_encode2_b(e, mode, st) : fmm_launch_encode2_a(e, blk, mode, st);
             if (s == FMM_OK) ++*launches;
@@ -194,15 +270,17 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     return s;
 }
 
-fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float* C, int64_t M, int64_t N,
+fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float* C, int64_t M, int64_t N, const Strip& strip,
                       cudaStream_t st, int* launches, bool after_encode)
 {
     GemmParams g;
     memset(&g, 0, sizeof(g));
     g.overlap_prev = after_encode ? 1 : 0;
-    g.qa = reinterpret_cast<const uint8_t*>(ws + L.qa);
-    g.qb = reinterpret_cast<const uint8_t*>(ws + L.qb);
-    g.sa = ws + L.sa; g.sb = ws + L.sb;
+    g.qa = reinterpret_cast<const uint8_t*>(ws + L.qa) + strip.m0 * L.k;
+    g.qb = reinterpret_cast<const uint8_t*>(ws + L.qb) + strip.n0 * L.k;
+    const bool e8 = plan->qp.scale_mode == FMM_SCALE_UE8M0_CEIL;
+    g.sa = ws + L.sa + (e8 ? strip.m0 / 128 * 512 : strip.m0 * 4 * (128 / plan->qp.block_k));
+    g.sb = ws + L.sb + (e8 ? strip.n0 / 128 * 512 : strip.n0 * 4);
     g.sa_term = (int64_t)L.sa_term; g.sb_term = (int64_t)L.sb_term;
     // The product kernel applies the innermost decoder only: leaf products of parent p land in the four
     // blocks of parent p's (2m x 2n) matrix.  For one level that matrix is C itself; for more levels the
@@ -213,7 +291,8 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     const int64_t parents = lv >= 2 ? fmm_ipow(plan->rank, lv - 1) : 1;
     const int64_t pm = lv >= 1 ? 2 * L.m : L.m, pn = lv >= 1 ? 2 * L.n : L.n;      // a parent's matrix
     float* dest = lv >= 2 ? reinterpret_cast<float*>(ws + L.dec[lv - 1]) : C;
-    g.C = dest; g.ldc = pn; g.Mfull = parents * pm; g.Nfull = pn;
+    g.C = dest + strip.m0 * pn + strip.n0; g.ldc = pn; g.Mfull = parents * pm; g.Nfull = pn;
+    g.msub = (int)(strip.m1 - strip.m0); g.nsub = (int)(strip.n1 - strip.n0);
     g.m = (int)L.m; g.n = (int)L.n; g.k = (int)L.k; g.terms = (int)L.terms;
     g.terms_per_group = plan->levels >= 2 ? plan->rank : (int)L.terms;
     g.out_start = plan->d_out_start; g.out = plan->d_out; g.status = plan->d_status;
@@ -421,6 +500,8 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
     }
     pstart.push_back((int)pentries.size());
 
+    p->lanes = new (std::nothrow) FmmHostLanes;
+    if (!p->lanes) { delete p; return FMM_ERR_ALLOC; }
     cudaError_t ce = cudaMalloc(&p->d_status, 64 * sizeof(int));
     if (ce == cudaSuccess) ce = cudaMalloc(&p->d_out_start, sizeof(int) * start.size());
     if (ce == cudaSuccess) ce = cudaMalloc(&p->d_out, sizeof(FmmOutEntry) * (entries.size() + 1));
@@ -444,6 +525,7 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
 fmm_status_t fmm_plan_destroy(fmm_plan_t* p)
 {
     if (!p) return FMM_ERR_INVALID_ARG;
+    delete p->lanes;
     if (p->d_status) cudaFree(p->d_status);
     if (p->d_out_start) cudaFree(p->d_out_start);
     if (p->d_out) cudaFree(p->d_out);
@@ -498,8 +580,8 @@ fmm_status_t fmm_encode_only(const fmm_plan_t* plan, const float* A, const float
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, st, &launches);
+    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
+    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
 }
@@ -512,7 +594,7 @@ fmm_status_t fmm_multiply_only(const fmm_plan_t* plan, float* C, int64_t M, int6
     fmm_status_t s = check_ws(plan, M, N, K, ws, ws_bytes, &L);
     if (s != FMM_OK) return s;
     int launches = 0;
-    s = multiply(plan, L, static_cast<char*>(ws), C, M, N, reinterpret_cast<cudaStream_t>(stream), &launches, false);
+    s = multiply(plan, L, static_cast<char*>(ws), C, M, N, {0, L.m, 0, L.n}, reinterpret_cast<cudaStream_t>(stream), &launches, false);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
 }
@@ -526,9 +608,9 @@ fmm_status_t fmm_matmul(const fmm_plan_t* plan, const float* A, const float* B, 
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, st, &launches);
-    if (s == FMM_OK) s = multiply(plan, L, static_cast<char*>(ws), C, M, N, st, &launches, true);
+    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
+    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
+    if (s == FMM_OK) s = multiply(plan, L, static_cast<char*>(ws), C, M, N, {0, L.m, 0, L.n}, st, &launches, true);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
 }
@@ -546,6 +628,69 @@ fmm_status_t fmm_host_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t
     return FMM_OK;
 }
 
+// One cudaMemcpyAsync per leaf block row / column of a strip: rows lo .. hi (whole rows), or columns lo .. hi, of each of the
+// `blocks` leaf blocks of a rows x cols matrix.
+static bool copy_strip(float* dst, const float* src, int64_t rows, int64_t cols, int blocks, bool by_rows, int64_t lo, int64_t hi,
+                       cudaMemcpyKind kind, cudaStream_t st)
+{
+    for (int b = 0; b < blocks; ++b) {
+        cudaError_t e;
+        if (by_rows) {
+            const int64_t at = (b * (rows / blocks) + lo) * cols;
+            e = cudaMemcpyAsync(dst + at, src + at, (size_t)((hi - lo) * cols) * 4, kind, st);
+        } else {
+            const int64_t at = b * (cols / blocks) + lo;
+            e = cudaMemcpy2DAsync(dst + at, (size_t)cols * 4, src + at, (size_t)cols * 4, (size_t)(hi - lo) * 4, (size_t)rows, kind, st);
+        }
+        if (e != cudaSuccess) { cudaGetLastError(); return false; }
+    }
+    return true;
+}
+
+// Host operands, at most one level: the transfers bound the call (n = 4096: 134 MB up at 55 GB/s = 2.4 ms, 67 MB down, against
+// 0.33 ms of kernels), and the link is full duplex.  So the smaller operand goes up first, the larger one in strips of leaf
+// rows (A) or columns (B); a strip is encoded and multiplied on one side stream while the next one is on its way, and its part
+// of C goes down on another while later strips still come up.  What remains beside the upload is the last strip's kernels
+// and download.  Strips of at least 4 MB (75 us), at most 8, cut at 256 rows / columns so that a strip has the tiles of
+// the whole product: the results are the same bits.
+static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* A, const float* B, float* C,
+                                       float* dA, float* dB, float* dC, int64_t M, int64_t N, int64_t K, int strips, bool by_rows,
+                                       HostLane& lane, cudaStream_t st)
+{
+    const int blocks = 1 << plan->levels;
+    const cudaMemcpyKind up = cudaMemcpyHostToDevice, down = cudaMemcpyDeviceToHost;
+    int launches = 0;
+    auto sig = [](cudaEvent_t e, cudaStream_t from, cudaStream_t to) {
+        if (cudaEventRecord(e, from) == cudaSuccess && cudaStreamWaitEvent(to, e, 0) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    };
+    // whatever happens below, the caller's stream waits for what has been enqueued on the side streams
+    auto join = [&](fmm_status_t s) {
+        const bool ok = sig(lane.done[0], lane.comp, st) && sig(lane.done[1], lane.down, st);
+        return s == FMM_OK && !ok ? FMM_ERR_CUDA : s;
+    };
+    const int64_t ext = by_rows ? L.m : L.n, gran = ext % 256 == 0 ? 256 : 128, units = ext / gran;
+    if (cudaMemcpyAsync(by_rows ? dB : dA, by_rows ? B : A, (size_t)(by_rows ? K * N : M * K) * 4, up, st) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
+    if (!sig(lane.up[strips], st, lane.comp)) return join(FMM_ERR_CUDA);
+    fmm_status_t s = by_rows ? encode_side(plan, L, ws, dB, K, N, true, 0, L.n, false, lane.comp, &launches)
+                             : encode_side(plan, L, ws, dA, M, K, false, 0, L.m, false, lane.comp, &launches);
+    for (int i = 0; i < strips && s == FMM_OK; ++i) {
+        const int64_t lo = units * i / strips * gran, hi = units * (i + 1) / strips * gran;
+        Strip part = {0, L.m, 0, L.n};
+        if (by_rows) { part.m0 = lo; part.m1 = hi; } else { part.n0 = lo; part.n1 = hi; }
+        if (!copy_strip(by_rows ? dA : dB, by_rows ? A : B, by_rows ? M : K, by_rows ? K : N, blocks, by_rows, lo, hi, up, st) ||
+            !sig(lane.up[i], st, lane.comp)) return join(FMM_ERR_CUDA);
+        s = by_rows ? encode_side(plan, L, ws, dA, M, K, false, lo, hi, false, lane.comp, &launches)
+                    : encode_side(plan, L, ws, dB, K, N, true, lo, hi, false, lane.comp, &launches);
+        if (s == FMM_OK) s = multiply(plan, L, ws, dC, M, N, part, lane.comp, &launches, false);
+        if (s != FMM_OK) break;
+        if (!sig(lane.mul[i], lane.comp, lane.down) || !copy_strip(C, dC, M, N, blocks, by_rows, lo, hi, down, lane.down)) return join(FMM_ERR_CUDA);
+    }
+    plan->last_launches.store(launches, std::memory_order_relaxed);
+    return join(s);
+}
+
 fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float* B, float* C,
                              int64_t M, int64_t N, int64_t K, void* ws, size_t ws_bytes, void* stream)
 {
@@ -560,6 +705,31 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
     float* dB = reinterpret_cast<float*>(reinterpret_cast<char*>(dA) + host_align((size_t)M * K * 4));
     float* dC = reinterpret_cast<float*>(reinterpret_cast<char*>(dB) + host_align((size_t)K * N * 4));
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (plan->levels <= 1) {
+        FmmLayout L;
+        s = check_ws(plan, M, N, K, ws, inner, &L);
+        if (s != FMM_OK) return s;
+        const bool by_rows = M >= N;                         // the larger operand of the two
+        const int64_t ext = by_rows ? L.m : L.n, bytes = (by_rows ? M : N) * K * 4;
+        int64_t strips = bytes / (4 << 20);
+        if (strips > HOST_STRIPS) strips = HOST_STRIPS;
+        if (strips > ext / (ext % 256 == 0 ? 256 : 128)) strips = ext / (ext % 256 == 0 ? 256 : 128);
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        // pageable copies block the host in order, so they would gain nothing from the strips
+        auto pinned = [](const void* p) {
+            cudaPointerAttributes a;
+            return cudaPointerGetAttributes(&a, p) == cudaSuccess && a.type == cudaMemoryTypeHost;
+        };
+        if (strips > 1 && pinned(A) && pinned(B) && pinned(C) && cudaStreamIsCapturing(st, &capture) == cudaSuccess &&
+            capture == cudaStreamCaptureStatusNone) {
+            if (HostLane* lane = plan->lanes->acquire()) {
+                s = matmul_host_strips(plan, L, base, A, B, C, dA, dB, dC, M, N, K, (int)strips, by_rows, *lane, st);
+                plan->lanes->release(lane);
+                return s;
+            }
+        }
+        cudaGetLastError();
+    }
     if (cudaMemcpyAsync(dA, A, (size_t)M * K * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(dB, B, (size_t)K * N * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) {
         cudaGetLastError();

@@ -164,7 +164,7 @@ __device__ __forceinline__ void store_chunk_a(const EncodeParams& p, const float
 {
     constexpr int GROUP = BLK / 4;
     constexpr unsigned FULL = 0xffffffffu;
-    const int64_t term_codes = (int64_t)p.rows * p.cols;
+    const int64_t term_codes = p.q_term;
     const int my_r = lane & 7;
     uint8_t* qp = p.q_out + ((int64_t)b * p.R) * term_codes + (int64_t)i * p.cols + c * 128 + lane * 4;
 #pragma unroll
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(TILE ? 256 : 128, TILE ? 2 : 4) encode_b_kerne
     const int kc = blockIdx.y;                      // chunk of 128 k
     const int b = blockIdx.z;
     const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
-    const int64_t term_codes = (int64_t)p.rows * p.cols;
+    const int64_t term_codes = p.q_term;
 
     float raw[4][16];
     float blk_amax[FMM_MAX_RANK], blk_inv[FMM_MAX_RANK];
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
     const int b = blockIdx.z;
     const int k0 = kb * 32 + khalf * 16;
     const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
-    const int64_t term_codes = (int64_t)p.rows * p.cols;
+    const int64_t term_codes = p.q_term;
 
     float raw[4][16];
 #pragma unroll
@@ -520,7 +520,7 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
     const int b = blockIdx.z;
     const int k0 = kc * 128 + warp * 32 + khalf * 16;
     const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
-    const int64_t term_codes = (int64_t)p.rows * p.cols;
+    const int64_t term_codes = p.q_term;
 
     float raw[4][16];
 #pragma unroll
@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
     const int kb = blockIdx.y;                                      // 32-k block
     const int k0 = kb * 32 + (lane & 7) * 4;
     const int b = blockIdx.z;
-    const int64_t term_codes = (int64_t)p.rows * p.cols;
+    const int64_t term_codes = p.q_term;
     const int my_r = lane & 7;
     // The block's 32 k x 32 columns of each of the 16 sub-blocks go through shared memory: the global loads are
     // whole 128-byte row segments (a thread reading its own 4 k x 1 column directly touches eight lines per warp

@@ -137,7 +137,7 @@ struct KParams {
     // at the innermost level; all terms at one level) feed one set of output blocks and are walked by one CTA
     // (pair) in order.  (Cutting the slots of a short last wave into narrower items does not pay: a tcgen05.mma of
     // half the width takes as long to issue, measured 4 % slower at n = 8192.)
-    int positions, terms_per_group, items;
+    int positions, tiles_n, terms_per_group, items;      // tiles_n: tile positions per row of positions
     const int* out_start; const FmmOutEntry* out;
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
     int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
@@ -196,7 +196,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     tc_fence_after();
     const uint32_t tmem_base = uniform(*tmem_slot);
 
-    const int tiles_n = p.n / BN;
+    const int tiles_n = p.tiles_n;
     const int kstages = p.k / BK;
     const int nkb = p.k / BLK;
     // ti-th product a CTA (pair) walks in work-item group grp: the parents of the group one after the other, the R
@@ -768,13 +768,14 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     using C = Cfg<BN, MODE, BLK, NCTA>;
     CUtensorMap tmA, tmB, tmC, tmSFA, tmSFB;
     const CUtensorMapSwizzle SW = CU_TENSOR_MAP_SWIZZLE_128B;
-    if (!make_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qa, (uint64_t)g.k, (uint64_t)g.terms * g.m, BK, BM, SW)) return FMM_ERR_CUDA;
-    if (!make_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qb, (uint64_t)g.k, (uint64_t)g.terms * g.n, BK, C::BROWS, SW)) return FMM_ERR_CUDA;
-    if (!make_map_2d(&tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.C, (uint64_t)g.Nfull, (uint64_t)g.Mfull, C::CH, 32,
-                     C::CH == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B)) return FMM_ERR_CUDA;
+    if (!make_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qa, (uint64_t)g.k, (uint64_t)(g.terms - 1) * g.m + g.msub, BK, BM, SW)) return FMM_ERR_CUDA;
+    if (!make_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qb, (uint64_t)g.k, (uint64_t)(g.terms - 1) * g.n + g.nsub, BK, C::BROWS, SW)) return FMM_ERR_CUDA;
+    if (!make_map_2d(&tmC, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, g.C, (uint64_t)(g.Nfull - g.n + g.nsub), (uint64_t)(g.Mfull - g.m + g.msub), C::CH, 32,
+                     C::CH == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, (uint64_t)g.Nfull)) return FMM_ERR_CUDA;
     if (C::MX) {
         // scale tiles as rows of 128 uint32 (one 512-byte atom per row)
-        const uint64_t atoms_a = (uint64_t)g.terms * (g.k / 128) * (g.m / 128), atoms_b = (uint64_t)g.terms * (g.k / 128) * (g.n / 128);
+        const uint64_t chunks = (uint64_t)g.terms * (g.k / 128);
+        const uint64_t atoms_a = (chunks - 1) * (g.m / 128) + g.msub / 128, atoms_b = (chunks - 1) * (g.n / 128) + g.nsub / 128;
         if (!make_map_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, g.sa, 128, atoms_a, 128, 1, CU_TENSOR_MAP_SWIZZLE_NONE)) return FMM_ERR_CUDA;
         if (!make_map_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, g.sb, 128, atoms_b, 128, C::SFB_ATOMS, CU_TENSOR_MAP_SWIZZLE_NONE)) return FMM_ERR_CUDA;
     } else {
@@ -790,7 +791,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
         }
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
     }
-    const int positions = (g.m / (BM * NCTA)) * (g.n / BN);
+    const int positions = (g.msub / (BM * NCTA)) * (g.nsub / BN);
     const int max_units = sms / NCTA;
     // Term groups as separate work items only where that shortens the longest CTA's list of terms (many terms on
     // few tile positions); otherwise one CTA (pair) walks all terms of its position.
@@ -809,7 +810,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.sa = static_cast<const uint8_t*>(g.sa); kp.sb = static_cast<const uint8_t*>(g.sb);
     kp.sa_term = g.sa_term; kp.sb_term = g.sb_term;
     kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.terms = g.terms;
-    kp.positions = positions; kp.terms_per_group = tpg;
+    kp.positions = positions; kp.tiles_n = g.nsub / BN; kp.terms_per_group = tpg;
     kp.items = slots;
     kp.out_start = g.out_start; kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
@@ -877,6 +878,7 @@ fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long li
 fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_t st, int* launches)
 {
     fmm_status_t s;
+    // chosen for the whole problem, also when this launch covers a strip of it: the strips' results do not depend on the cut
     const int ksplit = fmm_split_choice(g, blk, mode);
     if (ksplit > 0) s = fmm_launch_split(g, blk, mode, ksplit, st);
     else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, st);

@@ -70,12 +70,12 @@ EncodeTiledFn get_encode_fn()
 }
 
 bool make_map_2d(CUtensorMap* tm, CUtensorMapDataType dt, int elt_bytes, const void* ptr, uint64_t inner, uint64_t outer,
-                 uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz)
+                 uint32_t box_inner, uint32_t box_outer, CUtensorMapSwizzle swz, uint64_t pitch = 0)      // pitch in elements, 0: inner
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
     cuuint64_t dims[2] = {inner, outer};
-    cuuint64_t strides[1] = {inner * (uint64_t)elt_bytes};
+    cuuint64_t strides[1] = {(pitch ? pitch : inner) * (uint64_t)elt_bytes};
     cuuint32_t box[2] = {box_inner, box_outer};
     cuuint32_t estr[2] = {1, 1};
     return fn(tm, dt, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

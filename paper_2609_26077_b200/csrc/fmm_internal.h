@@ -78,6 +78,7 @@ struct fmm_plan {
     float U[FMM_MAX_RANK][4], V[FMM_MAX_RANK][4], W[FMM_MAX_RANK][4];
     int terms;
     int device, sms;
+    struct FmmHostLanes* lanes;   // streams and events of fmm_matmul_host
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
     int* d_out_start;         // [terms + 1]
@@ -103,7 +104,8 @@ struct EncodeParams {
     int nq;                   // number of input blocks read (4, or 1 for a plain pass over one matrix)
     int R;                    // combinations per input matrix
     float coef[FMM_MAX_RANK][4];
-    uint8_t* q_out;           // codes, term t = b * R + r at q_out + t * rows * cols
+    uint8_t* q_out;           // codes, term t = b * R + r at q_out + t * q_term
+    int64_t q_term;           // rows * cols, or more when the launch covers a strip of the rows (A) / columns (B) of every term
     void* s_out;              // scales
     int64_t s_term_stride;    // bytes between the scale arrays of consecutive terms
     int s_step;               // rows (A side) / columns (B side) by which combination r is shifted inside a shared scale array
@@ -150,6 +152,8 @@ struct GemmParams {
     float* C; int64_t ldc;                  // full output
     int64_t Mfull, Nfull;
     int m, n, k, terms;
+    int msub, nsub;                         // output rows / columns of every leaf block this launch covers (m, n: all of them); the
+                                            // pointers above then point at the strip's first row and column
     const int* out_start; const FmmOutEntry* out;
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder tables (UE8M0 kernel)
     int order[FMM_MAX_RANK]; int steps;

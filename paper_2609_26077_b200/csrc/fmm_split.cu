@@ -409,10 +409,11 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     using C = SplitCfg<MODE, BLK>;
     CUtensorMap tmA, tmB, tmSFA, tmSFB;
     const CUtensorMapSwizzle SW = CU_TENSOR_MAP_SWIZZLE_128B;
-    if (!make_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qa, (uint64_t)g.k, (uint64_t)g.terms * g.m, BK, BM, SW)) return FMM_ERR_CUDA;
-    if (!make_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qb, (uint64_t)g.k, (uint64_t)g.terms * g.n, BK, C::BN, SW)) return FMM_ERR_CUDA;
+    if (!make_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qa, (uint64_t)g.k, (uint64_t)(g.terms - 1) * g.m + g.msub, BK, BM, SW)) return FMM_ERR_CUDA;
+    if (!make_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qb, (uint64_t)g.k, (uint64_t)(g.terms - 1) * g.n + g.nsub, BK, C::BN, SW)) return FMM_ERR_CUDA;
     if (C::MX) {
-        const uint64_t atoms_a = (uint64_t)g.terms * (g.k / 128) * (g.m / 128), atoms_b = (uint64_t)g.terms * (g.k / 128) * (g.n / 128);
+        const uint64_t chunks = (uint64_t)g.terms * (g.k / 128);
+        const uint64_t atoms_a = (chunks - 1) * (g.m / 128) + g.msub / 128, atoms_b = (chunks - 1) * (g.n / 128) + g.nsub / 128;
         if (!make_map_2d(&tmSFA, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, g.sa, 128, atoms_a, 128, 1, CU_TENSOR_MAP_SWIZZLE_NONE)) return FMM_ERR_CUDA;
         if (!make_map_2d(&tmSFB, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, g.sb, 128, atoms_b, 128, 1, CU_TENSOR_MAP_SWIZZLE_NONE)) return FMM_ERR_CUDA;
     } else {
@@ -431,7 +432,7 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     const int S = g.R * ksplit;
 
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = split_config<MODE, BLK>(S, (unsigned)(g.n / C::BN), (unsigned)(g.m / BM), (unsigned)(g.terms / g.R), st, attr);
+    cudaLaunchConfig_t cfg = split_config<MODE, BLK>(S, (unsigned)(g.nsub / C::BN), (unsigned)(g.msub / BM), (unsigned)(g.terms / g.R), st, attr);
     // right behind the encoders of the same call: set up while they drain, the producer warps wait before their first load
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
