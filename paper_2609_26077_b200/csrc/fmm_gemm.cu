@@ -138,7 +138,7 @@ struct KParams {
     // (pair) in order.  (Cutting the slots of a short last wave into narrower items does not pay: a tcgen05.mma of
     // half the width takes as long to issue, measured 4 % slower at n = 8192.)
     int positions, tiles_n, terms_per_group, items;      // tiles_n: tile positions per row of positions
-    const int* out_start; const FmmOutEntry* out;
+    const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
     int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
     int* status;
@@ -200,10 +200,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int kstages = p.k / BK;
     const int nkb = p.k / BLK;
     // ti-th product a CTA (pair) walks in work-item group grp: the parents of the group one after the other, the R
-    // products of a parent in the plan's walk order (identity unless the decoder is pair-fused)
+    // products of a parent in the plan's walk order
     auto term_of = [&](int grp, int ti) {
         if constexpr (C::MX) return grp * p.terms_per_group + (ti / p.R) * p.R + p.order[ti % p.R];
-        else return grp * p.terms_per_group + ti;
+        else return p.walk[grp * p.terms_per_group + ti].term;
     };
     const int row_blocks_a = p.m / 128, row_blocks_b = p.n / 128;
 
@@ -256,9 +256,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int slot = w;
                 const int grp = slot / p.positions, pos = slot - grp * p.positions;
                 const int tn = pos % tiles_n;
-                const int t_end = (grp + 1) * p.terms_per_group;
                 const int tm = pos / tiles_n;
-                for (int t = t_end - p.terms_per_group; t < t_end && ok; ++t) {
+                for (int ti = 0; ti < p.terms_per_group && ok; ++ti) {
+                    const int t = term_of(grp, ti);
                     const uint8_t* sb_t = p.sb + (long long)t * p.sb_term + (long long)tn * BN * 4;
                     const uint8_t* sa_t = p.sa + (long long)t * p.sa_term + (long long)(tm * NCTA + cta_rank) * BM * (C::KB_PER_STAGE * 4);
                     for (int ks = 0; ks < kstages; ++ks) {
@@ -288,11 +288,11 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int slot = w;
                 const int grp = slot / p.positions, pos = slot - grp * p.positions;
                 const int tm = pos / tiles_n, tn = pos % tiles_n;
-                const int t_end = (grp + 1) * p.terms_per_group;
-                for (int t = t_end - p.terms_per_group; t < t_end && ok; ++t) {
+                const int s_end = (grp + 1) * p.terms_per_group;
+                for (int s = s_end - p.terms_per_group; s < s_end && ok; ++s) {
                     if (!mbar_wait_warp(bar_dfull, dphase, ctl, 401)) { ok = false; break; }
                     dphase ^= 1u;
-                    const int o0 = p.out_start[t], o1 = p.out_start[t + 1];
+                    const int o0 = p.walk[s].out0, o1 = p.walk[s].out1;
                     if (lane == 0) bulk_wait<0>();     // the previous term's writes to these tiles have landed
                     __syncwarp();
                     for (int o = o0; o < o1; ++o) {
@@ -446,7 +446,15 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int nch = cw / 32;
             const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + h * cw;
             for (int ti = 0, left = p.terms_per_group; left > 0 && ok; ++ti, --left) {
-                const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;
+                const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;      // FP32 scales: the step of the walk
+                // FP32 scales: the sum starts from `carry` times the previous product's, still in the registers (the test of ti
+                // says nothing that the table does not, and is worth 1.5 % of the block-32 kernel's time)
+                const float carry = (C::MX || ti == 0) ? 0.0f : p.walk[t].carry;
+                const unsigned long long carry2 = pack2(carry, carry);
+                if (carry == 0.0f) {                    // not a product with zero: the sum before may not be finite
+#pragma unroll
+                    for (int i = 0; i < (C::MX ? 1 : C::CW / 2); ++i) acc2[i] = 0ull;
+                }
                 if (C::MX) {
                     if (!mbar_wait_warp(bar_tfull(0), bphase, ctl, 301)) { ok = false; break; }
                     tc_fence_after();
@@ -534,7 +542,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     static_assert(!C::ROWS4 || C::KB_PER_STAGE == 4 || C::KB_PER_STAGE == 1, "block 32 or 128");
                     static_assert(!C::DUMP || C::ROWS4, "the output warp expects the four-row register layout");
 #pragma unroll
-                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = 0ull;         // acc2[k * (CW/8) + j]: row slot k, column group j
+                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);         // acc2[k * (CW/8) + j]: row slot k, column group j
                     constexpr int JG = C::CW / 8;                               // column groups of eight per warp
                     constexpr int KB = C::KB_PER_STAGE;
                     // A-side scales of the thread's four rows (q*32 + lane/4 + 8k of this CTA's 128), per K block
@@ -605,7 +613,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (!ok) break;
                 } else {
 #pragma unroll
-                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = 0ull;
+                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);
                     // this thread's row (q*32 + lane of the CTA's 128) in the A-side part of a scale stage
                     const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + lane) * (C::KB_PER_STAGE * 4);
                     for (int ks = 0; ks < kstages && ok; ++ks) {
@@ -685,7 +693,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 // half-accumulated tiles, product kernel 3 % faster; evict-first on the operand loads was slower).
                 // The policy word is rebuilt here so that it is not live across the promotion loop.
                 const uint64_t pol_c = policy_evict_last();
-                const int o0 = p.out_start[t], o1 = p.out_start[t + 1];
+                const int o0 = p.walk[t].out0, o1 = p.walk[t].out1;
                 if (lane == 0) bulk_wait<0>();     // the previous term's writes to these tiles have landed
                 __syncwarp();
                 for (int o = o0; o < o1; ++o) {
@@ -812,7 +820,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.terms = g.terms;
     kp.positions = positions; kp.tiles_n = g.nsub / BN; kp.terms_per_group = tpg;
     kp.items = slots;
-    kp.out_start = g.out_start; kp.out = g.out; kp.status = g.status;
+    kp.walk = g.walk; kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
     kp.R = g.terms_per_group > 0 ? g.terms_per_group : 1;       // products per parent (1 for the cubic product)

@@ -9,13 +9,21 @@
 #define FMM_MAX_RANK 8
 #define FMM_MAX_LEVELS 3
 
-// One destination of a leaf product in C: block origin, weight, and whether this is the first
-// product written there (store) or a later one (accumulate).
+// One destination of a product in C: block origin, weight, and whether this is the first
+// product written there (store) or a later one (accumulate).  FP32 scales.
 struct FmmOutEntry {
     int row_off;   // element row of the destination block origin in C
     int col_off;   // element column
     float w;       // product of the W coefficients along the recursion path
     int first;     // 1: overwrite, 0: add
+};
+
+// One step of the fp32-scale product kernel's walk over the leaf products: which term it multiplies, the factor of the
+// previous step's sum that its accumulators start from, and where the sum goes (see choose_walk in fmm_api.cu).
+struct FmmWalkEntry {
+    int term;
+    float carry;              // 0 at the first product of a parent
+    int out0, out1;           // entries [out0, out1) of the FmmOutEntry table
 };
 
 // Store guard of the FMM_DEBUG build (the stand-in for a memory checker, which this library cannot count on
@@ -81,10 +89,9 @@ struct fmm_plan {
     struct FmmHostLanes* lanes;   // streams and events of fmm_matmul_host
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
-    int* d_out_start;         // [terms + 1]
+    FmmWalkEntry* d_walk;     // [terms]
     FmmOutEntry* d_out;       // [total entries], block offsets in units of leaf blocks (scaled at launch)
-    int n_out_total;
-    int order[FMM_MAX_RANK];  // walk order of the R products of a parent (identity unless the decoder is pair-fused)
+    int order[FMM_MAX_RANK];  // pair-fused decoder: walk order of the R products of a parent
     int steps;                // pair-fused decoder: steps per parent, ceil(R / 2)
     int* d_pair_start;        // [parents * steps + 1]
     FmmPairEntry* d_pair;     // entries of all steps
@@ -154,7 +161,7 @@ struct GemmParams {
     int m, n, k, terms;
     int msub, nsub;                         // output rows / columns of every leaf block this launch covers (m, n: all of them); the
                                             // pointers above then point at the strip's first row and column
-    const int* out_start; const FmmOutEntry* out;
+    const FmmWalkEntry* walk; const FmmOutEntry* out;  // walk and decoder of the fp32-scale kernel
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder tables (UE8M0 kernel)
     int order[FMM_MAX_RANK]; int steps;
     int device, sms;                        // the plan's device and its SM count
