@@ -30,6 +30,15 @@ __device__ __forceinline__ uint32_t pack4_e4m3(float a, float b, float c, float 
     return (uint32_t)cvt_e4m3x2(b, a) | ((uint32_t)cvt_e4m3x2(d, c) << 16);
 }
 
+// four codes of v * inv (the multiplications two per instruction)
+__device__ __forceinline__ uint32_t scaled_pack4(const float4& v, float inv)
+{
+    const unsigned long long i2 = pack2(inv, inv);
+    float a, b, c, d;
+    unpack2(mul2(pack2(v.x, v.y), i2), a, b); unpack2(mul2(pack2(v.z, v.w), i2), c, d);
+    return pack4_e4m3(a, b, c, d);
+}
+
 // Scale of one block from its amax.  Returns the multiplier applied before the cast and writes
 // the stored scale (fp32 mode) or the biased power-of-two exponent (UE8M0 mode).
 template <int MODE>
@@ -82,7 +91,11 @@ template <uint32_t NZ> __device__ __forceinline__ bool row_used(int r, int R)
 // adjacent.  Forms the R combinations v[r], reduces their block maxima with a transposing butterfly over the
 // 8 lanes (lane & 7) - afterwards each lane holds the maximum of combination (lane & 7) - and computes that
 // combination's multiplier `inv` and stored scale (s or e8) once per block instead of once per lane.
-template <int GROUP, int MODE, uint32_t NZ>
+//
+// PACKED: two elements per fp32x2 instruction, the same IEEE operations in half the issue slots (two-level kernels, whose
+// 49 combinations bind them to the issue rate: 217 -> 202 us for both sides at n = 8192; no gain in the one-level kernels,
+// which wait for memory, and 1 % slower at block 128, where the pairs cost registers).
+template <int GROUP, int MODE, uint32_t NZ, bool PACKED = true>
 __device__ __forceinline__ void combine_chunk(const EncodeParams& p, const float4 (&x)[4], int lane,
                                               float4 (&v)[FMM_MAX_RANK], float& inv, float& s, uint32_t& e8)
 {
@@ -98,14 +111,20 @@ __device__ __forceinline__ void combine_chunk(const EncodeParams& p, const float
             for (int j = 0; j < 4; ++j) {
                 const float cj = p.coef[r][j];
                 if (coef_used<NZ>(r, j, cj)) {
-                    if (!set) {
+                    const unsigned long long c2 = pack2(cj, cj);
+                    if (PACKED && !set) {
+                        unpack2(mul2(c2, pack2(x[j].x, x[j].y)), v[r].x, v[r].y); unpack2(mul2(c2, pack2(x[j].z, x[j].w)), v[r].z, v[r].w);
+                    } else if (PACKED) {
+                        unpack2(fma2(c2, pack2(x[j].x, x[j].y), pack2(v[r].x, v[r].y)), v[r].x, v[r].y);
+                        unpack2(fma2(c2, pack2(x[j].z, x[j].w), pack2(v[r].z, v[r].w)), v[r].z, v[r].w);
+                    } else if (!set) {
                         v[r].x = __fmul_rn(cj, x[j].x); v[r].y = __fmul_rn(cj, x[j].y);
                         v[r].z = __fmul_rn(cj, x[j].z); v[r].w = __fmul_rn(cj, x[j].w);
-                        set = true;
                     } else {
                         v[r].x = __fmaf_rn(cj, x[j].x, v[r].x); v[r].y = __fmaf_rn(cj, x[j].y, v[r].y);
                         v[r].z = __fmaf_rn(cj, x[j].z, v[r].z); v[r].w = __fmaf_rn(cj, x[j].w, v[r].w);
                     }
+                    set = true;
                 }
             }
             am[r] = fmaxf(fmaxf(fabsf(v[r].x), fabsf(v[r].y)), fmaxf(fabsf(v[r].z), fabsf(v[r].w)));
@@ -144,12 +163,13 @@ __device__ __forceinline__ float4 combine_outer(const EncodeParams& p, int r, co
         const float cj = p.coef[r][j];
         if (coef_used<NZ>(r, j, cj)) {
             const float4 a = raw[j][q2];
+            const unsigned long long c2 = pack2(cj, cj);
             if (!set) {
-                o.x = __fmul_rn(cj, a.x); o.y = __fmul_rn(cj, a.y); o.z = __fmul_rn(cj, a.z); o.w = __fmul_rn(cj, a.w);
+                unpack2(mul2(c2, pack2(a.x, a.y)), o.x, o.y); unpack2(mul2(c2, pack2(a.z, a.w)), o.z, o.w);
                 set = true;
             } else {
-                o.x = __fmaf_rn(cj, a.x, o.x); o.y = __fmaf_rn(cj, a.y, o.y);
-                o.z = __fmaf_rn(cj, a.z, o.z); o.w = __fmaf_rn(cj, a.w, o.w);
+                unpack2(fma2(c2, pack2(a.x, a.y), pack2(o.x, o.y)), o.x, o.y);
+                unpack2(fma2(c2, pack2(a.z, a.w), pack2(o.z, o.w)), o.z, o.w);
             }
         }
     }
@@ -166,16 +186,17 @@ __device__ __forceinline__ void store_chunk_a(const EncodeParams& p, const float
     constexpr unsigned FULL = 0xffffffffu;
     const int64_t term_codes = p.q_term;
     const int my_r = lane & 7;
-    uint8_t* qp = p.q_out + ((int64_t)b * p.R) * term_codes + (int64_t)i * p.cols + c * 128 + lane * 4;
+    uint8_t* row = p.q_out + ((int64_t)b * p.R) * term_codes + (int64_t)i * p.cols + c * 128;      // warp-uniform
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
         if (row_used<NZ>(r, p.R)) {
             const float inv_r = __shfl_sync(FULL, inv, (GROUP == 32) ? r : ((lane & 24) | r));
+            uint8_t* qp = row + (uint32_t)(lane * 4);
             if (FMM_GUARD(p.guard, qp, 4, 1101))
-            *reinterpret_cast<uint32_t*>(qp) = pack4_e4m3(__fmul_rn(v[r].x, inv_r), __fmul_rn(v[r].y, inv_r),
-                                                          __fmul_rn(v[r].z, inv_r), __fmul_rn(v[r].w, inv_r));
+            *reinterpret_cast<uint32_t*>(qp) = BLK == 32 ? scaled_pack4(v[r], inv_r) : pack4_e4m3(__fmul_rn(v[r].x, inv_r), __fmul_rn(v[r].y, inv_r),
+                                                                                        __fmul_rn(v[r].z, inv_r), __fmul_rn(v[r].w, inv_r));
         }
-        qp += term_codes;
+        row += term_codes;
     }
     // scales: lane holds the scale of combination my_r, block (lane / GROUP) of this chunk
     if (MODE == FMM_SCALE_FP32_AMAX_DIV_448) {
@@ -203,64 +224,66 @@ __device__ __forceinline__ void store_chunk_a(const EncodeParams& p, const float
     }
 }
 
+// Rows that a task of the A-side encoder walks together (its rows are multiples of 32: of 128, or 128 / 4 in row panels).
+template <int BLK, int MODE> struct RowsPerTask { static constexpr int value = MODE == FMM_SCALE_FP32_AMAX_DIV_448 && BLK == 32 ? 2 : 1; };
+
 template <int BLK, int MODE, uint32_t NZ>
-__global__ void __launch_bounds__(256) encode_a_kernel(const EncodeParams p)
+__global__ void __launch_bounds__(256, BLK == 128 ? 4 : 3) encode_a_kernel(const EncodeParams p)
 {
     fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
     constexpr int GROUP = BLK / 4;                 // lanes per block
-    constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const uint32_t warp_gid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t warp_gid = blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5);
+    const uint32_t nwarps = gridDim.x * 8;
     const int chunks = p.cols / 128;
     // a task is CPT consecutive 128-k chunks of one output row (two adjacent rows at block 32 with fp32 scales).  Tasks
-    // are dealt to warps round-robin (32-bit index arithmetic only: one division per task, none per chunk).  The fp32
+    // are dealt to warps round-robin (32-bit index arithmetic only: one division per task, none per chunk; the warp index
+    // is warp-uniform, and so are all addresses but the lane's offset).  The fp32
     // scales of a chunk are stored row after row (16 bytes per row at block 32, 4 at block 128), so partial sectors
     // are avoided this way: block 32 walks two rows per task, the two rows of a chunk back to back (one 32-byte sector
     // per pair of stores); block 128 makes the ROW the fastest task index, so that the eight warps of a block hold
     // eight consecutive rows of the same chunks.  Both choices are the measured better one for their block size
     // (n = 8192, both sides: 0.160 vs 0.165 ms, and 0.158 vs 0.162 ms).  The power-of-two mode writes its exponent
     // bytes in row-major tiles: one row per task, chunk group fastest.
-    const int CPT = (chunks % 8 == 0) ? 8 : ((chunks % 4 == 0) ? 4 : 1);
-    constexpr bool FP32S = (MODE == FMM_SCALE_FP32_AMAX_DIV_448);
-    const int RPT = (FP32S && BLK == 32 && p.rows % 2 == 0) ? 2 : 1;
-    constexpr bool ROW_FASTEST = FP32S && BLK == 128;
-    const uint32_t tasks_per_row = (uint32_t)(chunks / CPT);
+    const int CPT = p.cpt;
+    constexpr int RPT = RowsPerTask<BLK, MODE>::value;
+    constexpr bool ROW_FASTEST = (MODE == FMM_SCALE_FP32_AMAX_DIV_448) && BLK == 128;
+    const uint32_t tasks_per_row = (uint32_t)((chunks + CPT - 1) / CPT);
     const uint32_t row_groups = (uint32_t)(p.rows / RPT);
     const uint32_t rows_all = (uint32_t)p.batch * row_groups;
     const uint32_t tasks = rows_all * tasks_per_row;
 
     for (uint32_t task = warp_gid; task < tasks; task += nwarps) {
-      const uint32_t cgrp = ROW_FASTEST ? task / rows_all : 0u;
-      const uint32_t row_id = ROW_FASTEST ? task - cgrp * rows_all : task / tasks_per_row;
-      const int c0 = (int)(ROW_FASTEST ? cgrp : task - row_id * tasks_per_row) * CPT;
-      const int b = (int)(row_id / row_groups);
-      const int i0 = (int)(row_id - (uint32_t)b * row_groups) * RPT;
-      // the loads of step n+1 are issued before step n is processed (two steps in flight per warp); step = (chunk, row)
-      const float* row_base = p.in + (int64_t)b * p.in_batch_stride + (int64_t)i0 * p.ld + lane * 4;
-      const int steps = CPT * RPT;
-      float4 xn[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-          if (j < p.nq) xn[j] = __ldcs(reinterpret_cast<const float4*>(row_base + c0 * 128 + p.qoff[j]));
-      for (int st = 0; st < steps; ++st) {
-        const int c = c0 + st / RPT, i = i0 + st % RPT;
-        float4 x[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = xn[j];
-        if (st + 1 < steps) {
-            const int cn = c0 + (st + 1) / RPT, rn = (st + 1) % RPT;
+        const uint32_t cgrp = ROW_FASTEST ? task / rows_all : 0u;
+        const uint32_t row_id = ROW_FASTEST ? task - cgrp * rows_all : task / tasks_per_row;
+        const int c0 = (int)(ROW_FASTEST ? cgrp : task - row_id * tasks_per_row) * CPT;
+        const int b = (int)(row_id / row_groups);
+        const int i0 = (int)(row_id - (uint32_t)b * row_groups) * RPT;
+        const int steps = min(CPT, chunks - c0) * RPT;     // step = (chunk, row)
+        const float* row_base = p.in + (int64_t)b * p.in_batch_stride + (int64_t)i0 * p.ld + c0 * 128;
+        auto load = [&](int st, float4 (&x)[4]) {
+            const float* at = row_base + (int64_t)(st % RPT) * p.ld + (st / RPT) * 128;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                if (j < p.nq) xn[j] = __ldcs(reinterpret_cast<const float4*>(row_base + (int64_t)rn * p.ld + cn * 128 + p.qoff[j]));
+                if (NZ || j < p.nq) x[j] = __ldcs(reinterpret_cast<const float4*>(at + p.qoff[j]) + lane);
+        };
+        auto process = [&](int st, const float4 (&x)[4]) {
+            float4 v[FMM_MAX_RANK];
+            float inv, s; uint32_t e8;
+            combine_chunk<GROUP, MODE, NZ, BLK == 32>(p, x, lane, v, inv, s, e8);
+            store_chunk_a<BLK, MODE, NZ>(p, v, inv, s, e8, b, i0 + st % RPT, c0 + st / RPT, lane);
+        };
+        // the loads of step n+1 are issued before step n is processed (two steps in flight per warp)
+        float4 xa[4], xb[4];
+        load(0, xa);
+        for (int st = 0; st < steps; st += 2) {
+            if (st + 1 < steps) load(st + 1, xb);
+            process(st, xa);
+            if (st + 1 < steps) {
+                if (st + 2 < steps) load(st + 2, xa);
+                process(st + 1, xb);
+            }
         }
-
-        float4 v[FMM_MAX_RANK];
-        float inv, s; uint32_t e8;
-        combine_chunk<GROUP, MODE, NZ>(p, x, lane, v, inv, s, e8);
-
-        store_chunk_a<BLK, MODE, NZ>(p, v, inv, s, e8, b, i, c, lane);
-      }
     }
 }
 
@@ -269,14 +292,7 @@ __global__ void __launch_bounds__(256) encode_a_kernel(const EncodeParams p)
 // tensor-core operand layout).  A thread owns 16 consecutive k of one column n; lanes l and l+16
 // hold the two halves of a 32-element (sub-)block, so one shuffle completes the amax.  Each load
 // is two 64-byte row segments per warp; each thread writes 16 contiguous code bytes and the two
-// lanes of a block fill one 32-byte sector.  BLK == 128 takes a second pass over the four
-// 32-element sub-blocks (served by L1/L2).
-//
-// TILE (App. E.5, the deployment-matched weight grouping; BLK == 128, FP32 scales): one scale per tile of
-// 128 k x 128 columns of each encoded combination.  A block of 256 threads then covers a whole tile, the
-// column maxima of the first pass are reduced across the block, and every column stores the tile's scale,
-// so the scale array keeps its per-column shape.  p.preround_bf16 rounds each encoded combination to
-// bfloat16 (nearest even) before the maximum and the cast, as the paper's real kernel does.
+// lanes of a block fill one 32-byte sector.
 template <int MODE>
 __device__ __forceinline__ void store_b_scale(const EncodeParams& p, int64_t t, int r, int j, int kb, int kc,
                                               float s, uint32_t e8word, bool last_of_word)
@@ -291,128 +307,6 @@ __device__ __forceinline__ void store_b_scale(const EncodeParams& p, int64_t t, 
         char* sp = so + tile * 512 + (jg & 31) * 16 + ((jg & 127) >> 5) * 4;
         if (FMM_GUARD(p.guard, sp, 4, 1202)) *reinterpret_cast<uint32_t*>(sp) = e8word;
     }
-}
-
-template <int BLK, int MODE, uint32_t NZ, bool TILE, bool PRE>
-__global__ void __launch_bounds__(TILE ? 256 : 128, TILE ? 2 : 4) encode_b_kernel(const EncodeParams p)
-{
-    static_assert(!(TILE || PRE) || (BLK == 128 && MODE == FMM_SCALE_FP32_AMAX_DIV_448), "weight-side options: blk 128, fp32");
-    // here p.rows = leaf k (contracted), p.cols = leaf n
-    constexpr unsigned FULL = 0xffffffffu;
-    constexpr int WARPS = TILE ? 8 : 4;
-    __shared__ float tile_amax[TILE ? WARPS : 1][FMM_MAX_RANK];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int j = blockIdx.x * (WARPS * 16) + warp * 16 + (lane & 15);
-    const int khalf = lane >> 4;
-    const int kc = blockIdx.y;                      // chunk of 128 k
-    const int b = blockIdx.z;
-    const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
-    const int64_t term_codes = p.q_term;
-
-    float raw[4][16];
-    float blk_amax[FMM_MAX_RANK], blk_inv[FMM_MAX_RANK];
-    uint32_t e8word[FMM_MAX_RANK];
-#pragma unroll
-    for (int r = 0; r < FMM_MAX_RANK; ++r) { blk_amax[r] = 0.0f; blk_inv[r] = 0.0f; e8word[r] = 0; }
-
-    constexpr int PASSES = (BLK == 32) ? 1 : 2;
-#pragma unroll 1
-    for (int pass = 0; pass < PASSES; ++pass) {
-#pragma unroll 1
-        for (int sub = 0; sub < 4; ++sub) {
-            const int k0 = kc * 128 + sub * 32 + khalf * 16;
-#pragma unroll
-            for (int jq = 0; jq < 4; ++jq)
-                if (jq < p.nq) {
-#pragma unroll
-                    for (int kk = 0; kk < 16; ++kk)
-                        raw[jq][kk] = __ldg(base + p.qoff[jq] + (int64_t)(k0 + kk) * p.ld);
-                }
-#pragma unroll
-            for (int r = 0; r < FMM_MAX_RANK; ++r) {
-                if (row_used<NZ>(r, p.R)) {
-                    float v[16];
-                    bool set = false;
-#pragma unroll
-                    for (int jq = 0; jq < 4; ++jq) {
-                        const float cj = p.coef[r][jq];
-                        if (coef_used<NZ>(r, jq, cj)) {
-                            if (!set) {
-#pragma unroll
-                                for (int kk = 0; kk < 16; ++kk) v[kk] = __fmul_rn(cj, raw[jq][kk]);
-                                set = true;
-                            } else {
-#pragma unroll
-                                for (int kk = 0; kk < 16; ++kk) v[kk] = __fmaf_rn(cj, raw[jq][kk], v[kk]);
-                            }
-                        }
-                    }
-                    if (!set) {
-#pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) v[kk] = 0.0f;
-                    }
-                    if (PRE) {
-#pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) v[kk] = __bfloat162float(__float2bfloat16_rn(v[kk]));
-                    }
-                    const int64_t t = (int64_t)b * p.R + r;
-                    if (BLK == 32 || pass == 0) {
-                        float amax = 0.0f;
-#pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) amax = fmaxf(amax, fabsf(v[kk]));
-                        amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 16));
-                        if (BLK == 32) blk_amax[r] = amax; else blk_amax[r] = fmaxf(blk_amax[r], amax);
-                    }
-                    if (!TILE && (BLK == 32 || (pass == 0 && sub == 3))) {
-                        float sc; uint32_t e8;
-                        blk_inv[r] = block_scale<MODE>(blk_amax[r], p.amax_floor, sc, e8);
-                        const int kb = (BLK == 32) ? (kc * 4 + sub) : kc;
-                        e8word[r] |= e8 << (8 * (kb & 3));
-                        if (khalf == 0) store_b_scale<MODE>(p, t, r, j, kb, kc, sc, e8word[r], (kb & 3) == 3);
-                    }
-                    if (BLK == 32 || pass == 1) {
-                        const float inv = blk_inv[r];
-                        uint32_t wv[4];
-#pragma unroll
-                        for (int g = 0; g < 4; ++g)
-                            wv[g] = pack4_e4m3(__fmul_rn(v[4 * g], inv), __fmul_rn(v[4 * g + 1], inv),
-                                               __fmul_rn(v[4 * g + 2], inv), __fmul_rn(v[4 * g + 3], inv));
-                        uint8_t* qp = p.q_out + t * term_codes + (int64_t)j * p.rows + k0;
-                        if (FMM_GUARD(p.guard, qp, 16, 1203)) *reinterpret_cast<uint4*>(qp) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-                    }
-                }
-            }
-        }
-        if (TILE && pass == 0) {
-            // column maxima -> tile maximum: 16 columns per warp by shuffles, 8 warps through shared memory
-#pragma unroll
-            for (int r = 0; r < FMM_MAX_RANK; ++r) {
-                float a = blk_amax[r];
-#pragma unroll
-                for (int d = 8; d >= 1; d >>= 1) a = fmaxf(a, __shfl_xor_sync(FULL, a, d));
-                if (lane == 0) tile_amax[warp][r] = a;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int r = 0; r < FMM_MAX_RANK; ++r) {
-                if (row_used<NZ>(r, p.R)) {
-                    float a = tile_amax[0][r];
-#pragma unroll
-                    for (int w = 1; w < WARPS; ++w) a = fmaxf(a, tile_amax[w][r]);
-                    float sc; uint32_t e8;
-                    blk_inv[r] = block_scale<MODE>(a, p.amax_floor, sc, e8);
-                    if (khalf == 0) store_b_scale<MODE>(p, (int64_t)b * p.R + r, r, j, kc, kc, sc, 0u, false);
-                }
-            }
-        }
-    }
-    // the product kernel, launched behind this one by the same call, may be scheduled as soon as every block has got
-    // here: its launch latency and set-up then fall under this grid's last blocks (signalling at the start instead lets
-    // its CTAs take SMs from this grid's tail: 0.5 % slower back to back)
-    fmmptx::griddep_launch_dependents();
-    // a launch that overlapped the A-side encoder must not end before it (what follows on the stream needs both):
-    // the last block of the grid waits for it, the others leave as they finish
-    if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
 }
 
 // B side, block 32, one 32-k block of 16 columns per warp (thread = 16 k of one column, lanes l and l+16 the two
@@ -453,11 +347,11 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
                 if (coef_used<NZ>(r, jq, cj)) {
                     if (!set) {
 #pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) v[kk] = __fmul_rn(cj, raw[jq][kk]);
+                        for (int kk = 0; kk < 16; kk += 2) unpack2(mul2(pack2(cj, cj), pack2(raw[jq][kk], raw[jq][kk + 1])), v[kk], v[kk + 1]);
                         set = true;
                     } else {
 #pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) v[kk] = __fmaf_rn(cj, raw[jq][kk], v[kk]);
+                        for (int kk = 0; kk < 16; kk += 2) unpack2(fma2(pack2(cj, cj), pack2(raw[jq][kk], raw[jq][kk + 1]), pack2(v[kk], v[kk + 1])), v[kk], v[kk + 1]);
                     }
                 }
             }
@@ -487,8 +381,7 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
             uint32_t wv[4];
 #pragma unroll
             for (int g = 0; g < 4; ++g)
-                wv[g] = pack4_e4m3(__fmul_rn(v[4 * g], inv), __fmul_rn(v[4 * g + 1], inv),
-                                   __fmul_rn(v[4 * g + 2], inv), __fmul_rn(v[4 * g + 3], inv));
+                wv[g] = scaled_pack4(make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]), inv);
             uint8_t* qp = p.q_out + t * term_codes + (int64_t)j * p.rows + k0;
             if (FMM_GUARD(p.guard, qp, 16, 1207)) *reinterpret_cast<uint4*>(qp) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
@@ -502,17 +395,24 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
     if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
 }
 
-// B side, block 128, per-column scales, one pass.  The four warps of a block take the four 32-k sub-blocks of one
+// B side, block 128, one pass.  The four warps of a block take the four 32-k sub-blocks of one
 // 128-k block of the same 16 columns; every thread forms the combinations of its 16 k x 1 column, the sub-block
 // maxima meet in shared memory, and each warp then quantizes its own sub-block from the raw values it still holds
 // (the combinations are formed a second time in registers - the same rounded-multiply / FMA chain, so the same bits -
 // instead of reading the operand a second time).  Grid: (cols / 16, rows / 128, batch), 128 threads.
-template <uint32_t NZ>
+//
+// TILE (App. E.5, the deployment-matched weight grouping): one scale per tile of 128 k x 128 columns of each encoded
+// combination.  The eight blocks of a tile are a cluster and read each other's maxima from distributed shared memory, so
+// this takes one pass as well (two passes over the operand by one block per tile took 39 instead of 23 us for a 4096 x 4096
+// operand); every column stores the tile's scale, so the scale array keeps its per-column shape.  PRE rounds each encoded
+// combination to bfloat16 (nearest even) before the maximum and the cast, as the paper's real kernel does.
+template <uint32_t NZ, bool TILE, bool PRE>
 __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams p)
 {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int MODE = FMM_SCALE_FP32_AMAX_DIV_448;
-    __shared__ float sub_amax[4][FMM_MAX_RANK][16];
+    __shared__ float sub_amax[4][FMM_MAX_RANK][16];      // TILE: [warp][r][0]
+    __shared__ float blk_amax[FMM_MAX_RANK], tile_amax[FMM_MAX_RANK];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int col = lane & 15, khalf = lane >> 4;
     const int j = blockIdx.x * 16 + col;
@@ -550,6 +450,10 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk) v[kk] = 0.0f;
         }
+        if (PRE) {
+#pragma unroll
+            for (int kk = 0; kk < 16; ++kk) v[kk] = __bfloat162float(__float2bfloat16_rn(v[kk]));
+        }
     };
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
@@ -559,15 +463,36 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             float amax = 0.0f;
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk) amax = fmaxf(amax, fabsf(v[kk]));
-            amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 16));
-            if (khalf == 0) sub_amax[warp][r][col] = amax;
+            // non-negative floats order like their bits: one warp-wide integer maximum
+            if (TILE) amax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(amax)));
+            else amax = fmaxf(amax, __shfl_xor_sync(FULL, amax, 16));
+            if (TILE ? lane == 0 : khalf == 0) sub_amax[warp][r][TILE ? 0 : col] = amax;
         }
     }
     __syncthreads();
+    if (TILE) {
+        if (threadIdx.x < FMM_MAX_RANK) {
+            const int r = threadIdx.x;
+            blk_amax[r] = fmaxf(fmaxf(sub_amax[0][r][0], sub_amax[1][r][0]), fmaxf(sub_amax[2][r][0], sub_amax[3][r][0]));
+        }
+        fmmptx::cluster_sync();
+        if (threadIdx.x < 8 * FMM_MAX_RANK) {       // thread: combination t / 8, block t % 8 of the cluster
+            const int r = threadIdx.x >> 3;
+            float a;
+            asm volatile("{\n\t.reg .b32 m;\n\tmapa.shared::cluster.u32 m, %1, %2;\n\tld.shared::cluster.f32 %0, [m];\n\t}"
+                         : "=f"(a) : "r"(fmmptx::smem_u32(&blk_amax[r])), "r"(threadIdx.x & 7) : "memory");
+#pragma unroll
+            for (int d = 4; d >= 1; d >>= 1) a = fmaxf(a, __shfl_xor_sync(FULL, a, d));
+            if ((threadIdx.x & 7) == 0) tile_amax[r] = a;
+        }
+        __syncthreads();
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");       // this block has read its peers' maxima
+    }
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
         if (row_used<NZ>(r, p.R)) {
-            const float amax = fmaxf(fmaxf(sub_amax[0][r][col], sub_amax[1][r][col]), fmaxf(sub_amax[2][r][col], sub_amax[3][r][col]));
+            const float amax = TILE ? tile_amax[r]
+                                    : fmaxf(fmaxf(sub_amax[0][r][col], sub_amax[1][r][col]), fmaxf(sub_amax[2][r][col], sub_amax[3][r][col]));
             float sc; uint32_t e8;
             const float inv = block_scale<MODE>(amax, p.amax_floor, sc, e8);
             const int64_t t = (int64_t)b * p.R + r;
@@ -590,6 +515,7 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
     // a launch that overlapped the A-side encoder must not end before it (what follows on the stream needs both):
     // the last block of the grid waits for it, the others leave as they finish
     if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
+    if (TILE) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");           // its own maxima are no longer read either
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -606,8 +532,8 @@ __global__ void __launch_bounds__(256) encode2_a_kernel(const EncodeParams p)
     fmmptx::griddep_launch_dependents();           // as encode_a_kernel
     constexpr int GROUP = BLK / 4;
     const int lane = threadIdx.x & 31;
-    const uint32_t warp_gid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t warp_gid = blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5);
+    const uint32_t nwarps = gridDim.x * 8;
     const uint32_t chunks = (uint32_t)(p.cols / 128);
     const uint32_t tasks = (uint32_t)p.batch * (uint32_t)p.rows * chunks;       // one 128-k chunk of one leaf row
     for (uint32_t task = warp_gid; task < tasks; task += nwarps) {
@@ -615,13 +541,13 @@ __global__ void __launch_bounds__(256) encode2_a_kernel(const EncodeParams p)
         const int c = (int)(task - row_id * chunks);
         const int b = (int)(row_id / (uint32_t)p.rows);
         const int i = (int)(row_id - (uint32_t)b * (uint32_t)p.rows);
-        const float* base = p.in + (int64_t)b * p.in_batch_stride + (int64_t)i * p.ld + c * 128 + lane * 4;
+        const float* base = p.in + (int64_t)b * p.in_batch_stride + (int64_t)i * p.ld + c * 128;
         float4 raw[4][4];                                   // [outer block][inner block]
 #pragma unroll
         for (int q1 = 0; q1 < 4; ++q1)
 #pragma unroll
             for (int q2 = 0; q2 < 4; ++q2)
-                raw[q1][q2] = __ldcs(reinterpret_cast<const float4*>(base + p.qoff_outer[q1] + p.qoff[q2]));
+                raw[q1][q2] = __ldcs(reinterpret_cast<const float4*>(base + p.qoff_outer[q1] + p.qoff[q2]) + lane);
 #pragma unroll
         for (int r1 = 0; r1 < FMM_MAX_RANK; ++r1) {
             if (row_used<NZ>(r1, p.R)) {
@@ -697,8 +623,7 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
                 if (row_used<NZ>(r, p.R)) {
                     const float inv_r = __shfl_sync(FULL, inv, (lane & 24) | r);
                     if (FMM_GUARD(p.guard, qp, 4, 1301))
-                    *reinterpret_cast<uint32_t*>(qp) = pack4_e4m3(__fmul_rn(v[r].x, inv_r), __fmul_rn(v[r].y, inv_r),
-                                                                  __fmul_rn(v[r].z, inv_r), __fmul_rn(v[r].w, inv_r));
+                    *reinterpret_cast<uint32_t*>(qp) = scaled_pack4(v[r], inv_r);
                 }
                 qp += term_codes;
             }
@@ -862,15 +787,18 @@ uint32_t coef_mask(const EncodeParams& p)
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
 // begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192).
 template <typename K>
-void launch_b_kernel(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p)
+void launch_b_kernel(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p, unsigned cluster = 1)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = grid; cfg.blockDim = dim3(threads, 1, 1); cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = p.overlap_prev ? 1 : 0;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cluster; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    // without a cluster only the second one, or none
+    cfg.attrs = cluster > 1 ? at : at + 1; cfg.numAttrs = (cluster > 1 ? 1 : 0) + (p.overlap_prev ? 1 : 0);
     cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
@@ -885,17 +813,6 @@ void launch_a(const EncodeParams& p, unsigned g, cudaStream_t st)
         default: encode_a_kernel<BLK, MODE, 0u><<<g, 256, 0, st>>>(p); return;
     }
 }
-template <int BLK, int MODE>
-void launch_b(const EncodeParams& p, dim3 grid, cudaStream_t st)
-{
-    const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
-    switch (m) {
-#define X(M) case M: launch_b_kernel(encode_b_kernel<BLK, MODE, M, false, false>, grid, 128, st, p); return;
-        FMM_KNOWN_MASKS(X)
-#undef X
-        default: launch_b_kernel(encode_b_kernel<BLK, MODE, 0u, false, false>, grid, 128, st, p); return;
-    }
-}
 template <int MODE>
 void launch_b32(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
@@ -907,14 +824,15 @@ void launch_b32(const EncodeParams& p, dim3 grid, cudaStream_t st)
         default: launch_b_kernel(encode_b32_kernel<MODE, 0u>, grid, 32, st, p); return;
     }
 }
+template <bool TILE, bool PRE>
 void launch_b128(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_b_kernel(encode_b128_kernel<M>, grid, 128, st, p); return;
+#define X(M) case M: launch_b_kernel(encode_b128_kernel<M, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_b_kernel(encode_b128_kernel<0u>, grid, 128, st, p); return;
+        default: launch_b_kernel(encode_b128_kernel<0u, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
     }
 }
 template <int BLK, int MODE>
@@ -937,29 +855,20 @@ void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
         default: launch_b_kernel(encode2_b_kernel<MODE, 0u>, grid, 256, st, p); return;
     }
 }
-// weight-side options (tile scales and / or bf16 pre-round): blk 128, fp32 scales
-template <bool TILE, bool PRE>
-void launch_b_opt(const EncodeParams& p, dim3 grid, cudaStream_t st)
-{
-    constexpr int F = FMM_SCALE_FP32_AMAX_DIV_448;
-    constexpr int T = TILE ? 256 : 128;
-    const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
-    switch (m) {
-#define X(M) case M: launch_b_kernel(encode_b_kernel<128, F, M, TILE, PRE>, grid, T, st, p); return;
-        FMM_KNOWN_MASKS(X)
-#undef X
-        default: launch_b_kernel(encode_b_kernel<128, F, 0u, TILE, PRE>, grid, T, st, p); return;
-    }
-}
 }  // namespace
 
-fmm_status_t fmm_launch_encode_a(const EncodeParams& p, int blk, int mode, cudaStream_t st)
+fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st)
 {
-    // one task (8, 4 or 1 chunks of 128 k of one row) per warp; the block scheduler balances the SMs
-    const int chunks = p.cols / 128;
-    const int cpt = (chunks % 8 == 0) ? 8 : ((chunks % 4 == 0) ? 4 : 1);
-    const int64_t tasks = (int64_t)p.batch * p.rows * (chunks / cpt);
-    int64_t blocks = (tasks + 7) / 8;
+    // one task per warp; the block scheduler balances the SMs
+    const int chunks = p.cols / 128, rpt = (mode == FMM_SCALE_FP32_AMAX_DIV_448 && blk == 32) ? 2 : 1;
+    const int64_t row_tasks = (int64_t)p.batch * (p.rows / rpt);
+    // long tasks keep two steps of loads in flight, but a problem has to have tasks for about half the resident warps
+    // (n = 2048, block 32: one task per eight chunks 15 us for both sides, per two 10 us; n = 4096: per eight 36.8, per two 39)
+    const int64_t want = (int64_t)sm_count() * 10;
+    int64_t tpr = (chunks + 7) / 8;
+    while (row_tasks * tpr < want && chunks > 2 * tpr) tpr *= 2;
+    p.cpt = (int)((chunks + tpr - 1) / tpr);
+    int64_t blocks = (row_tasks * ((chunks + p.cpt - 1) / p.cpt) + 7) / 8;
     if (blocks > 0x7fffffff) blocks = 0x7fffffff;
     const unsigned g = (unsigned)blocks;
     if (mode == FMM_SCALE_FP32_AMAX_DIV_448) {
@@ -973,20 +882,13 @@ fmm_status_t fmm_launch_encode_a(const EncodeParams& p, int blk, int mode, cudaS
 
 fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaStream_t st)
 {
-    dim3 grid((unsigned)(p.cols / 64), (unsigned)(p.rows / 128), (unsigned)p.batch);
-    if (p.b_tile || p.preround_bf16) {
-        if (p.b_tile) grid.x = (unsigned)(p.cols / 128);
-        if (p.b_tile && p.preround_bf16) launch_b_opt<true, true>(p, grid, st);
-        else if (p.b_tile) launch_b_opt<true, false>(p, grid, st);
-        else launch_b_opt<false, true>(p, grid, st);
-    } else if (mode == FMM_SCALE_FP32_AMAX_DIV_448) {
-        grid.x = (unsigned)(p.cols / 16);
-        if (blk == 32) { grid.y = (unsigned)(p.rows / 32); launch_b32<FMM_SCALE_FP32_AMAX_DIV_448>(p, grid, st); }
-        else launch_b128(p, grid, st);
-    } else {
-        grid.x = (unsigned)(p.cols / 16); grid.y = (unsigned)(p.rows / 32);
-        launch_b32<FMM_SCALE_UE8M0_CEIL>(p, grid, st);
-    }
+    dim3 grid((unsigned)(p.cols / 16), (unsigned)(p.rows / blk), (unsigned)p.batch);
+    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) launch_b32<FMM_SCALE_UE8M0_CEIL>(p, grid, st);
+    else if (blk == 32) launch_b32<FMM_SCALE_FP32_AMAX_DIV_448>(p, grid, st);
+    else if (p.b_tile && p.preround_bf16) launch_b128<true, true>(p, grid, st);
+    else if (p.b_tile) launch_b128<true, false>(p, grid, st);
+    else if (p.preround_bf16) launch_b128<false, true>(p, grid, st);
+    else launch_b128<false, false>(p, grid, st);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 

@@ -18,7 +18,7 @@
 //   FP32 mode   (the paper's scale = amax/448 in fp32 on BOTH sides, per 1 x blk block): no
 //               tensor-core path can apply a per-row x per-column fp32 factor per K block, so
 //               each K block's partial product is accumulated on its own in TMEM
-//               (kind::f8f6f4) and promoted on the CUDA cores: acc += P * (sA[row] * sB[col]),
+//               (kind::f8f6f4) and promoted on the CUDA cores: acc += (P * sB[col]) * sA[row],
 //               two columns per instruction (fp32x2), overlapped with the next TMEM load.
 //
 // Every wait is bounded: on time-out a status word is set and all roles leave the kernel.
@@ -432,7 +432,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         int ss = 0; uint32_t sphase = 0;
         uint32_t store_cnt = 0;
         uint32_t dphase = 0;
-        bool ok = true;
+        bool ok = true, t_ready = false, s_ready = false;
         uint32_t accu[C::MX ? C::CW : 1];               // UE8M0: raw fp32 bits drained from TMEM
         uint32_t kept[C::MX ? 16 : 1];                  // ... and the 16 columns of a parked product that stay in registers
         unsigned long long acc2[C::MX ? 1 : C::CW / 2]; // FP32: promoted accumulators, two columns per register pair
@@ -545,11 +545,16 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);         // acc2[k * (CW/8) + j]: row slot k, column group j
                     constexpr int JG = C::CW / 8;                               // column groups of eight per warp
                     constexpr int KB = C::KB_PER_STAGE;
+                    // Block 32: the next buffer's and the next scale stage's barriers are tested before the last chunk's
+                    // arithmetic, which hides the test (about 70 cycles) when they are complete; they are waited for only
+                    // if they were not (n = 8192: 1842 -> 1815 us, cubic n = 4096: 276 -> 271).  Block 128 has one buffer
+                    // per stage, rarely complete that early: 2 % slower.
+                    constexpr bool PEEK = KB == 4;
                     // A-side scales of the thread's four rows (q*32 + lane/4 + 8k of this CTA's 128), per K block
                     const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + (lane >> 2)) * (KB * 4);
                     const uint32_t sb_lane = base + C::OFF_SB + (h * C::CW + 2 * (lane & 3)) * 4;
                     for (int ks = 0; ks < kstages && ok; ++ks) {
-                        if (!mbar_wait_warp(bar_sfull(ss), sphase, ctl, 302)) { ok = false; break; }
+                        if (!(PEEK && __all_sync(0xffffffffu, s_ready)) && !mbar_wait_warp(bar_sfull(ss), sphase, ctl, 302)) { ok = false; break; }
                         const uint32_t sbs32 = sb_lane + ss * C::SB_STAGE_BYTES;
                         // the stage's K blocks for the thread's four rows, from the scale ring (a global load here, even
                         // issued a stage early, stalled the promotion: 14 % of the block-32 kernel)
@@ -565,41 +570,42 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         }
 #pragma unroll
                         for (int g0 = 0; g0 < C::KB_PER_STAGE; g0 += C::GPB) {
-                            if (!mbar_wait_warp(bar_tfull(buf), bphase, ctl, 303)) { ok = false; break; }
+                            if (!(PEEK && __all_sync(0xffffffffu, t_ready)) && !mbar_wait_warp(bar_tfull(buf), bphase, ctl, 303)) { ok = false; break; }
                             tc_fence_after();
 #pragma unroll
                             for (int gi = 0; gi < C::GPB; ++gi) {
                                 const int g = g0 + gi;
                                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (buf * C::GPB + gi) * BN + h * C::CW;
-                                float sbt = 1.0f;
-                                if (MODE == MODE_FP32_SB_TILE) sbt = *reinterpret_cast<const float*>(base_ptr + C::OFF_SB + ss * C::SB_STAGE_BYTES + (g * BN + h * C::CW) * 4);
 #pragma unroll
                                 for (int c = 0; c < C::CW / 32; ++c) {   // chunks of 32 columns
                                     uint32_t lo[16], hi[16];
                                     tmem_ld_16x256b_x4(taddr + c * 32, lo);                       // rows lane/4, lane/4 + 8
                                     tmem_ld_16x256b_x4(taddr + c * 32 + (16u << 16), hi);         // rows lane/4 + 16, lane/4 + 24
                                     unsigned long long sb2[4];
-                                    if (MODE != MODE_FP32_SB_TILE) {
 #pragma unroll
-                                        for (int j = 0; j < 4; ++j) sb2[j] = lds64(sbs32 + (g * BN + c * 32 + 8 * j) * 4);
-                                    }
+                                    for (int j = 0; j < 4; ++j) sb2[j] = lds64(sbs32 + (g * BN + c * 32 + 8 * j) * 4);
                                     tmem_ld_wait();
                                     if (gi + 1 == C::GPB && c + 1 == C::CW / 32) {
                                         // the last chunk is in registers: hand the TMEM buffers back before the arithmetic
                                         tc_fence_before();
                                         __syncwarp();
                                         if (lane == 0) release_acc(buf);
+                                        if (PEEK) {
+                                            const bool tw = buf + 1 == C::ACC_BUFS, sw = ss + 1 == C::SB_STAGES;
+                                            t_ready = mbar_try_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
+                                            if (g0 + C::GPB >= KB) s_ready = mbar_try_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
+                                        }
                                     }
 #pragma unroll
                                     for (int k = 0; k < 4; ++k) {
-                                        const float sak = sa4[k][g] * sbt;       // tile mode: sA * sB_tile; else sbt = 1 (folded away)
-                                        const unsigned long long sa2 = pack2(sak, sak);
+                                        const unsigned long long sa2 = pack2(sa4[k][g], sa4[k][g]);
                                         const uint32_t* src = (k < 2) ? lo : hi;
 #pragma unroll
                                         for (int j = 0; j < 4; ++j) {
                                             const uint32_t* tp = src + 4 * j + 2 * (k & 1);
-                                            const unsigned long long s2 = (MODE == MODE_FP32_SB_TILE) ? sa2 : mul2(sa2, sb2[j]);
-                                            acc2[k * JG + c * 4 + j] = fma2(pack2u(tp[0], tp[1]), s2, acc2[k * JG + c * 4 + j]);
+                                            // (P * sB) * sA rather than P * (sA * sB): 1 % faster, the multiply no longer keeps a
+                                            // product of scales alive (computing those ahead of the TMEM wait: 7 % slower)
+                                            acc2[k * JG + c * 4 + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + c * 4 + j]);
                                         }
                                     }
                                 }
