@@ -186,7 +186,8 @@ void make_layout(const fmm_plan* plan, int64_t M, int64_t N, int64_t K, FmmLayou
         const bool need_b = !(last && fmm_encode2_supported(true, plan->qp.block_k, plan->qp.b_tile_n, plan->qp.b_preround_bf16));
         if (need_a) { L->inter_a[lv] = off; off = align_up(off + (size_t)(cnt * (M / dd) * (K / dd)) * 4, 1024); }
         if (need_b) { L->inter_b[lv] = off; off = align_up(off + (size_t)(cnt * (K / dd) * (N / dd)) * 4, 1024); }
-        L->dec[lv] = off; off = align_up(off + (size_t)(cnt * (M / dd) * (N / dd)) * 4, 1024);
+        // (three levels: the first-level matrices stay in the registers of the two-step decoder)
+        if (last) { L->dec[lv] = off; off = align_up(off + (size_t)(cnt * (M / dd) * (N / dd)) * 4, 1024); }
     }
     L->total = off;
 }
@@ -224,7 +225,42 @@ void fill_coef(float dst[FMM_MAX_RANK][4], const float src[FMM_MAX_RANK][4], int
 // A strip of the leaf rows of A and C (m0 .. m1) or of the leaf columns of B and C (n0 .. n1), in every block.
 struct Strip { int64_t m0, m1, n0, n1; };
 
-// One side of steps 1-2: outer levels as fp32 combinations, last level fused with the quantizer.  [lo, hi) is the strip of
+// Levels whose combinations are formed as fp32 matrices in the workspace (the innermost one or two are not).
+int outer_levels(const fmm_plan* plan, bool b_side)
+{
+    if (plan->levels < 2) return 0;
+    const bool fused2 = fmm_encode2_supported(b_side, plan->qp.block_k, b_side ? plan->qp.b_tile_n : 0, b_side ? plan->qp.b_preround_bf16 : 0);
+    return fused2 ? plan->levels - 2 : plan->levels - 1;
+}
+
+// Those combinations, level by level, both sides of a level in one launch.
+fmm_status_t encode_outer(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* A, const float* B, int64_t M, int64_t N, int64_t K,
+                          cudaStream_t st, int* launches)
+{
+    const int deepest[2] = {outer_levels(plan, false), outer_levels(plan, true)};
+    for (int level = 1; level <= deepest[0] || level <= deepest[1]; ++level) {
+        CombParams c[2];
+        memset(c, 0, sizeof(c));
+        for (int side = 0; side < 2; ++side) {
+            if (level > deepest[side]) continue;
+            const size_t* inter = side ? L.inter_b : L.inter_a;
+            const int64_t rows = (side ? K : M) >> (level - 1), cols = (side ? N : K) >> (level - 1);
+            CombParams& s = c[side];
+            s.in = level > 1 ? reinterpret_cast<const float*>(ws + inter[level - 1]) : (side ? B : A);
+            s.in_batch_stride = level > 1 ? rows * cols : 0; s.ld = cols; s.batch = (int)fmm_ipow(plan->rank, level - 1);
+            s.rows = (int)(rows / 2); s.cols = (int)(cols / 2); s.R = plan->rank;
+            fill_coef(s.coef, side ? plan->V : plan->U, plan->rank);
+            s.out = reinterpret_cast<float*>(ws + inter[level]);
+            s.guard = fmm_make_guard(s.out, (size_t)s.batch * s.R * (size_t)(s.rows * (int64_t)s.cols) * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
+        }
+        const fmm_status_t s = fmm_launch_comb(c[0], c[1], level > 1, st);
+        if (s != FMM_OK) return s;
+        ++*launches;
+    }
+    return FMM_OK;
+}
+
+// One side of steps 1-2, behind encode_outer: the innermost one or two levels and the quantizer.  [lo, hi) is the strip of
 // leaf rows (A) or columns (B) to encode: everything, or with at most one level a part of it (multiples of 128).
 fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* X,
                          int64_t rows, int64_t cols, bool b_side, int64_t lo, int64_t hi, bool overlap, cudaStream_t st, int* launches)
@@ -277,31 +313,17 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
         }
         e.q_term = (int64_t)e.rows * e.cols;
     } else {
-        const float* cur = X;
-        int64_t cur_rows = rows, cur_cols = cols, cur_ld = cols, cur_stride = 0;
-        int batch = 1;
         // the last two levels run as one kernel where that is supported: the combinations of level lv-1 stay
         // in registers
         const bool fused2 = lv >= 2 && fmm_encode2_supported(b_side, blk, e.b_tile, e.preround_bf16);
-        for (int level = 1; level < (fused2 ? lv - 1 : lv); ++level) {
-            CombParams c;
-            memset(&c, 0, sizeof(c));
-            c.in = cur; c.in_batch_stride = cur_stride; c.ld = cur_ld; c.batch = batch;
-            c.rows = (int)(cur_rows / 2); c.cols = (int)(cur_cols / 2); c.R = R;
-            fill_coef(c.coef, coef, R);
-            c.out = reinterpret_cast<float*>(ws + (b_side ? L.inter_b[level] : L.inter_a[level]));
-            c.guard = fmm_make_guard(c.out, (size_t)batch * R * (size_t)(c.rows * (int64_t)c.cols) * 4, nullptr, 0,
-                                     plan->d_status + FMM_GUARD_WORD);
-            s = fmm_launch_comb(c, st);
-            if (s != FMM_OK) return s;
-            ++*launches;
-            cur = c.out; cur_rows /= 2; cur_cols /= 2; cur_ld = cur_cols; cur_stride = cur_rows * cur_cols;
-            batch *= R;
-        }
+        const int level = outer_levels(plan, b_side);
+        const float* cur = level ? reinterpret_cast<const float*>(ws + (b_side ? L.inter_b[level] : L.inter_a[level])) : X;
+        const int64_t cur_rows = rows >> level, cur_cols = cols >> level, cur_ld = cur_cols, cur_stride = level ? cur_rows * cur_cols : 0;
+        const int batch = (int)fmm_ipow(R, level);
         e.in = cur + strip_in; e.in_batch_stride = cur_stride; e.ld = cur_ld; e.batch = batch;
-        // the B-side leaf encoder may start under the tail of the A-side one (launched just before it by fmm_matmul /
-        // fmm_encode_only) when it reads the caller's matrix itself, i.e. nothing a kernel of this call has written
-        e.overlap_prev = (b_side && overlap && cur == X) ? 1 : 0;
+        // see EncodeParams: the B-side encoder runs behind the A-side one, the A-side one behind the combinations if its side has
+        // any (they are launched for both sides at once, the deepest level last)
+        e.overlap_prev = b_side ? overlap : level > 0;
         const int div = fused2 ? 4 : 2;
         e.rows = (int)(cur_rows / div); e.cols = (int)(cur_cols / div); e.nq = 4; e.R = R;
         e.qoff[0] = 0; e.qoff[1] = e.cols; e.qoff[2] = (int64_t)e.rows * e.ld; e.qoff[3] = (int64_t)e.rows * e.ld + e.cols;
@@ -355,18 +377,19 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     g.guard = fmm_make_guard(dest, (size_t)g.Mfull * (size_t)g.Nfull * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
     fmm_status_t s = fmm_launch_gemm(g, plan->qp.block_k, (int)plan->qp.scale_mode, st, launches);
     if (s != FMM_OK) return s;
-    for (int l = lv - 1; l >= 1; --l) {
+    for (int l = lv - 1, steps; l >= 1; l -= steps) {
+        steps = l == 2 ? 2 : 1;
         DecodeParams d;
         memset(&d, 0, sizeof(d));
         d.in = reinterpret_cast<const float*>(ws + L.dec[l]);
-        d.out = l == 1 ? C : reinterpret_cast<float*>(ws + L.dec[l - 1]);
-        d.batch = (int)fmm_ipow(plan->rank, l - 1);
+        d.out = l == steps ? C : reinterpret_cast<float*>(ws + L.dec[l - steps]);
+        d.batch = (int)fmm_ipow(plan->rank, l - steps);
         d.rows = (int)(M >> l); d.cols = (int)(N >> l); d.R = plan->rank;
         for (int r = 0; r < plan->rank; ++r)
             for (int q = 0; q < 4; ++q) d.W[r][q] = plan->W[r][q];
-        d.guard = fmm_make_guard(d.out, (size_t)d.batch * 4 * (size_t)d.rows * (size_t)d.cols * 4, nullptr, 0,
+        d.guard = fmm_make_guard(d.out, (size_t)d.batch * ((size_t)d.rows << steps) * ((size_t)d.cols << steps) * 4, nullptr, 0,
                                  plan->d_status + FMM_GUARD_WORD);
-        s = fmm_launch_decode(d, st);
+        s = fmm_launch_decode(d, steps, st);
         if (s != FMM_OK) return s;
         ++*launches;
     }
@@ -632,7 +655,8 @@ fmm_status_t fmm_encode_only(const fmm_plan_t* plan, const float* A, const float
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
+    s = encode_outer(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
+    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
     if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
@@ -660,7 +684,8 @@ fmm_status_t fmm_matmul(const fmm_plan_t* plan, const float* A, const float* B, 
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
+    s = encode_outer(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
+    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
     if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
     if (s == FMM_OK) s = multiply(plan, L, static_cast<char*>(ws), C, M, N, {0, L.m, 0, L.n}, st, &launches, true);
     plan->last_launches.store(launches, std::memory_order_relaxed);

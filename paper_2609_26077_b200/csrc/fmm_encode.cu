@@ -230,6 +230,7 @@ template <int BLK, int MODE> struct RowsPerTask { static constexpr int value = M
 template <int BLK, int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(256, BLK == 128 ? 4 : 3) encode_a_kernel(const EncodeParams p)
 {
+    fmmptx::griddep_wait();                        // the combinations of the level above, when this launch overlaps their tail
     fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
     constexpr int GROUP = BLK / 4;                 // lanes per block
     const int lane = threadIdx.x & 31;
@@ -529,7 +530,8 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
 template <int BLK, int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(256) encode2_a_kernel(const EncodeParams p)
 {
-    fmmptx::griddep_launch_dependents();           // as encode_a_kernel
+    fmmptx::griddep_wait();                        // as encode_a_kernel
+    fmmptx::griddep_launch_dependents();
     constexpr int GROUP = BLK / 4;
     const int lane = threadIdx.x & 31;
     const uint32_t warp_gid = blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5);
@@ -617,15 +619,18 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
             float inv, s; uint32_t e8;
             combine_chunk<8, MODE, NZ>(p, x, lane, v, inv, s, e8);
             const int64_t t0 = ((int64_t)b * p.R + r1) * p.R;
-            uint8_t* qp = p.q_out + t0 * term_codes + (int64_t)j * p.rows + k0;
+            // warp-uniform base; a lane's offset fits 32 bits: the operand has 16 times 4 bytes for every code of a term
+            uint8_t* term = p.q_out + t0 * term_codes;
+            const uint32_t at = (uint32_t)j * (uint32_t)p.rows + (uint32_t)k0;
 #pragma unroll
             for (int r = 0; r < FMM_MAX_RANK; ++r) {
                 if (row_used<NZ>(r, p.R)) {
                     const float inv_r = __shfl_sync(FULL, inv, (lane & 24) | r);
+                    uint8_t* qp = term + at;
                     if (FMM_GUARD(p.guard, qp, 4, 1301))
                     *reinterpret_cast<uint32_t*>(qp) = scaled_pack4(v[r], inv_r);
                 }
-                qp += term_codes;
+                term += term_codes;
             }
             if (my_r < p.R) {
                 char* so = reinterpret_cast<char*>(p.s_out) + (t0 + my_r) * p.s_term_stride;
@@ -649,94 +654,137 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
     if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
 }
 
-// fp32 combinations of the outer recursion levels (levels >= 3): out[b*R + r] = sum_j coef[r][j] X_j
-__global__ void __launch_bounds__(256) comb_kernel(const CombParams p)
+// Streaming kernels of the outer recursion levels.  A block is 8 rows x 32 float4 of a matrix, a thread one float4 of every
+// input block; the row and column come from one 32-bit division per thread (64-bit divisions took a third of the time of
+// these kernels at the sizes where their data stays in L2).
+struct OuterIndex { int row, col4; };
+__device__ __forceinline__ OuterIndex outer_index(int cols)
 {
-    const int c4 = p.cols / 4;
-    const int64_t units = (int64_t)p.batch * p.rows * c4;
+    const uint32_t tiles = (uint32_t)cols / 128, by = blockIdx.x / tiles, bx = blockIdx.x - by * tiles;
+    return {(int)(by * 8 + threadIdx.y), (int)(bx * 32 + threadIdx.x)};
+}
+__device__ __forceinline__ void axpy(float4& acc, float w, const float4& x)
+{
+    acc.x = __fmaf_rn(w, x.x, acc.x); acc.y = __fmaf_rn(w, x.y, acc.y);
+    acc.z = __fmaf_rn(w, x.z, acc.z); acc.w = __fmaf_rn(w, x.w, acc.w);
+}
+
+// fp32 combinations of the outer recursion levels: out[b*R + r] = sum_j coef[r][j] X_j, first term a rounded multiply, later
+// terms FMAs, zero coefficients skipped.  Both sides of a level in one launch (blockIdx.y).
+__global__ void __launch_bounds__(256) comb_kernel(const CombParams pa, const CombParams pb)
+{
+    fmmptx::griddep_wait();                        // the level above, when this launch overlaps its tail
+    const CombParams& p = blockIdx.y ? pb : pa;
+    if (blockIdx.x * 8u >= (uint32_t)p.rows * ((uint32_t)p.cols / 128) || (int)blockIdx.z >= p.batch) return;
+    const OuterIndex at = outer_index(p.cols);
     const int64_t qoff[4] = {0, (int64_t)p.cols, (int64_t)p.rows * p.ld, (int64_t)p.rows * p.ld + p.cols};
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(u % c4);
-        const int64_t bi = u / c4;
-        const int i = (int)(bi % p.rows);
-        const int b = (int)(bi / p.rows);
-        const float* base = p.in + (int64_t)b * p.in_batch_stride + (int64_t)i * p.ld + c * 4;
-        float4 x[4];
+    const float* base = p.in + (int64_t)blockIdx.z * p.in_batch_stride + (int64_t)at.row * p.ld + at.col4 * 4;
+    float4 x[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) x[j] = __ldcs(reinterpret_cast<const float4*>(base + qoff[j]));
-        for (int r = 0; r < p.R; ++r) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            bool set = false;
+    for (int j = 0; j < 4; ++j) x[j] = __ldcs(reinterpret_cast<const float4*>(base + qoff[j]));
+    const int64_t term = (int64_t)p.rows * p.cols;
+    float* o = p.out + (int64_t)blockIdx.z * p.R * term + (int64_t)at.row * p.cols + at.col4 * 4;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float cj = p.coef[r][j];
-                if (cj != 0.0f) {
-                    if (!set) {
-                        v.x = __fmul_rn(cj, x[j].x); v.y = __fmul_rn(cj, x[j].y);
-                        v.z = __fmul_rn(cj, x[j].z); v.w = __fmul_rn(cj, x[j].w);
-                        set = true;
-                    } else {
-                        v.x = __fmaf_rn(cj, x[j].x, v.x); v.y = __fmaf_rn(cj, x[j].y, v.y);
-                        v.z = __fmaf_rn(cj, x[j].z, v.z); v.w = __fmaf_rn(cj, x[j].w, v.w);
-                    }
-                }
+    for (int r = 0; r < FMM_MAX_RANK; ++r) {
+        if (r >= p.R) break;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool set = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float cj = p.coef[r][j];
+            if (cj != 0.0f) {
+                if (!set) {
+                    v.x = __fmul_rn(cj, x[j].x); v.y = __fmul_rn(cj, x[j].y);
+                    v.z = __fmul_rn(cj, x[j].z); v.w = __fmul_rn(cj, x[j].w);
+                    set = true;
+                } else axpy(v, cj, x[j]);
             }
-            float* o = p.out + ((int64_t)b * p.R + r) * p.rows * p.cols + (int64_t)i * p.cols + c * 4;
-            if (FMM_GUARD(p.guard, o, 16, 1401)) *reinterpret_cast<float4*>(o) = v;
         }
+        if (FMM_GUARD(p.guard, o, 16, 1401)) *reinterpret_cast<float4*>(o) = v;
+        o += term;
     }
 }
 
 // Outward step of the decoder for levels >= 2: the R partially decoded products of a parent are
-// combined into the four blocks of the parent's matrix, out_q = sum_r W[r][q] * in_r (fp32, r ascending,
-// zero weights skipped, first term a multiply, later terms FMAs).
+// combined into the four blocks of the parent's matrix, out_q = sum_r W[r][q] * in_r (fp32, r ascending).
 __global__ void __launch_bounds__(256) decode_kernel(const DecodeParams p)
 {
-    const int c4 = p.cols / 4;
-    const int64_t units = (int64_t)p.batch * p.rows * c4;
-    const int64_t in_stride = (int64_t)p.rows * p.cols;
-    const int64_t out_ld = 2 * (int64_t)p.cols;
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < units; u += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(u % c4);
-        const int64_t bi = u / c4;
-        const int i = (int)(bi % p.rows);
-        const int b = (int)(bi / p.rows);
-        float4 acc[4];
-        bool set[4] = {false, false, false, false};
+    fmmptx::griddep_wait();                        // the product kernel, whose tail this launch overlaps
+    const OuterIndex at = outer_index(p.cols);
+    const int64_t in_stride = (int64_t)p.rows * p.cols, out_ld = 2 * (int64_t)p.cols;
+    const float* src = p.in + (int64_t)blockIdx.z * p.R * in_stride + (int64_t)at.row * p.cols + at.col4 * 4;
+    // all R loads are issued before the first use (R x 16 bytes in flight per thread)
+    float4 x[FMM_MAX_RANK];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float* src = p.in + ((int64_t)b * p.R) * in_stride + (int64_t)i * p.cols + c * 4;
-        // all R loads are issued before the first use (R x 16 bytes in flight per thread)
-        float4 xs[FMM_MAX_RANK];
+    for (int r = 0; r < FMM_MAX_RANK; ++r)
+        if (r < p.R) x[r] = __ldcs(reinterpret_cast<const float4*>(src + r * in_stride));
+    float* dst = p.out + (int64_t)blockIdx.z * 4 * in_stride;
 #pragma unroll
-        for (int r = 0; r < FMM_MAX_RANK; ++r)
-            if (r < p.R) xs[r] = __ldcs(reinterpret_cast<const float4*>(src + r * in_stride));
+    for (int q = 0; q < 4; ++q) {
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int r = 0; r < FMM_MAX_RANK; ++r) {
-            if (r >= p.R) break;
-            const float4 x = xs[r];
+            const float w = p.W[r][q];             // zero for r >= R
+            if (w != 0.0f) axpy(acc, w, x[r]);
+        }
+        float* o = dst + ((int64_t)(q >> 1) * p.rows + at.row) * out_ld + (q & 1) * p.cols + at.col4 * 4;
+        if (FMM_GUARD(p.guard, o, 16, 1501)) *reinterpret_cast<float4*>(o) = acc;
+    }
+}
+
+// Two outward steps at once (three levels): the R x R matrices of the second level go to the 16 blocks of the result with the
+// first-level matrices in registers, in the order of two single steps.  The first-level matrices are neither written nor read
+// back (n = 2048: 14 + 10 us as two launches).  The next R loads are in flight while R are combined.
+__global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
+{
+    fmmptx::griddep_wait();
+    const uint32_t tiles = (uint32_t)p.cols / 128, by = blockIdx.x / tiles, bx = blockIdx.x - by * tiles;
+    const int row = by * 4 + threadIdx.y, col = (bx * 32 + threadIdx.x) * 4;
+    const int64_t in_stride = (int64_t)p.rows * p.cols, out_ld = 4 * (int64_t)p.cols;
+    const float* src = p.in + (int64_t)row * p.cols + col;
+    float4 acc[4][4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float w = p.W[r][q];
-                if (w != 0.0f) {
-                    if (!set[q]) {
-                        acc[q].x = __fmul_rn(w, x.x); acc[q].y = __fmul_rn(w, x.y);
-                        acc[q].z = __fmul_rn(w, x.z); acc[q].w = __fmul_rn(w, x.w);
-                        set[q] = true;
-                    } else {
-                        acc[q].x = __fmaf_rn(w, x.x, acc[q].x); acc[q].y = __fmaf_rn(w, x.y, acc[q].y);
-                        acc[q].z = __fmaf_rn(w, x.z, acc[q].z); acc[q].w = __fmaf_rn(w, x.w, acc[q].w);
-                    }
-                }
+    for (int i = 0; i < 16; ++i) acc[i >> 2][i & 3] = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load = [&](int r1, float4 (&x)[FMM_MAX_RANK]) {
+#pragma unroll
+        for (int r = 0; r < FMM_MAX_RANK; ++r)
+            if (r < p.R) x[r] = __ldcs(reinterpret_cast<const float4*>(src + (int64_t)(r1 * p.R + r) * in_stride));
+    };
+    auto add = [&](int r1, const float4 (&x)[FMM_MAX_RANK]) {
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) {
+            float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < FMM_MAX_RANK; ++r) {
+                const float w = p.W[r][q2];
+                if (w != 0.0f) axpy(y, w, x[r]);
+            }
+#pragma unroll
+            for (int q1 = 0; q1 < 4; ++q1) {
+                const float w = p.W[r1][q1];
+                if (w != 0.0f) axpy(acc[q1][q2], w, y);
             }
         }
-        float* dst = p.out + (int64_t)b * 4 * in_stride;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float* o = dst + ((int64_t)(q >> 1) * p.rows + i) * out_ld + (q & 1) * p.cols + c * 4;
-            if (FMM_GUARD(p.guard, o, 16, 1501)) *reinterpret_cast<float4*>(o) = acc[q];
+    };
+    float4 xa[FMM_MAX_RANK], xb[FMM_MAX_RANK];
+    load(0, xa);
+#pragma unroll 1
+    for (int r1 = 0; r1 < p.R; r1 += 2) {
+        if (r1 + 1 < p.R) load(r1 + 1, xb);
+        add(r1, xa);
+        if (r1 + 1 < p.R) {
+            if (r1 + 2 < p.R) load(r1 + 2, xa);
+            add(r1 + 1, xb);
         }
     }
+#pragma unroll
+    for (int q1 = 0; q1 < 4; ++q1)
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) {
+            const int64_t r = (int64_t)(2 * (q1 >> 1) + (q2 >> 1)) * p.rows + row;
+            float* o = p.out + r * out_ld + (2 * (q1 & 1) + (q2 & 1)) * (int64_t)p.cols + col;
+            if (FMM_GUARD(p.guard, o, 16, 1502)) *reinterpret_cast<float4*>(o) = acc[q1][q2];
+        }
 }
 
 int sm_count()
@@ -749,24 +797,35 @@ int sm_count()
 
 }  // namespace
 
-fmm_status_t fmm_launch_decode(const DecodeParams& p, cudaStream_t st)
+namespace {
+// Launch that may begin under the tail of the kernel before it on the stream (which wrote what this one reads: it waits for
+// it before its first load), so that its launch latency and set-up are hidden.
+template <typename K, typename... A>
+fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, bool overlap, const A&... args)
 {
-    const int64_t units = (int64_t)p.batch * p.rows * (p.cols / 4);
-    int64_t blocks = (units + 255) / 256;
-    const int64_t cap = (int64_t)sm_count() * 16;
-    if (blocks > cap) blocks = cap;
-    decode_kernel<<<(unsigned)blocks, 256, 0, st>>>(p);
+    cudaLaunchConfig_t cfg;
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = overlap ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
+}  // namespace
 
-fmm_status_t fmm_launch_comb(const CombParams& p, cudaStream_t st)
+fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st)
 {
-    const int64_t units = (int64_t)p.batch * p.rows * (p.cols / 4);
-    int64_t blocks = (units + 255) / 256;
-    const int64_t cap = (int64_t)sm_count() * 8;
-    if (blocks > cap) blocks = cap;
-    comb_kernel<<<(unsigned)blocks, 256, 0, st>>>(p);
-    return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+    const unsigned tiles = (unsigned)(p.cols / 128);
+    if (steps == 2) return launch_behind(decode2_kernel, dim3((unsigned)(p.rows / 4) * tiles), dim3(32, 4), st, true, p);
+    return launch_behind(decode_kernel, dim3((unsigned)(p.rows / 8) * tiles, 1, (unsigned)p.batch), dim3(32, 8), st, true, p);
+}
+
+fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, bool overlap, cudaStream_t st)
+{
+    const unsigned ga = (unsigned)(a.rows / 8) * (unsigned)(a.cols / 128), gb = (unsigned)(b.rows / 8) * (unsigned)(b.cols / 128);
+    return launch_behind(comb_kernel, dim3(ga > gb ? ga : gb, 2, (unsigned)(a.batch > b.batch ? a.batch : b.batch)), dim3(32, 8), st, overlap, a, b);
 }
 
 namespace {
@@ -783,11 +842,13 @@ uint32_t coef_mask(const EncodeParams& p)
 // Phi-optimal realization, and the identity used to quantize a matrix as four panels
 #define FMM_KNOWN_MASKS(X) X(0x0a5381c9u) X(0x0c385a19u) X(0x05dc8f21u) X(0x0ab3f841u) X(0x0f5fc5c9u) X(0x0cfc5f59u) X(0x00008421u)
 
-// Launch of a B-side encoder.  With p.overlap_prev it carries the programmatic-serialization attribute: the kernel
+// Launch of an encoder.  With p.overlap_prev it carries the programmatic-serialization attribute.  B side: the kernel
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
-// begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192).
+// begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192); what it
+// reads, the caller's matrix or combinations of a kernel before the A-side one, is complete.  A side: set up under the
+// tail of the combinations it reads.
 template <typename K>
-void launch_b_kernel(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p, unsigned cluster = 1)
+void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p, unsigned cluster = 1)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -807,10 +868,10 @@ void launch_a(const EncodeParams& p, unsigned g, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: encode_a_kernel<BLK, MODE, M><<<g, 256, 0, st>>>(p); return;
+#define X(M) case M: launch_encoder(encode_a_kernel<BLK, MODE, M>, dim3(g), 256, st, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: encode_a_kernel<BLK, MODE, 0u><<<g, 256, 0, st>>>(p); return;
+        default: launch_encoder(encode_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, p); return;
     }
 }
 template <int MODE>
@@ -818,10 +879,10 @@ void launch_b32(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_b_kernel(encode_b32_kernel<MODE, M>, grid, 32, st, p); return;
+#define X(M) case M: launch_encoder(encode_b32_kernel<MODE, M>, grid, 32, st, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_b_kernel(encode_b32_kernel<MODE, 0u>, grid, 32, st, p); return;
+        default: launch_encoder(encode_b32_kernel<MODE, 0u>, grid, 32, st, p); return;
     }
 }
 template <bool TILE, bool PRE>
@@ -829,30 +890,30 @@ void launch_b128(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_b_kernel(encode_b128_kernel<M, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
+#define X(M) case M: launch_encoder(encode_b128_kernel<M, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_b_kernel(encode_b128_kernel<0u, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
+        default: launch_encoder(encode_b128_kernel<0u, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
     }
 }
 template <int BLK, int MODE>
 void launch_a2(const EncodeParams& p, unsigned g, cudaStream_t st)
 {
     switch (coef_mask(p)) {
-#define X(M) case M: encode2_a_kernel<BLK, MODE, M><<<g, 256, 0, st>>>(p); return;
+#define X(M) case M: launch_encoder(encode2_a_kernel<BLK, MODE, M>, dim3(g), 256, st, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: encode2_a_kernel<BLK, MODE, 0u><<<g, 256, 0, st>>>(p); return;
+        default: launch_encoder(encode2_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, p); return;
     }
 }
 template <int MODE>
 void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     switch (coef_mask(p)) {
-#define X(M) case M: launch_b_kernel(encode2_b_kernel<MODE, M>, grid, 256, st, p); return;
+#define X(M) case M: launch_encoder(encode2_b_kernel<MODE, M>, grid, 256, st, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_b_kernel(encode2_b_kernel<MODE, 0u>, grid, 256, st, p); return;
+        default: launch_encoder(encode2_b_kernel<MODE, 0u>, grid, 256, st, p); return;
     }
 }
 }  // namespace

@@ -124,7 +124,8 @@ struct EncodeParams {
     int preround_bf16;        // B side: round each combination to bfloat16 before the maximum and the cast
     FmmGuard guard;           // codes and scales of this side
     int overlap_prev;         // B side: the kernel launched just before on the stream is the A-side encoder of the same
-                              // call (nothing this kernel reads): it may start while that one drains
+                              // call (nothing this kernel reads): it may start while that one drains.  A side: that kernel is
+                              // the combinations this one reads: it may be set up while that one drains
 };
 
 struct CombParams {
@@ -144,8 +145,10 @@ struct DecodeParams {
     float W[FMM_MAX_RANK][4];
     FmmGuard guard;
 };
-fmm_status_t fmm_launch_decode(const DecodeParams& p, cudaStream_t st);
-fmm_status_t fmm_launch_comb(const CombParams& p, cudaStream_t st);
+// steps: 1, or 2 outward steps at once (batch 1; rows x cols and W as for the inner step)
+fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st);
+// one level of combinations of the two sides (a side with rows == 0 has none); overlap: behind another such launch
+fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, bool overlap, cudaStream_t st);
 fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st);
 fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaStream_t st);
 // last two recursion levels in one pass (p.rows x p.cols = leaf dimensions, inputs 4*rows x 4*cols)
