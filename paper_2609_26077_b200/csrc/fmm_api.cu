@@ -8,7 +8,7 @@
 #include <vector>
 #include "fmm_internal.h"
 
-constexpr int HOST_STRIPS = 8;
+constexpr int HOST_STRIPS = 9;
 
 // Side streams and events of one fmm_matmul_host call in flight.
 struct HostLane {
@@ -726,33 +726,48 @@ fmm_status_t fmm_host_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t
     return FMM_OK;
 }
 
-// One cudaMemcpyAsync per leaf block row / column of a strip: rows lo .. hi (whole rows), or columns lo .. hi, of each of the
-// `blocks` leaf blocks of a rows x cols matrix.
+// The strip [lo, hi) of the rows (columns) of each of the `blocks` leaf blocks of a rows x cols matrix, as one copy.
 static bool copy_strip(float* dst, const float* src, int64_t rows, int64_t cols, int blocks, bool by_rows, int64_t lo, int64_t hi,
                        cudaMemcpyKind kind, cudaStream_t st)
 {
+    if (by_rows) {
+        // a "row" of this copy is the strip's rows of one block, which are contiguous
+        const size_t pitch = (size_t)(rows / blocks) * (size_t)cols * 4, width = (size_t)((hi - lo) * cols) * 4;
+        const int64_t at = lo * cols;
+        if (blocks == 1 || pitch > 0x7fffffff) {
+            for (int b = 0; b < blocks; ++b)
+                if (cudaMemcpyAsync(dst + b * (int64_t)(pitch / 4) + at, src + b * (int64_t)(pitch / 4) + at, width, kind, st) != cudaSuccess) { cudaGetLastError(); return false; }
+        } else if (cudaMemcpy2DAsync(dst + at, pitch, src + at, pitch, width, (size_t)blocks, kind, st) != cudaSuccess) { cudaGetLastError(); return false; }
+        return true;
+    }
     for (int b = 0; b < blocks; ++b) {
-        cudaError_t e;
-        if (by_rows) {
-            const int64_t at = (b * (rows / blocks) + lo) * cols;
-            e = cudaMemcpyAsync(dst + at, src + at, (size_t)((hi - lo) * cols) * 4, kind, st);
-        } else {
-            const int64_t at = b * (cols / blocks) + lo;
-            e = cudaMemcpy2DAsync(dst + at, (size_t)cols * 4, src + at, (size_t)cols * 4, (size_t)(hi - lo) * 4, (size_t)rows, kind, st);
-        }
-        if (e != cudaSuccess) { cudaGetLastError(); return false; }
+        const int64_t at = b * (cols / blocks) + lo;
+        if (cudaMemcpy2DAsync(dst + at, (size_t)cols * 4, src + at, (size_t)cols * 4, (size_t)(hi - lo) * 4, (size_t)rows, kind, st) != cudaSuccess) { cudaGetLastError(); return false; }
     }
     return true;
+}
+
+// Borders of the strips in sixteenths of the leaf extent.  A copy costs about 12 us besides its bytes while the link is used
+// both ways, so strips are few where the upload bounds the call and more where the download, which cannot begin before the
+// first strip has been multiplied, does too (n = 4096: nine 2.93 ms, five 3.10; 8192 x 1024 x 2048: 1.77 and 1.63).  The first
+// is short to start the download, the last short because its products and download follow the upload.
+static const int* strip_borders(int64_t upload, int64_t download, int* count)
+{
+    static const int nine[] = {0, 2, 4, 6, 8, 10, 12, 14, 15, 16}, five[] = {0, 2, 6, 10, 14, 16}, four[] = {0, 8, 12, 14, 16}, two[] = {0, 8, 16};
+    if (upload >= (32 << 20) && 5 * download > 3 * upload) { *count = 9; return nine; }
+    if (upload >= (32 << 20)) { *count = 5; return five; }
+    if (upload >= (12 << 20)) { *count = 4; return four; }
+    *count = upload >= (8 << 20) ? 2 : 1;
+    return two;
 }
 
 // Host operands, at most one level: the transfers bound the call (n = 4096: 134 MB up at 55 GB/s = 2.4 ms, 67 MB down, against
 // 0.33 ms of kernels), and the link is full duplex.  So the smaller operand goes up first, the larger one in strips of leaf
 // rows (A) or columns (B); a strip is encoded and multiplied on one side stream while the next one is on its way, and its part
 // of C goes down on another while later strips still come up.  What remains beside the upload is the last strip's kernels
-// and download.  Strips of at least 4 MB (75 us), at most 8, cut at 256 rows / columns so that a strip has the tiles of
-// the whole product: the results are the same bits.
+// and download.  A strip is computed by the kernel that the whole product would take, so the results are the same bits.
 static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* A, const float* B, float* C,
-                                       float* dA, float* dB, float* dC, int64_t M, int64_t N, int64_t K, int strips, bool by_rows,
+                                       float* dA, float* dB, float* dC, int64_t M, int64_t N, int64_t K, int strips, const int* borders, bool by_rows,
                                        HostLane& lane, cudaStream_t st)
 {
     const int blocks = 1 << plan->levels;
@@ -768,13 +783,14 @@ static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L,
         const bool ok = sig(lane.done[0], lane.comp, st) && sig(lane.done[1], lane.down, st);
         return s == FMM_OK && !ok ? FMM_ERR_CUDA : s;
     };
-    const int64_t ext = by_rows ? L.m : L.n, gran = ext % 256 == 0 ? 256 : 128, units = ext / gran;
+    const int64_t units = (by_rows ? L.m : L.n) / 128;
     if (cudaMemcpyAsync(by_rows ? dB : dA, by_rows ? B : A, (size_t)(by_rows ? K * N : M * K) * 4, up, st) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
     if (!sig(lane.up[strips], st, lane.comp)) return join(FMM_ERR_CUDA);
     fmm_status_t s = by_rows ? encode_side(plan, L, ws, dB, K, N, true, 0, L.n, false, lane.comp, &launches)
                              : encode_side(plan, L, ws, dA, M, K, false, 0, L.m, false, lane.comp, &launches);
     for (int i = 0; i < strips && s == FMM_OK; ++i) {
-        const int64_t lo = units * i / strips * gran, hi = units * (i + 1) / strips * gran;
+        const int64_t lo = units * borders[i] / 16 * 128, hi = units * borders[i + 1] / 16 * 128;
+        if (lo == hi) continue;
         Strip part = {0, L.m, 0, L.n};
         if (by_rows) { part.m0 = lo; part.m1 = hi; } else { part.n0 = lo; part.n1 = hi; }
         if (!copy_strip(by_rows ? dA : dB, by_rows ? A : B, by_rows ? M : K, by_rows ? K : N, blocks, by_rows, lo, hi, up, st) ||
@@ -808,10 +824,9 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
         s = check_ws(plan, M, N, K, ws, inner, &L);
         if (s != FMM_OK) return s;
         const bool by_rows = M >= N;                         // the larger operand of the two
-        const int64_t ext = by_rows ? L.m : L.n, bytes = (by_rows ? M : N) * K * 4;
-        int64_t strips = bytes / (4 << 20);
-        if (strips > HOST_STRIPS) strips = HOST_STRIPS;
-        if (strips > ext / (ext % 256 == 0 ? 256 : 128)) strips = ext / (ext % 256 == 0 ? 256 : 128);
+        int strips = 1;
+        const int* borders = strip_borders((by_rows ? M : N) * K * 4, M * N * 4, &strips);
+        if ((by_rows ? L.m : L.n) < 256) strips = 1;
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
         // pageable copies block the host in order, so they would gain nothing from the strips
         auto pinned = [](const void* p) {
@@ -821,7 +836,7 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
         if (strips > 1 && pinned(A) && pinned(B) && pinned(C) && cudaStreamIsCapturing(st, &capture) == cudaSuccess &&
             capture == cudaStreamCaptureStatusNone) {
             if (HostLane* lane = plan->lanes->acquire()) {
-                s = matmul_host_strips(plan, L, base, A, B, C, dA, dB, dC, M, N, K, (int)strips, by_rows, *lane, st);
+                s = matmul_host_strips(plan, L, base, A, B, C, dA, dB, dC, M, N, K, strips, borders, by_rows, *lane, st);
                 plan->lanes->release(lane);
                 return s;
             }

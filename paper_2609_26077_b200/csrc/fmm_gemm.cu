@@ -575,36 +575,63 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             for (int gi = 0; gi < C::GPB; ++gi) {
                                 const int g = g0 + gi;
                                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (buf * C::GPB + gi) * BN + h * C::CW;
-#pragma unroll
-                                for (int c = 0; c < C::CW / 32; ++c) {   // chunks of 32 columns
-                                    uint32_t lo[16], hi[16];
-                                    tmem_ld_16x256b_x4(taddr + c * 32, lo);                       // rows lane/4, lane/4 + 8
-                                    tmem_ld_16x256b_x4(taddr + c * 32 + (16u << 16), hi);         // rows lane/4 + 16, lane/4 + 24
-                                    unsigned long long sb2[4];
-#pragma unroll
-                                    for (int j = 0; j < 4; ++j) sb2[j] = lds64(sbs32 + (g * BN + c * 32 + 8 * j) * 4);
-                                    tmem_ld_wait();
-                                    if (gi + 1 == C::GPB && c + 1 == C::CW / 32) {
-                                        // the last chunk is in registers: hand the TMEM buffers back before the arithmetic
-                                        tc_fence_before();
-                                        __syncwarp();
-                                        if (lane == 0) release_acc(buf);
-                                        if (PEEK) {
-                                            const bool tw = buf + 1 == C::ACC_BUFS, sw = ss + 1 == C::SB_STAGES;
-                                            t_ready = mbar_try_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
-                                            if (g0 + C::GPB >= KB) s_ready = mbar_try_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
-                                        }
+                                // the last chunk is in registers: hand the TMEM buffers back before the arithmetic
+                                auto release = [&]() {
+                                    tc_fence_before();
+                                    __syncwarp();
+                                    if (lane == 0) release_acc(buf);
+                                    if (PEEK) {
+                                        const bool tw = buf + 1 == C::ACC_BUFS, sw = ss + 1 == C::SB_STAGES;
+                                        t_ready = mbar_try_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
+                                        if (g0 + C::GPB >= KB) s_ready = mbar_try_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
                                     }
+                                };
+                                // (P * sB) * sA rather than P * (sA * sB): 1 % faster, the multiply no longer keeps a
+                                // product of scales alive (computing those ahead of the TMEM wait: 7 % slower)
+                                if constexpr (C::CW == 64) {
+                                    // two chunks of 16 rows x 64 columns, the second one's load under the first one's arithmetic
+                                    // (1.5 % of the cubic product at n = 4096 against chunks of 32 x 32 without the overlap)
+                                    uint32_t lo[32], hi[32];
+                                    unsigned long long sb2[8];
+                                    tmem_ld_16x256b_x8(taddr, lo);                        // rows lane/4, lane/4 + 8
+#pragma unroll
+                                    for (int j = 0; j < 8; ++j) sb2[j] = lds64(sbs32 + (g * BN + 8 * j) * 4);
+                                    tmem_ld_wait();
+                                    tmem_ld_16x256b_x8(taddr + (16u << 16), hi);          // rows lane/4 + 16, lane/4 + 24
 #pragma unroll
                                     for (int k = 0; k < 4; ++k) {
+                                        if (k == 2) {
+                                            tmem_ld_wait();
+                                            if (gi + 1 == C::GPB) release();
+                                        }
                                         const unsigned long long sa2 = pack2(sa4[k][g], sa4[k][g]);
                                         const uint32_t* src = (k < 2) ? lo : hi;
 #pragma unroll
-                                        for (int j = 0; j < 4; ++j) {
+                                        for (int j = 0; j < 8; ++j) {
                                             const uint32_t* tp = src + 4 * j + 2 * (k & 1);
-                                            // (P * sB) * sA rather than P * (sA * sB): 1 % faster, the multiply no longer keeps a
-                                            // product of scales alive (computing those ahead of the TMEM wait: 7 % slower)
-                                            acc2[k * JG + c * 4 + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + c * 4 + j]);
+                                            acc2[k * JG + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + j]);
+                                        }
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int c = 0; c < C::CW / 32; ++c) {   // chunks of 32 columns
+                                        uint32_t lo[16], hi[16];
+                                        tmem_ld_16x256b_x4(taddr + c * 32, lo);                       // rows lane/4, lane/4 + 8
+                                        tmem_ld_16x256b_x4(taddr + c * 32 + (16u << 16), hi);         // rows lane/4 + 16, lane/4 + 24
+                                        unsigned long long sb2[4];
+#pragma unroll
+                                        for (int j = 0; j < 4; ++j) sb2[j] = lds64(sbs32 + (g * BN + c * 32 + 8 * j) * 4);
+                                        tmem_ld_wait();
+                                        if (gi + 1 == C::GPB && c + 1 == C::CW / 32) release();
+#pragma unroll
+                                        for (int k = 0; k < 4; ++k) {
+                                            const unsigned long long sa2 = pack2(sa4[k][g], sa4[k][g]);
+                                            const uint32_t* src = (k < 2) ? lo : hi;
+#pragma unroll
+                                            for (int j = 0; j < 4; ++j) {
+                                                const uint32_t* tp = src + 4 * j + 2 * (k & 1);
+                                                acc2[k * JG + c * 4 + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + c * 4 + j]);
+                                            }
                                         }
                                     }
                                 }
@@ -861,19 +888,19 @@ fmm_status_t launch_shape(const GemmParams& g, cudaStream_t st)
             // the output warp it runs as fast as with 256-column tiles and none, 0.81 ms at n = 8192, and the cubic
             // product, which has a single store per tile, is 20 % slower.)
             if (g.k / BK >= 16) {
-                if ((g.m % 256) == 0) return launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st);
+                if ((g.msub % 256) == 0) return launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st);
                 return launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
             }
         }
         if constexpr (BLK == 128) {
             // one promotion per 128 k: 256-column tiles with two TMEM accumulators
-            if ((g.m % 256) == 0 && (g.n % 256) == 0) return launch<256, MODE, BLK, 2>(g, st);
+            if ((g.msub % 256) == 0 && (g.nsub % 256) == 0) return launch<256, MODE, BLK, 2>(g, st);
         }
-        if ((g.m % 256) == 0) return launch<128, MODE, BLK, 2>(g, st);
+        if ((g.msub % 256) == 0) return launch<128, MODE, BLK, 2>(g, st);
         return launch<128, MODE, BLK, 1>(g, st);
     } else {
-        if ((g.m % 256) == 0 && (g.n % 256) == 0) return launch<256, MODE, 32, 2>(g, st);
-        if ((g.n % 256) == 0) return launch<256, MODE, 32, 1>(g, st);
+        if ((g.msub % 256) == 0 && (g.nsub % 256) == 0) return launch<256, MODE, 32, 2>(g, st);
+        if ((g.nsub % 256) == 0) return launch<256, MODE, 32, 1>(g, st);
         return launch<128, MODE, 32, 1>(g, st);
     }
 }

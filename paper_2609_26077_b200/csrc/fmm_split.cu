@@ -275,8 +275,8 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 const uint32_t* tp = src + 4 * j + 2 * (k & 1);
-                                const unsigned long long s2 = (MODE == MODE_FP32_SB_TILE) ? sa2 : mul2(sa2, sb2[j]);
-                                acc2[k * JG + c * 4 + j] = fma2(pack2u(tp[0], tp[1]), s2, acc2[k * JG + c * 4 + j]);
+                                const unsigned long long v = pack2u(tp[0], tp[1]);
+                                acc2[k * JG + c * 4 + j] = fma2((MODE == MODE_FP32_SB_TILE) ? v : mul2(v, sb2[j]), sa2, acc2[k * JG + c * 4 + j]);
                             }
                         }
                     }
@@ -442,16 +442,16 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
 }
 
 // Time models of the two product kernels in microseconds, fitted to measurements of both at leaves of 128 to 4096 in every
-// direction and zero to three levels (34 shapes of rank 7 and 13 cubic ones per mode; the choice they give loses 1 % on
-// the better of the two in the mean).  The persistent kernel needs R * (k * c + o) per wave of tile positions: c per stage
+// direction and zero to three levels (35 shapes of rank 7 and 13 cubic ones per mode; the choice they give loses 0.5 to 2 %
+// on the better of the two in the mean).  The persistent kernel needs R * (k * c + o) per wave of tile positions: c per stage
 // of 128 k, o per term for the chain from the first load to the output; CTA pairs and single CTAs have their own.  The
 // cluster kernel needs lat + (f + k * c) per wave of clusters, f being set-up, exchange and output (f_alone without an
 // exchange).  So it takes the products of few tiles, whatever their K: leaves of 128 to 1024 (block 32) or 1536 (else).
 struct SplitModel { float c_pair, o_pair, c_one, o_one, f, c, f_alone, lat; };
-constexpr SplitModel SPLIT_MX = {0.36f, 3.95f, 0.27f, 2.6f, 3.8f, 0.40f, 4.5f, 1.2f};
-constexpr SplitModel SPLIT_B32 = {0.80f, 5.95f, 0.74f, 4.8f, 3.8f, 2.00f, 3.9f, 1.9f};
-constexpr SplitModel SPLIT_B128 = {0.68f, 6.6f, 0.42f, 3.35f, 4.5f, 0.75f, 4.05f, 1.85f};
-constexpr SplitModel SPLIT_TILE = {0.37f, 6.45f, 0.33f, 3.6f, 4.0f, 0.84f, 3.8f, 1.9f};
+constexpr SplitModel SPLIT_MX = {0.37f, 4.05f, 0.40f, 1.9f, 3.3f, 0.73f, 3.9f, 0.65f};
+constexpr SplitModel SPLIT_B32 = {0.80f, 5.8f, 0.75f, 4.15f, 3.7f, 2.15f, 4.25f, 1.25f};
+constexpr SplitModel SPLIT_B128 = {0.68f, 3.9f, 0.47f, 2.4f, 3.9f, 0.65f, 4.3f, 1.9f};
+constexpr SplitModel SPLIT_TILE = {0.36f, 4.75f, 0.33f, 3.05f, 4.1f, 0.68f, 3.9f, 1.4f};
 
 template <int MODE, int BLK>
 int choose_split(const GemmParams& g, const SplitModel& m, int pair_bn, int one_bn)
