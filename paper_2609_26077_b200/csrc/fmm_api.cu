@@ -151,87 +151,6 @@ void choose_walk(int R, const float (*W)[4], int* order, float* carry)
     for (int i = 1; i < R; ++i) carry[i] = ratio[order[i - 1]][order[i]];
 }
 
-// The same for the UE8M0 kernel, whose sums stay in TMEM, where only adding and subtracting products is free (the carries are
-// 0, 1 or -1), and whose epilogue sends two sums as one update (parked: first of a pair; odd R: one sum is sent alone, at
-// any place).  Sums, pairs and their order are chosen together: fewest block updates over all walks, by a dynamic programme
-// over (products used, product that begins the next unit).  11 -> 9 updates for the Phi-optimal realization, 9 -> 7 for
-// Strassen, 9 -> 6 for the Winograd form against pairs of single products.
-void choose_pairs(int R, const float (*W)[4], int* order, float* carry, bool* parked)
-{
-    constexpr int END = FMM_MAX_RANK;                // "no next product"
-    // blocks fed by the sum that ends in a when the next product, b, carries it with factor c - 1
-    unsigned char mask[FMM_MAX_RANK][FMM_MAX_RANK + 1][3];
-    auto bits = [](int m) { return (m & 1) + ((m >> 1) & 1) + ((m >> 2) & 1) + ((m >> 3) & 1); };
-    for (int a = 0; a < R; ++a)
-        for (int b = 0; b <= END; ++b)
-            for (int c = 0; c < 3; ++c) {
-                int m = 0;
-                for (int q = 0; q < 4; ++q)
-                    if ((b < R ? emitted_weight(W[a][q], (float)(c - 1), W[b][q]) : W[a][q]) != 0.0f) m |= 1 << q;
-                mask[a][b][c] = (unsigned char)m;
-            }
-    // best carry into b (b == END: none) for a sum that ends in a and is sent with the blocks `with`
-    auto one = [&](int a, int b, int with, int& c) {
-        int best = 9;
-        for (int k : {1, 0, 2}) { const int n = bits(mask[a][b][k] | with); if (n < best && (b != END || k == 1)) { best = n; c = k; } }
-        return best;
-    };
-    auto two = [&](int a, int b, int next, int& ca, int& cb) {
-        int best = 9;
-        for (int k : {1, 0, 2}) { int c = 1; const int n = one(b, next, mask[a][b][k], c); if (n < best) { best = n; ca = k; cb = c; } }
-        return best;
-    };
-    struct State { short cost; signed char prev_next, kind; short prev_set; };      // kind: 1 single, 2 pair (its second product)
-    std::vector<State> dp((size_t)(1 << R) * 2 * (END + 1), State{999, -1, 0, 0});
-    auto at = [&](int set, int single, int next) -> State& { return dp[((size_t)set * 2 + single) * (END + 1) + next]; };
-    const int full = (1 << R) - 1;
-    for (int n = 0; n < R; ++n) at(0, 0, n).cost = 0;
-    std::vector<signed char> via((size_t)(1 << R) * 2 * (END + 1), -1);              // second product of the pair that led here
-    for (int set = 0; set < full; ++set)
-        for (int single = 0; single < 2; ++single)
-            for (int a = 0; a < R; ++a) {
-                if ((set & (1 << a)) || at(set, single, a).cost >= 999) continue;
-                const int cost = at(set, single, a).cost;
-                auto relax = [&](int nset, int nsingle, int next, int add, int kind, int b) {
-                    if (next == END ? nset != full : (nset >> next) & 1) return;
-                    State& s = at(nset, nsingle, next);
-                    if (cost + add < s.cost) {
-                        s = State{(short)(cost + add), (signed char)a, (signed char)kind, (short)(set * 2 + single)};
-                        via[((size_t)nset * 2 + nsingle) * (END + 1) + next] = (signed char)b;
-                    }
-                };
-                int c, c2;
-                if ((R & 1) && !single)
-                    for (int next = 0; next <= END; ++next)
-                        if (next < R || next == END) relax(set | (1 << a), 1, next, one(a, next, 0, c), 1, -1);
-                for (int b = 0; b < R; ++b) {
-                    if (b == a || (set & (1 << b))) continue;
-                    for (int next = 0; next <= END; ++next)
-                        if (next < R || next == END) relax(set | (1 << a) | (1 << b), single, next, two(a, b, next, c, c2), 2, b);
-                }
-            }
-    // walk back from the end
-    int set = full, single = R & 1, next = END, pos = R;
-    for (int i = 0; i < FMM_MAX_RANK; ++i) { carry[i] = 0.0f; parked[i] = false; }
-    while (pos > 0) {
-        const State s = at(set, single, next);
-        const int a = s.prev_next, b = via[((size_t)set * 2 + single) * (END + 1) + next];
-        int c = 1, c2 = 1;
-        if (s.kind == 1) {
-            one(a, next, 0, c);
-            if (pos < R) carry[pos] = (float)(c - 1);
-            order[--pos] = a;
-        } else {
-            two(a, b, next, c, c2);
-            if (pos < R) carry[pos] = (float)(c2 - 1);
-            order[--pos] = b; carry[pos] = (float)(c - 1);
-            order[--pos] = a; parked[pos] = true;
-        }
-        next = a; set = s.prev_set >> 1; single = s.prev_set & 1;
-    }
-    carry[0] = 0.0f;
-}
-
 fmm_status_t check_shape(const fmm_plan* plan, int64_t M, int64_t N, int64_t K)
 {
     if (M <= 0 || N <= 0 || K <= 0) return FMM_ERR_SHAPE;
@@ -449,7 +368,9 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     g.msub = (int)(strip.m1 - strip.m0); g.nsub = (int)(strip.n1 - strip.n0);
     g.m = (int)L.m; g.n = (int)L.n; g.k = (int)L.k; g.terms = (int)L.terms;
     g.terms_per_group = plan->levels >= 2 ? plan->rank : (int)L.terms;
-    g.walk = plan->d_walk; g.out = plan->d_out; g.pair = plan->d_pair; g.status = plan->d_status;
+    g.walk = plan->d_walk; g.out = plan->d_out; g.status = plan->d_status;
+    g.pair_start = plan->d_pair_start; g.pair = plan->d_pair; g.steps = plan->steps;
+    for (int r = 0; r < FMM_MAX_RANK; ++r) g.order[r] = plan->order[r];
     g.device = plan->device; g.sms = plan->sms;
     g.R = lv >= 1 ? plan->rank : 1; g.nq = lv >= 1 ? 4 : 1; g.W = plan->W;
     g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0;
@@ -560,56 +481,113 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
             for (int j = 0; j < 4; ++j) { p->U[r][j] = U[r * 4 + j]; p->V[r][j] = V[r * 4 + j]; p->W[r][j] = W[r * 4 + j]; }
     p->terms = (int)fmm_ipow(rank, levels);
 
-    // Walk and decoder table of the product kernel (Sec. 2.1 decode, innermost level; outer levels are decoded afterwards).
-    // row_off / col_off are in units of leaf blocks inside the stack of parent matrices.
-    const bool e8 = qp->scale_mode == FMM_SCALE_UE8M0_CEIL;
-    int order[FMM_MAX_RANK] = {0};
-    float carry[FMM_MAX_RANK] = {0.0f};          // UE8M0: -1, 0 or 1, see choose_pairs
-    bool parked[FMM_MAX_RANK] = {false};
-    if (levels >= 1) { if (e8) choose_pairs(rank, p->W, order, carry, parked); else choose_walk(rank, p->W, order, carry); }
+    // Walk and decoder table of the fp32-scale product kernel (Sec. 2.1 decode, innermost level; outer levels are decoded
+    // afterwards).  row_off / col_off are in units of leaf blocks inside the stack of parent matrices.
+    int walk_order[FMM_MAX_RANK] = {0};
+    float walk_carry[FMM_MAX_RANK] = {0.0f};
+    if (levels >= 1) choose_walk(rank, p->W, walk_order, walk_carry);
     std::vector<FmmWalkEntry> walk(p->terms);
     std::vector<FmmOutEntry> entries;
-    std::vector<FmmPairEntry> pairs;
     const int parents = levels >= 1 ? p->terms / rank : 1;
-    for (int parent = 0; parent < parents; ++parent) {
-        bool touched[4] = {false};
-        float sign = 1.0f, before[4] = {0.0f};   // UE8M0: the accumulators hold sign * S; weights of the parked sum
-        for (int s = 0; s < rank; ++s) {
-            const int r = order[s];
-            FmmWalkEntry& we = walk[parent * rank + s];
-            we.term = parent * rank + r;
-            // UE8M0: T_s = T_(s-1) + x * M_s with T = sign * S and S_s = M_s + carry * S_(s-1)  =>  x = carry * sign
-            we.carry = e8 ? carry[s] * sign : carry[s];
-            if (e8) sign = carry[s] == 0.0f ? 1.0f : sign * carry[s];
-            we.out0 = (int)(e8 ? pairs.size() : entries.size());
-            for (int q = 0; q < 4; ++q) {
-                float w = levels == 0 ? (q == 0 ? 1.0f : 0.0f) : p->W[r][q];
-                if (s + 1 < rank) w = emitted_weight(w, carry[s + 1], p->W[order[s + 1]][q]);
-                if (e8) w *= sign;
-                if (parked[s]) { before[q] = w; continue; }
-                const float wA = (s > 0 && parked[s - 1]) ? before[q] : 0.0f;
-                if (w == 0.0f && wA == 0.0f) continue;
-                const int row = parent * 2 + (q >> 1), col = q & 1, first = touched[q] ? 0 : 1;
-                if (e8) pairs.push_back({row, col, wA, w, first});
-                else entries.push_back({row, col, w, first});
-                touched[q] = true;
-            }
-            we.out1 = (int)(e8 ? pairs.size() : entries.size());
+    std::vector<char> touched((size_t)parents * 4, 0);
+    for (int t = 0; t < p->terms; ++t) {
+        walk[t].out0 = walk[t].out1 = (int)entries.size();
+        if (levels == 0) {
+            FmmOutEntry e; e.row_off = 0; e.col_off = 0; e.w = 1.0f; e.first = 1;
+            entries.push_back(e);
+            walk[t].term = 0; walk[t].carry = 0.0f; walk[t].out1 = 1;
+            continue;
         }
+        const int parent = t / rank, s = t % rank, r = walk_order[s];
+        walk[t].term = parent * rank + r; walk[t].carry = walk_carry[s];
+        for (int q = 0; q < 4; ++q) {
+            const float w = s + 1 < rank ? emitted_weight(p->W[r][q], walk_carry[s + 1], p->W[walk_order[s + 1]][q]) : p->W[r][q];
+            if (w == 0.0f) continue;
+            FmmOutEntry e;
+            e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.w = w;
+            e.first = touched[(size_t)parent * 4 + q] ? 0 : 1;
+            touched[(size_t)parent * 4 + q] = 1;
+            entries.push_back(e);
+        }
+        walk[t].out1 = (int)entries.size();
     }
+
+    // Pair-fused decoder: pair up the R products of a parent so that the pairs' unions of destination blocks are as
+    // small as possible in total (exhaustive over the matchings: R <= 8), walk the pairs one after the other.
+    for (int r = 0; r < FMM_MAX_RANK; ++r) p->order[r] = r;
+    p->steps = levels >= 1 ? (rank + 1) / 2 : 1;
+    std::vector<int> pstart;
+    std::vector<FmmPairEntry> pentries;
+    if (levels >= 1) {
+        auto mask = [&](int r) { int m = 0; for (int q = 0; q < 4; ++q) if (p->W[r][q] != 0.0f) m |= 1 << q; return m; };
+        auto bits = [](int m) { return (m & 1) + ((m >> 1) & 1) + ((m >> 2) & 1) + ((m >> 3) & 1); };
+        int best_cost = 1 << 30, best[FMM_MAX_RANK], cur[FMM_MAX_RANK];
+        bool used[FMM_MAX_RANK] = {false};
+        // recursive matching: always pair the lowest unused product with some other one (or leave it single once)
+        struct Rec {
+            static void go(int n, int R, int cost, bool single_used, bool* used, int* cur, int& best_cost, int* best,
+                           const int* masks, int (*bitsf)(int))
+            {
+                if (cost >= best_cost) return;
+                int a = -1;
+                for (int r = 0; r < R; ++r) if (!used[r]) { a = r; break; }
+                if (a < 0) { best_cost = cost; for (int i = 0; i < R; ++i) best[i] = cur[i]; return; }
+                used[a] = true;
+                for (int b = a + 1; b < R; ++b) {
+                    if (used[b]) continue;
+                    used[b] = true; cur[n] = a; cur[n + 1] = b;
+                    go(n + 2, R, cost + bitsf(masks[a] | masks[b]), single_used, used, cur, best_cost, best, masks, bitsf);
+                    used[b] = false;
+                }
+                if ((R & 1) && !single_used) {
+                    // the single product goes last in the walk: remember it at the end of cur
+                    cur[R - 1] = a;
+                    // shift: pairs fill cur[0 .. R-2]
+                    go(n, R, cost + bitsf(masks[a]), true, used, cur, best_cost, best, masks, bitsf);
+                }
+                used[a] = false;
+            }
+        };
+        int masks[FMM_MAX_RANK];
+        for (int r = 0; r < rank; ++r) masks[r] = mask(r);
+        Rec::go(0, rank, 0, false, used, cur, best_cost, best, masks, +bits);
+        for (int r = 0; r < rank; ++r) p->order[r] = best[r];
+        std::vector<char> ptouched((size_t)parents * 4, 0);
+        for (int parent = 0; parent < parents; ++parent)
+            for (int s = 0; s < p->steps; ++s) {
+                pstart.push_back((int)pentries.size());
+                const bool pairstep = 2 * s + 1 < rank;
+                const int ra = pairstep ? p->order[2 * s] : -1, rb = pairstep ? p->order[2 * s + 1] : p->order[2 * s];
+                for (int q = 0; q < 4; ++q) {
+                    const float wa = ra >= 0 ? p->W[ra][q] : 0.0f, wb = p->W[rb][q];
+                    if (wa == 0.0f && wb == 0.0f) continue;
+                    FmmPairEntry e;
+                    e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.wA = wa; e.wB = wb;
+                    e.first = ptouched[(size_t)parent * 4 + q] ? 0 : 1;
+                    ptouched[(size_t)parent * 4 + q] = 1;
+                    pentries.push_back(e);
+                }
+            }
+    } else {
+        pstart.push_back(0);
+        FmmPairEntry e; e.row_off = 0; e.col_off = 0; e.wA = 0.0f; e.wB = 1.0f; e.first = 1;
+        pentries.push_back(e);
+    }
+    pstart.push_back((int)pentries.size());
 
     p->lanes = new (std::nothrow) FmmHostLanes;
     if (!p->lanes) { delete p; return FMM_ERR_ALLOC; }
     cudaError_t ce = cudaMalloc(&p->d_status, 64 * sizeof(int));
     if (ce == cudaSuccess) ce = cudaMalloc(&p->d_walk, sizeof(FmmWalkEntry) * walk.size());
+    if (ce == cudaSuccess) ce = cudaMalloc(&p->d_out, sizeof(FmmOutEntry) * (entries.size() + 1));
     if (ce == cudaSuccess) ce = cudaMemset(p->d_status, 0, 64 * sizeof(int));
     if (ce == cudaSuccess) ce = cudaMemcpy(p->d_walk, walk.data(), sizeof(FmmWalkEntry) * walk.size(), cudaMemcpyHostToDevice);
-    const void* table = e8 ? static_cast<const void*>(pairs.data()) : entries.data();
-    const size_t bytes = e8 ? sizeof(FmmPairEntry) * pairs.size() : sizeof(FmmOutEntry) * entries.size();
-    void* d_table = nullptr;
-    if (ce == cudaSuccess) ce = cudaMalloc(&d_table, bytes + 1);
-    if (e8) p->d_pair = static_cast<FmmPairEntry*>(d_table); else p->d_out = static_cast<FmmOutEntry*>(d_table);
-    if (ce == cudaSuccess && bytes) ce = cudaMemcpy(d_table, table, bytes, cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess && !entries.empty())
+        ce = cudaMemcpy(p->d_out, entries.data(), sizeof(FmmOutEntry) * entries.size(), cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = cudaMalloc(&p->d_pair_start, sizeof(int) * pstart.size());
+    if (ce == cudaSuccess) ce = cudaMalloc(&p->d_pair, sizeof(FmmPairEntry) * (pentries.size() + 1));
+    if (ce == cudaSuccess) ce = cudaMemcpy(p->d_pair_start, pstart.data(), sizeof(int) * pstart.size(), cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess) ce = cudaMemcpy(p->d_pair, pentries.data(), sizeof(FmmPairEntry) * pentries.size(), cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) {
         cudaGetLastError();
         fmm_plan_destroy(p);
@@ -626,6 +604,7 @@ fmm_status_t fmm_plan_destroy(fmm_plan_t* p)
     if (p->d_status) cudaFree(p->d_status);
     if (p->d_walk) cudaFree(p->d_walk);
     if (p->d_out) cudaFree(p->d_out);
+    if (p->d_pair_start) cudaFree(p->d_pair_start);
     if (p->d_pair) cudaFree(p->d_pair);
     delete p;
     return FMM_OK;

@@ -41,8 +41,6 @@ constexpr int NUM_THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
 constexpr int REGS_AT_LAUNCH = 168;
 static_assert(NUM_THREADS * (REGS_AT_LAUNCH + 8) > 65536, "REGS_AT_LAUNCH must be the launch-bound maximum");
 
-constexpr uint32_t IDESC_NEGATE_A = 1u << 13;      // instruction descriptor: multiply with -A
-
 template <int BN, int MODE, int BLK, int NCTA>
 struct Cfg {
     static constexpr bool MX = (MODE == FMM_SCALE_UE8M0_CEIL);
@@ -140,7 +138,9 @@ struct KParams {
     // (pair) in order.  (Cutting the slots of a short last wave into narrower items does not pay: a tcgen05.mma of
     // half the width takes as long to issue, measured 4 % slower at n = 8192.)
     int positions, tiles_n, terms_per_group, items;      // tiles_n: tile positions per row of positions
-    const FmmWalkEntry* walk; const FmmOutEntry* out; const FmmPairEntry* pair;    // out: FP32 scales, pair: UE8M0
+    const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
+    const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
+    int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
     FmmGuard guard;
@@ -201,7 +201,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int nkb = p.k / BLK;
     // ti-th product a CTA (pair) walks in work-item group grp: the parents of the group one after the other, the R
     // products of a parent in the plan's walk order
-    auto term_of = [&](int grp, int ti) { return p.walk[grp * p.terms_per_group + ti].term; };
+    auto term_of = [&](int grp, int ti) {
+        if constexpr (C::MX) return grp * p.terms_per_group + (ti / p.R) * p.R + p.order[ti % p.R];
+        else return p.walk[grp * p.terms_per_group + ti].term;
+    };
     const int row_blocks_a = p.m / 128, row_blocks_b = p.n / 128;
 
     if (warp < EPI_WARP0) {
@@ -364,13 +367,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             if (C::MX) idesc_full = (1u << 23) | ((uint32_t)(BN >> 3) << 17) | (MDIM << 24);
             else idesc_full = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | (MDIM << 24);
             for (int w = unit; w < p.items && ok; w += units) {
-                uint32_t idesc = idesc_full, keep = 0;
+                const uint32_t idesc = idesc_full;
                 for (int t = 0; t < p.terms_per_group && ok; ++t) {
                     if (C::MX) {
-                        // UE8M0: a sum goes on in the accumulators, with this term's S_r negated where the walk subtracts it
-                        const float carry = t == 0 ? 0.0f : p.walk[w / p.positions * p.terms_per_group + t].carry;
-                        keep = carry != 0.0f ? 1u : 0u;
-                        idesc = carry < 0.0f ? idesc_full | IDESC_NEGATE_A : idesc_full;
                         if (!mbar_wait_warp(bar_tempty(0), bphase ^ 1u, ctl, 201)) { ok = false; break; }
                         tc_fence_after();
                     }
@@ -390,7 +389,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
                             for (int j = 0; j < BK / 32; ++j) {
                                 const uint32_t id = idesc | ((uint32_t)j << 29) | ((uint32_t)j << 4);
-                                mma_mxf8<NCTA>(tmem_base, adesc + 2 * j, bdesc + 2 * j, id, (ks > 0 || j > 0) ? 1u : keep, tsfa, tsfb);
+                                mma_mxf8<NCTA>(tmem_base, adesc + 2 * j, bdesc + 2 * j, id, (ks > 0 || j > 0) ? 1u : 0u, tsfa, tsfb);
                             }
                         } else {
 #pragma unroll
@@ -447,7 +446,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const int nch = cw / 32;
             const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + h * cw;
             for (int ti = 0, left = p.terms_per_group; left > 0 && ok; ++ti, --left) {
-                const int t = grp * p.terms_per_group + ti;      // the step of the walk
+                const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;      // FP32 scales: the step of the walk
                 // FP32 scales: the sum starts from `carry` times the previous product's, still in the registers (the test of ti
                 // says nothing that the table does not, and is worth 1.5 % of the block-32 kernel's time)
                 const float carry = (C::MX || ti == 0) ? 0.0f : p.walk[t].carry;
@@ -467,11 +466,11 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     __syncwarp();
                     if (lane == 0) release_acc(0);
                     bphase ^= 1u;
-                    // ---- pair-fused post-addition (see FmmPairEntry).  First sum of a pair: park it - CW - 16
+                    // ---- pair-fused post-addition (see FmmPairEntry).  First product of a step: park it - CW - 16
                     // columns in this warp's part of the TMEM hold area, 16 in registers - and go on to the next product.
-                    const int o0 = p.walk[t].out0, o1 = p.walk[t].out1;
+                    const int ri = ti % p.R;
                     const uint32_t hold_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + C::OFF_HOLD + h * C::HOLD_T;
-                    if (o0 == o1) {
+                    if ((ri & 1) == 0 && ri + 1 < p.R) {
 #pragma unroll
                         for (int c = 0; c < C::HOLD_T / 32; ++c) tmem_st32(hold_taddr + c * 32, &accu[c * 32]);
                         tmem_st16(hold_taddr + (C::HOLD_T / 32) * 32, &accu[(C::HOLD_T / 32) * 32]);
@@ -480,8 +479,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         tmem_st_wait();
                         continue;
                     }
-                    // second sum of a pair, or an unpaired one: one weighted update per destination block
+                    // second product of a step, or an unpaired one: one weighted update per destination block
                     const uint64_t pol_c = policy_evict_last();
+                    const int sidx = (t / p.R) * p.steps + (ri >> 1);
+                    const int o0 = p.pair_start[sidx], o1 = p.pair_start[sidx + 1];
                     if (lane == 0) bulk_wait<0>();     // the previous step's writes to these tiles have landed
                     __syncwarp();
                     for (int o = o0; o < o1; ++o) {
@@ -853,7 +854,9 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.positions = positions; kp.tiles_n = g.nsub / BN; kp.terms_per_group = tpg;
     kp.items = slots;
     kp.walk = g.walk; kp.out = g.out; kp.status = g.status;
-    kp.pair = g.pair;
+    kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
+    for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
+    kp.R = g.terms_per_group > 0 ? g.terms_per_group : 1;       // products per parent (1 for the cubic product)
     kp.c_base = g.C; kp.ldc = g.Nfull; kp.guard = g.guard;
 
     cudaLaunchConfig_t cfg;

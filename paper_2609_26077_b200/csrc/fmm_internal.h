@@ -18,13 +18,12 @@ struct FmmOutEntry {
     int first;     // 1: overwrite, 0: add
 };
 
-// One step of the product kernel's walk over the leaf products: which term it multiplies, what its accumulators start from
-// and where the sum goes (see choose_walk and choose_pairs in fmm_api.cu).
+// One step of the fp32-scale product kernel's walk over the leaf products: which term it multiplies, the factor of the
+// previous step's sum that its accumulators start from, and where the sum goes (see choose_walk in fmm_api.cu).
 struct FmmWalkEntry {
     int term;
-    float carry;              // FP32 scales: the accumulators start from carry times the previous step's sum.  UE8M0: they keep
-                              // that sum, and this term's product is added (1) or subtracted (-1).  0: they start from zero.
-    int out0, out1;           // entries [out0, out1) of the FmmOutEntry / FmmPairEntry table; UE8M0: none = park the sum
+    float carry;              // 0 at the first product of a parent
+    int out0, out1;           // entries [out0, out1) of the FmmOutEntry table
 };
 
 // Store guard of the FMM_DEBUG build (the stand-in for a memory checker, which this library cannot count on
@@ -59,11 +58,14 @@ static inline FmmGuard fmm_make_guard(const void* a, size_t na, const void* b, s
 // status word that receives guard violations: plan->d_status[FMM_GUARD_WORD]
 #define FMM_GUARD_WORD 2
 
-// Pair-fused decoder (UE8M0 product kernel): the epilogue keeps sum A on chip until the next step's sum B is done and sends
-// ONE weighted update wA * A + wB * B to every output block either of them feeds.  An unpaired sum is sent with wA = 0.
+// Pair-fused decoder (UE8M0 product kernel): the R products of a parent are walked in an order in which consecutive
+// products (2s, 2s+1) form a step; the epilogue keeps product A on chip until product B is done and sends ONE weighted
+// update wA * M_A + wB * M_B to every output block either of them feeds, which cuts the number of block updates that
+// go through L2 (18 -> 11 for the Phi-optimal realization, 12 -> 9 for Strassen).  An unpaired last product is a step
+// with wA = 0.
 struct FmmPairEntry {
     int row_off, col_off;     // destination block, in units of leaf blocks
-    float wA, wB;             // weights of the parked and of this step's sum (wA = 0: nothing parked, or not used)
+    float wA, wB;             // weights of the step's first and second product (wA = 0: first product absent / not used)
     int first;                // 1: overwrite, 0: add
 };
 
@@ -89,7 +91,10 @@ struct fmm_plan {
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
     FmmWalkEntry* d_walk;     // [terms]
     FmmOutEntry* d_out;       // [total entries], block offsets in units of leaf blocks (scaled at launch)
-    FmmPairEntry* d_pair;     // UE8M0: in place of d_out
+    int order[FMM_MAX_RANK];  // pair-fused decoder: walk order of the R products of a parent
+    int steps;                // pair-fused decoder: steps per parent, ceil(R / 2)
+    int* d_pair_start;        // [parents * steps + 1]
+    FmmPairEntry* d_pair;     // entries of all steps
     // kernels launched by the most recent call on this plan; written once, at the end of a call (calls take the
     // plan as const, and two host threads may share one)
     mutable std::atomic<int> last_launches;
@@ -160,7 +165,9 @@ struct GemmParams {
     int m, n, k, terms;
     int msub, nsub;                         // output rows / columns of every leaf block this launch covers (m, n: all of them); the
                                             // pointers above then point at the strip's first row and column
-    const FmmWalkEntry* walk; const FmmOutEntry* out; const FmmPairEntry* pair;    // out: FP32 scales, pair: UE8M0
+    const FmmWalkEntry* walk; const FmmOutEntry* out;  // walk and decoder of the fp32-scale kernel
+    const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder tables (UE8M0 kernel)
+    int order[FMM_MAX_RANK]; int steps;
     int device, sms;                        // the plan's device and its SM count
     int R, nq;                              // products per parent; blocks of a parent's matrix (4, or 1 for the cubic product)
     const float (*W)[4];                    // innermost decoder, R x 4 (host pointer; unused when nq == 1)
