@@ -920,8 +920,8 @@ fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_
 {
     fmm_status_t s;
     // chosen for the whole problem, also when this launch covers a strip of it: the strips' results do not depend on the cut
-    const int ksplit = fmm_split_choice(g, blk, mode);
-    if (ksplit > 0) s = fmm_launch_split(g, blk, mode, ksplit, st);
+    const SplitChoice split = fmm_split_choice(g, blk, mode);
+    if (split.ksplit > 0) s = fmm_launch_split(g, blk, mode, split, st);
     else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, st);
     else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, st);
     else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, st);

@@ -182,9 +182,11 @@ struct GemmParams {
 fmm_status_t fmm_stats_guard_read(int* code);
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st);
 fmm_status_t fmm_launch_guard_selftest(int* status, cudaStream_t st);
-// K shares per term with which the cluster kernel (fmm_split.cu) takes this product; 0: the persistent kernel is faster
-int fmm_split_choice(const GemmParams& p, int blk, int mode);
-fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, int ksplit, cudaStream_t st);
+// How the cluster kernel (fmm_split.cu) takes this product: K shares per term and columns per tile; 0 shares: the persistent
+// kernel is faster
+struct SplitChoice { int ksplit, bn; };
+SplitChoice fmm_split_choice(const GemmParams& p, int blk, int mode);
+fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, SplitChoice c, cudaStream_t st);
 fmm_status_t fmm_launch_gemm(const GemmParams& p, int blk, int mode, cudaStream_t st, int* launches);
 
 static inline int64_t fmm_ipow(int64_t b, int e) { int64_t r = 1; while (e-- > 0) r *= b; return r; }

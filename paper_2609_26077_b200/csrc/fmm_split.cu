@@ -1,20 +1,23 @@
 // Product kernel for problems with few output tiles (the operation is the one of fmm_gemm.cu).
 //
-// A cluster of CTAs owns one 128 x 128 tile position of one parent: CTA j multiplies one of the parent's R terms (of the
-// cubic product, which has one term: one share of K), so the terms that the persistent kernel of fmm_gemm.cu walks one after the other run side by side.  The
-// partial products then meet in distributed shared memory: every CTA leaves its 128 x 128 fp32 tile in its own shared
-// memory (over the operand ring, which is drained by then), and after a cluster barrier CTA j forms the weighted sums of
-// its share of the rows, out_q = sum_j W[j][q] * M_j in ascending j, and writes each output element once.  Nothing is
-// read back from C, no partial result goes through L2, and the order of the sum is fixed.
+// A cluster of CTAs owns one tile position (128 x 128; with FP32 scales also 128 x 64 or 128 x 32) of one parent: CTA j
+// multiplies one of the parent's R terms (of the cubic product, which has one term: one share of K), so the terms that the
+// persistent kernel of fmm_gemm.cu walks one after the other run side by side.  The partial products then meet in
+// distributed shared memory: every CTA leaves its fp32 tile in its own shared memory (over the operand ring, which is
+// drained by then), and after a cluster barrier CTA j forms the weighted sums of its share of the rows,
+// out_q = sum_j W[j][q] * M_j in ascending j, and writes each output element once.  Nothing is read back from C, no
+// partial result goes through L2, and the order of the sum is fixed.
 //
 // Bound: latency (launch, first operand load, the chain MMA -> promotion -> exchange), which is why the work is spread
 // over as many SMs as the problem has (tile, term, K share) triples.  Two CTAs fit an SM, so that one exchanges or
-// waits for its first operands while the other multiplies.
+// waits for its first operands while the other multiplies.  Promotion and exchange take time in proportion to the tile's
+// columns, so where the narrower tiles still find room at once they are the faster ones (see the time models below).
 //
 //   warp 0  TMA producer of the operand tiles (UE8M0: and of the scale tiles)
 //   warp 1  tcgen05.mma issuer
 //   warp 2  FP32 scales: producer of both sides' scales
 //   warps 4..7  promotion (FP32 scales) or drain (UE8M0), exchange, weighted sums: one TMEM lane quadrant each
+#include <algorithm>
 #include "fmm_gemm_common.cuh"
 
 namespace {
@@ -33,10 +36,11 @@ struct SplitParams {
     FmmGuard guard;
 };
 
-template <int MODE, int BLK>
+template <int MODE, int BLK, int BN_>
 struct SplitCfg {
     static constexpr bool MX = (MODE == FMM_SCALE_UE8M0_CEIL);
-    static constexpr int BN = 128;
+    static constexpr int BN = BN_;                           // columns of a tile
+    static_assert(BN == 128 || (!MX && (BN == 64 || BN == 32)), "tile widths");
     static constexpr int EPI_WARPS = 4, EPI_WARP0 = 4, THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
     static constexpr int REGS_AT_LAUNCH = 128;               // 65536 / (2 CTAs x 256 threads)
     static constexpr int REGS_CTRL = 56, REGS_EPI = 200;
@@ -54,11 +58,12 @@ struct SplitCfg {
     static constexpr int OFF_BAR = OFF_S + S_STAGES * S_BYTES;
     static constexpr int OFF_TILE = 0;                       // the finished partial product, over the operand ring
     static constexpr int BUFS = MX ? 1 : 2;                  // TMEM accumulators
-    static constexpr int TMEM_COLS = 256;
+    static constexpr int TMEM_COLS = MX ? 256 : BUFS * BN;
     static constexpr int NUM_BARS = 2 * STAGES + 2 * S_STAGES + 2 * BUFS;
     static constexpr int SMEM_BYTES = OFF_BAR + NUM_BARS * 8 + 16 + 1024;   // + alignment slack
     static_assert(SMEM_BYTES + 1024 <= 233472 / 2, "two CTAs per SM");
-    static_assert(BM * BN * 4 <= OFF_SF, "the exchange tile lies inside the operand ring");
+    static constexpr int ROW_BYTES = BN * 4;                 // exchange tile: bytes and 16-byte pieces per row
+    static_assert(BM * ROW_BYTES <= OFF_SF, "the exchange tile lies inside the operand ring");
 };
 
 __device__ __forceinline__ uint32_t cluster_id_x()
@@ -72,13 +77,12 @@ __device__ __forceinline__ float4 ld_cluster128(uint32_t addr)
     return v;
 }
 
-template <int MODE, int BLK>
-__global__ void __launch_bounds__(SplitCfg<MODE, BLK>::THREADS, 2)
+template <int MODE, int BLK, int BN>
+__global__ void __launch_bounds__(SplitCfg<MODE, BLK, BN>::THREADS, 2)
 fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmSFA, const __grid_constant__ CUtensorMap tmSFB, const SplitParams p)
 {
-    using C = SplitCfg<MODE, BLK>;
-    constexpr int BN = C::BN;
+    using C = SplitCfg<MODE, BLK, BN>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;       // the same offset in every CTA of the cluster
@@ -209,7 +213,7 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const int q = warp & 3;            // TMEM lane quadrant this warp may access
         const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16);
         bool ok = true;
-        // The exchange tile: row-major fp32, 512 bytes per row, the row's 16-byte pieces permuted by piece ^ (row & 7).
+        // The exchange tile: row-major fp32, the row's 16-byte pieces permuted by piece ^ (row & 7).
         if constexpr (C::MX) {
             ok = mbar_wait_warp(bar_tfull(0), 0, ctl, 321);
             tc_fence_after();
@@ -221,7 +225,7 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 tmem_ld_wait();
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
-                    sts128(tile + row * 512 + (((c * 8 + i) ^ (row & 7)) << 4),
+                    sts128(tile + row * C::ROW_BYTES + (((c * 8 + i) ^ (row & 7)) << 4),
                            make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])));
             }
         } else {
@@ -293,22 +297,23 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                 for (int j = 0; j < JG; ++j) {
                     const int piece = 2 * j + ((lane & 3) >> 1);
-                    sts64(tile + row * 512 + ((piece ^ rr) << 4) + (lane & 1) * 8, acc2[k * JG + j]);
+                    sts64(tile + row * C::ROW_BYTES + ((piece ^ rr) << 4) + (lane & 1) * 8, acc2[k * JG + j]);
                 }
             }
         }
         cluster_sync();                                      // every CTA's partial product is in its shared memory
 
-        // ---- weighted sums of this CTA's share of the rows, one row (of 128 columns) per warp and step; the remote loads
-        // of the next row are in flight while this one is summed and stored (remote shared memory delivers 12 bytes per
-        // clock and SM, 4.5k cycles for the 64 KB of a CTA, measured)
-        const int r0 = BM * rank / S, r1 = BM * (rank + 1) / S;
+        // ---- weighted sums of this CTA's share of the rows, 128 / BN rows per warp and step; the remote loads
+        // of the next step are in flight while this one is summed and stored (remote shared memory delivers 12 bytes per
+        // clock and SM, 4.5k cycles for the 64 KB of a CTA with 128 columns, measured)
+        constexpr int LANES = BN / 4, RPW = 32 / LANES;       // lanes per row, rows per warp and step
+        const int r0 = BM * rank / S, r1 = BM * (rank + 1) / S, piece = lane % LANES;
         uint32_t peer[FMM_MAX_RANK];
 #pragma unroll
         for (int j = 0; j < FMM_MAX_RANK; ++j) peer[j] = map_to_cta(tile, j < S ? j : 0);
-        float* c_tile = p.C + ((long long)parent * (p.nq == 4 ? 2 : 1) * p.m + tm * BM) * p.ldc + tn * BN + lane * 4;
+        float* c_tile = p.C + ((long long)parent * (p.nq == 4 ? 2 : 1) * p.m + tm * BM) * p.ldc + tn * BN + piece * 4;
         auto fetch = [&](int row, float4 (&v)[FMM_MAX_RANK]) {
-            const uint32_t off = row * 512 + ((lane ^ (row & 7)) << 4);
+            const uint32_t off = row * C::ROW_BYTES + ((piece ^ (row & 7)) << 4);
 #pragma unroll
             for (int j = 0; j < FMM_MAX_RANK; ++j) if (j < S) v[j] = ld_cluster128(peer[j] + off);
         };
@@ -327,15 +332,16 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
         };
         float4 v0[FMM_MAX_RANK], v1[FMM_MAX_RANK];
-        int row = r0 + q;
+        constexpr int STEP = C::EPI_WARPS * RPW;
+        int row = r0 + q * RPW + lane / LANES;
         if (row < r1) fetch(row, v0);
 #pragma unroll 1
-        for (; row < r1; row += 2 * C::EPI_WARPS) {
-            const bool more1 = row + C::EPI_WARPS < r1, more2 = row + 2 * C::EPI_WARPS < r1;
-            if (more1) fetch(row + C::EPI_WARPS, v1);
+        for (; row < r1; row += 2 * STEP) {
+            const bool more1 = row + STEP < r1, more2 = row + 2 * STEP < r1;
+            if (more1) fetch(row + STEP, v1);
             sum_and_store(row, v0);
-            if (more2) fetch(row + 2 * C::EPI_WARPS, v0);
-            if (more1) sum_and_store(row + C::EPI_WARPS, v1);
+            if (more2) fetch(row + 2 * STEP, v0);
+            if (more1) sum_and_store(row + STEP, v1);
         }
         (void)ok;
     }
@@ -356,12 +362,12 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // The kernel's shared memory limit, raised once per device.
-template <int MODE, int BLK>
+template <int MODE, int BLK, int BN>
 bool prepare_split(int dev)
 {
     static std::atomic<bool> attr_set[64];
     if (dev >= 0 && dev < 64 && attr_set[dev].load(std::memory_order_acquire)) return true;
-    if (cudaFuncSetAttribute(fmm_split_kernel<MODE, BLK>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitCfg<MODE, BLK>::SMEM_BYTES) != cudaSuccess) {
+    if (cudaFuncSetAttribute(fmm_split_kernel<MODE, BLK, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitCfg<MODE, BLK, BN>::SMEM_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -369,14 +375,14 @@ bool prepare_split(int dev)
     return true;
 }
 
-template <int MODE, int BLK>
+template <int MODE, int BLK, int BN>
 cudaLaunchConfig_t split_config(int S, unsigned tiles_n, unsigned tiles_m, unsigned parents, cudaStream_t st, cudaLaunchAttribute* attr)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3(tiles_n * S, tiles_m, parents);
-    cfg.blockDim = dim3(SplitCfg<MODE, BLK>::THREADS, 1, 1);
-    cfg.dynamicSmemBytes = SplitCfg<MODE, BLK>::SMEM_BYTES;
+    cfg.blockDim = dim3(SplitCfg<MODE, BLK, BN>::THREADS, 1, 1);
+    cfg.dynamicSmemBytes = SplitCfg<MODE, BLK, BN>::SMEM_BYTES;
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = S; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -385,7 +391,8 @@ cudaLaunchConfig_t split_config(int S, unsigned tiles_n, unsigned tiles_m, unsig
 }
 
 // How many clusters of S CTAs the device holds at once (clusters stay inside a GPC, so this is less than SMs * 2 / S).  The
-// runtime counts one CTA per SM for a kernel that allocates TMEM; two are resident (3.1 warps per scheduler, measured).
+// runtime counts one CTA per SM for a kernel that allocates TMEM; two are resident (3.1 warps per scheduler, measured).  Asked for the widest
+// tile: the narrower ones are resident as often, two to an SM by their registers.
 template <int MODE, int BLK>
 int resident_clusters(int dev, int S)
 {
@@ -393,8 +400,8 @@ int resident_clusters(int dev, int S)
     if (dev >= 0 && dev < 64) { const int n = known[dev][S].load(std::memory_order_relaxed); if (n > 0) return n; }
     int n = 0;
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = split_config<MODE, BLK>(S, 1, 1, 1, nullptr, attr);
-    if (!prepare_split<MODE, BLK>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK>, &cfg) != cudaSuccess || n <= 0) {
+    const cudaLaunchConfig_t cfg = split_config<MODE, BLK, 128>(S, 1, 1, 1, nullptr, attr);
+    if (!prepare_split<MODE, BLK, 128>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK, 128>, &cfg) != cudaSuccess || n <= 0) {
         cudaGetLastError();
         return 0;
     }
@@ -403,10 +410,10 @@ int resident_clusters(int dev, int S)
     return n;
 }
 
-template <int MODE, int BLK>
+template <int MODE, int BLK, int BN>
 fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
 {
-    using C = SplitCfg<MODE, BLK>;
+    using C = SplitCfg<MODE, BLK, BN>;
     CUtensorMap tmA, tmB, tmSFA, tmSFB;
     const CUtensorMapSwizzle SW = CU_TENSOR_MAP_SWIZZLE_128B;
     if (!make_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, g.qa, (uint64_t)g.k, (uint64_t)(g.terms - 1) * g.m + g.msub, BK, BM, SW)) return FMM_ERR_CUDA;
@@ -419,7 +426,7 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     } else {
         tmSFA = tmA; tmSFB = tmB;       // unused in this mode
     }
-    if (!prepare_split<MODE, BLK>(g.device)) return FMM_ERR_CUDA;
+    if (!prepare_split<MODE, BLK, BN>(g.device)) return FMM_ERR_CUDA;
     SplitParams p;
     p.sa = static_cast<const uint8_t*>(g.sa); p.sb = static_cast<const uint8_t*>(g.sb);
     p.sa_term = g.sa_term; p.sb_term = g.sb_term;
@@ -432,64 +439,80 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     const int S = g.R * ksplit;
 
     cudaLaunchAttribute attr[2];
-    cudaLaunchConfig_t cfg = split_config<MODE, BLK>(S, (unsigned)(g.nsub / C::BN), (unsigned)(g.msub / BM), (unsigned)(g.terms / g.R), st, attr);
+    cudaLaunchConfig_t cfg = split_config<MODE, BLK, BN>(S, (unsigned)(g.nsub / C::BN), (unsigned)(g.msub / BM), (unsigned)(g.terms / g.R), st, attr);
     // right behind the encoders of the same call: set up while they drain, the producer warps wait before their first load
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = g.overlap_prev ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, fmm_split_kernel<MODE, BLK>, tmA, tmB, tmSFA, tmSFB, p) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
+    if (cudaLaunchKernelEx(&cfg, fmm_split_kernel<MODE, BLK, BN>, tmA, tmB, tmSFA, tmSFB, p) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
     return FMM_OK;
 }
 
 // Time models of the two product kernels in microseconds, fitted to measurements of both at leaves of 128 to 4096 in every
-// direction and zero to three levels (35 shapes of rank 7 and 13 cubic ones per mode; the choice they give loses 0.5 to 2 %
-// on the better of the two in the mean).  The persistent kernel needs R * (k * c + o) per wave of tile positions: c per stage
-// of 128 k, o per term for the chain from the first load to the output; CTA pairs and single CTAs have their own.  The
-// cluster kernel needs lat + (f + k * c) per wave of clusters, f being set-up, exchange and output (f_alone without an
-// exchange).  So it takes the products of few tiles, whatever their K: leaves of 128 to 1024 (block 32) or 1536 (else).
-struct SplitModel { float c_pair, o_pair, c_one, o_one, f, c, f_alone, lat; };
-constexpr SplitModel SPLIT_MX = {0.37f, 4.05f, 0.40f, 1.9f, 3.3f, 0.73f, 3.9f, 0.65f};
-constexpr SplitModel SPLIT_B32 = {0.80f, 5.8f, 0.75f, 4.15f, 3.7f, 2.15f, 4.25f, 1.25f};
-constexpr SplitModel SPLIT_B128 = {0.68f, 3.9f, 0.47f, 2.4f, 3.9f, 0.65f, 4.3f, 1.9f};
-constexpr SplitModel SPLIT_TILE = {0.36f, 4.75f, 0.33f, 3.05f, 4.1f, 0.68f, 3.9f, 1.4f};
+// direction and zero to three levels (some 20 shapes of rank 7 and 13 cubic ones per mode; the choice they give loses 0.5
+// to 2 % on the best one in the mean).  The persistent kernel needs base + R * (k * c + o) per wave of tile positions: c per
+// stage of 128 k, o per term for the chain from the first load to the output; CTA pairs and single CTAs have their own.  The
+// cluster kernel needs lat + waves * (f + k * c), f being set-up, exchange and output; f and c depend on the tile's width.
+// With FP32 scales a cluster that ends makes room for the next at once, so waves is a fraction there; with UE8M0 the
+// clusters of a wave end together.  So the cluster kernel takes the products of few tiles, whatever their K: leaves of 128
+// to 1024 (block 32) or 1536 (else), and it takes tiles of 64 or 32 columns as long as about all of them are resident at
+// once.  Rank 7, block 32, one level, 128 columns -> the width chosen: n = 256 8.6 -> 5.1 us, n = 512 10.7 -> 7.2,
+// n = 1024 18.5 -> 14.0, 512 x 4096 x 1024 40.6 -> 19.7, 256 x 8192 x 256 74.7 -> 27.6.
+struct SplitModel { float c_pair, o_pair, c_one, o_one, base, lat; int widths; float f[3], c[3]; };   // f, c: 128, 64, 32 columns
+constexpr SplitModel SPLIT_MX = {0.37f, 4.05f, 0.40f, 1.9f, 0.0f, 0.65f, 1, {3.3f, 0.f, 0.f}, {0.73f, 0.f, 0.f}};
+constexpr SplitModel SPLIT_B32 = {0.81f, 3.5f, 0.93f, 2.85f, 7.2f, 1.45f, 3, {7.3f, 5.05f, 3.05f}, {2.28f, 1.39f, 0.94f}};
+constexpr SplitModel SPLIT_B128 = {0.67f, 4.85f, 0.39f, 2.7f, 2.3f, 1.3f, 3, {7.45f, 4.95f, 3.75f}, {0.68f, 0.43f, 0.35f}};
+constexpr SplitModel SPLIT_TILE = {0.45f, 5.0f, 0.34f, 2.6f, 2.5f, 1.3f, 3, {7.45f, 4.95f, 3.85f}, {0.55f, 0.38f, 0.32f}};
 
 template <int MODE, int BLK>
-int choose_split(const GemmParams& g, const SplitModel& m, int pair_bn, int one_bn)
+SplitChoice choose_split(const GemmParams& g, const SplitModel& m, int pair_bn, int one_bn)
 {
     const int kst = g.k / BK;
-    const long long parents = g.terms / g.R, tiles = (long long)(g.m / BM) * (g.n / 128) * parents;
+    const long long parents = g.terms / g.R;
     // the persistent kernel: see launch_shape for its tiles
     const bool pair = g.m % 256 == 0 && g.n % pair_bn == 0;
     const int bn = pair ? pair_bn : (g.n % one_bn == 0 ? one_bn : 128);
     const long long positions = (long long)(g.m / (pair ? 256 : 128)) * (g.n / bn) * parents;
     const int units = pair ? g.sms / 2 : g.sms;
-    float best_time = (float)((positions + units - 1) / units) * g.R * (kst * (pair ? m.c_pair : m.c_one) + (pair ? m.o_pair : m.o_one));
-    int best = 0;
+    float best_time = m.base + (float)((positions + units - 1) / units) * g.R * (kst * (pair ? m.c_pair : m.c_one) + (pair ? m.o_pair : m.o_one));
+    SplitChoice best = {0, 0};
     for (int ks = 1; g.R * ks <= FMM_MAX_RANK && ks <= kst; ks *= 2) {
-        const int S = g.R * ks, cap = resident_clusters<MODE, BLK>(g.device, S);
+        const int cap = resident_clusters<MODE, BLK>(g.device, g.R * ks);
         if (cap <= 0) break;
-        const float time = m.lat + (float)((tiles + cap - 1) / cap) * ((S > 1 ? m.f : m.f_alone) + ((kst + ks - 1) / ks) * m.c);
-        if (time < best_time) { best_time = time; best = ks; }
+        for (int w = 0; w < m.widths; ++w) {
+            const long long tiles = (long long)(g.m / BM) * (g.n / (128 >> w)) * parents;
+            const float waves = MODE == FMM_SCALE_UE8M0_CEIL ? (float)((tiles + cap - 1) / cap) : std::max(1.0f, (float)tiles / cap);
+            const float time = m.lat + waves * (m.f[w] + ((kst + ks - 1) / ks) * m.c[w]);
+            if (time < best_time) { best_time = time; best = {ks, 128 >> w}; }
+        }
         if (g.R > 1) break;
     }
     return best;
 }
 
+template <int BN>
+fmm_status_t launch_fp32(const GemmParams& g, int blk, int ksplit, cudaStream_t st)
+{
+    if (blk == 32) return launch_split<MODE_FP32_COLUMN, 32, BN>(g, ksplit, st);
+    if (g.sb_tile) return launch_split<MODE_FP32_SB_TILE, 128, BN>(g, ksplit, st);
+    return launch_split<MODE_FP32_COLUMN, 128, BN>(g, ksplit, st);
+}
+
 }  // namespace
 
-int fmm_split_choice(const GemmParams& g, int blk, int mode)
+SplitChoice fmm_split_choice(const GemmParams& g, int blk, int mode)
 {
-    if (g.m / BM > 65535 || g.terms / g.R > 65535) return 0;          // grid dimensions
+    if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0};     // grid dimensions
     if (mode == FMM_SCALE_UE8M0_CEIL) return choose_split<FMM_SCALE_UE8M0_CEIL, 32>(g, SPLIT_MX, 256, 256);
     if (blk == 32) return choose_split<MODE_FP32_COLUMN, 32>(g, SPLIT_B32, 128, 128);
     if (g.sb_tile) return choose_split<MODE_FP32_SB_TILE, 128>(g, SPLIT_TILE, 256, 128);
     return choose_split<MODE_FP32_COLUMN, 128>(g, SPLIT_B128, 256, 128);
 }
 
-fmm_status_t fmm_launch_split(const GemmParams& g, int blk, int mode, int ksplit, cudaStream_t st)
+fmm_status_t fmm_launch_split(const GemmParams& g, int blk, int mode, SplitChoice c, cudaStream_t st)
 {
-    if (mode == FMM_SCALE_UE8M0_CEIL) return launch_split<FMM_SCALE_UE8M0_CEIL, 32>(g, ksplit, st);
-    if (blk == 32) return launch_split<MODE_FP32_COLUMN, 32>(g, ksplit, st);
-    if (g.sb_tile) return launch_split<MODE_FP32_SB_TILE, 128>(g, ksplit, st);
-    return launch_split<MODE_FP32_COLUMN, 128>(g, ksplit, st);
+    if (mode == FMM_SCALE_UE8M0_CEIL) return launch_split<FMM_SCALE_UE8M0_CEIL, 32, 128>(g, c.ksplit, st);
+    if (c.bn == 32) return launch_fp32<32>(g, blk, c.ksplit, st);
+    if (c.bn == 64) return launch_fp32<64>(g, blk, c.ksplit, st);
+    return launch_fp32<128>(g, blk, c.ksplit, st);
 }

@@ -1,7 +1,7 @@
 """The product kernel for few output tiles (a cluster of CTAs per tile, partial products exchanged in distributed shared
 memory): every mode at the sizes where its indexing can go wrong - one tile, one K stage, fewer and more K stages than
 operand slots, clusters of 7 (rank 7), 8 (rank 8, or eight K shares) and 2 (a K that does not divide evenly), several
-parents - against the oracle, and bit for bit from call to call."""
+parents, and (FP32 scales) tiles of 32, 64 and 128 columns - against the oracle, and bit for bit from call to call."""
 import numpy as np
 import pytest
 import torch
@@ -14,7 +14,8 @@ pytestmark = pytest.mark.gpu
 
 SHAPES = [("strassen", 1, (256, 256, 256)), ("phi_optimal", 1, (256, 1792, 768)), ("winograd", 1, (768, 1024, 256)),
           ("cubic8", 1, (256, 512, 512)), ("phi_optimal", 2, (512, 1024, 1536)), ("winograd", 3, (1024, 1024, 1024)),
-          ("cubic", 0, (128, 128, 128)), ("cubic", 0, (128, 1920, 256)), ("cubic", 0, (256, 4096, 128))]
+          ("cubic", 0, (128, 128, 128)), ("cubic", 0, (128, 1920, 256)), ("cubic", 0, (256, 4096, 128)), ("cubic", 0, (1024, 2048, 1024)),
+          ("winograd", 1, (1024, 1024, 1024)), ("winograd", 1, (1280, 1280, 1280))]
 
 
 @pytest.mark.parametrize("blk,mode,tile", [(32, "fp32", 0), (32, "ue8m0", 0), (128, "fp32", 0), (128, "fp32", 128)])
