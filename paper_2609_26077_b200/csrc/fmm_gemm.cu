@@ -22,6 +22,7 @@
 //               two columns per instruction (fp32x2), overlapped with the next TMEM load.
 //
 // Every wait is bounded: on time-out a status word is set and all roles leave the kernel.
+#include <algorithm>
 #include "fmm_gemm_common.cuh"
 
 namespace {
@@ -133,6 +134,7 @@ struct KParams {
     const uint8_t* sa; const uint8_t* sb;   // scale arrays (bytes); fp32 mode only
     long long sa_term, sb_term;
     int m, n, k, terms;
+    int msub, nsub;                          // rows and columns of a leaf that this launch multiplies (m and n, or a strip)
     // Work items.  A slot is (term group, tile position): the terms of one group (the R products of one parent
     // at the innermost level; all terms at one level) feed one set of output blocks and are walked by one CTA
     // (pair) in order.  (Cutting the slots of a short last wave into narrower items does not pay: a tcgen05.mma of
@@ -261,15 +263,19 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     const int t = term_of(grp, ti);
                     const uint8_t* sb_t = p.sb + (long long)t * p.sb_term + (long long)tn * BN * 4;
                     const uint8_t* sa_t = p.sa + (long long)t * p.sa_term + (long long)(tm * NCTA + cta_rank) * BM * (C::KB_PER_STAGE * 4);
+                    // a tile that hangs over the edge: only the scales that exist (those of its other rows or columns are
+                    // whatever the ring held, as their products are never stored)
+                    const int sb_bytes = min(BN, p.nsub - tn * BN) * 4;
+                    const bool rows = (tm * NCTA + cta_rank) * BM < p.msub;
                     for (int ks = 0; ks < kstages; ++ks) {
                         if (!mbar_wait_warp(bar_sempty(ss), sphase ^ 1u, ctl, 102)) { ok = false; break; }
                         if (elect_one()) {
-                            mbar_expect_tx(bar_sfull(ss), C::SB_STAGE_BYTES);
+                            mbar_expect_tx(bar_sfull(ss), C::KB_PER_STAGE * (sb_bytes + (rows ? BM * 4 : 0)));
 #pragma unroll
                             for (int g = 0; g < C::KB_PER_STAGE; ++g)
                                 bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + g * BN * 4,
-                                          sb_t + (long long)(ks * C::KB_PER_STAGE + g) * p.n * 4, BN * 4, bar_sfull(ss));
-                            bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + C::SB_PART_BYTES,
+                                          sb_t + (long long)(ks * C::KB_PER_STAGE + g) * p.n * 4, sb_bytes, bar_sfull(ss));
+                            if (rows) bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + C::SB_PART_BYTES,
                                       sa_t + (long long)ks * p.m * (C::KB_PER_STAGE * 4), BM * C::KB_PER_STAGE * 4, bar_sfull(ss));
                         }
                         if (++ss == C::SB_STAGES) { ss = 0; sphase ^= 1u; }
@@ -288,11 +294,12 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int slot = w;
                 const int grp = slot / p.positions, pos = slot - grp * p.positions;
                 const int tm = pos / tiles_n, tn = pos % tiles_n;
+                const bool rows = (tm * NCTA + cta_rank) * BM < p.msub;        // else this CTA's half hangs over the edge
                 const int s_end = (grp + 1) * p.terms_per_group;
                 for (int s = s_end - p.terms_per_group; s < s_end && ok; ++s) {
                     if (!mbar_wait_warp(bar_dfull, dphase, ctl, 401)) { ok = false; break; }
                     dphase ^= 1u;
-                    const int o0 = p.walk[s].out0, o1 = p.walk[s].out1;
+                    const int o0 = p.walk[s].out0, o1 = rows ? p.walk[s].out1 : o0;
                     if (lane == 0) bulk_wait<0>();     // the previous term's writes to these tiles have landed
                     __syncwarp();
                     for (int o = o0; o < o1; ++o) {
@@ -444,6 +451,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             // columns this warp owns, in 32-column chunks
             constexpr int cw = C::CW;
             const int nch = cw / 32;
+            // rows and columns that hang over the leaf's edge are multiplied and staged like the others, but never stored (the
+            // test stands where the store is issued: leaving the loops early instead makes the weight-tile kernel 5 % slower)
+            auto live = [&]() { return row_in_leaf < p.msub && (BN == 128 || tn * BN + h * cw < p.nsub); };
             const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + h * cw;
             for (int ti = 0, left = p.terms_per_group; left > 0 && ok; ++ti, --left) {
                 const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;      // FP32 scales: the step of the walk
@@ -522,7 +532,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             }
                             fence_proxy_async();
                             __syncwarp();
-                            if (lane == 0) {
+                            if (lane == 0 && live()) {
                                 if (FMM_GUARD(p.guard, p.c_base + (long long)row0 * p.ldc + col0 + c * C::CH, (31 * p.ldc + C::CH) * 4, 1703)) {
                                     if (ent.first) tma_store_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
                                     else tma_reduce_add_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
@@ -771,7 +781,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         }
                         fence_proxy_async();
                         __syncwarp();
-                        if (lane == 0) {
+                        if (lane == 0 && live()) {
                             if (FMM_GUARD(p.guard, p.c_base + (long long)row0 * p.ldc + col0 + c * C::CH, (31 * p.ldc + C::CH) * 4, 1702)) {
                                 if (ent.first) tma_store_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
                                 else tma_reduce_add_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
@@ -803,6 +813,19 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 }
 
 // --------------------------------------------------------------------------------- host side
+// Tile positions of a leaf of m x n, the ones that hang over its edges included.
+int tile_positions(int m, int n, int ncta, int bn) { return (m + BM * ncta - 1) / (BM * ncta) * ((n + bn - 1) / bn); }
+
+// Term groups as separate work items only where that shortens the longest CTA's list of terms (many terms on few tile
+// positions); otherwise one CTA (pair) walks all terms of its position.
+int terms_per_item(const GemmParams& g, int positions, int units)
+{
+    const int tpg = (g.terms_per_group > 0 && g.terms % g.terms_per_group == 0) ? g.terms_per_group : g.terms;
+    const long long one = (long long)((positions + units - 1) / units) * g.terms;
+    const long long many = ((long long)positions * (g.terms / tpg) + units - 1) / units * tpg;
+    return many >= one ? g.terms : tpg;
+}
+
 template <int BN, int MODE, int BLK, int NCTA>
 fmm_status_t launch(const GemmParams& g, cudaStream_t st)
 {
@@ -832,16 +855,9 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
         }
         if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
     }
-    const int positions = (g.msub / (BM * NCTA)) * (g.nsub / BN);
+    const int tiles_n = (g.nsub + BN - 1) / BN, positions = tile_positions(g.msub, g.nsub, NCTA, BN);
     const int max_units = sms / NCTA;
-    // Term groups as separate work items only where that shortens the longest CTA's list of terms (many terms on
-    // few tile positions); otherwise one CTA (pair) walks all terms of its position.
-    int tpg = (g.terms_per_group > 0 && g.terms % g.terms_per_group == 0) ? g.terms_per_group : g.terms;
-    {
-        const long long one = (long long)((positions + max_units - 1) / max_units) * g.terms;
-        const long long many = (long long)((positions * (g.terms / tpg) + max_units - 1) / max_units) * tpg;
-        if (many >= one) tpg = g.terms;
-    }
+    const int tpg = terms_per_item(g, positions, max_units);
     const int slots = positions * (g.terms / tpg);
     // as few CTAs (pairs) as finish in the same number of waves: every unit then gets the same number of items, and
     // fewer units contend for L2 (256 positions: 64 pairs in 4 waves instead of 74 pairs with a ragged fourth wave)
@@ -850,8 +866,8 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     KParams kp;
     kp.sa = static_cast<const uint8_t*>(g.sa); kp.sb = static_cast<const uint8_t*>(g.sb);
     kp.sa_term = g.sa_term; kp.sb_term = g.sb_term;
-    kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.terms = g.terms;
-    kp.positions = positions; kp.tiles_n = g.nsub / BN; kp.terms_per_group = tpg;
+    kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.msub = g.msub; kp.nsub = g.nsub; kp.terms = g.terms;
+    kp.positions = positions; kp.tiles_n = tiles_n; kp.terms_per_group = tpg;
     kp.items = slots;
     kp.walk = g.walk; kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
@@ -878,37 +894,64 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     return FMM_OK;
 }
 
-template <int MODE, int BLK>
-fmm_status_t launch_shape(const GemmParams& g, cudaStream_t st)
+// The tile shapes each kind of product can be launched with, and the time of one: base + L * (kst * c + o) in microseconds,
+// L being the terms that the busiest CTA (pair) walks, kst the stages of 128 k, o a term's chain from the first load to its
+// output (o_cubic: of the cubic product, which writes every tile once).  A leaf need not be a multiple of the tile: what
+// hangs over the edge is multiplied and not stored, so a leaf of an odd number of 128-row or 128-column blocks may take the
+// wide tiles as well, at the price of a part of its last row or column of tiles.  Fitted, together with the cluster kernel's
+// model (fmm_split.cu), to the times of every shape for some 200 problems per kind, leaves of 128 to 8192 in every direction
+// and zero to three levels; the choice by these models costs 0.4 to 1 % more than the best one in the mean.  Product kernel
+// against the rule before, which gave wide tiles only to leaves that are multiples of them: UE8M0 8192 x 8192 x 8448 one
+// level 674 -> 492 us, cubic 4096 x 1024 x 4224 47.6 -> 26.4; block 128 8192 x 8192 x 8448 956 -> 787; weight tiles
+// 888 -> 664.
+struct ShapeModel { int ncta, bn; float c, o, o_cubic; };
+constexpr ShapeModel MODEL_MX[] = {{2, 256, 0.26f, 3.9f, 3.6f}, {1, 256, 0.35f, 3.4f, 2.7f}, {1, 128, 0.22f, 1.7f, 1.2f}};
+constexpr ShapeModel MODEL_B32[] = {{2, 128, 0.71f, 3.6f, 2.2f}, {1, 128, 0.67f, 3.55f, 1.85f}};
+constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 5.6f, 3.9f}, {1, 128, 0.28f, 2.5f, 1.8f}};
+constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.34f, 4.8f, 2.35f}, {1, 128, 0.26f, 2.4f, 1.15f}};
+constexpr float BASE_MX = 3.3f, BASE_B32 = 6.0f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
+
+template <int N>
+GemmShape best_shape(const GemmParams& g, int m, int n, const ShapeModel (&models)[N], float base)
 {
-    // Pairs of CTAs whenever the leaf shape allows it; single CTAs otherwise.  The UE8M0 kernel wants the
-    // widest tile (least operand traffic per MMA); the FP32-scale kernels are bound by the promotion
-    // on the CUDA cores and use 128-column tiles, whose four TMEM accumulators let the MMA issuer run
-    // further ahead of the promoting warps.
-    if constexpr (MODE != FMM_SCALE_UE8M0_CEIL) {
-        if constexpr (BLK == 32 && MODE == FMM_SCALE_FP32_AMAX_DIV_448) {
-            // long terms: post-addition by the output warp.  (Block 128 does not gain from it: with 128-column tiles and
-            // the output warp it runs as fast as with 256-column tiles and none, 0.81 ms at n = 8192, and the cubic
-            // product, which has a single store per tile, is 20 % slower.)
-            if (g.k / BK >= 16) {
-                if ((g.msub % 256) == 0) return launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st);
-                return launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
-            }
-        }
-        if constexpr (BLK == 128) {
-            // one promotion per 128 k: 256-column tiles with two TMEM accumulators
-            if ((g.msub % 256) == 0 && (g.nsub % 256) == 0) return launch<256, MODE, BLK, 2>(g, st);
-        }
-        if ((g.msub % 256) == 0) return launch<128, MODE, BLK, 2>(g, st);
-        return launch<128, MODE, BLK, 1>(g, st);
+    GemmShape best = {0, 0, 0.0f};
+    for (const ShapeModel& s : models) {
+        const int positions = tile_positions(m, n, s.ncta, s.bn), units = g.sms / s.ncta, tpg = terms_per_item(g, positions, units);
+        const long long longest = ((long long)positions * (g.terms / tpg) + units - 1) / units * tpg;
+        const float time = base + (float)longest * ((float)(g.k / BK) * s.c + (g.R > 1 ? s.o : s.o_cubic));
+        if (best.ncta == 0 || time < best.time) best = {s.ncta, s.bn, time};
+    }
+    return best;
+}
+
+template <int MODE, int BLK>
+fmm_status_t launch_shape(const GemmParams& g, int blk, int mode, cudaStream_t st)
+{
+    const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
+    if constexpr (MODE == FMM_SCALE_UE8M0_CEIL) {
+        if (s.ncta == 2) return launch<256, MODE, 32, 2>(g, st);
+        return s.bn == 256 ? launch<256, MODE, 32, 1>(g, st) : launch<128, MODE, 32, 1>(g, st);
+    } else if constexpr (BLK == 128) {
+        // one promotion per 128 k: 256-column tiles with two TMEM accumulators in a pair
+        return s.ncta == 2 ? launch<256, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     } else {
-        if ((g.msub % 256) == 0 && (g.nsub % 256) == 0) return launch<256, MODE, 32, 2>(g, st);
-        if ((g.nsub % 256) == 0) return launch<256, MODE, 32, 1>(g, st);
-        return launch<128, MODE, 32, 1>(g, st);
+        // bound by the promotion on the CUDA cores: 128-column tiles, whose four TMEM accumulators let the MMA issuer run
+        // further ahead of the promoting warps.  Long terms: post-addition by the output warp.  (Block 128 does not gain
+        // from it: with 128-column tiles and the output warp it runs as fast as with 256-column tiles and none, 0.81 ms at
+        // n = 8192, and the cubic product, which has a single store per tile, is 20 % slower.)
+        if (g.k / BK >= 16) return s.ncta == 2 ? launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st) : launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
+        return s.ncta == 2 ? launch<128, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     }
 }
 
 }  // namespace
+
+GemmShape fmm_gemm_shape(const GemmParams& g, int blk, int mode, int m, int n)
+{
+    if (mode == FMM_SCALE_UE8M0_CEIL) return best_shape(g, m, n, MODEL_MX, BASE_MX);
+    if (blk == 32) return best_shape(g, m, n, MODEL_B32, BASE_B32);
+    return g.sb_tile ? best_shape(g, m, n, MODEL_TILE, BASE_TILE) : best_shape(g, m, n, MODEL_B128, BASE_B128);
+}
 
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st)
 {
@@ -922,10 +965,10 @@ fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_
     // chosen for the whole problem, also when this launch covers a strip of it: the strips' results do not depend on the cut
     const SplitChoice split = fmm_split_choice(g, blk, mode);
     if (split.ksplit > 0) s = fmm_launch_split(g, blk, mode, split, st);
-    else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, st);
-    else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, st);
-    else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, st);
-    else s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 128>(g, st);
+    else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, blk, mode, st);
+    else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, blk, mode, st);
+    else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, blk, mode, st);
+    else s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 128>(g, blk, mode, st);
     if (s == FMM_OK && launches) *launches += 1;
     return s;
 }

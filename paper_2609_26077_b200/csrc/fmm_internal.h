@@ -182,6 +182,10 @@ struct GemmParams {
 fmm_status_t fmm_stats_guard_read(int* code);
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st);
 fmm_status_t fmm_launch_guard_selftest(int* status, cudaStream_t st);
+// Tile shape (CTAs per tile, columns) with which the persistent kernel takes a leaf of m x n, and its time in microseconds by the
+// model the choice is made with
+struct GemmShape { int ncta, bn; float time; };
+GemmShape fmm_gemm_shape(const GemmParams& p, int blk, int mode, int m, int n);
 // How the cluster kernel (fmm_split.cu) takes this product: K shares per term and columns per tile; 0 shares: the persistent
 // kernel is faster
 struct SplitChoice { int ksplit, bn; };

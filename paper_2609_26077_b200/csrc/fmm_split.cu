@@ -448,40 +448,33 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     return FMM_OK;
 }
 
-// Time models of the two product kernels in microseconds, fitted to measurements of both at leaves of 128 to 4096 in every
-// direction and zero to three levels (some 20 shapes of rank 7 and 13 cubic ones per mode; the choice they give loses 0.5
-// to 2 % on the best one in the mean).  The persistent kernel needs base + R * (k * c + o) per wave of tile positions: c per
-// stage of 128 k, o per term for the chain from the first load to the output; CTA pairs and single CTAs have their own.  The
-// cluster kernel needs lat + waves * (f + k * c), f being set-up, exchange and output; f and c depend on the tile's width.
-// With FP32 scales a cluster that ends makes room for the next at once, so waves is a fraction there; with UE8M0 the
-// clusters of a wave end together.  So the cluster kernel takes the products of few tiles, whatever their K: leaves of 128
-// to 1024 (block 32) or 1536 (else), and it takes tiles of 64 or 32 columns as long as about all of them are resident at
-// once.  Rank 7, block 32, one level, 128 columns -> the width chosen: n = 256 8.6 -> 5.1 us, n = 512 10.7 -> 7.2,
+// Time model of the cluster kernel in microseconds, fitted together with the one of the persistent kernel (fmm_gemm_shape): lat +
+// waves * (f + k * c), k in stages of 128, f being set-up, exchange and output; f and c depend on the tile's width.  A
+// cluster that ends makes room for the next at once, so waves is a fraction (of the places; without an exchange the CTAs of
+// an SM get in each other's way, and `alone` of the places count).  So the cluster kernel takes the products of few tiles,
+// whatever their K: leaves of 128 to 1024, and it takes tiles of 64 or 32 columns as long as about all of them are resident
+// at once.  Rank 7, block 32, one level, 128 columns -> the width chosen: n = 256 8.6 -> 5.1 us, n = 512 10.7 -> 7.2,
 // n = 1024 18.5 -> 14.0, 512 x 4096 x 1024 40.6 -> 19.7, 256 x 8192 x 256 74.7 -> 27.6.
-struct SplitModel { float c_pair, o_pair, c_one, o_one, base, lat; int widths; float f[3], c[3]; };   // f, c: 128, 64, 32 columns
-constexpr SplitModel SPLIT_MX = {0.37f, 4.05f, 0.40f, 1.9f, 0.0f, 0.65f, 1, {3.3f, 0.f, 0.f}, {0.73f, 0.f, 0.f}};
-constexpr SplitModel SPLIT_B32 = {0.81f, 3.5f, 0.93f, 2.85f, 7.2f, 1.45f, 3, {7.3f, 5.05f, 3.05f}, {2.28f, 1.39f, 0.94f}};
-constexpr SplitModel SPLIT_B128 = {0.67f, 4.85f, 0.39f, 2.7f, 2.3f, 1.3f, 3, {7.45f, 4.95f, 3.75f}, {0.68f, 0.43f, 0.35f}};
-constexpr SplitModel SPLIT_TILE = {0.45f, 5.0f, 0.34f, 2.6f, 2.5f, 1.3f, 3, {7.45f, 4.95f, 3.85f}, {0.55f, 0.38f, 0.32f}};
+struct SplitModel { float lat, alone; int widths; float f[3], c[3]; };       // f, c: 128, 64, 32 columns
+constexpr SplitModel SPLIT_MX = {0.65f, 0.67f, 1, {6.6f, 0.f, 0.f}, {0.33f, 0.f, 0.f}};
+constexpr SplitModel SPLIT_B32 = {1.7f, 0.89f, 3, {7.15f, 5.55f, 3.75f}, {2.02f, 1.31f, 0.82f}};
+constexpr SplitModel SPLIT_B128 = {1.55f, 0.85f, 3, {7.5f, 5.9f, 4.25f}, {0.61f, 0.34f, 0.34f}};
+constexpr SplitModel SPLIT_TILE = {1.55f, 0.88f, 3, {6.9f, 4.85f, 3.55f}, {0.47f, 0.37f, 0.33f}};
 
 template <int MODE, int BLK>
-SplitChoice choose_split(const GemmParams& g, const SplitModel& m, int pair_bn, int one_bn)
+SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persistent_time)
 {
     const int kst = g.k / BK;
     const long long parents = g.terms / g.R;
-    // the persistent kernel: see launch_shape for its tiles
-    const bool pair = g.m % 256 == 0 && g.n % pair_bn == 0;
-    const int bn = pair ? pair_bn : (g.n % one_bn == 0 ? one_bn : 128);
-    const long long positions = (long long)(g.m / (pair ? 256 : 128)) * (g.n / bn) * parents;
-    const int units = pair ? g.sms / 2 : g.sms;
-    float best_time = m.base + (float)((positions + units - 1) / units) * g.R * (kst * (pair ? m.c_pair : m.c_one) + (pair ? m.o_pair : m.o_one));
+    float best_time = persistent_time;
     SplitChoice best = {0, 0};
     for (int ks = 1; g.R * ks <= FMM_MAX_RANK && ks <= kst; ks *= 2) {
         const int cap = resident_clusters<MODE, BLK>(g.device, g.R * ks);
         if (cap <= 0) break;
+        const float places = g.R * ks > 1 ? (float)cap : cap * m.alone;
         for (int w = 0; w < m.widths; ++w) {
             const long long tiles = (long long)(g.m / BM) * (g.n / (128 >> w)) * parents;
-            const float waves = MODE == FMM_SCALE_UE8M0_CEIL ? (float)((tiles + cap - 1) / cap) : std::max(1.0f, (float)tiles / cap);
+            const float waves = std::max(1.0f, (float)tiles / places);
             const float time = m.lat + waves * (m.f[w] + ((kst + ks - 1) / ks) * m.c[w]);
             if (time < best_time) { best_time = time; best = {ks, 128 >> w}; }
         }
@@ -503,10 +496,11 @@ fmm_status_t launch_fp32(const GemmParams& g, int blk, int ksplit, cudaStream_t 
 SplitChoice fmm_split_choice(const GemmParams& g, int blk, int mode)
 {
     if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0};     // grid dimensions
-    if (mode == FMM_SCALE_UE8M0_CEIL) return choose_split<FMM_SCALE_UE8M0_CEIL, 32>(g, SPLIT_MX, 256, 256);
-    if (blk == 32) return choose_split<MODE_FP32_COLUMN, 32>(g, SPLIT_B32, 128, 128);
-    if (g.sb_tile) return choose_split<MODE_FP32_SB_TILE, 128>(g, SPLIT_TILE, 256, 128);
-    return choose_split<MODE_FP32_COLUMN, 128>(g, SPLIT_B128, 256, 128);
+    const float t = fmm_gemm_shape(g, blk, mode, g.m, g.n).time;
+    if (mode == FMM_SCALE_UE8M0_CEIL) return choose_split<FMM_SCALE_UE8M0_CEIL, 32>(g, SPLIT_MX, t);
+    if (blk == 32) return choose_split<MODE_FP32_COLUMN, 32>(g, SPLIT_B32, t);
+    if (g.sb_tile) return choose_split<MODE_FP32_SB_TILE, 128>(g, SPLIT_TILE, t);
+    return choose_split<MODE_FP32_COLUMN, 128>(g, SPLIT_B128, t);
 }
 
 fmm_status_t fmm_launch_split(const GemmParams& g, int blk, int mode, SplitChoice c, cudaStream_t st)
