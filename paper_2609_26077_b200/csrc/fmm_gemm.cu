@@ -557,8 +557,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     constexpr int KB = C::KB_PER_STAGE;
                     // Block 32: the next buffer's and the next scale stage's barriers are tested before the last chunk's
                     // arithmetic, which hides the test (about 70 cycles) when they are complete; they are waited for only
-                    // if they were not (n = 8192: 1842 -> 1815 us, cubic n = 4096: 276 -> 271).  Block 128 has one buffer
-                    // per stage, rarely complete that early: 2 % slower.
+                    // if they were not (n = 8192: 1792 -> 1740 us, cubic n = 4096: 268.5 -> 256.9).  With test_wait: try_wait
+                    // suspends the warp where the phase is not complete, which costs half of the gain and, on the barriers
+                    // that nothing follows on, 3.6 us per launch.  Block 128 has one buffer per stage, rarely complete that
+                    // early: no gain.
                     constexpr bool PEEK = KB == 4;
                     // A-side scales of the thread's four rows (q*32 + lane/4 + 8k of this CTA's 128), per K block
                     const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + (lane >> 2)) * (KB * 4);
@@ -593,8 +595,8 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                     if (lane == 0) release_acc(buf);
                                     if (PEEK) {
                                         const bool tw = buf + 1 == C::ACC_BUFS, sw = ss + 1 == C::SB_STAGES;
-                                        t_ready = mbar_try_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
-                                        if (g0 + C::GPB >= KB) s_ready = mbar_try_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
+                                        t_ready = mbar_test_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
+                                        if (g0 + C::GPB >= KB) s_ready = mbar_test_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
                                     }
                                 };
                                 // (P * sB) * sA rather than P * (sA * sB): 1 % faster, the multiply no longer keeps a
@@ -909,7 +911,7 @@ constexpr ShapeModel MODEL_MX[] = {{2, 256, 0.26f, 3.9f, 3.6f}, {1, 256, 0.35f, 
 constexpr ShapeModel MODEL_B32[] = {{2, 128, 0.71f, 3.6f, 2.2f}, {1, 128, 0.67f, 3.55f, 1.85f}};
 constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 5.6f, 3.9f}, {1, 128, 0.28f, 2.5f, 1.8f}};
 constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.34f, 4.8f, 2.35f}, {1, 128, 0.26f, 2.4f, 1.15f}};
-constexpr float BASE_MX = 3.3f, BASE_B32 = 6.0f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
+constexpr float BASE_MX = 3.3f, BASE_B32 = 2.4f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
 
 template <int N>
 GemmShape best_shape(const GemmParams& g, int m, int n, const ShapeModel (&models)[N], float base)
