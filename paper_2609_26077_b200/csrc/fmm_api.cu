@@ -100,57 +100,6 @@ double brent_residual(int rank, const float* U, const float* V, const float* W)
     return worst;
 }
 
-// Weight with which the running sum of a step goes to a block: w - c * w_next, c being the next step's carry; exactly zero
-// where that cancels but for the rounding of the coefficients (two units in the last place).
-float emitted_weight(float w, float carry, float w_next)
-{
-    const double x = (double)w - (double)carry * (double)w_next;
-    return fabs(x) <= 2.5e-7 * fabs((double)w) ? 0.0f : (float)x;
-}
-
-// The order in which the fp32-scale product kernel walks the R products of a parent, and what it carries from one to the
-// next.  Its accumulators need not start at zero: with S_t = M_t + c_t * S_{t-1} (the previous sum is still in registers)
-// C_q = sum_t W_t[q] M_t = sum_t (W_t[q] - c_{t+1} W_{t+1}[q]) S_t, so a ratio c that two neighbouring rows of W share in
-// several blocks saves an update of C in all but one of them.  The walk that saves most is a longest path over the R rows
-// (dynamic programme over subsets): 18 -> 12 block updates for the Phi-optimal realization, 14 -> 7 for the Winograd form,
-// 12 -> 10 for Strassen.  Ratios above 2 in magnitude are not used: a sum that grew by them would lose bits of M_t.
-void choose_walk(int R, const float (*W)[4], int* order, float* carry)
-{
-    int save[FMM_MAX_RANK][FMM_MAX_RANK];
-    float ratio[FMM_MAX_RANK][FMM_MAX_RANK];
-    for (int a = 0; a < R; ++a)
-        for (int b = 0; b < R; ++b) {
-            save[a][b] = 0; ratio[a][b] = 0.0f;
-            for (int q = 0; q < 4 && a != b; ++q) {
-                if (W[a][q] == 0.0f || W[b][q] == 0.0f) continue;
-                const float c = W[a][q] / W[b][q];
-                if (!(fabsf(c) <= 2.0f)) continue;
-                int n = 0;
-                for (int k = 0; k < 4; ++k) n += (W[a][k] != 0.0f) - (emitted_weight(W[a][k], c, W[b][k]) != 0.0f);
-                if (n > save[a][b]) { save[a][b] = n; ratio[a][b] = c; }
-            }
-        }
-    // best[set][last]: most updates saved by a walk over `set` that ends in `last`; from: the step before
-    static_assert(FMM_MAX_RANK <= 8, "subset table");
-    signed char best[1 << FMM_MAX_RANK][FMM_MAX_RANK], from[1 << FMM_MAX_RANK][FMM_MAX_RANK];
-    memset(best, -1, sizeof(best));
-    for (int r = 0; r < R; ++r) { best[1 << r][r] = 0; from[1 << r][r] = (signed char)r; }
-    for (int set = 1; set < (1 << R); ++set)
-        for (int a = 0; a < R; ++a) {
-            if (best[set][a] < 0) continue;
-            for (int b = 0; b < R; ++b) {
-                if (set & (1 << b)) continue;
-                const int next = set | (1 << b), v = best[set][a] + save[a][b];
-                if (v > best[next][b]) { best[next][b] = (signed char)v; from[next][b] = (signed char)a; }
-            }
-        }
-    int set = (1 << R) - 1, last = 0;
-    for (int r = 1; r < R; ++r) if (best[set][r] > best[set][last]) last = r;
-    for (int i = R - 1; i >= 0; --i) { order[i] = last; const int f = from[set][last]; set &= ~(1 << last); last = f; }
-    carry[0] = 0.0f;
-    for (int i = 1; i < R; ++i) carry[i] = ratio[order[i - 1]][order[i]];
-}
-
 fmm_status_t check_shape(const fmm_plan* plan, int64_t M, int64_t N, int64_t K)
 {
     if (M <= 0 || N <= 0 || K <= 0) return FMM_ERR_SHAPE;
@@ -483,9 +432,10 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
 
     // Walk and decoder table of the fp32-scale product kernel (Sec. 2.1 decode, innermost level; outer levels are decoded
     // afterwards).  row_off / col_off are in units of leaf blocks inside the stack of parent matrices.
-    int walk_order[FMM_MAX_RANK] = {0};
+    int walk_order[FMM_MAX_RANK];
     float walk_carry[FMM_MAX_RANK] = {0.0f};
-    if (levels >= 1) choose_walk(rank, p->W, walk_order, walk_carry);
+    for (int r = 0; r < FMM_MAX_RANK; ++r) walk_order[r] = r;
+    if (levels >= 1 && qp->scale_mode == FMM_SCALE_FP32_AMAX_DIV_448) fmm_choose_walk(rank, p->U, p->V, p->W, walk_order, walk_carry);
     std::vector<FmmWalkEntry> walk(p->terms);
     std::vector<FmmOutEntry> entries;
     const int parents = levels >= 1 ? p->terms / rank : 1;
@@ -501,7 +451,7 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
         const int parent = t / rank, s = t % rank, r = walk_order[s];
         walk[t].term = parent * rank + r; walk[t].carry = walk_carry[s];
         for (int q = 0; q < 4; ++q) {
-            const float w = s + 1 < rank ? emitted_weight(p->W[r][q], walk_carry[s + 1], p->W[walk_order[s + 1]][q]) : p->W[r][q];
+            const float w = s + 1 < rank ? fmm_emitted_weight(p->W[r][q], walk_carry[s + 1], p->W[walk_order[s + 1]][q]) : p->W[r][q];
             if (w == 0.0f) continue;
             FmmOutEntry e;
             e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.w = w;

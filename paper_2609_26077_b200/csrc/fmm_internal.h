@@ -5,8 +5,8 @@
 #include <stdint.h>
 #include <atomic>
 #include "../../include/fmm.h"
+#include "fmm_walk.h"
 
-#define FMM_MAX_RANK 8
 #define FMM_MAX_LEVELS 3
 
 // One destination of a product in C: block origin, weight, and whether this is the first
@@ -19,7 +19,7 @@ struct FmmOutEntry {
 };
 
 // One step of the fp32-scale product kernel's walk over the leaf products: which term it multiplies, the factor of the
-// previous step's sum that its accumulators start from, and where the sum goes (see choose_walk in fmm_api.cu).
+// previous step's sum that its accumulators start from, and where the sum goes (see fmm_walk.h).
 struct FmmWalkEntry {
     int term;
     float carry;              // 0 at the first product of a parent
