@@ -136,6 +136,24 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
                              int64_t M, int64_t N, int64_t K, void* workspace, size_t workspace_bytes,
                              void* cuda_stream);
 
+/* (No counterpart in the paper: the kernels' tile shapes, for tests and measurements.)
+ * How the leaf products of a call are multiplied. */
+typedef struct {
+    int kernel;                  /* 1: persistent kernel, a CTA or CTA pair walks the terms of a tile position;
+                                    2: cluster kernel, one CTA per term and tile (or per share of K, where there is one term) */
+    int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; cluster: 1 */
+    int columns;                 /* columns of a tile */
+    int k_shares;                /* cluster, one term: CTAs that share K (1, 2, 4, 8); otherwise 1 */
+    int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = a warp of its own writes the products out */
+} fmm_product_shape_t;
+/* The shape that fmm_matmul and fmm_multiply_only take for this problem size (host call; errors as fmm_matmul). */
+fmm_status_t fmm_product_shape(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K, fmm_product_shape_t* shape);
+/* From now on every call on this plan takes `shape` instead of the one that the library expects to be fastest; NULL: the
+ * library chooses again.  FMM_ERR_INVALID_ARG for a shape that does not exist for the plan's quantizer; a later call whose
+ * size cannot be multiplied that way (more K shares than chunks of 128 k) returns FMM_ERR_SHAPE.  Not while another thread
+ * uses the plan. */
+fmm_status_t fmm_force_product_shape(fmm_plan_t* plan, const fmm_product_shape_t* shape);
+
 /* The encoder alone (Sec. 2.1: x_r = <U_r, a>, y_r = <V_r, b>, formed in fp32 from the unquantized blocks; Sec. 2.2 /
  * App. D.1: quantized only afterwards; App. E.2: scale and cast per block) for both sides, into the workspace.
  * Arguments, shape rule and errors as fmm_matmul; C is not touched. */

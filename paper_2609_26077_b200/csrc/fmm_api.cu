@@ -292,11 +292,25 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     return s;
 }
 
-fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float* C, int64_t M, int64_t N, const Strip& strip,
-                      cudaStream_t st, int* launches, bool after_encode)
+// The part of the product kernel's parameters that its tile shape depends on.
+GemmParams product_params(const fmm_plan* plan, const FmmLayout& L, const Strip& strip)
 {
     GemmParams g;
     memset(&g, 0, sizeof(g));
+    g.msub = (int)(strip.m1 - strip.m0); g.nsub = (int)(strip.n1 - strip.n0);
+    g.m = (int)L.m; g.n = (int)L.n; g.k = (int)L.k; g.terms = (int)L.terms;
+    g.terms_per_group = plan->levels >= 2 ? plan->rank : (int)L.terms;
+    g.device = plan->device; g.sms = plan->sms;
+    g.R = plan->levels >= 1 ? plan->rank : 1; g.nq = plan->levels >= 1 ? 4 : 1; g.W = plan->W;
+    g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0;
+    g.forced = plan->forced;
+    return g;
+}
+
+fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float* C, int64_t M, int64_t N, const Strip& strip,
+                      cudaStream_t st, int* launches, bool after_encode)
+{
+    GemmParams g = product_params(plan, L, strip);
     g.overlap_prev = after_encode ? 1 : 0;
     g.qa = reinterpret_cast<const uint8_t*>(ws + L.qa) + strip.m0 * L.k;
     g.qb = reinterpret_cast<const uint8_t*>(ws + L.qb) + strip.n0 * L.k;
@@ -314,15 +328,9 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     const int64_t pm = lv >= 1 ? 2 * L.m : L.m, pn = lv >= 1 ? 2 * L.n : L.n;      // a parent's matrix
     float* dest = lv >= 2 ? reinterpret_cast<float*>(ws + L.dec[lv - 1]) : C;
     g.C = dest + strip.m0 * pn + strip.n0; g.ldc = pn; g.Mfull = parents * pm; g.Nfull = pn;
-    g.msub = (int)(strip.m1 - strip.m0); g.nsub = (int)(strip.n1 - strip.n0);
-    g.m = (int)L.m; g.n = (int)L.n; g.k = (int)L.k; g.terms = (int)L.terms;
-    g.terms_per_group = plan->levels >= 2 ? plan->rank : (int)L.terms;
     g.walk = plan->d_walk; g.out = plan->d_out; g.status = plan->d_status;
     g.pair_start = plan->d_pair_start; g.pair = plan->d_pair; g.steps = plan->steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) g.order[r] = plan->order[r];
-    g.device = plan->device; g.sms = plan->sms;
-    g.R = lv >= 1 ? plan->rank : 1; g.nq = lv >= 1 ? 4 : 1; g.W = plan->W;
-    g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0;
     g.guard = fmm_make_guard(dest, (size_t)g.Mfull * (size_t)g.Nfull * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
     fmm_status_t s = fmm_launch_gemm(g, plan->qp.block_k, (int)plan->qp.scale_mode, st, launches);
     if (s != FMM_OK) return s;
@@ -640,6 +648,29 @@ fmm_status_t fmm_matmul(const fmm_plan_t* plan, const float* A, const float* B, 
     if (s == FMM_OK) s = multiply(plan, L, static_cast<char*>(ws), C, M, N, {0, L.m, 0, L.n}, st, &launches, true);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
+}
+
+fmm_status_t fmm_product_shape(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K, fmm_product_shape_t* shape)
+{
+    if (!plan || !shape) return FMM_ERR_INVALID_ARG;
+    fmm_status_t s = check_device(plan);
+    if (s == FMM_OK) s = check_shape(plan, M, N, K);
+    if (s != FMM_OK) return s;
+    FmmLayout L;
+    make_layout(plan, M, N, K, &L);
+    const GemmParams g = product_params(plan, L, {0, L.m, 0, L.n});
+    *shape = fmm_choose_product(g, plan->qp.block_k, (int)plan->qp.scale_mode);
+    return shape->k_shares <= L.k / 128 ? FMM_OK : FMM_ERR_SHAPE;
+}
+
+fmm_status_t fmm_force_product_shape(fmm_plan_t* plan, const fmm_product_shape_t* shape)
+{
+    if (!plan) return FMM_ERR_INVALID_ARG;
+    if (!shape) { memset(&plan->forced, 0, sizeof(plan->forced)); return FMM_OK; }
+    if (!fmm_product_shape_exists(*shape, plan->qp.block_k, (int)plan->qp.scale_mode, plan->qp.b_tile_n == 128, plan->levels >= 1 ? plan->rank : 1))
+        return FMM_ERR_INVALID_ARG;
+    plan->forced = *shape;
+    return FMM_OK;
 }
 
 // Host-operand variant: [product workspace | A | B | C] in the caller's device buffer, 1024-byte aligned parts.

@@ -33,6 +33,7 @@ namespace {
 // it.  The output warp needs a fixed time per term, so this pays only when a term has many K stages (measured
 // cross-over near 16 stages of 128 k); the dispatcher picks the mode per launch.
 constexpr int MODE_FP32_OUT_WARP = 3;
+constexpr int OUT_WARP_STAGES = 16;        // ... K stages of a term from which on it is taken
 
 constexpr int EPI_WARPS = 8;               // two per TMEM lane quadrant, each half of the tile's columns
 constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, scale producer (FP32 modes), idle
@@ -927,22 +928,21 @@ GemmShape best_shape(const GemmParams& g, int m, int n, const ShapeModel (&model
 }
 
 template <int MODE, int BLK>
-fmm_status_t launch_shape(const GemmParams& g, int blk, int mode, cudaStream_t st)
+fmm_status_t launch_shape(const GemmParams& g, const fmm_product_shape_t& s, cudaStream_t st)
 {
-    const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
     if constexpr (MODE == FMM_SCALE_UE8M0_CEIL) {
-        if (s.ncta == 2) return launch<256, MODE, 32, 2>(g, st);
-        return s.bn == 256 ? launch<256, MODE, 32, 1>(g, st) : launch<128, MODE, 32, 1>(g, st);
+        if (s.ctas == 2) return launch<256, MODE, 32, 2>(g, st);
+        return s.columns == 256 ? launch<256, MODE, 32, 1>(g, st) : launch<128, MODE, 32, 1>(g, st);
     } else if constexpr (BLK == 128) {
         // one promotion per 128 k: 256-column tiles with two TMEM accumulators in a pair
-        return s.ncta == 2 ? launch<256, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
+        return s.ctas == 2 ? launch<256, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     } else {
         // bound by the promotion on the CUDA cores: 128-column tiles, whose four TMEM accumulators let the MMA issuer run
         // further ahead of the promoting warps.  Long terms: post-addition by the output warp.  (Block 128 does not gain
         // from it: with 128-column tiles and the output warp it runs as fast as with 256-column tiles and none, 0.81 ms at
         // n = 8192, and the cubic product, which has a single store per tile, is 20 % slower.)
-        if (g.k / BK >= 16) return s.ncta == 2 ? launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st) : launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
-        return s.ncta == 2 ? launch<128, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
+        if (s.output_warp) return s.ctas == 2 ? launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st) : launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
+        return s.ctas == 2 ? launch<128, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     }
 }
 
@@ -955,6 +955,31 @@ GemmShape fmm_gemm_shape(const GemmParams& g, int blk, int mode, int m, int n)
     return g.sb_tile ? best_shape(g, m, n, MODEL_TILE, BASE_TILE) : best_shape(g, m, n, MODEL_B128, BASE_B128);
 }
 
+fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
+{
+    if (g.forced.kernel) return g.forced;
+    const SplitChoice split = fmm_split_choice(g, blk, mode);
+    if (split.ksplit > 0) return {2, 1, split.bn, split.ksplit, 0};
+    const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
+    return {1, s.ncta, s.bn, 1, mode != FMM_SCALE_UE8M0_CEIL && blk == 32 && g.k / BK >= OUT_WARP_STAGES};
+}
+
+bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R)
+{
+    const bool mx = mode == FMM_SCALE_UE8M0_CEIL;
+    if (s.kernel == 2) {
+        const bool width = s.columns == 128 || (!mx && (s.columns == 64 || s.columns == 32));
+        const bool shares = s.k_shares == 1 || (R == 1 && (s.k_shares == 2 || s.k_shares == 4 || s.k_shares == 8));
+        return width && shares && s.ctas == 1 && !s.output_warp;
+    }
+    auto known = [&](const auto& models) {
+        for (const ShapeModel& m : models) if (m.ncta == s.ctas && m.bn == s.columns) return true;
+        return false;
+    };
+    if (s.kernel != 1 || s.k_shares != 1 || s.output_warp < 0 || s.output_warp > (!mx && blk == 32 ? 1 : 0)) return false;
+    return mx ? known(MODEL_MX) : blk == 32 ? known(MODEL_B32) : sb_tile ? known(MODEL_TILE) : known(MODEL_B128);
+}
+
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st)
 {
     bounded_wait_selftest_kernel<<<1, 32, 0, st>>>(status, limit_ns, 901);
@@ -964,13 +989,12 @@ fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long li
 fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_t st, int* launches)
 {
     fmm_status_t s;
-    // chosen for the whole problem, also when this launch covers a strip of it: the strips' results do not depend on the cut
-    const SplitChoice split = fmm_split_choice(g, blk, mode);
-    if (split.ksplit > 0) s = fmm_launch_split(g, blk, mode, split, st);
-    else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, blk, mode, st);
-    else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, blk, mode, st);
-    else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, blk, mode, st);
-    else s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 128>(g, blk, mode, st);
+    const fmm_product_shape_t shape = fmm_choose_product(g, blk, mode);
+    if (shape.kernel == 2) s = shape.k_shares <= g.k / BK ? fmm_launch_split(g, blk, mode, {shape.k_shares, shape.columns}, st) : FMM_ERR_SHAPE;
+    else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, shape, st);
+    else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, shape, st);
+    else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, shape, st);
+    else s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 128>(g, shape, st);
     if (s == FMM_OK && launches) *launches += 1;
     return s;
 }

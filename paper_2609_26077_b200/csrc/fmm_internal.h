@@ -86,6 +86,7 @@ struct fmm_plan {
     float U[FMM_MAX_RANK][4], V[FMM_MAX_RANK][4], W[FMM_MAX_RANK][4];
     int terms;
     int device, sms;
+    fmm_product_shape_t forced;   // fmm_force_product_shape; kernel 0: none
     struct FmmHostLanes* lanes;   // streams and events of fmm_matmul_host
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
@@ -174,6 +175,7 @@ struct GemmParams {
     int* status;
     int terms_per_group;                    // consecutive terms that feed the same output blocks (R at levels >= 2, else all)
     int sb_tile;                            // fp32 scales, blk 128: the B-side scale is constant over each 128-column tile
+    fmm_product_shape_t forced;             // kernel 0: the launcher chooses
     int overlap_prev;                       // the kernel launched just before on the stream is the B-side encoder of the same call:
                                             // the product kernel may be set up while that one drains (its loads wait for it)
     FmmGuard guard;                         // the output matrix (C, or the stack of parent matrices)
@@ -190,6 +192,10 @@ GemmShape fmm_gemm_shape(const GemmParams& p, int blk, int mode, int m, int n);
 // kernel is faster
 struct SplitChoice { int ksplit, bn; };
 SplitChoice fmm_split_choice(const GemmParams& p, int blk, int mode);
+// The forced shape, or the one that is expected to be fastest.  The kernel is chosen for the whole problem (m, n), also when
+// a launch covers a strip of it (msub, nsub): the strips' results do not depend on the cut
+fmm_product_shape_t fmm_choose_product(const GemmParams& p, int blk, int mode);
+bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R);
 fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, SplitChoice c, cudaStream_t st);
 fmm_status_t fmm_launch_gemm(const GemmParams& p, int blk, int mode, cudaStream_t st, int* launches);
 

@@ -20,7 +20,7 @@ SCALE_MODES = {"fp32": SCALE_FP32, "ue8m0": SCALE_UE8M0}
 
 EXPORTS = ["fmm_plan_create", "fmm_plan_destroy", "fmm_workspace_bytes", "fmm_matmul", "fmm_host_workspace_bytes",
            "fmm_matmul_host", "fmm_encode_only",
-           "fmm_multiply_only", "fmm_quantized_view", "fmm_ref_gemm_fp64", "fmm_error_stats",
+           "fmm_multiply_only", "fmm_product_shape", "fmm_force_product_shape", "fmm_quantized_view", "fmm_ref_gemm_fp64", "fmm_error_stats",
            "fmm_error_stats_scratch_bytes", "fmm_error_stats_noalloc", "fmm_error_stats_noalloc_max_elements",
            "fmm_device_status", "fmm_device_status_clear", "fmm_selftest_bounded_wait", "fmm_phi_gamma", "fmm_brent_residual",
            "fmm_last_launch_count", "fmm_status_string", "fmm_debug_build", "fmm_debug_violation",
@@ -30,6 +30,17 @@ EXPORTS = ["fmm_plan_create", "fmm_plan_destroy", "fmm_workspace_bytes", "fmm_ma
 class QuantParams(C.Structure):
     _fields_ = [("block_k", C.c_int), ("scale_mode", C.c_int), ("amax_floor", C.c_float), ("fp8_max", C.c_float),
                 ("b_tile_n", C.c_int), ("b_preround_bf16", C.c_int)]
+
+
+class ProductShape(C.Structure):
+    """fmm_product_shape_t: the kernel and tile shape of the leaf products."""
+    _fields_ = [("kernel", C.c_int), ("ctas", C.c_int), ("columns", C.c_int), ("k_shares", C.c_int), ("output_warp", C.c_int)]
+
+    def __iter__(self):
+        return iter((self.kernel, self.ctas, self.columns, self.k_shares, self.output_warp))
+
+
+KERNEL_PERSISTENT, KERNEL_CLUSTER = 1, 2
 
 
 class FmmError(RuntimeError):
@@ -61,6 +72,8 @@ def lib():
         ptr, i64, size = C.c_void_p, C.c_int64, C.c_size_t
         L.fmm_workspace_bytes.argtypes = [ptr, i64, i64, i64, ptr]
         L.fmm_host_workspace_bytes.argtypes = [ptr, i64, i64, i64, ptr]
+        L.fmm_product_shape.argtypes = [ptr, i64, i64, i64, ptr]
+        L.fmm_force_product_shape.argtypes = [ptr, ptr]
         L.fmm_quantized_view.argtypes = [ptr, i64, i64, i64, C.c_int, C.c_char] + [ptr] * 6
         L.fmm_matmul.argtypes = [ptr, ptr, ptr, ptr, i64, i64, i64, ptr, size, ptr]
         L.fmm_matmul_host.argtypes = [ptr, ptr, ptr, ptr, i64, i64, i64, ptr, size, ptr]
@@ -249,6 +262,17 @@ class Plan:
         _check(lib().fmm_multiply_only(self._h, out.data_ptr(), M, N, K,
                                        ws.data_ptr(), ws.numel(), _stream_ptr(stream)), "fmm_multiply_only")
         return out
+
+    def product_shape(self, M, N, K):
+        """The ProductShape that matmul takes for this size."""
+        s = ProductShape()
+        _check(lib().fmm_product_shape(self._h, M, N, K, C.byref(s)), "fmm_product_shape")
+        return s
+
+    def force_product_shape(self, kernel=None, ctas=1, columns=128, k_shares=1, output_warp=0):
+        """Every later call takes this shape; without arguments: the library chooses again."""
+        s = None if kernel is None else C.byref(ProductShape(kernel, ctas, columns, k_shares, output_warp))
+        _check(lib().fmm_force_product_shape(self._h, s), "fmm_force_product_shape")
 
     def quantized_view(self, M, N, K, term, side):
         vals = [C.c_size_t(), C.c_int64(), C.c_int64(), C.c_size_t(), C.c_int64(), C.c_int64()]

@@ -26,16 +26,23 @@ def test_few_tiles_match_oracle(name, levels, shape, blk, mode, tile):
     U, V, W = coeffs(name)
     plan = fmm.Plan(U, V, W, levels=levels, block_k=blk, scale_mode=mode, b_tile_n=tile)
     a, b = dev(A), dev(B)
-    out = torch.full((M, N), float("nan"), device="cuda")
-    first = plan.matmul(a, b, out=out).clone()
-    out.fill_(float("nan"))
-    assert torch.equal(plan.matmul(a, b, out=out), first)
-    assert plan.device_status() == (0, 0)
     want = O.fused_fmm(A, B, U, V, W, levels=levels, blk=blk, mode=MODES[mode], b_tile=tile)
-    got = first.cpu().numpy().astype(np.float64)
-    d = 1 << levels
-    for i in range(d):
-        for j in range(d):
-            s = np.s_[i * M // d:(i + 1) * M // d, j * N // d:(j + 1) * N // d]
-            assert np.linalg.norm(got[s] - want[s]) <= 2e-5 * np.linalg.norm(want[s]), f"block ({i},{j})"
-    assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
+    out = torch.full((M, N), float("nan"), device="cuda")
+    # every tile width of the kernel this test is about, and whatever the library chooses for the size
+    shares = max(s for s in (1, 2, 4, 8) if s <= K // 128) if name == "cubic" else 1
+    for columns in (None, 128) if mode == "ue8m0" else (None, 128, 64, 32):
+        if columns:
+            plan.force_product_shape(fmm.KERNEL_CLUSTER, 1, columns, shares)
+            assert plan.product_shape(M, N, K).kernel == fmm.KERNEL_CLUSTER
+        out.fill_(float("nan"))
+        first = plan.matmul(a, b, out=out).clone()
+        out.fill_(float("nan"))
+        assert torch.equal(plan.matmul(a, b, out=out), first)
+        assert plan.device_status() == (0, 0)
+        got = first.cpu().numpy().astype(np.float64)
+        d = 1 << levels
+        for i in range(d):
+            for j in range(d):
+                s = np.s_[i * M // d:(i + 1) * M // d, j * N // d:(j + 1) * N // d]
+                assert np.linalg.norm(got[s] - want[s]) <= 2e-5 * np.linalg.norm(want[s]), f"columns {columns}, block ({i},{j})"
+        assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want), f"columns {columns}"
