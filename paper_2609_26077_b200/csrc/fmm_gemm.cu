@@ -902,8 +902,10 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
 // output (o_cubic: of the cubic product, which writes every tile once).  A leaf need not be a multiple of the tile: what
 // hangs over the edge is multiplied and not stored, so a leaf of an odd number of 128-row or 128-column blocks may take the
 // wide tiles as well, at the price of a part of its last row or column of tiles.  Fitted, together with the cluster kernel's
-// model (fmm_split.cu), to the times of every shape for some 200 problems per kind, leaves of 128 to 8192 in every direction
-// and zero to three levels; the choice by these models costs 0.4 to 1 % more than the best one in the mean.  Product kernel
+// model (fmm_split.cu), to the times of every shape over leaves of 128 to 8192 in every direction and zero to three levels.
+// Over 60 random problems per kind (leaves of 128 to 5000) the choice is the fastest shape for 41 to 54 of them and costs, in
+// the mean, 1.7 % (block 32), 0.3 % (UE8M0), 1.4 % (block 128) and 1.7 % (weight tiles) more than the fastest; the worst are
+// single products of about 10 us, at up to 1.34 times.  Product kernel
 // against the rule before, which gave wide tiles only to leaves that are multiples of them: UE8M0 8192 x 8192 x 8448 one
 // level 674 -> 492 us, cubic 4096 x 1024 x 4224 47.6 -> 26.4; block 128 8192 x 8192 x 8448 956 -> 787; weight tiles
 // 888 -> 664.
