@@ -438,36 +438,34 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
             for (int j = 0; j < 4; ++j) { p->U[r][j] = U[r * 4 + j]; p->V[r][j] = V[r * 4 + j]; p->W[r][j] = W[r * 4 + j]; }
     p->terms = (int)fmm_ipow(rank, levels);
 
-    // Walk and decoder table of the fp32-scale product kernel (Sec. 2.1 decode, innermost level; outer levels are decoded
-    // afterwards).  row_off / col_off are in units of leaf blocks inside the stack of parent matrices.
-    int walk_order[FMM_MAX_RANK];
-    float walk_carry[FMM_MAX_RANK] = {0.0f};
-    for (int r = 0; r < FMM_MAX_RANK; ++r) walk_order[r] = r;
-    if (levels >= 1 && qp->scale_mode == FMM_SCALE_FP32_AMAX_DIV_448) fmm_choose_walk(rank, p->U, p->V, p->W, walk_order, walk_carry);
-    std::vector<FmmWalkEntry> walk(p->terms);
+    // Walks and decoder table of the fp32-scale product kernel (Sec. 2.1 decode, innermost level; outer levels are decoded
+    // afterwards), with carried sums and after them without.  row_off / col_off are in units of leaf blocks inside the stack
+    // of parent matrices.
+    std::vector<FmmWalkEntry> walk(2 * (size_t)p->terms);
     std::vector<FmmOutEntry> entries;
     const int parents = levels >= 1 ? p->terms / rank : 1;
-    std::vector<char> touched((size_t)parents * 4, 0);
-    for (int t = 0; t < p->terms; ++t) {
-        walk[t].out0 = walk[t].out1 = (int)entries.size();
-        if (levels == 0) {
-            FmmOutEntry e; e.row_off = 0; e.col_off = 0; e.w = 1.0f; e.first = 1;
-            entries.push_back(e);
-            walk[t].term = 0; walk[t].carry = 0.0f; walk[t].out1 = 1;
-            continue;
+    for (int carried = 1; carried >= 0; --carried) {
+        int order[FMM_MAX_RANK];
+        float carry[FMM_MAX_RANK] = {0.0f};
+        for (int r = 0; r < FMM_MAX_RANK; ++r) order[r] = r;
+        if (carried && levels >= 1 && qp->scale_mode == FMM_SCALE_FP32_AMAX_DIV_448) fmm_choose_walk(rank, p->U, p->V, p->W, order, carry);
+        std::vector<char> touched((size_t)parents * 4, 0);
+        for (int t = 0; t < p->terms; ++t) {
+            FmmWalkEntry& step = walk[t + (carried ? 0 : p->terms)];
+            step.out0 = (int)entries.size();
+            const int parent = levels ? t / rank : 0, s = levels ? t % rank : 0, r = order[s];
+            step.term = levels ? parent * rank + r : 0; step.carry = carry[s];
+            for (int q = 0; q < (levels ? 4 : 1); ++q) {
+                const float w = !levels ? 1.0f : s + 1 < rank ? fmm_emitted_weight(p->W[r][q], carry[s + 1], p->W[order[s + 1]][q]) : p->W[r][q];
+                if (w == 0.0f) continue;
+                FmmOutEntry e;
+                e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.w = w;
+                e.first = touched[(size_t)parent * 4 + q] ? 0 : 1;
+                touched[(size_t)parent * 4 + q] = 1;
+                entries.push_back(e);
+            }
+            step.out1 = (int)entries.size();
         }
-        const int parent = t / rank, s = t % rank, r = walk_order[s];
-        walk[t].term = parent * rank + r; walk[t].carry = walk_carry[s];
-        for (int q = 0; q < 4; ++q) {
-            const float w = s + 1 < rank ? fmm_emitted_weight(p->W[r][q], walk_carry[s + 1], p->W[walk_order[s + 1]][q]) : p->W[r][q];
-            if (w == 0.0f) continue;
-            FmmOutEntry e;
-            e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.w = w;
-            e.first = touched[(size_t)parent * 4 + q] ? 0 : 1;
-            touched[(size_t)parent * 4 + q] = 1;
-            entries.push_back(e);
-        }
-        walk[t].out1 = (int)entries.size();
     }
 
     // Pair-fused decoder: pair up the R products of a parent so that the pairs' unions of destination blocks are as

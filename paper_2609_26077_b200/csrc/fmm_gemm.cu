@@ -458,11 +458,13 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + h * cw;
             for (int ti = 0, left = p.terms_per_group; left > 0 && ok; ++ti, --left) {
                 const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;      // FP32 scales: the step of the walk
-                // FP32 scales: the sum starts from `carry` times the previous product's, still in the registers (the test of ti
-                // says nothing that the table does not, and is worth 1.5 % of the block-32 kernel's time)
-                const float carry = (C::MX || ti == 0) ? 0.0f : p.walk[t].carry;
+                // FP32 scales, no output warp: the sum starts from `carry` times the previous product's, still in the registers
+                // (the test of ti says nothing that the table does not).  With the output warp every product is summed on its
+                // own, see launch()
+                constexpr bool CARRY = !C::MX && !C::DUMP;
+                const float carry = (!CARRY || ti == 0) ? 0.0f : p.walk[t].carry;
                 const unsigned long long carry2 = pack2(carry, carry);
-                if (carry == 0.0f) {                    // not a product with zero: the sum before may not be finite
+                if (!CARRY || carry == 0.0f) {          // not a product with zero: the sum before may not be finite
 #pragma unroll
                     for (int i = 0; i < (C::MX ? 1 : C::CW / 2); ++i) acc2[i] = 0ull;
                 }
@@ -552,8 +554,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     // elements those loads were a quarter of the promotion) and four A-side scales instead of one.
                     static_assert(!C::ROWS4 || C::KB_PER_STAGE == 4 || C::KB_PER_STAGE == 1, "block 32 or 128");
                     static_assert(!C::DUMP || C::ROWS4, "the output warp expects the four-row register layout");
+                    // acc2[k * (CW/8) + j]: row slot k, column group j
 #pragma unroll
-                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);         // acc2[k * (CW/8) + j]: row slot k, column group j
+                    for (int i = 0; i < (CARRY ? C::CW / 2 : 0); ++i) acc2[i] = mul2(acc2[i], carry2);
                     constexpr int JG = C::CW / 8;                               // column groups of eight per warp
                     constexpr int KB = C::KB_PER_STAGE;
                     // Block 32: the next buffer's and the next scale stage's barriers are tested before the last chunk's
@@ -872,7 +875,12 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.msub = g.msub; kp.nsub = g.nsub; kp.terms = g.terms;
     kp.positions = positions; kp.tiles_n = tiles_n; kp.terms_per_group = tpg;
     kp.items = slots;
-    kp.walk = g.walk; kp.out = g.out; kp.status = g.status;
+    // The output warp's kernel walks the second half of the table, in which every product is summed on its own.  The updates
+    // that carried sums save are mostly hidden behind the next product there (n = 8192: Phi-optimal 0.9 % of the call,
+    // Winograd at 6144 0.4 %; Strassen at 4096 is 1.6 % faster without, Phi-optimal 2.3 % slower), and with 64 and more K
+    // blocks a term they cost the most accuracy: 1.19 times the error for Winograd, 1.20 for Phi-optimal (n = 4096)
+    kp.walk = C::DUMP ? g.walk + g.terms : g.walk;
+    kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
     kp.R = g.terms_per_group > 0 ? g.terms_per_group : 1;       // products per parent (1 for the cubic product)

@@ -90,7 +90,7 @@ struct fmm_plan {
     struct FmmHostLanes* lanes;   // streams and events of fmm_matmul_host
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
-    FmmWalkEntry* d_walk;     // [terms]
+    FmmWalkEntry* d_walk;     // [2 * terms]: with carried sums, and without
     FmmOutEntry* d_out;       // [total entries], block offsets in units of leaf blocks (scaled at launch)
     int order[FMM_MAX_RANK];  // pair-fused decoder: walk order of the R products of a parent
     int steps;                // pair-fused decoder: steps per parent, ceil(R / 2)
@@ -166,7 +166,7 @@ struct GemmParams {
     int m, n, k, terms;
     int msub, nsub;                         // output rows / columns of every leaf block this launch covers (m, n: all of them); the
                                             // pointers above then point at the strip's first row and column
-    const FmmWalkEntry* walk; const FmmOutEntry* out;  // walk and decoder of the fp32-scale kernel
+    const FmmWalkEntry* walk; const FmmOutEntry* out;  // walks (with carried sums, and from `terms` on without) and decoder of the fp32-scale kernel
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder tables (UE8M0 kernel)
     int order[FMM_MAX_RANK]; int steps;
     int device, sms;                        // the plan's device and its SM count
