@@ -124,6 +124,8 @@ void make_layout(const fmm_plan* plan, int64_t M, int64_t N, int64_t K, FmmLayou
     L->sb_term = (size_t)(L->n * nkb) * sbytes;
     L->sa = off; off = align_up(off + L->sa_term * L->terms, 1024);
     L->sb = off; off = align_up(off + L->sb_term * L->terms, 1024);
+    L->sb_down = L->sb;
+    if (sbytes == 4 && !plan->qp.b_tile_n) { L->sb_down = off; off = align_up(off + L->sb_term * L->terms, 1024); }
     for (int lv = 0; lv < FMM_MAX_LEVELS; ++lv) { L->inter_a[lv] = 0; L->inter_b[lv] = 0; L->dec[lv] = 0; }
     // fp32 combinations of the outer levels 1 .. levels-1
     for (int lv = 1; lv < plan->levels; ++lv) {
@@ -223,10 +225,11 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     e.s_out = ws + (b_side ? L.sb : L.sa);
     e.s_term_stride = (int64_t)(b_side ? L.sb_term : L.sa_term);
     e.amax_floor = plan->qp.amax_floor;
+    e.s_down = (int64_t)(L.sb_down - L.sb); e.down = fmm_scale_down(plan->qp);
     e.b_tile = b_side ? plan->qp.b_tile_n : 0;
     e.preround_bf16 = (b_side && plan->qp.b_preround_bf16) ? 1 : 0;
     e.guard = fmm_make_guard(e.q_out, (size_t)L.terms * (size_t)((b_side ? L.n : L.m) * L.k),
-                             e.s_out, (size_t)L.terms * (b_side ? L.sb_term : L.sa_term), plan->d_status + FMM_GUARD_WORD);
+                             e.s_out, (size_t)L.terms * (b_side ? L.sb_term : L.sa_term) + (b_side ? L.sb_down - L.sb : 0), plan->d_status + FMM_GUARD_WORD);
     // first element of the strip in every array
     const int64_t strip_in = b_side ? lo : lo * cols;
     e.q_out += lo * L.k;
@@ -316,8 +319,9 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     g.qb = reinterpret_cast<const uint8_t*>(ws + L.qb) + strip.n0 * L.k;
     const bool e8 = plan->qp.scale_mode == FMM_SCALE_UE8M0_CEIL;
     g.sa = ws + L.sa + (e8 ? strip.m0 / 128 * 512 : strip.m0 * 4 * (128 / plan->qp.block_k));
-    g.sb = ws + L.sb + (e8 ? strip.n0 / 128 * 512 : strip.n0 * 4);
+    g.sb = ws + L.sb_down + (e8 ? strip.n0 / 128 * 512 : strip.n0 * 4);
     g.sa_term = (int64_t)L.sa_term; g.sb_term = (int64_t)L.sb_term;
+    g.up = L.sb_down != L.sb ? 1.0f / fmm_scale_down(plan->qp) : 1.0f;
     // The product kernel applies the innermost decoder only: leaf products of parent p land in the four
     // blocks of parent p's (2m x 2n) matrix.  For one level that matrix is C itself; for more levels the
     // parents' matrices are stacked in the workspace and decoded outwards level by level (the same

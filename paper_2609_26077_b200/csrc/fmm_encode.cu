@@ -367,12 +367,13 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
             float sc; uint32_t e8;
             const float inv = block_scale<MODE>(amax, p.amax_floor, sc, e8);
             const int64_t t = (int64_t)b * p.R + r;
-            if (khalf == 0) {
+            if (MODE == FMM_SCALE_FP32_AMAX_DIV_448 || khalf == 0) {
                 char* so = reinterpret_cast<char*>(p.s_out) + t * p.s_term_stride;
                 const int jg = j + r * p.s_step;                   // column inside the scale array
                 if (MODE == FMM_SCALE_FP32_AMAX_DIV_448) {
-                    float* sp = reinterpret_cast<float*>(so) + (int64_t)kb * p.s_ld + jg;
-                    if (FMM_GUARD(p.guard, sp, 4, 1205)) *sp = sc;
+                    // the other half of the block's lanes writes the copy for the product kernels
+                    float* sp = reinterpret_cast<float*>(so + khalf * p.s_down) + (int64_t)kb * p.s_ld + jg;
+                    if (FMM_GUARD(p.guard, sp, 4, 1205)) *sp = khalf ? sc * p.down : sc;
                 } else {
                     const int64_t tile = (int64_t)kc * p.sf_blocks + (jg >> 7);
                     char* sp = so + tile * 512 + (jg & 31) * 16 + ((jg & 127) >> 5) * 4 + (kb & 3);
@@ -498,6 +499,11 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             const float inv = block_scale<MODE>(amax, p.amax_floor, sc, e8);
             const int64_t t = (int64_t)b * p.R + r;
             if (warp == 0 && khalf == 0) store_b_scale<MODE>(p, t, r, j, kc, kc, sc, 0u, false);
+            // the copy for the product kernels (the weight-tile kernel multiplies the two scales first and needs none)
+            if (!TILE && warp == 0 && khalf) {
+                float* sp = reinterpret_cast<float*>(reinterpret_cast<char*>(p.s_out) + t * p.s_term_stride + p.s_down) + (int64_t)kc * p.s_ld + j + r * p.s_step;
+                if (FMM_GUARD(p.guard, sp, 4, 1208)) *sp = sc * p.down;
+            }
             float v[16];
             combine(r, v);
             uint32_t wv[4];
@@ -637,6 +643,8 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
                 if (MODE == FMM_SCALE_FP32_AMAX_DIV_448) {
                     float* sp = reinterpret_cast<float*>(so) + (int64_t)kb * p.s_ld + j;
                     if (FMM_GUARD(p.guard, sp, 4, 1302)) *sp = s;
+                    float* sd = reinterpret_cast<float*>(reinterpret_cast<char*>(sp) + p.s_down);      // the copy for the product kernels
+                    if (FMM_GUARD(p.guard, sd, 4, 1304)) *sd = s * p.down;
                 } else {
                     const int64_t tile = (int64_t)(kb >> 2) * p.sf_blocks + (j >> 7);
                     char* sp = so + tile * 512 + (j & 31) * 16 + ((j & 127) >> 5) * 4 + (kb & 3);

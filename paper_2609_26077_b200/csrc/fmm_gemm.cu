@@ -19,7 +19,7 @@
 //               tensor-core path can apply a per-row x per-column fp32 factor per K block, so
 //               each K block's partial product is accumulated on its own in TMEM
 //               (kind::f8f6f4) and promoted on the CUDA cores: acc += (P * sB[col]) * sA[row],
-//               two columns per instruction (fp32x2), overlapped with the next TMEM load.
+//               sB scaled down by a power of two against overflow (fmm_scale_down), two columns per instruction (fp32x2), overlapped with the next TMEM load.
 //
 // Every wait is bounded: on time-out a status word is set and all roles leave the kernel.
 #include <algorithm>
@@ -144,6 +144,7 @@ struct KParams {
     const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
     int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
+    float up;                                 // one fp32 scale per column: factor of the sums (GemmParams)
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
     FmmGuard guard;
@@ -603,8 +604,8 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                         if (g0 + C::GPB >= KB) s_ready = mbar_test_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
                                     }
                                 };
-                                // (P * sB) * sA rather than P * (sA * sB): 1 % faster, the multiply no longer keeps a
-                                // product of scales alive (computing those ahead of the TMEM wait: 7 % slower)
+                                // (P * sB) * sA rather than P * (sA * sB): see fmm_scale_down (products of scales ahead of the
+                                // TMEM wait: 7 % slower; behind it, in order: 8 %)
                                 if constexpr (C::CW == 64) {
                                     // two chunks of 16 rows x 64 columns, the second one's load under the first one's arithmetic
                                     // (1.5 % of the cubic product at n = 4096 against chunks of 32 x 32 without the overlap)
@@ -722,13 +723,14 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     dphase ^= 1u;
                     // thread: rows lane/4 + 8k of the warp's 32-row chunk, column pairs 8j + 2(lane%4) of its 64 columns
                     const uint32_t dchunk = base + C::OFF_DUMP + (q * (BN / 32) + h * (C::CW / 32)) * 4096 + (lane & 1) * 8;
+                    const unsigned long long up2 = pack2(p.up, p.up);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int rr = (lane >> 2) + 8 * k;
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             const int pc = 2 * (j & 3) + ((lane & 3) >> 1);        // 16-byte piece of the 128-byte row
-                            sts64(dchunk + (j >> 2) * 4096 + rr * 128 + ((pc ^ (rr & 7)) << 4), acc2[k * 8 + j]);
+                            sts64(dchunk + (j >> 2) * 4096 + rr * 128 + ((pc ^ (rr & 7)) << 4), mul2(acc2[k * 8 + j], up2));
                         }
                     }
                     fence_proxy_async();          // the output warp may hand these chunks to the TMA engine as they are
@@ -761,7 +763,8 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         if (C::ROWS4) {
                             // four-row layout: rows lane/4 + 8k, column pairs 8j + 2(lane%4) of this 32-column chunk
                             const uint32_t sdst = stg + b * C::STAGING_BYTES + (lane & 1) * 8;
-                            const unsigned long long w2 = pack2(ent.w, ent.w);
+                            const float w = ent.w * p.up;
+                            const unsigned long long w2 = pack2(w, w);
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 const int rr = (lane >> 2) + 8 * k;
@@ -884,6 +887,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
     kp.R = g.terms_per_group > 0 ? g.terms_per_group : 1;       // products per parent (1 for the cubic product)
+    kp.up = g.up;
     kp.c_base = g.C; kp.ldc = g.Nfull; kp.guard = g.guard;
 
     cudaLaunchConfig_t cfg;

@@ -75,10 +75,18 @@ struct FmmLayout {            // byte offsets into the workspace
     size_t qa, qb;            // e4m3 codes, terms x m x k and terms x n x k
     size_t sa, sb;            // scales
     size_t sa_term, sb_term;  // bytes of scales per term
+    size_t sb_down;           // fp32 scales per column: the B-side scales times fmm_scale_down, as the product kernels read them
     size_t inter_a[FMM_MAX_LEVELS], inter_b[FMM_MAX_LEVELS];  // fp32 combinations of outer levels
     size_t dec[FMM_MAX_LEVELS];   // dec[l]: R^l partially decoded products of (M/2^l) x (N/2^l) fp32, l = 1 .. levels-1
     size_t total;
 };
+
+// The product kernels promote a K block's partial product P as (P * sB) * sA: P * (sA * sB) makes the block-32 kernel 5 to 7 %
+// slower.  |P| reaches 32 * 448^2 < 2^22.7 and sB 2^119.2, so P * sB could overflow (operands of B above 2e34) where the result
+// does not.  The B-side encoder therefore writes its scales a second time, times this power of two, for the product kernels
+// (n = 8192: 15 of 390 MB), and their sums are multiplied back up when they go out: the same bits for results above 1e-33.
+// With a clamp (amax_floor) so low that the smallest product would leave the normal range, 1.
+static inline float fmm_scale_down(const fmm_quant_params_t& qp) { return qp.amax_floor >= 3e-26f ? 0x1p-14f : 1.0f; }
 
 struct fmm_plan {
     int rank, levels;
@@ -116,6 +124,8 @@ struct EncodeParams {
     int64_t q_term;           // rows * cols, or more when the launch covers a strip of the rows (A) / columns (B) of every term
     void* s_out;              // scales
     int64_t s_term_stride;    // bytes between the scale arrays of consecutive terms
+    int64_t s_down;           // B side, one fp32 scale per column: bytes from a scale to its copy times `down` (fmm_scale_down)
+    float down;
     int s_step;               // rows (A side) / columns (B side) by which combination r is shifted inside a shared scale array
     int s_ld;                 // fp32 scales: columns of B / rows of A that the shared scale array covers
     int sf_blocks;            // UE8M0: number of 128-row blocks of the scale-tile array
@@ -159,8 +169,9 @@ fmm_status_t fmm_launch_encode2_b(const EncodeParams& p, int mode, cudaStream_t 
 
 struct GemmParams {
     const uint8_t* qa; const uint8_t* qb;   // terms x m x k, terms x n x k
-    const void* sa; const void* sb;
+    const void* sa; const void* sb;         // sb, one fp32 scale per column: times fmm_scale_down
     int64_t sa_term, sb_term;               // bytes per term
+    float up;                               // 1 / fmm_scale_down
     float* C; int64_t ldc;                  // full output
     int64_t Mfull, Nfull;
     int m, n, k, terms;

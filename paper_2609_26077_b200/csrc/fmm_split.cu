@@ -433,8 +433,9 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     p.m = g.m; p.n = g.n; p.k = g.k;
     p.R = g.R; p.ksplit = ksplit; p.nq = g.nq;
     memset(p.W, 0, sizeof(p.W));
-    if (g.nq == 4) for (int r = 0; r < g.R; ++r) for (int b = 0; b < 4; ++b) p.W[r][b] = g.W[r][b];
-    else for (int j = 0; j < ksplit; ++j) p.W[j][0] = 1.0f;
+    // times the factor that the sums were kept small by, see fmm_scale_down
+    if (g.nq == 4) for (int r = 0; r < g.R; ++r) for (int b = 0; b < 4; ++b) p.W[r][b] = g.W[r][b] * g.up;
+    else for (int j = 0; j < ksplit; ++j) p.W[j][0] = g.up;
     p.C = g.C; p.ldc = g.Nfull; p.status = g.status; p.guard = g.guard;
     const int S = g.R * ksplit;
 
