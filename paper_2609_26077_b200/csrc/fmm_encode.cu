@@ -294,21 +294,6 @@ __global__ void __launch_bounds__(256, BLK == 128 ? 4 : 3) encode_a_kernel(const
 // hold the two halves of a 32-element (sub-)block, so one shuffle completes the amax.  Each load
 // is two 64-byte row segments per warp; each thread writes 16 contiguous code bytes and the two
 // lanes of a block fill one 32-byte sector.
-template <int MODE>
-__device__ __forceinline__ void store_b_scale(const EncodeParams& p, int64_t t, int r, int j, int kb, int kc,
-                                              float s, uint32_t e8word, bool last_of_word)
-{
-    char* so = reinterpret_cast<char*>(p.s_out) + t * p.s_term_stride;
-    const int jg = j + r * p.s_step;                   // column inside the scale array
-    if (MODE == FMM_SCALE_FP32_AMAX_DIV_448) {
-        float* sp = reinterpret_cast<float*>(so) + (int64_t)kb * p.s_ld + jg;
-        if (FMM_GUARD(p.guard, sp, 4, 1201)) *sp = s;
-    } else if (last_of_word) {
-        const int64_t tile = (int64_t)kc * p.sf_blocks + (jg >> 7);
-        char* sp = so + tile * 512 + (jg & 31) * 16 + ((jg & 127) >> 5) * 4;
-        if (FMM_GUARD(p.guard, sp, 4, 1202)) *reinterpret_cast<uint32_t*>(sp) = e8word;
-    }
-}
 
 // B side, block 32, one 32-k block of 16 columns per warp (thread = 16 k of one column, lanes l and l+16 the two
 // halves of a block), so every thread issues all its loads at once.  A thread block is a single warp: the warps
@@ -498,11 +483,11 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             float sc; uint32_t e8;
             const float inv = block_scale<MODE>(amax, p.amax_floor, sc, e8);
             const int64_t t = (int64_t)b * p.R + r;
-            if (warp == 0 && khalf == 0) store_b_scale<MODE>(p, t, r, j, kc, kc, sc, 0u, false);
-            // the copy for the product kernels (the weight-tile kernel multiplies the two scales first and needs none)
-            if (!TILE && warp == 0 && khalf) {
-                float* sp = reinterpret_cast<float*>(reinterpret_cast<char*>(p.s_out) + t * p.s_term_stride + p.s_down) + (int64_t)kc * p.s_ld + j + r * p.s_step;
-                if (FMM_GUARD(p.guard, sp, 4, 1208)) *sp = sc * p.down;
+            // the upper half of the lanes writes the copy for the product kernels (the weight-tile kernel multiplies the two
+            // scales first and needs none)
+            if (warp == 0 && (!TILE || khalf == 0)) {
+                float* sp = reinterpret_cast<float*>(reinterpret_cast<char*>(p.s_out) + t * p.s_term_stride + khalf * p.s_down) + (int64_t)kc * p.s_ld + j + r * p.s_step;
+                if (FMM_GUARD(p.guard, sp, 4, 1201)) *sp = khalf ? sc * p.down : sc;
             }
             float v[16];
             combine(r, v);
