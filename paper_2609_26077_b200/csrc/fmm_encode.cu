@@ -227,8 +227,12 @@ __device__ __forceinline__ void store_chunk_a(const EncodeParams& p, const float
 // Rows that a task of the A-side encoder walks together (its rows are multiples of 32: of 128, or 128 / 4 in row panels).
 template <int BLK, int MODE> struct RowsPerTask { static constexpr int value = MODE == FMM_SCALE_FP32_AMAX_DIV_448 && BLK == 32 ? 2 : 1; };
 
+// Blocks per SM.  Block 128 with a known zero pattern: four, although 64 registers spill up to 48 bytes (both sides, n = 4096:
+// Winograd 39.1 us against 40.9 with three blocks, n = 8192 146.2 against 147.6).  Without one the spills are nine times that
+// and three blocks are faster (4096: 71.0 -> 67.5, 8192: 254 -> 234).  Block 32: three, and the 4 bytes that the power-of-two
+// kernel without a zero pattern spills then cost less than two blocks would (n = 4096: 51.5 against 56.6).
 template <int BLK, int MODE, uint32_t NZ>
-__global__ void __launch_bounds__(256, BLK == 128 ? 4 : 3) encode_a_kernel(const EncodeParams p)
+__global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_kernel(const EncodeParams p)
 {
     fmmptx::griddep_wait();                        // the combinations of the level above, when this launch overlaps their tail
     fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
@@ -832,8 +836,9 @@ uint32_t coef_mask(const EncodeParams& p)
 }
 
 // zero patterns with pre-instantiated kernels: U and V of Strassen, the Winograd form and the
-// Phi-optimal realization, and the identity used to quantize a matrix as four panels
-#define FMM_KNOWN_MASKS(X) X(0x0a5381c9u) X(0x0c385a19u) X(0x05dc8f21u) X(0x0ab3f841u) X(0x0f5fc5c9u) X(0x0cfc5f59u) X(0x00008421u)
+// Phi-optimal realization, and (one-level kernels) the identity used to quantize a matrix as four panels
+#define FMM_REALIZATION_MASKS(X) X(0x0a5381c9u) X(0x0c385a19u) X(0x05dc8f21u) X(0x0ab3f841u) X(0x0f5fc5c9u) X(0x0cfc5f59u)
+#define FMM_KNOWN_MASKS(X) FMM_REALIZATION_MASKS(X) X(0x00008421u)
 
 // Launch of an encoder.  With p.overlap_prev it carries the programmatic-serialization attribute.  B side: the kernel
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
@@ -894,7 +899,7 @@ void launch_a2(const EncodeParams& p, unsigned g, cudaStream_t st)
 {
     switch (coef_mask(p)) {
 #define X(M) case M: launch_encoder(encode2_a_kernel<BLK, MODE, M>, dim3(g), 256, st, p); return;
-        FMM_KNOWN_MASKS(X)
+        FMM_REALIZATION_MASKS(X)
 #undef X
         default: launch_encoder(encode2_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, p); return;
     }
@@ -904,7 +909,7 @@ void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     switch (coef_mask(p)) {
 #define X(M) case M: launch_encoder(encode2_b_kernel<MODE, M>, grid, 256, st, p); return;
-        FMM_KNOWN_MASKS(X)
+        FMM_REALIZATION_MASKS(X)
 #undef X
         default: launch_encoder(encode2_b_kernel<MODE, 0u>, grid, 256, st, p); return;
     }
