@@ -226,7 +226,7 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     e.s_term_stride = (int64_t)(b_side ? L.sb_term : L.sa_term);
     e.amax_floor = plan->qp.amax_floor;
     e.s_down = (int64_t)(L.sb_down - L.sb); e.down = fmm_scale_down(plan->qp);
-    e.b_tile = b_side ? plan->qp.b_tile_n : 0;
+    e.b_tile = (short)(b_side ? plan->qp.b_tile_n : 0);
     e.preround_bf16 = (b_side && plan->qp.b_preround_bf16) ? 1 : 0;
     e.guard = fmm_make_guard(e.q_out, (size_t)L.terms * (size_t)((b_side ? L.n : L.m) * L.k),
                              e.s_out, (size_t)L.terms * (b_side ? L.sb_term : L.sa_term) + (b_side ? L.sb_down - L.sb : 0), plan->d_status + FMM_GUARD_WORD);

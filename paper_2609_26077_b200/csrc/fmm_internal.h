@@ -131,13 +131,15 @@ struct EncodeParams {
     int sf_blocks;            // UE8M0: number of 128-row blocks of the scale-tile array
     int cpt;                  // A side: 128-k chunks per task (set by the launcher)
     float amax_floor;
-    int b_tile;               // B side: 128 = one fp32 scale per 128 x 128 tile (blk 128 only), 0 = per column
-    int preround_bf16;        // B side: round each combination to bfloat16 before the maximum and the cast
-    FmmGuard guard;           // codes and scales of this side
+    short b_tile;             // B side: 128 = one fp32 scale per 128 x 128 tile (blk 128 only), 0 = per column
+    short preround_bf16;      // B side: round each combination to bfloat16 before the maximum and the cast
     int overlap_prev;         // B side: the kernel launched just before on the stream is the A-side encoder of the same
                               // call (nothing this kernel reads): it may start while that one drains.  A side: that kernel is
                               // the combinations this one reads: it may be set up while that one drains
+    FmmGuard guard;           // codes and scales of this side
 };
+// a launch with more parameter bytes takes the host 0.35 us longer (n = 256: 10.2 -> 10.5 us a call)
+static_assert(sizeof(EncodeParams) <= 352, "encoder parameters");
 
 struct CombParams {
     const float* in;
