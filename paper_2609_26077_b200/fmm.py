@@ -221,7 +221,8 @@ class Plan:
             ws, nbytes = workspace.data_ptr(), workspace.numel()
         else:
             nbytes = self.workspace_bytes(M, N, K)
-            ws = self._own_workspace(nbytes, A.device)[1]
+            # the tensor is held until the call is enqueued: another thread may put a larger one in its place meanwhile
+            held, ws = self._own_workspace(nbytes, A.device)
         status = _lib.fmm_matmul(self._h, A.data_ptr(), B.data_ptr(), out.data_ptr(), M, N, K, ws, nbytes, _stream_ptr(stream))
         if status:
             _check(status, "fmm_matmul")
