@@ -784,14 +784,6 @@ __global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
         }
 }
 
-int sm_count()
-{
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);      // a cached host-side attribute: cheap
-    return n > 0 ? n : 148;
-}
-
 }  // namespace
 
 namespace {
@@ -923,7 +915,7 @@ fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t
     const int64_t row_tasks = (int64_t)p.batch * (p.rows / rpt);
     // long tasks keep two steps of loads in flight, but a problem has to have tasks for about half the resident warps
     // (n = 2048, block 32: one task per eight chunks 15 us for both sides, per two 10 us; n = 4096: per eight 36.8, per two 39)
-    const int64_t want = (int64_t)sm_count() * 10;
+    const int64_t want = (int64_t)fmm_sm_count() * 10;
     int64_t tpr = (chunks + 7) / 8;
     while (row_tasks * tpr < want && chunks > 2 * tpr) tpr *= 2;
     p.cpt = (int)((chunks + tpr - 1) / tpr);
@@ -962,7 +954,7 @@ fmm_status_t fmm_launch_encode2_a(const EncodeParams& p, int blk, int mode, cuda
 {
     const int64_t tasks = (int64_t)p.batch * p.rows * (p.cols / 128);
     int64_t blocks = (tasks + 7) / 8;
-    const int64_t cap = (int64_t)sm_count() * 64;
+    const int64_t cap = (int64_t)fmm_sm_count() * 64;
     if (blocks > cap) blocks = cap;
     const unsigned g = (unsigned)blocks;
     if (mode == FMM_SCALE_FP32_AMAX_DIV_448) {

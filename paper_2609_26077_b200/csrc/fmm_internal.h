@@ -212,4 +212,12 @@ bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, i
 fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, SplitChoice c, cudaStream_t st);
 fmm_status_t fmm_launch_gemm(const GemmParams& p, int blk, int mode, cudaStream_t st, int* launches);
 
+// SMs of the current device (a cached host-side attribute: cheap); 1 where it cannot be read
+static inline int fmm_sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) cudaGetLastError();
+    return n > 0 ? n : 1;
+}
+
 static inline int64_t fmm_ipow(int64_t b, int e) { int64_t r = 1; while (e-- > 0) r *= b; return r; }

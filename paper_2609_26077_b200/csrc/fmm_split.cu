@@ -390,22 +390,42 @@ cudaLaunchConfig_t split_config(int S, unsigned tiles_n, unsigned tiles_m, unsig
     return cfg;
 }
 
-// How many clusters of S CTAs the device holds at once (clusters stay inside a GPC, so this is less than SMs * 2 / S).  The
-// runtime counts one CTA per SM for a kernel that allocates TMEM; two are resident (3.1 warps per scheduler, measured).  Asked for the widest
-// tile: the narrower ones are resident as often, two to an SM by their registers.
+// CTAs that an SM holds, by what they take of its registers, shared memory and TMEM, and as the runtime counts them: one per SM
+// for a kernel that allocates TMEM, though two are resident (3.1 warps per scheduler, measured).
+template <int MODE, int BLK, int BN>
+bool ctas_per_sm(int dev, int* own, int* runtime)
+{
+    using C = SplitCfg<MODE, BLK, BN>;
+    int regs = 0, smem = 0, reserved = 0;
+    cudaFuncAttributes attr;
+    if (cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
+        cudaFuncGetAttributes(&attr, fmm_split_kernel<MODE, BLK, BN>) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(runtime, fmm_split_kernel<MODE, BLK, BN>, C::THREADS, C::SMEM_BYTES) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    *own = std::min(std::min(regs / (attr.numRegs * C::THREADS), smem / (C::SMEM_BYTES + reserved)), 512 / C::TMEM_COLS);
+    return *own > 0 && *runtime > 0;
+}
+
+// How many clusters of S CTAs the device holds at once: clusters stay inside a GPC, so this is less than SMs / S times the CTAs
+// of an SM.  Asked for the widest tile: the narrower ones are resident as often, two to an SM by their registers.
 template <int MODE, int BLK>
 int resident_clusters(int dev, int S)
 {
     static std::atomic<int> known[64][FMM_MAX_RANK + 1];
     if (dev >= 0 && dev < 64) { const int n = known[dev][S].load(std::memory_order_relaxed); if (n > 0) return n; }
-    int n = 0;
+    int n = 0, own = 0, runtime = 0;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = split_config<MODE, BLK, 128>(S, 1, 1, 1, nullptr, attr);
-    if (!prepare_split<MODE, BLK, 128>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK, 128>, &cfg) != cudaSuccess || n <= 0) {
+    if (!prepare_split<MODE, BLK, 128>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK, 128>, &cfg) != cudaSuccess || n <= 0 ||
+        !ctas_per_sm<MODE, BLK, 128>(dev, &own, &runtime)) {
         cudaGetLastError();
         return 0;
     }
-    n *= 2;
+    n = n * own / runtime;
     if (dev >= 0 && dev < 64) known[dev][S].store(n, std::memory_order_relaxed);
     return n;
 }

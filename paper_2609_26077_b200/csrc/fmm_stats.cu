@@ -17,7 +17,9 @@ static __device__ int g_stats_guard_code;
 
 namespace {
 
-constexpr int STAT_BLOCKS = 592;      // 4 x 148 SMs, all resident at 512 threads; at most the 1024 slots of g_noalloc_partials
+// 4 x 148 SMs, all resident at 512 threads; at most the 1024 slots of g_noalloc_partials.  A constant and not the device's count:
+// the partition of the sums, and with it their bits, are the same on every device
+constexpr int STAT_BLOCKS = 592;
 constexpr int STAT_THREADS = 512;
 constexpr int64_t STATS_MAX_DIM = (int64_t)1 << 30;    // per dimension, as for the product itself: M * N cannot overflow
 static_assert(STAT_BLOCKS <= 1024, "one scratch slot per reduction block");
@@ -279,7 +281,8 @@ fmm_status_t fmm_ref_gemm_fp64(const float* A, const float* B, double* Cref, int
     if ((uintptr_t)Cref & 15) return FMM_ERR_INVALID_ARG;
     const FmmGuard guard = fmm_make_guard(Cref, sizeof(double) * (size_t)M * (size_t)N, nullptr, 0, stats_guard_word());
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    if ((M / 64) * (N / 64) < 148) launch_ref<32>(A, B, Cref, M, N, K, guard, st);
+    // tiles of 64 only where they fill the device (the same bits either way)
+    if ((M / 64) * (N / 64) < fmm_sm_count()) launch_ref<32>(A, B, Cref, M, N, K, guard, st);
     else launch_ref<64>(A, B, Cref, M, N, K, guard, st);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }

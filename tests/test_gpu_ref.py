@@ -27,3 +27,11 @@ def test_reference_product_matches_the_cpu_product(M, K, N, aligned):
     want = O.ref_gemm(A, B)
     scale = np.abs(A.astype(np.float64)) @ np.abs(B.astype(np.float64))
     assert np.all(np.abs(got - want) <= 1e-13 * scale)
+
+
+def test_both_tile_sizes_give_the_same_bits():
+    # the size of the problem decides between tiles of 32 and of 64: a part of a large problem is the small problem's result
+    A, B = Wl.gaussian(1024, 272, 1024, seed=4)
+    whole = fmm.fmm_ref_gemm_fp64(dev(A), dev(B))
+    part = fmm.fmm_ref_gemm_fp64(dev(A[128:384]), dev(B[:, 64:320]))
+    assert torch.equal(whole[128:384, 64:320], part)
