@@ -39,6 +39,7 @@ struct FmmWalkSearch {
     float ratio[FMM_MAX_RANK][FMM_MAX_RANK];
     double norm2[FMM_MAX_RANK], size[FMM_MAX_RANK];    // |W_r|^2, |U_r|^2 |V_r|^2
     signed char left[1 << FMM_MAX_RANK][FMM_MAX_RANK]; // [rows walked][last of them]: most updates that the rest can save
+    double fresh[1 << FMM_MAX_RANK][FMM_MAX_RANK];     // least `extra` with which a walk has come to [rows walked][last], the last not carried into
     int cur[FMM_MAX_RANK], best[FMM_MAX_RANK];
     double best_extra;
 
@@ -65,6 +66,10 @@ struct FmmWalkSearch {
             const int saved = n ? save[cur[n - 1]][r] : 0;
             if (set >> r & 1 || saved + left[set | 1 << r][r] < most) continue;
             const double c2v = n ? (double)ratio[cur[n - 1]][r] * ratio[cur[n - 1]][r] * v : 0.0;
+            if (c2v == 0.0) {
+                if (extra >= fresh[set | 1 << r][r]) continue;
+                fresh[set | 1 << r][r] = extra;
+            }
             cur[n] = r;
             go(n + 1, set | 1 << r, most - saved, size[r] + c2v, extra + norm2[r] * c2v);
         }
@@ -92,6 +97,7 @@ static inline void fmm_choose_walk(int R, const float (*U)[4], const float (*V)[
             }
         }
     }
+    for (int set = 0; set < (1 << R); ++set) for (int r = 0; r < R; ++r) s.fresh[set][r] = HUGE_VAL;
     s.bound();
     int most = 0;
     for (int r = 0; r < R; ++r) if (s.left[1 << r][r] > most) most = s.left[1 << r][r];
