@@ -343,8 +343,8 @@ def run_ours(args):
                        "frac": flops_alg / (mul_ms * 1e-3) / 1e12 / fp8_peak,
                        "frac_spec": flops_alg / (mul_ms * 1e-3) / 1e12 / SPEC_FP8_TFLOPS,
                        "traffic": traffic,
-                       "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum, one-pass capture of this "
-                                          "command at this size" if traffic else None),
+                       "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum, one-pass capture of the "
+                                          "same product at this size" if traffic else None),
                        "algorithmic_bytes": gemm_bytes,
                        "peak_source": f"2 x {pk['source']} bf16 burst ({pk['bf16_tflops']} TF/s); spec {SPEC_FP8_TFLOPS} TF/s, {SPEC_HBM_GBS} GB/s",
                        "hbm_peak_gbs": hbm}
