@@ -125,7 +125,7 @@ void make_layout(const fmm_plan* plan, int64_t M, int64_t N, int64_t K, FmmLayou
     L->sa = off; off = align_up(off + L->sa_term * L->terms, 1024);
     L->sb = off; off = align_up(off + L->sb_term * L->terms, 1024);
     L->sb_down = L->sb;
-    if (sbytes == 4 && !plan->qp.b_tile_n) { L->sb_down = off; off = align_up(off + L->sb_term * L->terms, 1024); }
+    if (fmm_scale_per_column(plan->qp)) { L->sb_down = off; off = align_up(off + L->sb_term * L->terms, 1024); }
     for (int lv = 0; lv < FMM_MAX_LEVELS; ++lv) { L->inter_a[lv] = 0; L->inter_b[lv] = 0; L->dec[lv] = 0; }
     // fp32 combinations of the outer levels 1 .. levels-1
     for (int lv = 1; lv < plan->levels; ++lv) {
@@ -321,7 +321,7 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     g.sa = ws + L.sa + (e8 ? strip.m0 / 128 * 512 : strip.m0 * 4 * (128 / plan->qp.block_k));
     g.sb = ws + L.sb_down + (e8 ? strip.n0 / 128 * 512 : strip.n0 * 4);
     g.sa_term = (int64_t)L.sa_term; g.sb_term = (int64_t)L.sb_term;
-    g.up = L.sb_down != L.sb ? 1.0f / fmm_scale_down(plan->qp) : 1.0f;
+    g.up = fmm_scale_up(plan->qp);
     // The product kernel applies the innermost decoder only: leaf products of parent p land in the four
     // blocks of parent p's (2m x 2n) matrix.  For one level that matrix is C itself; for more levels the
     // parents' matrices are stacked in the workspace and decoded outwards level by level (the same
@@ -448,6 +448,7 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
     std::vector<FmmWalkEntry> walk(2 * (size_t)p->terms);
     std::vector<FmmOutEntry> entries;
     const int parents = levels >= 1 ? p->terms / rank : 1;
+    const float up = fmm_scale_up(*qp);
     for (int carried = 1; carried >= 0; --carried) {
         int order[FMM_MAX_RANK];
         float carry[FMM_MAX_RANK] = {0.0f};
@@ -463,7 +464,8 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
                 const float w = !levels ? 1.0f : s + 1 < rank ? fmm_emitted_weight(p->W[r][q], carry[s + 1], p->W[order[s + 1]][q]) : p->W[r][q];
                 if (w == 0.0f) continue;
                 FmmOutEntry e;
-                e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1; e.w = w;
+                e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1;
+                e.w = carried ? w * up : w;        // the output warp's kernel multiplies its sums, see fmm_scale_down
                 e.first = touched[(size_t)parent * 4 + q] ? 0 : 1;
                 touched[(size_t)parent * 4 + q] = 1;
                 entries.push_back(e);

@@ -144,7 +144,7 @@ struct KParams {
     const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
     int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
-    float up;                                 // one fp32 scale per column: factor of the sums (GemmParams)
+    float up;                                 // output warp: factor of the sums (GemmParams); the others have it in their weights
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
     FmmGuard guard;
@@ -763,8 +763,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         if (C::ROWS4) {
                             // four-row layout: rows lane/4 + 8k, column pairs 8j + 2(lane%4) of this 32-column chunk
                             const uint32_t sdst = stg + b * C::STAGING_BYTES + (lane & 1) * 8;
-                            const float w = ent.w * p.up;
-                            const unsigned long long w2 = pack2(w, w);
+                            const unsigned long long w2 = pack2(ent.w, ent.w);
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 const int rr = (lane >> 2) + 8 * k;

@@ -86,7 +86,10 @@ struct FmmLayout {            // byte offsets into the workspace
 // does not.  The B-side encoder therefore writes its scales a second time, times this power of two, for the product kernels
 // (n = 8192: 15 of 390 MB), and their sums are multiplied back up when they go out: the same bits for results above 1e-33.
 // With a clamp (amax_floor) so low that the smallest product would leave the normal range, 1.
+static inline bool fmm_scale_per_column(const fmm_quant_params_t& qp) { return qp.scale_mode == FMM_SCALE_FP32_AMAX_DIV_448 && qp.b_tile_n == 0; }
 static inline float fmm_scale_down(const fmm_quant_params_t& qp) { return qp.amax_floor >= 3e-26f ? 0x1p-14f : 1.0f; }
+// the factor that the sums, or their weights, carry in return
+static inline float fmm_scale_up(const fmm_quant_params_t& qp) { return fmm_scale_per_column(qp) ? 1.0f / fmm_scale_down(qp) : 1.0f; }
 
 struct fmm_plan {
     int rank, levels;
@@ -173,7 +176,7 @@ struct GemmParams {
     const uint8_t* qa; const uint8_t* qb;   // terms x m x k, terms x n x k
     const void* sa; const void* sb;         // sb, one fp32 scale per column: times fmm_scale_down
     int64_t sa_term, sb_term;               // bytes per term
-    float up;                               // 1 / fmm_scale_down
+    float up;                               // fmm_scale_up (the persistent kernel's weights without output warp have it in them)
     float* C; int64_t ldc;                  // full output
     int64_t Mfull, Nfull;
     int m, n, k, terms;
