@@ -143,12 +143,14 @@ struct KParams {
     int positions, tiles_n, terms_per_group, items;      // tiles_n: tile positions per row of positions
     const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
-    int order[FMM_MAX_RANK]; int steps; int R;         // walk order of the R products of a parent; steps = ceil(R / 2)
+    int order[FMM_MAX_RANK]; short steps, R;           // walk order of the R products of a parent; steps = ceil(R / 2)
     float up;                                 // output warp: factor of the sums (GemmParams); the others have it in their weights
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
     FmmGuard guard;
 };
+// no larger than it was: parameter bytes are host time per launch, see EncodeParams
+static_assert(sizeof(KParams) <= 208, "product kernel parameters");
 
 template <int BN, int MODE, int BLK, int NCTA>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
@@ -883,9 +885,9 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     // blocks a term they cost the most accuracy: 1.19 times the error for Winograd, 1.20 for Phi-optimal (n = 4096)
     kp.walk = C::DUMP ? g.walk + g.terms : g.walk;
     kp.out = g.out; kp.status = g.status;
-    kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = g.steps;
+    kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = (short)g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
-    kp.R = g.terms_per_group > 0 ? g.terms_per_group : 1;       // products per parent (1 for the cubic product)
+    kp.R = (short)(g.terms_per_group > 0 ? g.terms_per_group : 1);       // products per parent (1 for the cubic product)
     kp.up = g.up;
     kp.c_base = g.C; kp.ldc = g.Nfull; kp.guard = g.guard;
 
