@@ -92,7 +92,8 @@ fmm_status_t fmm_plan_destroy(fmm_plan_t* plan);
 
 /* Bytes of device workspace fmm_matmul / fmm_encode_only need for this problem size (host call).
  * The workspace holds what the fused regime of Sec. 2.2 / App. D.1 produces between its steps: the quantized
- * encoded combinations x_r, y_r of the R^levels leaves (e4m3 codes + one scale per block, App. E.2) and, for
+ * encoded combinations x_r, y_r of the R^levels leaves (e4m3 codes + one scale per block, App. E.2; fp32 scales per column of B a
+ * second time, times a power of two, as the product kernels read them) and, for
  * levels >= 2, the fp32 combinations of the outer levels and the partially decoded products of the level-by-level
  * recursion (Sec. 3).  Never the products M_r themselves: those go from the tensor cores straight into C. */
 fmm_status_t fmm_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K,
