@@ -36,7 +36,7 @@ constexpr int MODE_FP32_OUT_WARP = 3;
 constexpr int OUT_WARP_STAGES = 16;        // ... K stages of a term from which on it is taken
 
 constexpr int EPI_WARPS = 8;               // two per TMEM lane quadrant, each half of the tile's columns
-constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, scale producer (FP32 modes), idle
+constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, scale producer (FP32 modes), output warp
 constexpr int NUM_THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
 // setmaxnreg budget: the CTA's register pool is NUM_THREADS x (registers at launch); an increase
 // beyond what the decrease freed would block forever, so every split is checked (see Cfg).
@@ -46,10 +46,14 @@ static_assert(NUM_THREADS * (REGS_AT_LAUNCH + 8) > 65536, "REGS_AT_LAUNCH must b
 template <int BN, int MODE, int BLK, int NCTA>
 struct Cfg {
     static constexpr bool MX = (MODE == FMM_SCALE_UE8M0_CEIL);
-    // Register split between the four control warps and the eight epilogue warps.  The FP32-scale kernels give the
-    // promoting warps all they can (accumulators + a TMEM chunk + scales); the UE8M0 kernel's epilogue needs less and
-    // its producer and issuer, which also handle the scale tiles, spilled at 56.
-    static constexpr int REGS_CTRL = (MX || MODE == MODE_FP32_OUT_WARP) ? 72 : 56, REGS_EPI = (MX || MODE == MODE_FP32_OUT_WARP) ? 208 : 224;
+    // FP32 scales per column: the promoting warps read the accumulators with the 16-lane load shape, four rows x
+    // CW/4 columns per thread (see the promotion loop).  The weight-tile mode has no per-column scale loads to
+    // save and is faster with one row per thread.
+    static constexpr bool ROWS4 = !MX && MODE != MODE_FP32_SB_TILE;
+    // Register split between the four control warps and the eight epilogue warps.  The block-128 kernels give the
+    // promoting warps all they can (accumulators + two TMEM chunks + scales); the others' epilogue needs less, and their
+    // control warps, which also handle scale tiles or the output, or hold values not known to be uniform, spill at 56.
+    static constexpr int REGS_CTRL = ROWS4 && BLK == 128 ? 56 : 88, REGS_EPI = ROWS4 && BLK == 128 ? 224 : 208;
     static_assert(EPI_WARP0 * 32 * REGS_CTRL + EPI_WARPS * 32 * REGS_EPI <= NUM_THREADS * REGS_AT_LAUNCH, "register pool");
     // Warp index, CTA rank and TMEM base as values the compiler knows to be warp-uniform (see warp_uniform): 3 % of the
     // block-32 kernel at n = 8192 and 4096, 7 % of the single-CTA UE8M0 kernel at 1280 x 2816 x 3328.  Not for the UE8M0
@@ -63,10 +67,6 @@ struct Cfg {
     // and a second chunk in flight per warp was measured slower (more output traffic competing with the loads).
     static constexpr int STAGING_BUFS = (MX && NCTA == 2) ? 1 : 2;
     static constexpr bool DUMP = (MODE == MODE_FP32_OUT_WARP);
-    // FP32 scales per column: the promoting warps read the accumulators with the 16-lane load shape, four rows x
-    // CW/4 columns per thread (see the promotion loop).  The weight-tile mode has no per-column scale loads to
-    // save and is faster with one row per thread.
-    static constexpr bool ROWS4 = !MX && MODE != MODE_FP32_SB_TILE;
     static_assert(!DUMP || (BN == 128 && BK / BLK == 4), "output-warp mode: 128-column tiles, block 32");
     static constexpr int STAGES = (MX && NCTA == 2) ? 5 : ((A_BYTES + B_BYTES) > 40000 || DUMP ? 3 : 4);
     // DUMP (output-warp mode): shared-memory copy of a finished product, BM x BN fp32
@@ -97,13 +97,16 @@ struct Cfg {
     static constexpr int OFF_SF = OFF_DUMP + DUMP_BYTES;
     static constexpr int OFF_SB = OFF_SF + STAGES * SF_STAGE_BYTES;
     static constexpr int OFF_BAR = OFF_SB + SB_STAGES * SB_STAGE_BYTES;
-    static constexpr int NUM_BARS = 2 * STAGES + 2 * SB_STAGES + 8 + 2;
+    // FP32: the signals "K blocks multiplied" are a ring of their own, GROUPS per stage of the scale ring
+    static constexpr int GPB = MX ? 1 : ((KB_PER_STAGE >= 2 && 512 / BN >= 4) ? 2 : 1);
+    static constexpr int GROUPS = KB_PER_STAGE / GPB;
+    static constexpr int FULL_SLOTS = MX ? 1 : SB_STAGES * GROUPS;
+    static constexpr int NUM_BARS = 2 * STAGES + SB_STAGES + FULL_SLOTS + 4 + 2;
     static constexpr int SMEM_BYTES = OFF_BAR + NUM_BARS * 8 + 16 + 1024;   // + alignment slack
     // TMEM: MX: one BN-column accumulator, then per stage 4 SFA + 4*(BN/128) SFB columns.
     //       FP32: ring of 512/BN accumulators, one per K block in flight.
     // FP32: GPB consecutive K blocks ("granules") share one completion signal: their MMAs are issued back to
     // back into adjacent TMEM buffers and committed once, so the tensor pipe is not drained per K block.
-    static constexpr int GPB = MX ? 1 : ((KB_PER_STAGE >= 2 && 512 / BN >= 4) ? 2 : 1);
     static constexpr int ACC_BUFS = MX ? 1 : (512 / BN) / GPB;        // ring of (GPB x BN)-column super-buffers
     static constexpr int SF_COLS = 4 + 4 * SFB_ATOMS;
     // UE8M0: TMEM columns [0, BN) accumulator, [BN, BN + SF_COLS) the scale factors of the stage being multiplied (one
@@ -167,12 +170,11 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t bar0 = base + C::OFF_BAR;
     auto bar_full = [&](int s) { return bar0 + 8u * s; };
     auto bar_empty = [&](int s) { return bar0 + 8u * (C::STAGES + s); };
-    auto bar_sfull = [&](int s) { return bar0 + 8u * (2 * C::STAGES + s); };
-    auto bar_sempty = [&](int s) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + s); };
-    auto bar_tfull = [&](int b) { return bar0 + 8u * (2 * C::STAGES + 2 * C::SB_STAGES + b); };
-    auto bar_tempty = [&](int b) { return bar0 + 8u * (2 * C::STAGES + 2 * C::SB_STAGES + 4 + b); };
-    const uint32_t bar_dfull = bar0 + 8u * (2 * C::STAGES + 2 * C::SB_STAGES + 8);      // accumulator copy written
-    const uint32_t bar_dempty = bar_dfull + 8u;                                           // ... and consumed
+    auto bar_sempty = [&](int s) { return bar0 + 8u * (2 * C::STAGES + s); };
+    auto bar_tfull = [&](int b) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + b); };
+    auto bar_tempty = [&](int b) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + C::FULL_SLOTS + b); };
+    const uint32_t bar_dfull = bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + C::FULL_SLOTS + 4);      // accumulator copy written
+    const uint32_t bar_dempty = bar_dfull + 8u;                                                       // ... and consumed
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + C::OFF_BAR + C::NUM_BARS * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const Ctl ctl{abort_flag, p.status};
@@ -186,8 +188,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < C::STAGES; ++s) { mbar_init(bar_full(s), 1); mbar_init(bar_empty(s), 1); }
-        for (int s = 0; s < C::SB_STAGES; ++s) { mbar_init(bar_sfull(s), 1); mbar_init(bar_sempty(s), EPI_WARPS); }
-        for (int b = 0; b < 4; ++b) { mbar_init(bar_tfull(b), 1); mbar_init(bar_tempty(b), NCTA * EPI_WARPS); }
+        for (int s = 0; s < C::SB_STAGES; ++s) mbar_init(bar_sempty(s), EPI_WARPS);
+        // the first K blocks of a stage are signalled together with the stage's scales
+        for (int b = 0; b < C::FULL_SLOTS; ++b) mbar_init(bar_tfull(b), !C::MX && b % C::GROUPS == 0 ? 2 : 1);
+        for (int b = 0; b < 4; ++b) mbar_init(bar_tempty(b), NCTA * EPI_WARPS);
         mbar_init(bar_dfull, EPI_WARPS); mbar_init(bar_dempty, 1);
         *abort_flag = 0;
         fence_barrier_init();
@@ -274,13 +278,14 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     for (int ks = 0; ks < kstages; ++ks) {
                         if (!mbar_wait_warp(bar_sempty(ss), sphase ^ 1u, ctl, 102)) { ok = false; break; }
                         if (elect_one()) {
-                            mbar_expect_tx(bar_sfull(ss), C::KB_PER_STAGE * (sb_bytes + (rows ? BM * 4 : 0)));
+                            const uint32_t fb = bar_tfull(ss * C::GROUPS);
+                            mbar_expect_tx(fb, C::KB_PER_STAGE * (sb_bytes + (rows ? BM * 4 : 0)));
 #pragma unroll
                             for (int g = 0; g < C::KB_PER_STAGE; ++g)
                                 bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + g * BN * 4,
-                                          sb_t + (long long)(ks * C::KB_PER_STAGE + g) * p.n * 4, sb_bytes, bar_sfull(ss));
+                                          sb_t + (long long)(ks * C::KB_PER_STAGE + g) * p.n * 4, sb_bytes, fb);
                             if (rows) bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + C::SB_PART_BYTES,
-                                      sa_t + (long long)ks * p.m * (C::KB_PER_STAGE * 4), BM * C::KB_PER_STAGE * 4, bar_sfull(ss));
+                                      sa_t + (long long)ks * p.m * (C::KB_PER_STAGE * 4), BM * C::KB_PER_STAGE * 4, fb);
                         }
                         if (++ss == C::SB_STAGES) { ss = 0; sphase ^= 1u; }
                     }
@@ -371,7 +376,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         // one elected lane inside its wrapper.
         if (leader) {
             int stage = 0; uint32_t phase = 0;
-            int buf = 0; uint32_t bphase = 0;
+            int buf = 0, slot = 0; uint32_t bphase = 0;
             bool ok = true;
             constexpr uint32_t MDIM = (uint32_t)(BM * NCTA) >> 4;
             uint32_t idesc_full;
@@ -415,7 +420,8 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                         mma_f8f6f4<NCTA>(tmem_base + (buf * C::GPB + gi) * BN, adesc + 2 * jj, bdesc + 2 * jj, idesc, j > 0 ? 1u : 0u);
                                     }
                                 }
-                                tc_commit<NCTA>(bar_tfull(buf));
+                                tc_commit<NCTA>(bar_tfull(slot));
+                                if (++slot == C::FULL_SLOTS) slot = 0;
                                 if (++buf == C::ACC_BUFS) { buf = 0; bphase ^= 1u; }
                             }
                             if (!ok) break;
@@ -439,14 +445,60 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         auto release_acc = [&](int b) {
             if (NCTA == 2) mbar_arrive_cluster(bar_tempty(b) & PEER_BIT_MASK); else mbar_arrive(bar_tempty(b));
         };
-        int buf = 0; uint32_t bphase = 0;
-        int ss = 0; uint32_t sphase = 0;
+        int buf = 0, ss = 0;
+        uint32_t bphase = 0, sphase = 0;
         uint32_t store_cnt = 0;
         uint32_t dphase = 0;
-        bool ok = true, t_ready = false, s_ready = false;
+        bool ok = true;
         uint32_t accu[C::MX ? C::CW : 1];               // UE8M0: raw fp32 bits drained from TMEM
         uint32_t kept[C::MX ? 16 : 1];                  // ... and the 16 columns of a parked product that stay in registers
         unsigned long long acc2[C::MX ? 1 : C::CW / 2]; // FP32: promoted accumulators, two columns per register pair
+
+        // FP32 scales per column (ROWS4): the promotion, acc += (P * sB) * sA for every K block's partial product P, runs over
+        // chunks of 16 rows x 32 columns of TMEM with two register sets, the next chunk's load - of the next K block, stage or
+        // term as well - in flight while this one is added.  A stage's scales arrive on the barrier that says its first K
+        // blocks are multiplied: every wait costs a warp some 40 cycles that nothing hides with two warps to a scheduler.
+        // Block 32: 480 -> 440 cycles per 128 x 128 K block against 256 of arithmetic (cubic n = 4096 251 -> 234.5 us, n = 8192
+        // 1685 -> 1550 in bursts); block 128, n = 4096: 141.5 -> 129 in bursts.  The arithmetic alone runs at 293, with the
+        // TMEM loads and no barriers at 328, and the tensor cores' traffic costs another 40.  Measured around it: chunks of
+        // 64 columns 5 % slower; 16 promoting warps of a quarter of the columns 3 to 10 %; the next barrier tested ahead of
+        // the arithmetic 1.3 %, try_wait instead of test_wait 1 %; load shapes that are twice as fast need more scales a
+        // thread (16x64b, 16x32bx2: 2 to 12 %) or each scale twice (16x128b: 20 %); one set of barriers, and one issuing
+        // warp, per half of the columns gains nothing.
+        constexpr bool ROWS4 = C::ROWS4;
+        constexpr int KB = C::KB_PER_STAGE, CHUNKS = C::CW / 16;
+        constexpr int JG = C::CW / 8;                               // column groups of eight per warp
+        uint32_t set0[ROWS4 ? 16 : 1], set1[ROWS4 ? 16 : 1];
+        unsigned long long sb2[4];                                  // B-side scales of the chunk's 32 columns
+        float sa1[4];                                               // block 128: A-side scales of the thread's rows
+        const uint32_t tq = tmem_base + ((uint32_t)(q * 32) << 16) + h * C::CW;
+        // A-side scales of the thread's four rows (q*32 + lane/4 + 8k of this CTA's 128), per K block
+        const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + (lane >> 2)) * (KB * 4);
+        const uint32_t sb_lane = base + C::OFF_SB + (h * C::CW + 2 * (lane & 3)) * 4;
+        auto wait_full = [&](int slot, uint32_t phase) {
+            // test_wait: try_wait suspends the warp where the phase is not complete
+            const bool ready = mbar_test_wait(bar_tfull(slot), phase);
+            return __all_sync(0xffffffffu, ready) || mbar_wait_warp(bar_tfull(slot), phase, ctl, 303);
+        };
+        auto load_chunk = [&](uint32_t* r, int b, int gi, int i) {
+            tmem_ld_16x256b_x4(tq + (b * C::GPB + gi) * BN + (i >> 1) * 32 + ((uint32_t)(16 * (i & 1)) << 16), r);
+        };
+        auto load_sb = [&](unsigned long long (&d)[4], int s, int g, int cg) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d[j] = lds64(sb_lane + s * C::SB_STAGE_BYTES + (g * BN + cg * 32 + 8 * j) * 4);
+        };
+        auto load_sa1 = [&](float (&d)[4], int s) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[k] = lds32f(sa_lane + s * C::SB_STAGE_BYTES + 8 * k * 4);
+        };
+        if constexpr (ROWS4) {
+            ok = wait_full(0, 0);
+            tc_fence_after();
+            load_chunk(set0, 0, 0, 0);
+            load_sb(sb2, 0, 0, 0);
+            if constexpr (KB == 1) load_sa1(sa1, 0);
+            tmem_ld_wait16(set0);
+        }
         for (int w = unit; w < p.items && ok; w += units) {
             const int slot = w;
             const int grp = slot / p.positions, pos = slot - grp * p.positions;
@@ -471,7 +523,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
                     for (int i = 0; i < (C::MX ? 1 : C::CW / 2); ++i) acc2[i] = 0ull;
                 }
-                if (C::MX) {
+                if constexpr (C::MX) {
                     if (!mbar_wait_warp(bar_tfull(0), bphase, ctl, 301)) { ok = false; break; }
                     tc_fence_after();
 #pragma unroll
@@ -549,169 +601,117 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         }
                     }
                     continue;
-                } else if (C::ROWS4) {
+                } else if constexpr (ROWS4) {
                     // ---- per-column fp32 scales.  The accumulators are read with the
-                    // 16-lane load shape: a thread owns four rows (lane/4 + 8k) x CW/4 columns (8j + 2(lane%4), +1)
-                    // instead of one row x CW columns, so it needs CW/4 B-side scales per K block instead of CW (a
-                    // broadcast 16-byte shared-memory load returns 512 bytes to the register file; at one per four
-                    // elements those loads were a quarter of the promotion) and four A-side scales instead of one.
-                    static_assert(!C::ROWS4 || C::KB_PER_STAGE == 4 || C::KB_PER_STAGE == 1, "block 32 or 128");
-                    static_assert(!C::DUMP || C::ROWS4, "the output warp expects the four-row register layout");
-                    // acc2[k * (CW/8) + j]: row slot k, column group j
+                    // 16-lane load shape: a thread owns four rows (lane/4 + 8k) x CW/4 columns (8j + 2(lane%4), +1), so it
+                    // needs CW/4 B-side scales per K block instead of CW (a broadcast 16-byte shared-memory load returns 512
+                    // bytes to the register file; at one per four elements those loads were a quarter of the promotion) and
+                    // four A-side scales instead of one.
+                    static_assert(KB == 4 || KB == 1, "block 32 or 128");
+                    static_assert(CHUNKS % 2 == 0, "a K block begins with the first register set");
+                    // acc2[k * JG + j]: row slot k, column group j
 #pragma unroll
                     for (int i = 0; i < (CARRY ? C::CW / 2 : 0); ++i) acc2[i] = mul2(acc2[i], carry2);
-                    constexpr int JG = C::CW / 8;                               // column groups of eight per warp
-                    constexpr int KB = C::KB_PER_STAGE;
-                    // Block 32: the next buffer's and the next scale stage's barriers are tested before the last chunk's
-                    // arithmetic, which hides the test (about 70 cycles) when they are complete; they are waited for only
-                    // if they were not (n = 8192: 1792 -> 1740 us, cubic n = 4096: 268.5 -> 256.9).  With test_wait: try_wait
-                    // suspends the warp where the phase is not complete, which costs half of the gain and, on the barriers
-                    // that nothing follows on, 3.6 us per launch.  Block 128 has one buffer per stage, rarely complete that
-                    // early: no gain.
-                    constexpr bool PEEK = KB == 4;
-                    // A-side scales of the thread's four rows (q*32 + lane/4 + 8k of this CTA's 128), per K block
-                    const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + (lane >> 2)) * (KB * 4);
-                    const uint32_t sb_lane = base + C::OFF_SB + (h * C::CW + 2 * (lane & 3)) * 4;
+                    const bool more = left > 1 || w + units < p.items;          // another product after this one
                     for (int ks = 0; ks < kstages && ok; ++ks) {
-                        if (!(PEEK && __all_sync(0xffffffffu, s_ready)) && !mbar_wait_warp(bar_sfull(ss), sphase, ctl, 302)) { ok = false; break; }
-                        const uint32_t sbs32 = sb_lane + ss * C::SB_STAGE_BYTES;
-                        // the stage's K blocks for the thread's four rows, from the scale ring (a global load here, even
-                        // issued a stage early, stalled the promotion: 14 % of the block-32 kernel)
-                        float sa4[4][KB];
+                        const bool wrap = ss + 1 == C::SB_STAGES;
+                        const int sn = wrap ? 0 : ss + 1;
+                        const uint32_t pn = wrap ? sphase ^ 1u : sphase;
+                        // block 32: the stage's K blocks for the thread's four rows, from the scale ring (a global load here,
+                        // even issued a stage early, stalled the promotion: 14 % of the kernel)
+                        float sa4[KB == 4 ? 4 : 1][KB];
+                        if constexpr (KB == 4) {
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            if constexpr (KB == 4) {
+                            for (int k = 0; k < 4; ++k) {
                                 const float4 v4 = lds128(sa_lane + ss * C::SB_STAGE_BYTES + 8 * k * 16);
                                 sa4[k][0] = v4.x; sa4[k][1] = v4.y; sa4[k][2] = v4.z; sa4[k][3] = v4.w;
-                            } else {
-                                sa4[k][0] = lds32f(sa_lane + ss * C::SB_STAGE_BYTES + 8 * k * 4);
                             }
                         }
 #pragma unroll
-                        for (int g0 = 0; g0 < C::KB_PER_STAGE; g0 += C::GPB) {
-                            if (!(PEEK && __all_sync(0xffffffffu, t_ready)) && !mbar_wait_warp(bar_tfull(buf), bphase, ctl, 303)) { ok = false; break; }
-                            tc_fence_after();
+                        for (int g = 0; g < KB; ++g) {
+                            const int gi = g % C::GPB;
 #pragma unroll
-                            for (int gi = 0; gi < C::GPB; ++gi) {
-                                const int g = g0 + gi;
-                                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (buf * C::GPB + gi) * BN + h * C::CW;
-                                // the last chunk is in registers: hand the TMEM buffers back before the arithmetic
-                                auto release = [&]() {
-                                    tc_fence_before();
-                                    __syncwarp();
-                                    if (lane == 0) release_acc(buf);
-                                    if (PEEK) {
-                                        const bool tw = buf + 1 == C::ACC_BUFS, sw = ss + 1 == C::SB_STAGES;
-                                        t_ready = mbar_test_wait(bar_tfull(tw ? 0 : buf + 1), tw ? bphase ^ 1u : bphase);
-                                        if (g0 + C::GPB >= KB) s_ready = mbar_test_wait(bar_sfull(sw ? 0 : ss + 1), sw ? sphase ^ 1u : sphase);
-                                    }
-                                };
-                                // (P * sB) * sA rather than P * (sA * sB): see fmm_scale_down (products of scales ahead of the
-                                // TMEM wait: 7 % slower; behind it, in order: 8 %)
-                                if constexpr (C::CW == 64) {
-                                    // two chunks of 16 rows x 64 columns, the second one's load under the first one's arithmetic
-                                    // (1.5 % of the cubic product at n = 4096 against chunks of 32 x 32 without the overlap)
-                                    uint32_t lo[32], hi[32];
-                                    unsigned long long sb2[8];
-                                    tmem_ld_16x256b_x8(taddr, lo);                        // rows lane/4, lane/4 + 8
-#pragma unroll
-                                    for (int j = 0; j < 8; ++j) sb2[j] = lds64(sbs32 + (g * BN + 8 * j) * 4);
-                                    tmem_ld_wait();
-                                    tmem_ld_16x256b_x8(taddr + (16u << 16), hi);          // rows lane/4 + 16, lane/4 + 24
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) {
-                                        if (k == 2) {
-                                            tmem_ld_wait();
-                                            if (gi + 1 == C::GPB) release();
-                                        }
-                                        const unsigned long long sa2 = pack2(sa4[k][g], sa4[k][g]);
-                                        const uint32_t* src = (k < 2) ? lo : hi;
-#pragma unroll
-                                        for (int j = 0; j < 8; ++j) {
-                                            const uint32_t* tp = src + 4 * j + 2 * (k & 1);
-                                            acc2[k * JG + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + j]);
-                                        }
-                                    }
+                            for (int i = 0; i < CHUNKS; ++i) {
+                                uint32_t* cur = (i & 1) ? set1 : set0;
+                                uint32_t* nxt = (i & 1) ? set0 : set1;
+                                unsigned long long sbn[4];
+                                float san[4];
+                                int nb = buf;
+                                if (i + 1 < CHUNKS) {
+                                    load_chunk(nxt, buf, gi, i + 1);
+                                    if (i & 1) load_sb(sbn, ss, g, (i + 1) >> 1);
                                 } else {
-#pragma unroll
-                                    for (int c = 0; c < C::CW / 32; ++c) {   // chunks of 32 columns
-                                        uint32_t lo[16], hi[16];
-                                        tmem_ld_16x256b_x4(taddr + c * 32, lo);                       // rows lane/4, lane/4 + 8
-                                        tmem_ld_16x256b_x4(taddr + c * 32 + (16u << 16), hi);         // rows lane/4 + 16, lane/4 + 24
-                                        unsigned long long sb2[4];
-#pragma unroll
-                                        for (int j = 0; j < 4; ++j) sb2[j] = lds64(sbs32 + (g * BN + c * 32 + 8 * j) * 4);
-                                        tmem_ld_wait();
-                                        if (gi + 1 == C::GPB && c + 1 == C::CW / 32) release();
-#pragma unroll
-                                        for (int k = 0; k < 4; ++k) {
-                                            const unsigned long long sa2 = pack2(sa4[k][g], sa4[k][g]);
-                                            const uint32_t* src = (k < 2) ? lo : hi;
-#pragma unroll
-                                            for (int j = 0; j < 4; ++j) {
-                                                const uint32_t* tp = src + 4 * j + 2 * (k & 1);
-                                                acc2[k * JG + c * 4 + j] = fma2(mul2(pack2u(tp[0], tp[1]), sb2[j]), sa2, acc2[k * JG + c * 4 + j]);
-                                            }
-                                        }
-                                    }
-                                }
-                            }
-                            if (++buf == C::ACC_BUFS) { buf = 0; bphase ^= 1u; }
-                        }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(bar_sempty(ss));
-                        if (++ss == C::SB_STAGES) { ss = 0; sphase ^= 1u; }
-                    }
-                    if (!ok) break;
-                } else {
-#pragma unroll
-                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);
-                    // this thread's row (q*32 + lane of the CTA's 128) in the A-side part of a scale stage
-                    const uint32_t sa_lane = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + lane) * (C::KB_PER_STAGE * 4);
-                    for (int ks = 0; ks < kstages && ok; ++ks) {
-                        if (!mbar_wait_warp(bar_sfull(ss), sphase, ctl, 302)) { ok = false; break; }
-                        float sa[C::KB_PER_STAGE];
-#pragma unroll
-                        for (int g = 0; g < C::KB_PER_STAGE; ++g) sa[g] = lds32f(sa_lane + ss * C::SB_STAGE_BYTES + g * 4);
-                        const uint8_t* sbs = base_ptr + C::OFF_SB + ss * C::SB_STAGE_BYTES;
-#pragma unroll
-                        for (int g0 = 0; g0 < C::KB_PER_STAGE; g0 += C::GPB) {
-                            if (!mbar_wait_warp(bar_tfull(buf), bphase, ctl, 303)) { ok = false; break; }
-                            tc_fence_after();
-#pragma unroll
-                            for (int gi = 0; gi < C::GPB; ++gi) {
-                                const int g = g0 + gi;
-                                const ulonglong2* sbg = reinterpret_cast<const ulonglong2*>(sbs + (g * BN + h * C::CW) * 4);
-                                float sab = sa[g];
-                                if (MODE == MODE_FP32_SB_TILE) sab *= *reinterpret_cast<const float*>(sbs + (g * BN + h * C::CW) * 4);
-                                const unsigned long long sa2 = pack2(sab, sab);
-                                const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (buf * C::GPB + gi) * BN + h * C::CW;
-                                uint32_t tmp[32];
-#pragma unroll
-                                for (int c = 0; c < C::CW / 32; ++c) {
-                                    tmem_ld32(taddr + c * 32, tmp);      // a TMEM load round trip is a few tens of cycles
-                                    tmem_ld_wait();
-                                    if (gi + 1 == C::GPB && c + 1 == C::CW / 32) {
+                                    if (gi + 1 == C::GPB) {
                                         // the last chunk is in registers: hand the TMEM buffers back before the arithmetic
                                         tc_fence_before();
                                         __syncwarp();
                                         if (lane == 0) release_acc(buf);
+                                        nb = buf + 1 == C::ACC_BUFS ? 0 : buf + 1;
+                                        // (without another product the loads below fetch what nobody uses)
+                                        if (g + 1 < KB) ok = ok && wait_full(ss * C::GROUPS + (g + 1) / C::GPB, sphase);
+                                        else if (ks + 1 < kstages || more) ok = ok && wait_full(sn * C::GROUPS, pn);
+                                        tc_fence_after();
                                     }
+                                    load_chunk(nxt, nb, (gi + 1) % C::GPB, 0);
+                                    load_sb(sbn, g + 1 < KB ? ss : sn, (g + 1) % KB, 0);
+                                    if constexpr (KB == 1) load_sa1(san, sn);
+                                }
+                                // (P * sB) * sA rather than P * (sA * sB): see fmm_scale_down
 #pragma unroll
-                                    for (int i = 0; i < 8; ++i) {
-                                        const uint32_t* tp = tmp + 4 * i;
-                                        unsigned long long s01 = sa2, s23 = sa2;        // tile mode: sA * sB_tile
-                                        if (MODE != MODE_FP32_SB_TILE) {
-                                            const ulonglong2 s4 = sbg[c * 8 + i];        // four column scales
-                                            s01 = mul2(sa2, s4.x); s23 = mul2(sa2, s4.y);
-                                        }
-                                        acc2[c * 16 + 2 * i] = fma2(pack2u(tp[0], tp[1]), s01, acc2[c * 16 + 2 * i]);
-                                        acc2[c * 16 + 2 * i + 1] = fma2(pack2u(tp[2], tp[3]), s23, acc2[c * 16 + 2 * i + 1]);
+                                for (int k2 = 0; k2 < 2; ++k2) {
+                                    const int k = 2 * (i & 1) + k2;
+                                    const float s = KB == 4 ? sa4[KB == 4 ? k : 0][g] : sa1[k];
+                                    const unsigned long long sa2 = pack2(s, s);
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j) {
+                                        unsigned long long& acc = acc2[k * JG + (i >> 1) * 4 + j];
+                                        acc = fma2(mul2(pack2u(cur[4 * j + 2 * k2], cur[4 * j + 2 * k2 + 1]), sb2[j]), sa2, acc);
                                     }
                                 }
+                                if (i & 1) {
+#pragma unroll
+                                    for (int j = 0; j < 4; ++j) sb2[j] = sbn[j];
+                                }
+                                tmem_ld_wait16(nxt);
+                                if (KB == 1 && i + 1 == CHUNKS) {
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) sa1[k] = san[k];
+                                }
+                                if (i + 1 == CHUNKS) buf = nb;
                             }
-                            if (++buf == C::ACC_BUFS) { buf = 0; bphase ^= 1u; }
                         }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar_sempty(ss));
+                        ss = sn; sphase = pn;
+                    }
+                    if (!ok) break;
+                } else {
+                    // ---- weight tiles: one scale per row and K block, sA * sB_tile; a thread owns one row
+                    static_assert(C::GPB == 1 && KB == 1, "block 128");
+#pragma unroll
+                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);
+                    const uint32_t sa_row = base + C::OFF_SB + C::SB_PART_BYTES + (q * 32 + lane) * 4;
+                    for (int ks = 0; ks < kstages && ok; ++ks) {
+                        if (!mbar_wait_warp(bar_tfull(ss), sphase, ctl, 303)) { ok = false; break; }
+                        tc_fence_after();
+                        const float s = lds32f(sa_row + ss * C::SB_STAGE_BYTES) * lds32f(base + C::OFF_SB + h * C::CW * 4 + ss * C::SB_STAGE_BYTES);
+                        const unsigned long long s2 = pack2(s, s);
+#pragma unroll
+                        for (int c = 0; c < C::CW / 32; ++c) {
+                            // (the next chunk's load under this one's arithmetic, as above: 1.5 to 2 % slower)
+                            uint32_t tmp[32];
+                            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * BN + h * C::CW + c * 32, tmp);
+                            tmem_ld_wait();
+                            if (c + 1 == C::CW / 32) {
+                                // the last chunk is in registers: hand the TMEM buffer back before the arithmetic
+                                tc_fence_before();
+                                __syncwarp();
+                                if (lane == 0) release_acc(buf);
+                            }
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) acc2[c * 16 + j] = fma2(pack2u(tmp[2 * j], tmp[2 * j + 1]), s2, acc2[c * 16 + j]);
+                        }
+                        if (++buf == C::ACC_BUFS) buf = 0;
                         __syncwarp();
                         if (lane == 0) mbar_arrive(bar_sempty(ss));
                         if (++ss == C::SB_STAGES) { ss = 0; sphase ^= 1u; }
@@ -723,16 +723,16 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     // as 32 x 32 chunks in the 128-byte-swizzled layout of the output tensor map
                     if (!mbar_wait_warp(bar_dempty, dphase ^ 1u, ctl, 304)) { ok = false; break; }
                     dphase ^= 1u;
-                    // thread: rows lane/4 + 8k of the warp's 32-row chunk, column pairs 8j + 2(lane%4) of its 64 columns
+                    // thread: rows lane/4 + 8k of the warp's 32-row chunk, column pairs 8j + 2(lane%4) of its columns
                     const uint32_t dchunk = base + C::OFF_DUMP + (q * (BN / 32) + h * (C::CW / 32)) * 4096 + (lane & 1) * 8;
                     const unsigned long long up2 = pack2(p.up, p.up);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int rr = (lane >> 2) + 8 * k;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
+                        for (int j = 0; j < JG; ++j) {
                             const int pc = 2 * (j & 3) + ((lane & 3) >> 1);        // 16-byte piece of the 128-byte row
-                            sts64(dchunk + (j >> 2) * 4096 + rr * 128 + ((pc ^ (rr & 7)) << 4), mul2(acc2[k * 8 + j], up2));
+                            sts64(dchunk + (j >> 2) * 4096 + rr * 128 + ((pc ^ (rr & 7)) << 4), mul2(acc2[k * JG + j], up2));
                         }
                     }
                     fence_proxy_async();          // the output warp may hand these chunks to the TMA engine as they are
