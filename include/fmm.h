@@ -145,7 +145,7 @@ typedef struct {
     int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; cluster: 1 */
     int columns;                 /* columns of a tile */
     int k_shares;                /* cluster, one term: CTAs that share K (1, 2, 4, 8); otherwise 1 */
-    int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = a warp of its own writes the products out */
+    int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = every product is summed on its own and written by warps of its own; 0 = sums are carried from product to product */
 } fmm_product_shape_t;
 /* The shape that fmm_matmul and fmm_multiply_only take for this problem size (host call; errors as fmm_matmul). */
 fmm_status_t fmm_product_shape(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K, fmm_product_shape_t* shape);

@@ -448,13 +448,12 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
     std::vector<FmmWalkEntry> walk(2 * (size_t)p->terms);
     std::vector<FmmOutEntry> entries;
     const int parents = levels >= 1 ? p->terms / rank : 1;
-    const float up = fmm_scale_up(*qp);
     for (int carried = 1; carried >= 0; --carried) {
         int order[FMM_MAX_RANK];
         float carry[FMM_MAX_RANK] = {0.0f};
         for (int r = 0; r < FMM_MAX_RANK; ++r) order[r] = r;
         if (carried && levels >= 1 && qp->scale_mode == FMM_SCALE_FP32_AMAX_DIV_448) fmm_choose_walk(rank, p->U, p->V, p->W, order, carry);
-        std::vector<char> touched((size_t)parents * 4, 0);
+        std::vector<int> touched((size_t)parents * 4, -1);         // the last update of a block
         for (int t = 0; t < p->terms; ++t) {
             FmmWalkEntry& step = walk[t + (carried ? 0 : p->terms)];
             step.out0 = (int)entries.size();
@@ -465,9 +464,10 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
                 if (w == 0.0f) continue;
                 FmmOutEntry e;
                 e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1;
-                e.w = carried ? w * up : w;        // the output warp's kernel multiplies its sums, see fmm_scale_down
-                e.first = touched[(size_t)parent * 4 + q] ? 0 : 1;
-                touched[(size_t)parent * 4 + q] = 1;
+                e.w = w;
+                int& last = touched[(size_t)parent * 4 + q];
+                e.gap = last < 0 ? 0 : (int)entries.size() - last;
+                last = (int)entries.size();
                 entries.push_back(e);
             }
             step.out1 = (int)entries.size();

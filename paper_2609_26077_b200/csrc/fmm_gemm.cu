@@ -6,9 +6,10 @@
 // owns an output tile POSITION - the same (NCTA*128) x BN tile in every output block of C - and
 // walks all terms for it, so the W-weighted accumulation into C is race-free and deterministic.
 //
-//   warp 0      TMA producer: K-major e4m3 tiles of S_r and T_r (128-byte swizzle) + their scales.
+//   warp 0      TMA producer: K-major e4m3 tiles of S_r and T_r (128-byte swizzle), and where warp 2 does not their scales.
 //               In a pair each CTA loads its own 128 rows of S_r and its own half of the T_r tile.
 //   warp 1      tcgen05.mma issuer (the even CTA of a pair issues for both), fp32 accumulators in TMEM
+//   warps 2, 3  FP32 scales: scale producer, or (block 32) the two output warps, see MODE_FP32_OUT_WARP
 //   warps 4..11 epilogue (two warpgroups, given most of the register file with setmaxnreg): TMEM -> registers -> (x W[r][q]) -> swizzled smem -> TMA store / TMA
 //               add-reduce into the C blocks (the read-modify-write happens in L2, not in the SM)
 //
@@ -27,16 +28,17 @@
 
 namespace {
 
-// Internal fourth mode: FP32 scales (per column, as mode 0) with a dedicated output warp.  The promoting warps hand
-// a finished product to it through a shared-memory copy of the (unweighted) accumulators and go straight on with
-// the next term; the W-weighted stores / add-reductions then overlap the next term's promotion instead of stalling
-// it.  The output warp needs a fixed time per term, so this pays only when a term has many K stages (measured
-// cross-over near 16 stages of 128 k); the dispatcher picks the mode per launch.
+// Internal fourth mode: FP32 scales (per column, as mode 0) with two output warps.  The promoting warps hand a finished
+// product to them through a shared-memory copy of the (unweighted) accumulators, half of the rows to each, and go straight on
+// with the next term; the W-weighted stores / add-reductions then overlap the next term's promotion instead of stalling it.
+// One output warp was the bound of all but the longest terms: n = 4096, T* (16 stages a term) 265 -> 249 us, 4096 x 2048 x 4096
+// 153 -> 139; cubic and n = 8192 as before.  To make room one warp produces operands and scales.  Four output warps in a
+// block of 512 threads: short terms 5 % faster still, cubic 8 % slower (the promotion loop compiled for fewer registers).
 constexpr int MODE_FP32_OUT_WARP = 3;
-constexpr int OUT_WARP_STAGES = 16;        // ... K stages of a term from which on it is taken
+constexpr int SEPARATE_STAGES = 16;        // block 32: K stages of a term from which on every product is summed on its own, see launch()
 
 constexpr int EPI_WARPS = 8;               // two per TMEM lane quadrant, each half of the tile's columns
-constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, scale producer (FP32 modes), output warp
+constexpr int EPI_WARP0 = 4;               // warps 0..3: operand producer, MMA issuer, and two that produce scales or write the output
 constexpr int NUM_THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
 // setmaxnreg budget: the CTA's register pool is NUM_THREADS x (registers at launch); an increase
 // beyond what the decrease freed would block forever, so every split is checked (see Cfg).
@@ -50,10 +52,12 @@ struct Cfg {
     // CW/4 columns per thread (see the promotion loop).  The weight-tile mode has no per-column scale loads to
     // save and is faster with one row per thread.
     static constexpr bool ROWS4 = !MX && MODE != MODE_FP32_SB_TILE;
-    // Register split between the four control warps and the eight epilogue warps.  The block-128 kernels give the
-    // promoting warps all they can (accumulators + two TMEM chunks + scales); the others' epilogue needs less, and their
-    // control warps, which also handle scale tiles or the output, or hold values not known to be uniform, spill at 56.
-    static constexpr int REGS_CTRL = ROWS4 && BLK == 128 ? 56 : 88, REGS_EPI = ROWS4 && BLK == 128 ? 224 : 208;
+    static constexpr bool DUMP = (MODE == MODE_FP32_OUT_WARP);
+    // Register split between the four control warps and the eight epilogue warps.  Block 128 gives the promoting warps all
+    // they can (accumulators, two TMEM chunks, scales).  Block 32 with output warps needs less: with 176 to 200 registers
+    // ptxas finds a promotion loop that is 3 % faster than with 208 or more, with 168 it is 3 % slower (cubic n = 4096 233.4,
+    // 240.9, 247.5 us; block 128 is 2 to 7 % slower with fewer than 224).  Every split is one that ptxas spills nothing with.
+    static constexpr int REGS_CTRL = !ROWS4 || DUMP ? 88 : BLK == 32 ? 72 : 56, REGS_EPI = !ROWS4 ? 208 : DUMP ? 192 : BLK == 32 ? 216 : 224;
     static_assert(EPI_WARP0 * 32 * REGS_CTRL + EPI_WARPS * 32 * REGS_EPI <= NUM_THREADS * REGS_AT_LAUNCH, "register pool");
     // Warp index, CTA rank and TMEM base as values the compiler knows to be warp-uniform (see warp_uniform): 3 % of the
     // block-32 kernel at n = 8192 and 4096, 7 % of the single-CTA UE8M0 kernel at 1280 x 2816 x 3328.  Not for the UE8M0
@@ -66,7 +70,6 @@ struct Cfg {
     // The UE8M0 pair kernel keeps one staging chunk per epilogue warp: its shared memory goes to the operand stages,
     // and a second chunk in flight per warp was measured slower (more output traffic competing with the loads).
     static constexpr int STAGING_BUFS = (MX && NCTA == 2) ? 1 : 2;
-    static constexpr bool DUMP = (MODE == MODE_FP32_OUT_WARP);
     static_assert(!DUMP || (BN == 128 && BK / BLK == 4), "output-warp mode: 128-column tiles, block 32");
     static constexpr int STAGES = (MX && NCTA == 2) ? 5 : ((A_BYTES + B_BYTES) > 40000 || DUMP ? 3 : 4);
     // DUMP (output-warp mode): shared-memory copy of a finished product, BM x BN fp32
@@ -80,7 +83,7 @@ struct Cfg {
     static constexpr int SFB_ATOMS = BN / 128;
     static constexpr int SF_STAGE_BYTES = MX ? (512 + SFB_ATOMS * 512) : 0;
     static constexpr int KB_PER_STAGE = BK / BLK;
-    // depth of the scale ring: scales are small, so in the block-32 kernel with the output warp, which has the room,
+    // depth of the scale ring: scales are small, so in the block-32 kernel with output warps, which has the room,
     // they run several stages ahead of the operand tiles (2.5 % for the cubic product at n = 8192, neutral for rank 7)
     static constexpr int SB_STAGES = STAGES + (DUMP ? 5 : 1);
     // FP32 modes: one stage of the scale ring = the B-side scales of the stage's K blocks (KB x BN fp32, stored
@@ -92,7 +95,7 @@ struct Cfg {
     static constexpr int OFF_A = 0;
     static constexpr int OFF_B = OFF_A + STAGES * A_BYTES;
     static constexpr int OFF_STG = OFF_B + STAGES * B_BYTES;
-    static constexpr int OUT_BUFS = 8;          // DUMP: staging chunks of the output warp (TMA stores in flight)
+    static constexpr int OUT_BUFS = 8;          // DUMP: staging chunks of the two output warps
     static constexpr int OFF_DUMP = OFF_STG + (DUMP ? OUT_BUFS * 4096 : EPI_WARPS * STAGING_BUFS * STAGING_BYTES);
     static constexpr int OFF_SF = OFF_DUMP + DUMP_BYTES;
     static constexpr int OFF_SB = OFF_SF + STAGES * SF_STAGE_BYTES;
@@ -101,7 +104,7 @@ struct Cfg {
     static constexpr int GPB = MX ? 1 : ((KB_PER_STAGE >= 2 && 512 / BN >= 4) ? 2 : 1);
     static constexpr int GROUPS = KB_PER_STAGE / GPB;
     static constexpr int FULL_SLOTS = MX ? 1 : SB_STAGES * GROUPS;
-    static constexpr int NUM_BARS = 2 * STAGES + SB_STAGES + FULL_SLOTS + 4 + 2;
+    static constexpr int NUM_BARS = 2 * STAGES + SB_STAGES + FULL_SLOTS + 4 + 4;
     static constexpr int SMEM_BYTES = OFF_BAR + NUM_BARS * 8 + 16 + 1024;   // + alignment slack
     // TMEM: MX: one BN-column accumulator, then per stage 4 SFA + 4*(BN/128) SFB columns.
     //       FP32: ring of 512/BN accumulators, one per K block in flight.
@@ -147,7 +150,7 @@ struct KParams {
     const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
     int order[FMM_MAX_RANK]; short steps, R;           // walk order of the R products of a parent; steps = ceil(R / 2)
-    float up;                                 // output warp: factor of the sums (GemmParams); the others have it in their weights
+    float up;                                 // factor of the sums (GemmParams)
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
     FmmGuard guard;
@@ -173,8 +176,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     auto bar_sempty = [&](int s) { return bar0 + 8u * (2 * C::STAGES + s); };
     auto bar_tfull = [&](int b) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + b); };
     auto bar_tempty = [&](int b) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + C::FULL_SLOTS + b); };
-    const uint32_t bar_dfull = bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + C::FULL_SLOTS + 4);      // accumulator copy written
-    const uint32_t bar_dempty = bar_dfull + 8u;                                                       // ... and consumed
+    // DUMP: half of the rows of the accumulator copy is written, and consumed
+    auto bar_dfull = [&](int i) { return bar0 + 8u * (2 * C::STAGES + C::SB_STAGES + C::FULL_SLOTS + 4 + i); };
+    auto bar_dempty = [&](int i) { return bar_dfull(i) + 16u; };
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + C::OFF_BAR + C::NUM_BARS * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const Ctl ctl{abort_flag, p.status};
@@ -192,7 +196,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         // the first K blocks of a stage are signalled together with the stage's scales
         for (int b = 0; b < C::FULL_SLOTS; ++b) mbar_init(bar_tfull(b), !C::MX && b % C::GROUPS == 0 ? 2 : 1);
         for (int b = 0; b < 4; ++b) mbar_init(bar_tempty(b), NCTA * EPI_WARPS);
-        mbar_init(bar_dfull, EPI_WARPS); mbar_init(bar_dempty, 1);
+        for (int i = 0; i < 2; ++i) { mbar_init(bar_dfull(i), EPI_WARPS / 2); mbar_init(bar_dempty(i), 1); }
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -217,6 +221,44 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     };
     const int row_blocks_a = p.m / 128, row_blocks_b = p.n / 128;
 
+    // FP32 modes: the scales of the stages, in the order in which the promoting warps need them
+    struct ScaleProducer {
+        int w, ti, ks, ss;                          // the next stage's item, product and place in K, its place in the ring
+        uint32_t phase;
+        int sb_bytes; bool rows;
+        const uint8_t* sa; const uint8_t* sb;       // of stage 0 of the product
+        __device__ __forceinline__ void begin(int unit) { w = unit; ti = 0; ks = 0; ss = 0; phase = 0; }
+    };
+    constexpr int AHEAD = 2;
+    auto produce_scales = [&](ScaleProducer& c) {
+        if (c.w >= p.items) return true;
+        if (c.ks == 0) {
+            const int grp = c.w / p.positions, pos = c.w - grp * p.positions, tm = pos / tiles_n, tn = pos % tiles_n;
+            const int t = term_of(grp, c.ti);
+            c.sb = p.sb + (long long)t * p.sb_term + (long long)tn * BN * 4;
+            c.sa = p.sa + (long long)t * p.sa_term + (long long)(tm * NCTA + cta_rank) * BM * (C::KB_PER_STAGE * 4);
+            // a tile that hangs over the edge: only the scales that exist (those of its other rows or columns are whatever the
+            // ring held, as their products are never stored)
+            c.sb_bytes = min(BN, p.nsub - tn * BN) * 4;
+            c.rows = (tm * NCTA + cta_rank) * BM < p.msub;
+        }
+        if (!mbar_wait_warp(bar_sempty(c.ss), c.phase ^ 1u, ctl, 102)) return false;
+        if (elect_one()) {
+            const uint32_t fb = bar_tfull(c.ss * C::GROUPS), dst = base + C::OFF_SB + c.ss * C::SB_STAGE_BYTES;
+            mbar_expect_tx(fb, C::KB_PER_STAGE * (c.sb_bytes + (c.rows ? BM * 4 : 0)));
+#pragma unroll
+            for (int g = 0; g < C::KB_PER_STAGE; ++g)
+                bulk_load(dst + g * BN * 4, c.sb + (long long)(c.ks * C::KB_PER_STAGE + g) * p.n * 4, c.sb_bytes, fb);
+            if (c.rows) bulk_load(dst + C::SB_PART_BYTES, c.sa + (long long)c.ks * p.m * (C::KB_PER_STAGE * 4), BM * C::KB_PER_STAGE * 4, fb);
+        }
+        if (++c.ss == C::SB_STAGES) { c.ss = 0; c.phase ^= 1u; }
+        if (++c.ks == kstages) {
+            c.ks = 0;
+            if (++c.ti == p.terms_per_group) { c.ti = 0; c.w += units; }
+        }
+        return true;
+    };
+
     if (warp < EPI_WARP0) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(C::REGS_CTRL));
     if (warp == 0) {
@@ -226,6 +268,13 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             griddep_wait();        // the encoders' output is complete and visible (no-op unless launched to overlap them)
             int stage = 0; uint32_t phase = 0;
             bool ok = true;
+            ScaleProducer scales;
+            if constexpr (C::DUMP) {
+                // the scales run AHEAD stages in front of the operands; their ring is longer by more than that, so that the
+                // wait for a place in it is never longer than the one for the operands' place
+                scales.begin(unit);
+                for (int i = 0; i < AHEAD && ok; ++i) ok = produce_scales(scales);
+            }
             for (int w = unit; w < p.items && ok; w += units) {
                 const int slot = w;
                 const int grp = slot / p.positions, pos = slot - grp * p.positions;
@@ -250,126 +299,88 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             }
                         }
                         if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
+                        if constexpr (C::DUMP) { if (!produce_scales(scales)) { ok = false; break; } }
                     }
                 }
             }
         }
-    } else if (warp == 2) {
-        // ------------------------------------------------------------------ FP32 modes: producer of the B-side scales
+    } else if (warp == 2 && !C::MX && !C::DUMP) {
+        // ------------------------------------------------------------------ FP32 modes: producer of the scales
         // (its own thread and ring: the operand producer above has no registers to spare, and the scale ring is
         // released by the promoting warps, not by the tensor pipe)
-        if (!C::MX) {
-            griddep_wait();        // as the operand producer
-            int ss = 0; uint32_t sphase = 0;
-            bool ok = true;
-            for (int w = unit; w < p.items && ok; w += units) {
-                const int slot = w;
-                const int grp = slot / p.positions, pos = slot - grp * p.positions;
-                const int tn = pos % tiles_n;
-                const int tm = pos / tiles_n;
-                for (int ti = 0; ti < p.terms_per_group && ok; ++ti) {
-                    const int t = term_of(grp, ti);
-                    const uint8_t* sb_t = p.sb + (long long)t * p.sb_term + (long long)tn * BN * 4;
-                    const uint8_t* sa_t = p.sa + (long long)t * p.sa_term + (long long)(tm * NCTA + cta_rank) * BM * (C::KB_PER_STAGE * 4);
-                    // a tile that hangs over the edge: only the scales that exist (those of its other rows or columns are
-                    // whatever the ring held, as their products are never stored)
-                    const int sb_bytes = min(BN, p.nsub - tn * BN) * 4;
-                    const bool rows = (tm * NCTA + cta_rank) * BM < p.msub;
-                    for (int ks = 0; ks < kstages; ++ks) {
-                        if (!mbar_wait_warp(bar_sempty(ss), sphase ^ 1u, ctl, 102)) { ok = false; break; }
-                        if (elect_one()) {
-                            const uint32_t fb = bar_tfull(ss * C::GROUPS);
-                            mbar_expect_tx(fb, C::KB_PER_STAGE * (sb_bytes + (rows ? BM * 4 : 0)));
-#pragma unroll
-                            for (int g = 0; g < C::KB_PER_STAGE; ++g)
-                                bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + g * BN * 4,
-                                          sb_t + (long long)(ks * C::KB_PER_STAGE + g) * p.n * 4, sb_bytes, fb);
-                            if (rows) bulk_load(base + C::OFF_SB + ss * C::SB_STAGE_BYTES + C::SB_PART_BYTES,
-                                      sa_t + (long long)ks * p.m * (C::KB_PER_STAGE * 4), BM * C::KB_PER_STAGE * 4, fb);
-                        }
-                        if (++ss == C::SB_STAGES) { ss = 0; sphase ^= 1u; }
+        griddep_wait();            // as the operand producer
+        ScaleProducer scales;
+        scales.begin(unit);
+        while (scales.w < p.items && produce_scales(scales)) { }
+    } else if (C::DUMP && warp >= 2) {
+        // ------------------------------------------------------------------ FP32 scales, block 32: output warps
+        const int half = warp - 2;                                           // rows 64 half .. 64 half + 63 of the tile
+        constexpr int BUFS = C::OUT_BUFS / 2, CHS = 2 * (BN / 32);           // staging chunks; chunks of the copy
+        const uint32_t dump = base + C::OFF_DUMP + half * CHS * 4096, stg = base + C::OFF_STG + half * BUFS * 4096;
+        const uint64_t pol_c = policy_evict_last();                         // see the note on the C tiles' L2 policy below
+        uint32_t dphase = 0, cnt = 0;
+        bool ok = true;
+        for (int w = unit; w < p.items && ok; w += units) {
+            const int grp = w / p.positions, pos = w - grp * p.positions;
+            const int tm = pos / tiles_n, tn = pos % tiles_n;
+            const bool rows = (tm * NCTA + cta_rank) * BM < p.msub;            // else this CTA's half hangs over the edge
+            const int s_end = (grp + 1) * p.terms_per_group;
+            for (int s = s_end - p.terms_per_group; s < s_end && ok; ++s) {
+                const int o0 = p.walk[s].out0, o1 = rows ? p.walk[s].out1 : o0;
+                if (!mbar_wait_warp(bar_dfull(half), dphase, ctl, 401)) { ok = false; break; }
+                dphase ^= 1u;
+                bool any_direct = false;
+                for (int o = o0; o < o1; ++o) {
+                    const FmmOutEntry ent = p.out[o];
+                    const int row0 = ent.row_off * p.m + (tm * NCTA + cta_rank) * BM + half * 64, col0 = ent.col_off * p.n + tn * BN;
+                    // A weight of exactly 1 needs no copy: the promoting warps stored the chunks in the swizzled layout the
+                    // tensor map expects (and made them visible to the TMA engine), so they go out as they are.
+                    const bool direct = (ent.w == 1.0f);
+                    any_direct |= direct;
+                    // this warp's previous update of the same block, `gap` updates of CHS bulk groups ago, has landed
+                    if (lane == 0) {
+                        if (ent.gap == 1) bulk_wait<0>();
+                        else if (ent.gap == 2) bulk_wait<CHS>();
+                        else if (ent.gap >= 3) bulk_wait<2 * CHS>();
                     }
-                }
-            }
-        }
-    } else if (warp == 3) {
-        // ------------------------------------------------------------------ FP32 modes, 128-column tiles: output warp
-        if (C::DUMP) {
-            const uint32_t stg = base + C::OFF_STG + lane * 128;          // this lane's row of a staging chunk
-            const uint32_t dump = base + C::OFF_DUMP + lane * 128;        // ... and of a chunk of the accumulator copy
-            uint32_t dphase = 0, store_cnt = 0;
-            bool ok = true;
-            for (int w = unit; w < p.items && ok; w += units) {
-                const int slot = w;
-                const int grp = slot / p.positions, pos = slot - grp * p.positions;
-                const int tm = pos / tiles_n, tn = pos % tiles_n;
-                const bool rows = (tm * NCTA + cta_rank) * BM < p.msub;        // else this CTA's half hangs over the edge
-                const int s_end = (grp + 1) * p.terms_per_group;
-                for (int s = s_end - p.terms_per_group; s < s_end && ok; ++s) {
-                    if (!mbar_wait_warp(bar_dfull, dphase, ctl, 401)) { ok = false; break; }
-                    dphase ^= 1u;
-                    const int o0 = p.walk[s].out0, o1 = rows ? p.walk[s].out1 : o0;
-                    if (lane == 0) bulk_wait<0>();     // the previous term's writes to these tiles have landed
-                    __syncwarp();
-                    for (int o = o0; o < o1; ++o) {
-                        const FmmOutEntry ent = p.out[o];
-                        const int row0 = ent.row_off * p.m + (tm * NCTA + cta_rank) * BM;
-                        const int col0 = ent.col_off * p.n + tn * BN;
-                        // A weight of exactly 1 needs no copy: the promoting warps stored the chunks in the swizzled layout
-                        // the tensor map expects (and made them visible to the TMA engine), so they go out as they are.
-                        const bool direct = (ent.w == 1.0f);
 #pragma unroll 1
-                        for (int ch0 = 0; ch0 < (BM / 32) * (BN / 32); ch0 += C::OUT_BUFS / 2) {
-                            // OUT_BUFS/2 chunks of 32 rows x 32 columns per round (one proxy fence and one bulk group per
-                            // round, two rounds in flight); other weights are applied on the way through registers.
-                            const uint32_t b0 = (store_cnt & 1u) * (C::OUT_BUFS / 2);
-                            if (!direct) {
-                                if (lane == 0) bulk_wait_read<1>();
-                                __syncwarp();
-#pragma unroll 1
-                                for (int k = 0; k < C::OUT_BUFS / 2; ++k) {
-                                    const uint32_t src = dump + (ch0 + k) * 4096;
-                                    const uint32_t dst = stg + (b0 + k) * 4096;
-                                    // same physical piece on both sides (the swizzle is kept); the lane-dependent order only
-                                    // spreads the 32 rows over the shared-memory banks.  All loads are issued before the
-                                    // first store.
-                                    float4 v[8];
+                    for (int ch = 0; ch < CHS; ++ch) {
+                        const uint32_t from = dump + ch * 4096, to = stg + (cnt % BUFS) * 4096;
+                        if (!direct) {
+                            if (lane == 0) bulk_wait_read<BUFS - 1>();
+                            __syncwarp();
+                            // same physical piece on both sides (the swizzle is kept); the lane-dependent order only
+                            // spreads the 32 rows over the shared-memory banks.  All loads are issued before the first store.
+                            float4 v[8];
 #pragma unroll
-                                    for (int i4 = 0; i4 < 8; ++i4) v[i4] = lds128(src + ((i4 ^ (lane & 7)) << 4));
+                            for (int i4 = 0; i4 < 8; ++i4) v[i4] = lds128(from + lane * 128 + ((i4 ^ (lane & 7)) << 4));
 #pragma unroll
-                                    for (int i4 = 0; i4 < 8; ++i4) {
-                                        v[i4].x *= ent.w; v[i4].y *= ent.w; v[i4].z *= ent.w; v[i4].w *= ent.w;
-                                        sts128(dst + ((i4 ^ (lane & 7)) << 4), v[i4]);
-                                    }
-                                }
-                                fence_proxy_async();
-                                __syncwarp();
+                            for (int i4 = 0; i4 < 8; ++i4) {
+                                v[i4].x *= ent.w; v[i4].y *= ent.w; v[i4].z *= ent.w; v[i4].w *= ent.w;
+                                sts128(to + lane * 128 + ((i4 ^ (lane & 7)) << 4), v[i4]);
                             }
-                            if (lane == 0) {
-                                const uint64_t pol_c = policy_evict_last();     // see the note on the C tiles' L2 policy below
-                                const uint32_t src0 = direct ? (base + C::OFF_DUMP + ch0 * 4096) : (base + C::OFF_STG + b0 * 4096);
-#pragma unroll 1
-                                for (int k = 0; k < C::OUT_BUFS / 2; ++k) {
-                                    const int ch = ch0 + k;
-                                    const int r = row0 + (ch / (BN / 32)) * 32, c = col0 + (ch % (BN / 32)) * 32;
-                                    if (!FMM_GUARD(p.guard, p.c_base + (long long)r * p.ldc + c, (31 * p.ldc + 32) * 4, 1701)) continue;
-                                    if (ent.first) tma_store_2d_hint(&tmC, c, r, src0 + k * 4096, pol_c);
-                                    else tma_reduce_add_2d_hint(&tmC, c, r, src0 + k * 4096, pol_c);
-                                }
-                                bulk_commit();
+                            fence_proxy_async();
+                            __syncwarp();
+                            ++cnt;
+                        }
+                        if (lane == 0) {
+                            const uint32_t src = direct ? from : to;
+                            const int r = row0 + ch / (BN / 32) * 32, c = col0 + ch % (BN / 32) * 32;
+                            if (FMM_GUARD(p.guard, p.c_base + (long long)r * p.ldc + c, (31 * p.ldc + 32) * 4, 1701)) {
+                                if (ent.gap == 0) tma_store_2d_hint(&tmC, c, r, src, pol_c);
+                                else tma_reduce_add_2d_hint(&tmC, c, r, src, pol_c);
                             }
-                            if (!direct) ++store_cnt;
+                            bulk_commit();
                         }
                     }
-                    // the TMA engine has read the copy for the last time (chunks sent as they are), and so has every lane
-                    if (lane == 0) bulk_wait_read<0>();
-                    // every lane has read the copy for the last time
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_dempty);
                 }
+                // the TMA engine has read the copy for the last time (chunks sent as they are), and so has every lane
+                if (lane == 0 && any_direct) bulk_wait_read<0>();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_dempty(half));
             }
-            if (lane == 0) bulk_wait<0>();
         }
+        if (lane == 0) bulk_wait<0>();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (even CTA only in a pair)
         // The whole warp walks the loops (convergent, warp-uniform operands); each tcgen05 instruction is issued by
@@ -513,13 +524,11 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16) + h * cw;
             for (int ti = 0, left = p.terms_per_group; left > 0 && ok; ++ti, --left) {
                 const int t = C::MX ? term_of(grp, ti) : grp * p.terms_per_group + ti;      // FP32 scales: the step of the walk
-                // FP32 scales, no output warp: the sum starts from `carry` times the previous product's, still in the registers
-                // (the test of ti says nothing that the table does not).  With the output warp every product is summed on its
-                // own, see launch()
-                constexpr bool CARRY = !C::MX && !C::DUMP;
-                const float carry = (!CARRY || ti == 0) ? 0.0f : p.walk[t].carry;
+                // FP32 scales: the sum starts from `carry` times the previous product's, still in the registers (the test of ti
+                // says nothing that the table does not)
+                const float carry = (C::MX || ti == 0) ? 0.0f : p.walk[t].carry;
                 const unsigned long long carry2 = pack2(carry, carry);
-                if (!CARRY || carry == 0.0f) {          // not a product with zero: the sum before may not be finite
+                if (carry == 0.0f) {                    // not a product with zero: the sum before may not be finite
 #pragma unroll
                     for (int i = 0; i < (C::MX ? 1 : C::CW / 2); ++i) acc2[i] = 0ull;
                 }
@@ -611,7 +620,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     static_assert(CHUNKS % 2 == 0, "a K block begins with the first register set");
                     // acc2[k * JG + j]: row slot k, column group j
 #pragma unroll
-                    for (int i = 0; i < (CARRY ? C::CW / 2 : 0); ++i) acc2[i] = mul2(acc2[i], carry2);
+                    for (int i = 0; i < C::CW / 2; ++i) acc2[i] = mul2(acc2[i], carry2);
                     const bool more = left > 1 || w + units < p.items;          // another product after this one
                     for (int ks = 0; ks < kstages && ok; ++ks) {
                         const bool wrap = ss + 1 == C::SB_STAGES;
@@ -719,9 +728,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     if (!ok) break;
                 }
                 if (C::DUMP) {
-                    // ---- hand the finished product to the output warp: rows q*32 + lane, columns h*CW .. of the tile,
+                    // ---- hand the finished product to the output warps: rows q*32 + lane, columns h*CW .. of the tile,
                     // as 32 x 32 chunks in the 128-byte-swizzled layout of the output tensor map
-                    if (!mbar_wait_warp(bar_dempty, dphase ^ 1u, ctl, 304)) { ok = false; break; }
+                    if (!mbar_wait_warp(bar_dempty(q >> 1), dphase ^ 1u, ctl, 304)) { ok = false; break; }
                     dphase ^= 1u;
                     // thread: rows lane/4 + 8k of the warp's 32-row chunk, column pairs 8j + 2(lane%4) of its columns
                     const uint32_t dchunk = base + C::OFF_DUMP + (q * (BN / 32) + h * (C::CW / 32)) * 4096 + (lane & 1) * 8;
@@ -735,9 +744,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             sts64(dchunk + (j >> 2) * 4096 + rr * 128 + ((pc ^ (rr & 7)) << 4), mul2(acc2[k * JG + j], up2));
                         }
                     }
-                    fence_proxy_async();          // the output warp may hand these chunks to the TMA engine as they are
+                    fence_proxy_async();          // the output warps may hand these chunks to the TMA engine as they are
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(bar_dfull);
+                    if (lane == 0) mbar_arrive(bar_dfull(q >> 1));
                     continue;
                 }
                 // ---- post-addition: W-weighted scatter of this product into its C blocks
@@ -765,7 +774,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         if (C::ROWS4) {
                             // four-row layout: rows lane/4 + 8k, column pairs 8j + 2(lane%4) of this 32-column chunk
                             const uint32_t sdst = stg + b * C::STAGING_BYTES + (lane & 1) * 8;
-                            const unsigned long long w2 = pack2(ent.w, ent.w);
+                            const unsigned long long w2 = pack2(ent.w * p.up, ent.w * p.up);
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {
                                 const int rr = (lane >> 2) + 8 * k;
@@ -786,14 +795,14 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                                 unpack2(acc2[c * (C::CH / 2) + i4 * 2], v.x, v.y);
                                 unpack2(acc2[c * (C::CH / 2) + i4 * 2 + 1], v.z, v.w);
                             }
-                            v.x *= ent.w; v.y *= ent.w; v.z *= ent.w; v.w *= ent.w;
+                            v.x *= ent.w; v.y *= ent.w; v.z *= ent.w; v.w *= ent.w;        // weight tiles: p.up is 1
                             sts128(dst + ((i4 ^ swz) << 4), v);
                         }
                         fence_proxy_async();
                         __syncwarp();
                         if (lane == 0 && live()) {
                             if (FMM_GUARD(p.guard, p.c_base + (long long)row0 * p.ldc + col0 + c * C::CH, (31 * p.ldc + C::CH) * 4, 1702)) {
-                                if (ent.first) tma_store_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
+                                if (ent.gap == 0) tma_store_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
                                 else tma_reduce_add_2d_hint(&tmC, col0 + c * C::CH, row0, stg + b * C::STAGING_BYTES, pol_c);
                             }
                             bulk_commit();
@@ -837,7 +846,7 @@ int terms_per_item(const GemmParams& g, int positions, int units)
 }
 
 template <int BN, int MODE, int BLK, int NCTA>
-fmm_status_t launch(const GemmParams& g, cudaStream_t st)
+fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 {
     using C = Cfg<BN, MODE, BLK, NCTA>;
     CUtensorMap tmA, tmB, tmC, tmSFA, tmSFB;
@@ -879,11 +888,11 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st)
     kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.msub = g.msub; kp.nsub = g.nsub; kp.terms = g.terms;
     kp.positions = positions; kp.tiles_n = tiles_n; kp.terms_per_group = tpg;
     kp.items = slots;
-    // The output warp's kernel walks the second half of the table, in which every product is summed on its own.  The updates
-    // that carried sums save are mostly hidden behind the next product there (n = 8192: Phi-optimal 0.9 % of the call,
-    // Winograd at 6144 0.4 %; Strassen at 4096 is 1.6 % faster without, Phi-optimal 2.3 % slower), and with 64 and more K
-    // blocks a term they cost the most accuracy: 1.19 times the error for Winograd, 1.20 for Phi-optimal (n = 4096)
-    kp.walk = C::DUMP ? g.walk + g.terms : g.walk;
+    // In the second half of the table every product is summed on its own: with 64 and more K blocks a term the updates that
+    // carried sums save are hidden behind the next product (n = 8192: Phi-optimal 0.9 % of the call, Winograd at 6144 0.4 %;
+    // Strassen at 4096 is 1.6 % faster without, Phi-optimal 2.3 % slower), and they cost the most accuracy: 1.19 times the
+    // error for Winograd, 1.20 for Phi-optimal (n = 4096)
+    kp.walk = separate ? g.walk + g.terms : g.walk;
     kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = (short)g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
@@ -942,6 +951,11 @@ GemmShape best_shape(const GemmParams& g, int m, int n, const ShapeModel (&model
     return best;
 }
 
+// Block 32: whether the products are written by the output warps.  They need a fixed time per term: with fewer K stages the
+// promoting warps would wait for them (three levels n = 2048, two stages: 131 us with, 117 without; two levels 3072 x 2048 x 3072,
+// four stages: 121.0 and 123.5; 4096 x 2048 x 4096, eight stages: 138.9 and 153.2).
+bool output_warps(const GemmParams& g, const fmm_product_shape_t& s) { return s.output_warp || g.k / BK >= 4; }
+
 template <int MODE, int BLK>
 fmm_status_t launch_shape(const GemmParams& g, const fmm_product_shape_t& s, cudaStream_t st)
 {
@@ -953,10 +967,10 @@ fmm_status_t launch_shape(const GemmParams& g, const fmm_product_shape_t& s, cud
         return s.ctas == 2 ? launch<256, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     } else {
         // bound by the promotion on the CUDA cores: 128-column tiles, whose four TMEM accumulators let the MMA issuer run
-        // further ahead of the promoting warps.  Long terms: post-addition by the output warp.  (Block 128 does not gain
-        // from it: with 128-column tiles and the output warp it runs as fast as with 256-column tiles and none, 0.81 ms at
+        // further ahead of the promoting warps.  Post-addition by the output warps.  (Block 128 does not gain
+        // from them: with 128-column tiles and an output warp it runs as fast as with 256-column tiles and none, 0.81 ms at
         // n = 8192, and the cubic product, which has a single store per tile, is 20 % slower.)
-        if (s.output_warp) return s.ctas == 2 ? launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st) : launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st);
+        if (output_warps(g, s)) return s.ctas == 2 ? launch<128, MODE_FP32_OUT_WARP, BLK, 2>(g, st, s.output_warp) : launch<128, MODE_FP32_OUT_WARP, BLK, 1>(g, st, s.output_warp);
         return s.ctas == 2 ? launch<128, MODE, BLK, 2>(g, st) : launch<128, MODE, BLK, 1>(g, st);
     }
 }
@@ -976,7 +990,7 @@ fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
     const SplitChoice split = fmm_split_choice(g, blk, mode);
     if (split.ksplit > 0) return {2, 1, split.bn, split.ksplit, 0};
     const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
-    return {1, s.ncta, s.bn, 1, mode != FMM_SCALE_UE8M0_CEIL && blk == 32 && g.k / BK >= OUT_WARP_STAGES};
+    return {1, s.ncta, s.bn, 1, mode != FMM_SCALE_UE8M0_CEIL && blk == 32 && g.k / BK >= SEPARATE_STAGES};
 }
 
 bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R)

@@ -9,13 +9,13 @@
 
 #define FMM_MAX_LEVELS 3
 
-// One destination of a product in C: block origin, weight, and whether this is the first
-// product written there (store) or a later one (accumulate).  FP32 scales.
+// One destination of a product in C: block origin, weight, and whether this is the first product written there (store) or a
+// later one (accumulate, behind the one before).  FP32 scales.
 struct FmmOutEntry {
     int row_off;   // element row of the destination block origin in C
     int col_off;   // element column
     float w;       // product of the W coefficients along the recursion path
-    int first;     // 1: overwrite, 0: add
+    int gap;       // 0: overwrite; else add, and the previous update of this block is so many updates ago
 };
 
 // One step of the fp32-scale product kernel's walk over the leaf products: which term it multiplies, the factor of the
@@ -176,7 +176,7 @@ struct GemmParams {
     const uint8_t* qa; const uint8_t* qb;   // terms x m x k, terms x n x k
     const void* sa; const void* sb;         // sb, one fp32 scale per column: times fmm_scale_down
     int64_t sa_term, sb_term;               // bytes per term
-    float up;                               // fmm_scale_up (the persistent kernel's weights without output warp have it in them)
+    float up;                               // fmm_scale_up
     float* C; int64_t ldc;                  // full output
     int64_t Mfull, Nfull;
     int m, n, k, terms;
