@@ -8,7 +8,7 @@
 #include <vector>
 #include "fmm_internal.h"
 
-constexpr int HOST_STRIPS = 9;
+constexpr int HOST_STRIPS = 8;
 
 // Side streams and events of one fmm_matmul_host call in flight.
 struct HostLane {
@@ -713,12 +713,13 @@ static bool copy_strip(float* dst, const float* src, int64_t rows, int64_t cols,
 
 // Borders of the strips in sixteenths of the leaf extent.  A copy costs about 12 us besides its bytes while the link is used
 // both ways, so strips are few where the upload bounds the call and more where the download, which cannot begin before the
-// first strip has been multiplied, does too (n = 4096: nine 2.93 ms, five 3.10; 8192 x 1024 x 2048: 1.77 and 1.63).  The first
-// is short to start the download, the last short because its products and download follow the upload.
+// first strip has been multiplied, does too (n = 4096: eight 2.88 ms, five 3.13).  Of the
+// few, the first is short to start the download, the last short because its products and download follow the upload; more
+// equal or smaller strips cost more copies than they gain (n = 4096: nine with a shorter end 2.90, eleven 2.98, sixteen 3.34).
 static const int* strip_borders(int64_t upload, int64_t download, int* count)
 {
-    static const int nine[] = {0, 2, 4, 6, 8, 10, 12, 14, 15, 16}, five[] = {0, 2, 6, 10, 14, 16}, four[] = {0, 8, 12, 14, 16}, two[] = {0, 8, 16};
-    if (upload >= (32 << 20) && 5 * download > 3 * upload) { *count = 9; return nine; }
+    static const int eight[] = {0, 2, 4, 6, 8, 10, 12, 14, 16}, five[] = {0, 2, 6, 10, 14, 16}, four[] = {0, 8, 12, 14, 16}, two[] = {0, 8, 16};
+    if (upload >= (32 << 20) && 5 * download > 3 * upload) { *count = 8; return eight; }
     if (upload >= (32 << 20)) { *count = 5; return five; }
     if (upload >= (12 << 20)) { *count = 4; return four; }
     *count = upload >= (8 << 20) ? 2 : 1;
@@ -752,19 +753,26 @@ static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L,
     if (!sig(lane.up[strips], st, lane.comp)) return join(FMM_ERR_CUDA);
     fmm_status_t s = by_rows ? encode_side(plan, L, ws, dB, K, N, true, 0, L.n, false, lane.comp, &launches)
                              : encode_side(plan, L, ws, dA, M, K, false, 0, L.m, false, lane.comp, &launches);
+    // A strip of C goes down behind its product and the next strip's upload, that is with the upload after that one: a copy
+    // that starts while the other direction is busy takes some 45 us to get going, two that start together do not.
+    int last = -1;                             // the strip whose product was enqueued last
+    int64_t c_lo = 0, c_hi = 0;
+    auto send_down = [&]() {
+        return last < 0 || (sig(lane.mul[last], lane.comp, lane.down) && copy_strip(C, dC, M, N, blocks, by_rows, c_lo, c_hi, down, lane.down));
+    };
     for (int i = 0; i < strips && s == FMM_OK; ++i) {
         const int64_t lo = units * borders[i] / 16 * 128, hi = units * borders[i + 1] / 16 * 128;
         if (lo == hi) continue;
         Strip part = {0, L.m, 0, L.n};
         if (by_rows) { part.m0 = lo; part.m1 = hi; } else { part.n0 = lo; part.n1 = hi; }
         if (!copy_strip(by_rows ? dA : dB, by_rows ? A : B, by_rows ? M : K, by_rows ? K : N, blocks, by_rows, lo, hi, up, st) ||
-            !sig(lane.up[i], st, lane.comp)) return join(FMM_ERR_CUDA);
+            !sig(lane.up[i], st, lane.comp) || !send_down()) return join(FMM_ERR_CUDA);
         s = by_rows ? encode_side(plan, L, ws, dA, M, K, false, lo, hi, false, lane.comp, &launches)
                     : encode_side(plan, L, ws, dB, K, N, true, lo, hi, false, lane.comp, &launches);
         if (s == FMM_OK) s = multiply(plan, L, ws, dC, M, N, part, lane.comp, &launches, false);
-        if (s != FMM_OK) break;
-        if (!sig(lane.mul[i], lane.comp, lane.down) || !copy_strip(C, dC, M, N, blocks, by_rows, lo, hi, down, lane.down)) return join(FMM_ERR_CUDA);
+        last = i; c_lo = lo; c_hi = hi;
     }
+    if (s == FMM_OK && !send_down()) s = FMM_ERR_CUDA;
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return join(s);
 }
