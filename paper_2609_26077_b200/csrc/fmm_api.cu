@@ -204,7 +204,7 @@ fmm_status_t encode_outer(const fmm_plan* plan, const FmmLayout& L, char* ws, co
             s.out = reinterpret_cast<float*>(ws + inter[level]);
             s.guard = fmm_make_guard(s.out, (size_t)s.batch * s.R * (size_t)(s.rows * (int64_t)s.cols) * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
         }
-        const fmm_status_t s = fmm_launch_comb(c[0], c[1], level > 1, st);
+        const fmm_status_t s = fmm_launch_comb(c[0], c[1], st);
         if (s != FMM_OK) return s;
         ++*launches;
     }
@@ -243,7 +243,7 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
         const int64_t ext = hi - lo;               // rows of A / columns of B in this launch
         const bool panels = b_side ? (ext % (e.b_tile ? 512 : 256) == 0) : (ext % 4 == 0);
         e.in = X + strip_in; e.in_batch_stride = 0; e.ld = cols; e.batch = 1;
-        e.overlap_prev = b_side && overlap ? 1 : 0;
+        e.overlap_prev = overlap ? 1 : 0;
         e.s_ld = (int)(b_side ? cols : rows); e.sf_blocks = (int)((b_side ? cols : rows) / 128);
         if (panels) {
             e.nq = 4; e.R = 4;
@@ -273,9 +273,7 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
         const int64_t cur_rows = rows >> level, cur_cols = cols >> level, cur_ld = cur_cols, cur_stride = level ? cur_rows * cur_cols : 0;
         const int batch = (int)fmm_ipow(R, level);
         e.in = cur + strip_in; e.in_batch_stride = cur_stride; e.ld = cur_ld; e.batch = batch;
-        // see EncodeParams: the B-side encoder runs behind the A-side one, the A-side one behind the combinations if its side has
-        // any (they are launched for both sides at once, the deepest level last)
-        e.overlap_prev = b_side ? overlap : level > 0;
+        e.overlap_prev = overlap ? 1 : 0;
         const int div = fused2 ? 4 : 2;
         e.rows = (int)(cur_rows / div); e.cols = (int)(cur_cols / div); e.nq = 4; e.R = R;
         e.qoff[0] = 0; e.qoff[1] = e.cols; e.qoff[2] = (int64_t)e.rows * e.ld; e.qoff[3] = (int64_t)e.rows * e.ld + e.cols;

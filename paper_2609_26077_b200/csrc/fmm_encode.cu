@@ -234,7 +234,7 @@ template <int BLK, int MODE> struct RowsPerTask { static constexpr int value = M
 template <int BLK, int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_kernel(const EncodeParams p)
 {
-    fmmptx::griddep_wait();                        // the combinations of the level above, when this launch overlaps their tail
+    fmmptx::griddep_wait();                        // whatever is before this launch on the stream (launch_encoder)
     fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
     constexpr int GROUP = BLK / 4;                 // lanes per block
     const int lane = threadIdx.x & 31;
@@ -670,7 +670,7 @@ __device__ __forceinline__ void axpy(float4& acc, float w, const float4& x)
 // terms FMAs, zero coefficients skipped.  Both sides of a level in one launch (blockIdx.y).
 __global__ void __launch_bounds__(256) comb_kernel(const CombParams pa, const CombParams pb)
 {
-    fmmptx::griddep_wait();                        // the level above, when this launch overlaps its tail
+    fmmptx::griddep_wait();                        // the level above, or whatever is before the call on the stream
     const CombParams& p = blockIdx.y ? pb : pa;
     if (blockIdx.x * 8u >= (uint32_t)p.rows * ((uint32_t)p.cols / 128) || (int)blockIdx.z >= p.batch) return;
     const OuterIndex at = outer_index(p.cols);
@@ -787,10 +787,10 @@ __global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
 }  // namespace
 
 namespace {
-// Launch that may begin under the tail of the kernel before it on the stream (which wrote what this one reads: it waits for
-// it before its first load), so that its launch latency and set-up are hidden.
+// Launch that may begin under the tail of what is before it on the stream (the kernel waits for that before its first load),
+// so that its launch latency and set-up are hidden.
 template <typename K, typename... A>
-fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, bool overlap, const A&... args)
+fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, const A&... args)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -798,7 +798,7 @@ fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, boo
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = overlap ? 1 : 0;
+    cfg.attrs = at; cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, args...);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
@@ -807,14 +807,14 @@ fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, boo
 fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st)
 {
     const unsigned tiles = (unsigned)(p.cols / 128);
-    if (steps == 2) return launch_behind(decode2_kernel, dim3((unsigned)(p.rows / 4) * tiles), dim3(32, 4), st, true, p);
-    return launch_behind(decode_kernel, dim3((unsigned)(p.rows / 8) * tiles, 1, (unsigned)p.batch), dim3(32, 8), st, true, p);
+    if (steps == 2) return launch_behind(decode2_kernel, dim3((unsigned)(p.rows / 4) * tiles), dim3(32, 4), st, p);
+    return launch_behind(decode_kernel, dim3((unsigned)(p.rows / 8) * tiles, 1, (unsigned)p.batch), dim3(32, 8), st, p);
 }
 
-fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, bool overlap, cudaStream_t st)
+fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, cudaStream_t st)
 {
     const unsigned ga = (unsigned)(a.rows / 8) * (unsigned)(a.cols / 128), gb = (unsigned)(b.rows / 8) * (unsigned)(b.cols / 128);
-    return launch_behind(comb_kernel, dim3(ga > gb ? ga : gb, 2, (unsigned)(a.batch > b.batch ? a.batch : b.batch)), dim3(32, 8), st, overlap, a, b);
+    return launch_behind(comb_kernel, dim3(ga > gb ? ga : gb, 2, (unsigned)(a.batch > b.batch ? a.batch : b.batch)), dim3(32, 8), st, a, b);
 }
 
 namespace {
@@ -835,8 +835,11 @@ uint32_t coef_mask(const EncodeParams& p)
 // Launch of an encoder.  With p.overlap_prev it carries the programmatic-serialization attribute.  B side: the kernel
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
 // begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192); what it
-// reads, the caller's matrix or combinations of a kernel before the A-side one, is complete.  A side: set up under the
-// tail of the combinations it reads.
+// reads, the caller's matrix or combinations of a kernel before the A-side one, is complete.  A side: its launch latency falls
+// under the tail of whatever is before it, the caller's kernels or the previous call, whose operands and workspace it touches
+// only behind its wait (2 us of a call at every size: n = 256 10.3 -> 7.9 us of device time, 1024 block 128 16.4 -> 14.2,
+// 1280 x 3328 x 2816 UE8M0 42.0 -> 40.0).  The product kernels do not signal early for it: its blocks would take the
+// places of their last CTAs' successors (Winograd, block 128, n = 4096 127 -> 137).
 template <typename K>
 void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p, unsigned cluster = 1)
 {
