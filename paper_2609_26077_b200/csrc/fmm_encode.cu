@@ -429,11 +429,11 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             if (coef_used<NZ>(r, jq, cj)) {
                 if (!set) {
 #pragma unroll
-                    for (int kk = 0; kk < 16; ++kk) v[kk] = __fmul_rn(cj, raw[jq][kk]);
+                    for (int kk = 0; kk < 16; kk += 2) unpack2(mul2(pack2(cj, cj), pack2(raw[jq][kk], raw[jq][kk + 1])), v[kk], v[kk + 1]);
                     set = true;
                 } else {
 #pragma unroll
-                    for (int kk = 0; kk < 16; ++kk) v[kk] = __fmaf_rn(cj, raw[jq][kk], v[kk]);
+                    for (int kk = 0; kk < 16; kk += 2) unpack2(fma2(pack2(cj, cj), pack2(raw[jq][kk], raw[jq][kk + 1]), pack2(v[kk], v[kk + 1])), v[kk], v[kk + 1]);
                 }
             }
         }
@@ -498,8 +498,7 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             uint32_t wv[4];
 #pragma unroll
             for (int g = 0; g < 4; ++g)
-                wv[g] = pack4_e4m3(__fmul_rn(v[4 * g], inv), __fmul_rn(v[4 * g + 1], inv),
-                                   __fmul_rn(v[4 * g + 2], inv), __fmul_rn(v[4 * g + 3], inv));
+                wv[g] = scaled_pack4(make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]), inv);
             uint8_t* qp = p.q_out + t * term_codes + (int64_t)j * p.rows + k0;
             if (FMM_GUARD(p.guard, qp, 16, 1204)) *reinterpret_cast<uint4*>(qp) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
