@@ -211,10 +211,10 @@ fmm_status_t encode_outer(const fmm_plan* plan, const FmmLayout& L, char* ws, co
     return FMM_OK;
 }
 
-// One side of steps 1-2, behind encode_outer: the innermost one or two levels and the quantizer.  [lo, hi) is the strip of
-// leaf rows (A) or columns (B) to encode: everything, or with at most one level a part of it (multiples of 128).
-fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* X,
-                         int64_t rows, int64_t cols, bool b_side, int64_t lo, int64_t hi, bool overlap, cudaStream_t st, int* launches)
+// Parameters of one side of steps 1-2, behind encode_outer: the innermost one or two levels and the quantizer.  [lo, hi) is the
+// strip of leaf rows (A) or columns (B) to encode: everything, or with at most one level a part of it (multiples of 128).
+EncodeParams encode_params(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* X,
+                           int64_t rows, int64_t cols, bool b_side, int64_t lo, int64_t hi, bool overlap)
 {
     const int R = plan->rank, lv = plan->levels;
     const int blk = plan->qp.block_k, mode = (int)plan->qp.scale_mode;
@@ -234,7 +234,6 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
     const int64_t strip_in = b_side ? lo : lo * cols;
     e.q_out += lo * L.k;
     e.s_out = static_cast<char*>(e.s_out) + (mode == FMM_SCALE_UE8M0_CEIL ? lo / 128 * 512 : lo * 4 * (b_side ? 1 : 128 / blk));
-    fmm_status_t s;
     if (lv == 0) {
         // Plain quantization of the matrix itself.  The matrix is cut into four panels (row panels of A,
         // column panels of B) that are handled like four "combinations" with identity coefficients, so
@@ -282,14 +281,39 @@ fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, con
         e.s_step = 0; e.s_ld = b_side ? e.cols : e.rows; e.sf_blocks = (b_side ? e.cols : e.rows) / 128;
         e.q_term = (int64_t)e.rows * e.cols;
         if (b_side) e.cols = (int)(hi - lo); else e.rows = (int)(hi - lo);
-        if (fused2) {
-            s = b_side ? fmm_launch_encode2_b(e, mode, st) : fmm_launch_encode2_a(e, blk, mode, st);
+    }
+    return e;
+}
+
+fmm_status_t encode_side(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* X,
+                         int64_t rows, int64_t cols, bool b_side, int64_t lo, int64_t hi, bool overlap, cudaStream_t st, int* launches)
+{
+    const int blk = plan->qp.block_k, mode = (int)plan->qp.scale_mode;
+    const EncodeParams e = encode_params(plan, L, ws, X, rows, cols, b_side, lo, hi, overlap);
+    fmm_status_t s;
+    if (plan->levels >= 2 && fmm_encode2_supported(b_side, blk, e.b_tile, e.preround_bf16))
+        s = b_side ? fmm_launch_encode2_b(e, mode, st) : fmm_launch_encode2_a(e, blk, mode, st);
+    else
+        s = b_side ? fmm_launch_encode_b(e, blk, mode, st) : fmm_launch_encode_a(e, blk, mode, st);
+    if (s == FMM_OK) ++*launches;
+    return s;
+}
+
+// Steps 1-2 of a whole call.
+fmm_status_t encode_all(const fmm_plan* plan, const FmmLayout& L, char* ws, const float* A, const float* B, int64_t M, int64_t N, int64_t K,
+                        cudaStream_t st, int* launches)
+{
+    if (plan->levels <= 1) {
+        fmm_status_t s;
+        if (fmm_launch_encode_both(encode_params(plan, L, ws, A, M, K, false, 0, L.m, true), encode_params(plan, L, ws, B, K, N, true, 0, L.n, true),
+                                   plan->qp.block_k, (int)plan->qp.scale_mode, st, &s)) {
             if (s == FMM_OK) ++*launches;
             return s;
         }
     }
-    s = b_side ? fmm_launch_encode_b(e, blk, mode, st) : fmm_launch_encode_a(e, blk, mode, st);
-    if (s == FMM_OK) ++*launches;
+    fmm_status_t s = encode_outer(plan, L, ws, A, B, M, N, K, st, launches);
+    if (s == FMM_OK) s = encode_side(plan, L, ws, A, M, K, false, 0, L.m, true, st, launches);
+    if (s == FMM_OK) s = encode_side(plan, L, ws, B, K, N, true, 0, L.n, true, st, launches);
     return s;
 }
 
@@ -615,9 +639,7 @@ fmm_status_t fmm_encode_only(const fmm_plan_t* plan, const float* A, const float
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_outer(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
+    s = encode_all(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;
 }
@@ -644,9 +666,7 @@ fmm_status_t fmm_matmul(const fmm_plan_t* plan, const float* A, const float* B, 
     if (s != FMM_OK) return s;
     int launches = 0;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    s = encode_outer(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), A, M, K, false, 0, L.m, true, st, &launches);
-    if (s == FMM_OK) s = encode_side(plan, L, static_cast<char*>(ws), B, K, N, true, 0, L.n, true, st, &launches);
+    s = encode_all(plan, L, static_cast<char*>(ws), A, B, M, N, K, st, &launches);
     if (s == FMM_OK) s = multiply(plan, L, static_cast<char*>(ws), C, M, N, {0, L.m, 0, L.n}, st, &launches, true);
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return s;

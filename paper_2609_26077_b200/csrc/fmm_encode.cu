@@ -227,19 +227,11 @@ __device__ __forceinline__ void store_chunk_a(const EncodeParams& p, const float
 // Rows that a task of the A-side encoder walks together (its rows are multiples of 32: of 128, or 128 / 4 in row panels).
 template <int BLK, int MODE> struct RowsPerTask { static constexpr int value = MODE == FMM_SCALE_FP32_AMAX_DIV_448 && BLK == 32 ? 2 : 1; };
 
-// Blocks per SM.  Block 128 with a known zero pattern: four, although 64 registers spill up to 48 bytes (both sides, n = 4096:
-// Winograd 39.1 us against 40.9 with three blocks, n = 8192 146.2 against 147.6).  Without one the spills are nine times that
-// and three blocks are faster (4096: 71.0 -> 67.5, 8192: 254 -> 234).  Block 32: three, and the 4 bytes that the power-of-two
-// kernel without a zero pattern spills then cost less than two blocks would (n = 4096: 51.5 against 56.6).
 template <int BLK, int MODE, uint32_t NZ>
-__global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_kernel(const EncodeParams p)
+__device__ __forceinline__ void encode_a_tasks(const EncodeParams& p, uint32_t warp_gid, uint32_t nwarps)
 {
-    fmmptx::griddep_wait();                        // whatever is before this launch on the stream (launch_encoder)
-    fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
     constexpr int GROUP = BLK / 4;                 // lanes per block
     const int lane = threadIdx.x & 31;
-    const uint32_t warp_gid = blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5);
-    const uint32_t nwarps = gridDim.x * 8;
     const int chunks = p.cols / 128;
     // a task is CPT consecutive 128-k chunks of one output row (two adjacent rows at block 32 with fp32 scales).  Tasks
     // are dealt to warps round-robin (32-bit index arithmetic only: one division per task, none per chunk; the warp index
@@ -292,6 +284,18 @@ __global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_k
     }
 }
 
+// Blocks per SM.  Block 128 with a known zero pattern: four, although 64 registers spill up to 48 bytes (both sides, n = 4096:
+// Winograd 39.1 us against 40.9 with three blocks, n = 8192 146.2 against 147.6).  Without one the spills are nine times that
+// and three blocks are faster (4096: 71.0 -> 67.5, 8192: 254 -> 234).  Block 32: three, and the 4 bytes that the power-of-two
+// kernel without a zero pattern spills then cost less than two blocks would (n = 4096: 51.5 against 56.6).
+template <int BLK, int MODE, uint32_t NZ>
+__global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_kernel(const EncodeParams p)
+{
+    fmmptx::griddep_wait();                        // whatever is before this launch on the stream (launch_encoder)
+    fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
+    encode_a_tasks<BLK, MODE, NZ>(p, blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5), gridDim.x * 8);
+}
+
 // ---------------------------------------------------------------------------------------------
 // B side.  Blocks run along k, the strided axis of row-major B, and the output is K-major (the
 // tensor-core operand layout).  A thread owns 16 consecutive k of one column n; lanes l and l+16
@@ -305,7 +309,7 @@ __global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_k
 // warps of one 128-k chunk per block; blocks of two to eight warps side by side, covering 128- to 512-byte row
 // segments, are within 1 %).  Grid: (cols / 16, rows / 32, batch), 32 threads.
 template <int MODE, uint32_t NZ>
-__global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p)
+__device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x;
@@ -377,6 +381,11 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
             if (FMM_GUARD(p.guard, qp, 16, 1207)) *reinterpret_cast<uint4*>(qp) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
     }
+}
+
+// End of a B-side encoder.
+__device__ __forceinline__ void end_of_b_side()
+{
     // the product kernel, launched behind this one by the same call, may be scheduled as soon as every block has got
     // here: its launch latency and set-up then fall under this grid's last blocks (signalling at the start instead lets
     // its CTAs take SMs from this grid's tail: 0.5 % slower back to back)
@@ -384,6 +393,13 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
     // a launch that overlapped the A-side encoder must not end before it (what follows on the stream needs both):
     // the last block of the grid waits for it, the others leave as they finish
     if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
+}
+
+template <int MODE, uint32_t NZ>
+__global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p)
+{
+    encode_b32_block<MODE, NZ>(p);
+    end_of_b_side();
 }
 
 // B side, block 128, one pass.  The four warps of a block take the four 32-k sub-blocks of one
@@ -398,7 +414,7 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
 // operand); every column stores the tile's scale, so the scale array keeps its per-column shape.  PRE rounds each encoded
 // combination to bfloat16 (nearest even) before the maximum and the cast, as the paper's real kernel does.
 template <uint32_t NZ, bool TILE, bool PRE>
-__global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams p)
+__device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
 {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int MODE = FMM_SCALE_FP32_AMAX_DIV_448;
@@ -503,14 +519,34 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
             if (FMM_GUARD(p.guard, qp, 16, 1204)) *reinterpret_cast<uint4*>(qp) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
         }
     }
-    // the product kernel, launched behind this one by the same call, may be scheduled as soon as every block has got
-    // here: its launch latency and set-up then fall under this grid's last blocks (signalling at the start instead lets
-    // its CTAs take SMs from this grid's tail: 0.5 % slower back to back)
-    fmmptx::griddep_launch_dependents();
-    // a launch that overlapped the A-side encoder must not end before it (what follows on the stream needs both):
-    // the last block of the grid waits for it, the others leave as they finish
-    if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
+}
+
+template <uint32_t NZ, bool TILE, bool PRE>
+__global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams p)
+{
+    encode_b128_block<NZ, TILE, PRE>(p);
+    end_of_b_side();
     if (TILE) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");           // its own maxima are no longer read either
+}
+
+// Both sides of a call in one launch, for calls whose cost is their launches: the blocks of the B-side encoder, and behind
+// them (gridDim.y - pb.rows / BLK rows of blocks) warps for the A side's tasks.
+template <int BLK, int MODE, uint32_t NZA, uint32_t NZB, bool TILE, bool PRE>
+__global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) encode_both_kernel(const __grid_constant__ EncodeParams pa, const __grid_constant__ EncodeParams pb)
+{
+    fmmptx::griddep_wait();                        // whatever is before this launch on the stream
+    const uint32_t b_rows = (uint32_t)pb.rows / BLK;
+    const bool b_side = blockIdx.y < b_rows;
+    if (b_side) {
+        if constexpr (BLK == 32) encode_b32_block<MODE, NZB>(pb);
+        else encode_b128_block<NZB, TILE, PRE>(pb);
+    } else {
+        constexpr uint32_t WARPS = BLK / 32;
+        encode_a_tasks<BLK, MODE, NZA>(pa, ((blockIdx.y - b_rows) * gridDim.x + blockIdx.x) * WARPS + fmmptx::warp_uniform(threadIdx.x >> 5),
+                                       (gridDim.y - b_rows) * gridDim.x * WARPS);
+    }
+    fmmptx::griddep_launch_dependents();           // as end_of_b_side
+    if (TILE && b_side) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -641,13 +677,7 @@ __global__ void __launch_bounds__(256) encode2_b_kernel(const EncodeParams p)
             }
         }
     }
-    // the product kernel, launched behind this one by the same call, may be scheduled as soon as every block has got
-    // here: its launch latency and set-up then fall under this grid's last blocks (signalling at the start instead lets
-    // its CTAs take SMs from this grid's tail: 0.5 % slower back to back)
-    fmmptx::griddep_launch_dependents();
-    // a launch that overlapped the A-side encoder must not end before it (what follows on the stream needs both):
-    // the last block of the grid waits for it, the others leave as they finish
-    if (blockIdx.x + 1 == gridDim.x && blockIdx.y + 1 == gridDim.y && blockIdx.z + 1 == gridDim.z) fmmptx::griddep_wait();
+    end_of_b_side();
 }
 
 // Streaming kernels of the outer recursion levels.  A block is 8 rows x 32 float4 of a matrix, a thread one float4 of every
@@ -830,8 +860,10 @@ uint32_t coef_mask(const EncodeParams& p)
 // Phi-optimal realization, and (one-level kernels) the identity used to quantize a matrix as four panels
 #define FMM_REALIZATION_MASKS(X) X(0x0a5381c9u) X(0x0c385a19u) X(0x05dc8f21u) X(0x0ab3f841u) X(0x0f5fc5c9u) X(0x0cfc5f59u)
 #define FMM_KNOWN_MASKS(X) FMM_REALIZATION_MASKS(X) X(0x00008421u)
+// U and V of each
+#define FMM_KNOWN_MASK_PAIRS(X) X(0x0a5381c9u, 0x0c385a19u) X(0x05dc8f21u, 0x0ab3f841u) X(0x0f5fc5c9u, 0x0cfc5f59u) X(0x00008421u, 0x00008421u)
 
-// Launch of an encoder.  With p.overlap_prev it carries the programmatic-serialization attribute.  B side: the kernel
+// Launch of an encoder.  With `overlap` it carries the programmatic-serialization attribute.  B side: the kernel
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
 // begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192); what it
 // reads, the caller's matrix or combinations of a kernel before the A-side one, is complete.  A side: its launch latency falls
@@ -839,8 +871,8 @@ uint32_t coef_mask(const EncodeParams& p)
 // only behind its wait (2 us of a call at every size: n = 256 10.3 -> 7.9 us of device time, 1024 block 128 16.4 -> 14.2,
 // 1280 x 3328 x 2816 UE8M0 42.0 -> 40.0).  The product kernels do not signal early for it: its blocks would take the
 // places of their last CTAs' successors (Winograd, block 128, n = 4096 127 -> 137).
-template <typename K>
-void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const EncodeParams& p, unsigned cluster = 1)
+template <typename K, typename... P>
+void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, unsigned cluster, bool overlap, const P&... p)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -851,8 +883,8 @@ void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, cons
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     // without a cluster only the second one, or none
-    cfg.attrs = cluster > 1 ? at : at + 1; cfg.numAttrs = (cluster > 1 ? 1 : 0) + (p.overlap_prev ? 1 : 0);
-    cudaLaunchKernelEx(&cfg, kernel, p);
+    cfg.attrs = cluster > 1 ? at : at + 1; cfg.numAttrs = (cluster > 1 ? 1 : 0) + (overlap ? 1 : 0);
+    cudaLaunchKernelEx(&cfg, kernel, p...);
 }
 
 template <int BLK, int MODE>
@@ -860,10 +892,10 @@ void launch_a(const EncodeParams& p, unsigned g, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_encoder(encode_a_kernel<BLK, MODE, M>, dim3(g), 256, st, p); return;
+#define X(M) case M: launch_encoder(encode_a_kernel<BLK, MODE, M>, dim3(g), 256, st, 1, p.overlap_prev, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_encoder(encode_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, p); return;
+        default: launch_encoder(encode_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, 1, p.overlap_prev, p); return;
     }
 }
 template <int MODE>
@@ -871,10 +903,10 @@ void launch_b32(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_encoder(encode_b32_kernel<MODE, M>, grid, 32, st, p); return;
+#define X(M) case M: launch_encoder(encode_b32_kernel<MODE, M>, grid, 32, st, 1, p.overlap_prev, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_encoder(encode_b32_kernel<MODE, 0u>, grid, 32, st, p); return;
+        default: launch_encoder(encode_b32_kernel<MODE, 0u>, grid, 32, st, 1, p.overlap_prev, p); return;
     }
 }
 template <bool TILE, bool PRE>
@@ -882,46 +914,64 @@ void launch_b128(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     const uint32_t m = (p.nq == 4) ? coef_mask(p) : 0u;
     switch (m) {
-#define X(M) case M: launch_encoder(encode_b128_kernel<M, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
+#define X(M) case M: launch_encoder(encode_b128_kernel<M, TILE, PRE>, grid, 128, st, TILE ? 8 : 1, p.overlap_prev, p); return;
         FMM_KNOWN_MASKS(X)
 #undef X
-        default: launch_encoder(encode_b128_kernel<0u, TILE, PRE>, grid, 128, st, p, TILE ? 8 : 1); return;
+        default: launch_encoder(encode_b128_kernel<0u, TILE, PRE>, grid, 128, st, TILE ? 8 : 1, p.overlap_prev, p); return;
     }
 }
 template <int BLK, int MODE>
 void launch_a2(const EncodeParams& p, unsigned g, cudaStream_t st)
 {
     switch (coef_mask(p)) {
-#define X(M) case M: launch_encoder(encode2_a_kernel<BLK, MODE, M>, dim3(g), 256, st, p); return;
+#define X(M) case M: launch_encoder(encode2_a_kernel<BLK, MODE, M>, dim3(g), 256, st, 1, p.overlap_prev, p); return;
         FMM_REALIZATION_MASKS(X)
 #undef X
-        default: launch_encoder(encode2_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, p); return;
+        default: launch_encoder(encode2_a_kernel<BLK, MODE, 0u>, dim3(g), 256, st, 1, p.overlap_prev, p); return;
     }
 }
 template <int MODE>
 void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
 {
     switch (coef_mask(p)) {
-#define X(M) case M: launch_encoder(encode2_b_kernel<MODE, M>, grid, 256, st, p); return;
+#define X(M) case M: launch_encoder(encode2_b_kernel<MODE, M>, grid, 256, st, 1, p.overlap_prev, p); return;
         FMM_REALIZATION_MASKS(X)
 #undef X
-        default: launch_encoder(encode2_b_kernel<MODE, 0u>, grid, 256, st, p); return;
+        default: launch_encoder(encode2_b_kernel<MODE, 0u>, grid, 256, st, 1, p.overlap_prev, p); return;
     }
+}
+template <int BLK, int MODE, bool TILE, bool PRE>
+bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, cudaStream_t st)
+{
+    constexpr unsigned THREADS = BLK == 32 ? 32 : 128;
+    const unsigned gx = (unsigned)b.cols / 16, a_blocks = (a_warps + THREADS / 32 - 1) / (THREADS / 32);
+    const dim3 grid(gx, (unsigned)b.rows / BLK + (a_blocks + gx - 1) / gx);
+    const uint32_t ma = coef_mask(a), mb = coef_mask(b);
+#define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE>, grid, THREADS, st, TILE ? 8 : 1, true, a, b); return true; }
+    FMM_KNOWN_MASK_PAIRS(X)
+#undef X
+    return false;
+}
+
+// Tasks of the A-side encoder, one per warp; sets their length.  Long tasks keep two steps of loads in flight, but a problem has
+// to have tasks for about half the resident warps (n = 2048, block 32: one task per eight chunks 15 us for both sides, per two
+// 10 us; n = 4096: per eight 36.8, per two 39).
+int64_t a_side_tasks(EncodeParams& p, int blk, int mode)
+{
+    const int chunks = p.cols / 128, rpt = (mode == FMM_SCALE_FP32_AMAX_DIV_448 && blk == 32) ? 2 : 1;
+    const int64_t row_tasks = (int64_t)p.batch * (p.rows / rpt);
+    const int64_t want = (int64_t)fmm_sm_count() * 10;
+    int64_t tpr = (chunks + 7) / 8;
+    while (row_tasks * tpr < want && chunks > 2 * tpr) tpr *= 2;
+    p.cpt = (int)((chunks + tpr - 1) / tpr);
+    return row_tasks * ((chunks + p.cpt - 1) / p.cpt);
 }
 }  // namespace
 
 fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st)
 {
     // one task per warp; the block scheduler balances the SMs
-    const int chunks = p.cols / 128, rpt = (mode == FMM_SCALE_FP32_AMAX_DIV_448 && blk == 32) ? 2 : 1;
-    const int64_t row_tasks = (int64_t)p.batch * (p.rows / rpt);
-    // long tasks keep two steps of loads in flight, but a problem has to have tasks for about half the resident warps
-    // (n = 2048, block 32: one task per eight chunks 15 us for both sides, per two 10 us; n = 4096: per eight 36.8, per two 39)
-    const int64_t want = (int64_t)fmm_sm_count() * 10;
-    int64_t tpr = (chunks + 7) / 8;
-    while (row_tasks * tpr < want && chunks > 2 * tpr) tpr *= 2;
-    p.cpt = (int)((chunks + tpr - 1) / tpr);
-    int64_t blocks = (row_tasks * ((chunks + p.cpt - 1) / p.cpt) + 7) / 8;
+    int64_t blocks = (a_side_tasks(p, blk, mode) + 7) / 8;
     if (blocks > 0x7fffffff) blocks = 0x7fffffff;
     const unsigned g = (unsigned)blocks;
     if (mode == FMM_SCALE_FP32_AMAX_DIV_448) {
@@ -943,6 +993,29 @@ fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaS
     else if (p.preround_bf16) launch_b128<false, true>(p, grid, st);
     else launch_b128<false, false>(p, grid, st);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+
+// One launch for both sides where the call's cost is its launches (2.6 us of host time, 0.4 to 1.3 us of the device's): up to so
+// many warps per SM.  Above that the A side is better off with the registers and blocks of its own kernel.  Both ways, in us,
+// Phi-optimal, n = 512 / 1024 / 2048 / 3072: UE8M0 10.2, 9.7 / 14.0, 13.1 / 32.0, 32.5 / 57.9, 61.1; weight tiles 11.3, 10.0 /
+// 15.3, 14.4 / 38.9, 37.7 / 76.9, 80.1; block 128 9.3, 8.8 / 13.9, 13.5 / 39.4, 38.2 / 69.1, 72.1; block 32 15.2, 13.0 / 17.2, 17.7 /
+// 64.8, 64.8 / 107, 111 (768: 12.3, 12.9).  The B side's blocks come first: they take longer (the other way round nothing is gained).
+bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int mode, cudaStream_t st, fmm_status_t* status)
+{
+    if (a.nq != 4 || b.nq != 4 || a.batch != 1 || b.batch != 1) return false;
+    const int64_t warps = a_side_tasks(a, blk, mode);
+    const int64_t b_warps = (int64_t)(b.cols / 16) * (b.rows / 32);
+    if (warps + b_warps > (int64_t)fmm_sm_count() * (blk == 128 ? 32 : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? 16 : 4)) return false;
+    const unsigned w = (unsigned)warps;
+    bool known;
+    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) known = launch_both<32, FMM_SCALE_UE8M0_CEIL, false, false>(a, b, w, st);
+    else if (blk == 32) known = launch_both<32, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, st);
+    else if (b.b_tile && b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, true>(a, b, w, st);
+    else if (b.b_tile) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, false>(a, b, w, st);
+    else if (b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, true>(a, b, w, st);
+    else known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, st);
+    if (known) *status = cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+    return known;
 }
 
 bool fmm_encode2_supported(bool b_side, int blk, int b_tile, int preround_bf16)

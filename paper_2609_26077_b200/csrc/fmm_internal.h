@@ -166,6 +166,8 @@ fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st
 // one level of combinations of the two sides (a side with rows == 0 has none)
 fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, cudaStream_t st);
 fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st);
+// both sides of a small call in one launch: false if it is not one, or has coefficients without kernels of their own
+bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int mode, cudaStream_t st, fmm_status_t* status);
 fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaStream_t st);
 // last two recursion levels in one pass (p.rows x p.cols = leaf dimensions, inputs 4*rows x 4*cols)
 bool fmm_encode2_supported(bool b_side, int blk, int b_tile, int preround_bf16);
