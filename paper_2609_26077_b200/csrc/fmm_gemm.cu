@@ -931,10 +931,13 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 // against the rule before, which gave wide tiles only to leaves that are multiples of them: UE8M0 8192 x 8192 x 8448 one
 // level 674 -> 492 us, cubic 4096 x 1024 x 4224 47.6 -> 26.4; block 128 8192 x 8192 x 8448 956 -> 787; weight tiles
 // 888 -> 664.
+// Block 128: with the faster promotion the single CTAs have gained more than the pairs, whose constants are fitted again, to 666
+// problems (5 % faster on the 7 % of them that change; cubic n = 4096 122.3 -> 115.7 us a call, two levels 270 -> 257; the pairs stay at
+// n = 8192, 739 against 781, cubic 718 against 893).
 struct ShapeModel { int ncta, bn; float c, o, o_cubic; };
 constexpr ShapeModel MODEL_MX[] = {{2, 256, 0.26f, 3.9f, 3.6f}, {1, 256, 0.35f, 3.4f, 2.7f}, {1, 128, 0.22f, 1.7f, 1.2f}};
 constexpr ShapeModel MODEL_B32[] = {{2, 128, 0.71f, 3.6f, 2.2f}, {1, 128, 0.67f, 3.55f, 1.85f}};
-constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 5.6f, 3.9f}, {1, 128, 0.28f, 2.5f, 1.8f}};
+constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 6.0f, 5.1f}, {1, 128, 0.28f, 2.5f, 1.8f}};
 constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.34f, 4.8f, 2.35f}, {1, 128, 0.26f, 2.4f, 1.15f}};
 constexpr float BASE_MX = 3.3f, BASE_B32 = 2.4f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
 
