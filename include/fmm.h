@@ -111,7 +111,8 @@ fmm_status_t fmm_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t N, i
  *   the same holds for every call that takes a plan and touches the device.
  * Asynchronous on cuda_stream.  Calls sharing a workspace must be stream-ordered; a plan may be shared by host
  * threads (it is read-only during a call, apart from the launch counter below).  Towards other work on the stream a
- * call is ordinary stream-ordered work: its first kernel starts after everything enqueued before it has completed, and
+ * call is ordinary stream-ordered work: its first kernel, which is set up under the tail of what is enqueued before it, touches
+ * nothing until all of that has completed, and
  * whatever is enqueued after it starts after all of its kernels have completed.  Between themselves the kernels of one
  * call overlap where they do not depend on each other (programmatic dependent launch: the B-side encoder starts under
  * the A-side encoder's last wave, the product kernel is set up under the B-side encoder's last blocks). */
@@ -141,7 +142,8 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
  * How the leaf products of a call are multiplied. */
 typedef struct {
     int kernel;                  /* 1: persistent kernel, a CTA or CTA pair walks the terms of a tile position;
-                                    2: cluster kernel, one CTA per term and tile (or per share of K, where there is one term) */
+                                    2: cluster kernel, one CTA per term and tile (or per share of K, where there is one term);
+                                    4: the same, UE8M0, one CTA per two terms and tile */
     int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; cluster: 1 */
     int columns;                 /* columns of a tile */
     int k_shares;                /* cluster, one term: CTAs that share K (1, 2, 4, 8); otherwise 1 */

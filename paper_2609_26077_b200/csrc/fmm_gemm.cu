@@ -991,7 +991,7 @@ fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
 {
     if (g.forced.kernel) return g.forced;
     const SplitChoice split = fmm_split_choice(g, blk, mode);
-    if (split.ksplit > 0) return {2, 1, split.bn, split.ksplit, 0};
+    if (split.ksplit > 0) return {split.terms == 2 ? 4 : 2, 1, split.bn, split.ksplit, 0};
     const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
     return {1, s.ncta, s.bn, 1, mode != FMM_SCALE_UE8M0_CEIL && blk == 32 && g.k / BK >= SEPARATE_STAGES};
 }
@@ -999,6 +999,7 @@ fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
 bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R)
 {
     const bool mx = mode == FMM_SCALE_UE8M0_CEIL;
+    if (s.kernel == 4) return mx && R > 1 && s.ctas == 1 && s.columns == 128 && s.k_shares == 1 && !s.output_warp;
     if (s.kernel == 2) {
         const bool width = s.columns == 128 || (!mx && (s.columns == 64 || s.columns == 32));
         const bool shares = s.k_shares == 1 || (R == 1 && (s.k_shares == 2 || s.k_shares == 4 || s.k_shares == 8));
@@ -1022,7 +1023,8 @@ fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_
 {
     fmm_status_t s;
     const fmm_product_shape_t shape = fmm_choose_product(g, blk, mode);
-    if (shape.kernel == 2) s = shape.k_shares <= g.k / BK ? fmm_launch_split(g, blk, mode, {shape.k_shares, shape.columns}, st) : FMM_ERR_SHAPE;
+    if (shape.kernel == 2 || shape.kernel == 4)
+        s = shape.k_shares <= g.k / BK ? fmm_launch_split(g, blk, mode, {shape.k_shares, shape.columns, shape.kernel / 2}, st) : FMM_ERR_SHAPE;
     else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, shape, st);
     else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, shape, st);
     else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, shape, st);

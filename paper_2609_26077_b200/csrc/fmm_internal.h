@@ -208,7 +208,7 @@ struct GemmShape { int ncta, bn; float time; };
 GemmShape fmm_gemm_shape(const GemmParams& p, int blk, int mode, int m, int n);
 // How the cluster kernel (fmm_split.cu) takes this product: K shares per term and columns per tile; 0 shares: the persistent
 // kernel is faster
-struct SplitChoice { int ksplit, bn; };
+struct SplitChoice { int ksplit, bn, terms; };        // terms: of a CTA
 SplitChoice fmm_split_choice(const GemmParams& p, int blk, int mode);
 // The forced shape, or the one that is expected to be fastest.  The kernel is chosen for the whole problem (m, n), also when
 // a launch covers a strip of it (msub, nsub): the strips' results do not depend on the cut

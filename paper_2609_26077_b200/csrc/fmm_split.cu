@@ -13,6 +13,11 @@
 // waits for its first operands while the other multiplies.  Promotion and exchange take time in proportion to the tile's
 // columns, so where the narrower tiles still find room at once they are the faster ones (see the time models below).
 //
+// With UE8M0 scales a CTA may multiply two of the terms, one after the other: clusters of ceil(R / 2) fit the GPCs where clusters
+// of 7 leave 86 of 296 places empty, and hold 64 tiles at once instead of 30.  The first product waits in registers until the
+// operand ring is free; three halves of 64 columns fit over the ring, so the exchange goes in two passes.  (With FP32 scales the
+// registers hold the running sums, and neither TMEM nor shared memory has room for another product beside a second CTA.)
+//
 //   warp 0  TMA producer of the operand tiles (UE8M0: and of the scale tiles)
 //   warp 1  tcgen05.mma issuer
 //   warp 2  FP32 scales: producer of both sides' scales
@@ -36,9 +41,10 @@ struct SplitParams {
     FmmGuard guard;
 };
 
-template <int MODE, int BLK, int BN_>
+template <int MODE, int BLK, int BN_, int TPC = 1>
 struct SplitCfg {
     static constexpr bool MX = (MODE == FMM_SCALE_UE8M0_CEIL);
+    static_assert(TPC == 1 || (TPC == 2 && MX), "terms per CTA");
     static constexpr int BN = BN_;                           // columns of a tile
     static_assert(BN == 128 || (!MX && (BN == 64 || BN == 32)), "tile widths");
     static constexpr int EPI_WARPS = 4, EPI_WARP0 = 4, THREADS = (EPI_WARP0 + EPI_WARPS) * 32;
@@ -64,6 +70,9 @@ struct SplitCfg {
     static_assert(SMEM_BYTES + 1024 <= 233472 / 2, "two CTAs per SM");
     static constexpr int ROW_BYTES = BN * 4;                 // exchange tile: bytes and 16-byte pieces per row
     static_assert(BM * ROW_BYTES <= OFF_SF, "the exchange tile lies inside the operand ring");
+    // two terms: halves of 64 columns, [first product's left | second product's, one half after the other | first's right]
+    static constexpr int HALF_BYTES = BM * 64 * 4;
+    static_assert(TPC == 1 || 3 * HALF_BYTES <= OFF_SF, "three halves lie inside the operand ring");
 };
 
 __device__ __forceinline__ uint32_t cluster_id_x()
@@ -77,12 +86,12 @@ __device__ __forceinline__ float4 ld_cluster128(uint32_t addr)
     return v;
 }
 
-template <int MODE, int BLK, int BN>
-__global__ void __launch_bounds__(SplitCfg<MODE, BLK, BN>::THREADS, 2)
+template <int MODE, int BLK, int BN, int TPC>
+__global__ void __launch_bounds__(SplitCfg<MODE, BLK, BN, TPC>::THREADS, 2)
 fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmSFA, const __grid_constant__ CUtensorMap tmSFB, const SplitParams p)
 {
-    using C = SplitCfg<MODE, BLK, BN>;
+    using C = SplitCfg<MODE, BLK, BN, TPC>;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;       // the same offset in every CTA of the cluster
@@ -117,10 +126,10 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t tmem_base = warp_uniform(*tmem_slot);
 
     // grid (S * tiles_n, tiles_m, parents), clusters of S along x: no index needs a division
-    const int S = p.R * p.ksplit, rank = (int)warp_uniform(cluster_ctarank());
+    const int S = TPC == 2 ? (p.R + 1) / 2 : p.R * p.ksplit, rank = (int)warp_uniform(cluster_ctarank());
     const int parent = blockIdx.z, tm = blockIdx.y, tn = (int)warp_uniform(cluster_id_x());
-    const int r = p.R == 1 ? 0 : rank, kpart = p.R == 1 ? rank : 0;
-    const int t = parent * p.R + r;
+    const int r = p.R == 1 ? 0 : TPC * rank, kpart = p.R == 1 ? rank : 0;
+    const int t0 = parent * p.R + r, nt = TPC == 2 && r + 1 < p.R ? 2 : 1;       // this CTA's terms: t0 .. t0 + nt - 1
     const int kstages = p.k / BK;
     const int ks0 = kstages * kpart / p.ksplit, ks1 = kstages * (kpart + 1) / p.ksplit;
     const uint32_t tile = base + C::OFF_TILE;
@@ -132,8 +141,10 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             griddep_wait();        // the encoders' output is complete and visible (no-op unless launched to overlap them)
             int stage = 0; uint32_t phase = 0;
             const int nq4 = p.k / BK, row_blocks_a = p.m / 128, row_blocks_b = p.n / 128;
+            bool ok = true;
+            for (int t = t0; t < t0 + nt && ok; ++t)
             for (int ks = ks0; ks < ks1; ++ks) {
-                if (!mbar_wait_warp(bar_empty(stage), phase ^ 1u, ctl, 121)) break;
+                if (!mbar_wait_warp(bar_empty(stage), phase ^ 1u, ctl, 121)) { ok = false; break; }
                 if (elect_one()) {
                     mbar_expect_tx(bar_full(stage), C::TX_BYTES);
                     tma_load_2d<1>(base + C::OFF_A + stage * C::A_BYTES, &tmA, ks * BK, t * p.m + tm * BM, bar_full(stage));
@@ -150,8 +161,8 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             // ------------------------------------------------------------------ producer of both sides' fp32 scales
             griddep_wait();
             int ss = 0; uint32_t sphase = 0;
-            const uint8_t* sb_t = p.sb + (long long)t * p.sb_term + (long long)tn * BN * 4;
-            const uint8_t* sa_t = p.sa + (long long)t * p.sa_term + (long long)tm * BM * (C::KB * 4);
+            const uint8_t* sb_t = p.sb + (long long)t0 * p.sb_term + (long long)tn * BN * 4;
+            const uint8_t* sa_t = p.sa + (long long)t0 * p.sa_term + (long long)tm * BM * (C::KB * 4);
             for (int ks = ks0; ks < ks1; ++ks) {
                 if (!mbar_wait_warp(bar_sempty(ss), sphase ^ 1u, ctl, 122)) break;
                 if (elect_one()) {
@@ -171,6 +182,11 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int buf = 0; uint32_t bphase = 0;
             bool ok = true;
             constexpr uint32_t idesc = (C::MX ? (1u << 23) : (1u << 4)) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+            for (int tt = 0; tt < nt && ok; ++tt) {
+            if (tt > 0) {                                    // the first product has left its accumulator
+                if (!mbar_wait_warp(bar_tempty(0), 0, ctl, 223)) { ok = false; break; }
+                tc_fence_after();
+            }
             for (int ks = ks0; ks < ks1 && ok; ++ks) {
                 if (!mbar_wait_warp(bar_full(stage), phase, ctl, 221)) { ok = false; break; }
                 tc_fence_after();
@@ -205,8 +221,10 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if (++stage == C::STAGES) { stage = 0; phase ^= 1u; }
             }
             if (C::MX && ok) tc_commit<1>(bar_tfull(0));
+            }
         }
         cluster_sync();                                      // every CTA's partial product is in its shared memory
+        if (TPC == 2) { cluster_sync(); cluster_sync(); }    // as below
     } else {
         // ---------------------------------------------------------------------- promotion / drain, exchange, output
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(C::REGS_EPI));
@@ -214,6 +232,88 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         const uint32_t lane_taddr = tmem_base + ((uint32_t)(q * 32) << 16);
         bool ok = true;
         // The exchange tile: row-major fp32, the row's 16-byte pieces permuted by piece ^ (row & 7).
+        if constexpr (TPC == 2) {
+            uint32_t v[64];
+            auto put_half = [&](uint32_t region) {
+                const int row = q * 32 + lane;
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    sts128(tile + region * C::HALF_BYTES + row * 256 + ((i ^ (row & 7)) << 4),
+                           make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3])));
+            };
+            auto load_half = [&](int h) {
+                tmem_ld32(lane_taddr + h * 64, v); tmem_ld32(lane_taddr + h * 64 + 32, v + 32);
+                tmem_ld_wait();
+            };
+            // the first product waits in registers for the operand ring to be free
+            uint32_t first[128];
+            ok = mbar_wait_warp(bar_tfull(0), 0, ctl, 321);
+            tc_fence_after();
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tmem_ld32(lane_taddr + c * 32, first + c * 32);
+            tmem_ld_wait();
+            if (nt == 2) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_tempty(0));
+                ok = ok && mbar_wait_warp(bar_tfull(0), 1, ctl, 324);
+                tc_fence_after();
+                load_half(0);
+                put_half(1);
+            }
+#pragma unroll
+            for (int i = 0; i < 64; ++i) v[i] = first[i];
+            put_half(0);
+#pragma unroll
+            for (int i = 0; i < 64; ++i) v[i] = first[64 + i];
+            put_half(2);
+            cluster_sync();                                  // the left halves of every product, and the firsts' right ones
+            const int r0 = BM * rank / S, r1 = BM * (rank + 1) / S, piece = lane & 15;
+            uint32_t peer[FMM_MAX_RANK / 2];
+#pragma unroll
+            for (int j = 0; j < FMM_MAX_RANK / 2; ++j) peer[j] = map_to_cta(tile, j < S ? j : 0);
+            float* c_tile = p.C + ((long long)parent * 2 * p.m + tm * BM) * p.ldc + tn * BN + piece * 4;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                if (h == 1) {
+                    cluster_sync();                          // the second products' left halves have been read
+                    if (nt == 2) { load_half(1); put_half(1); }
+                    cluster_sync();                          // their right halves are there
+                }
+                // two rows per warp and step, as below; product j is CTA j / 2's first or second
+                auto fetch = [&](int row, float4 (&x)[FMM_MAX_RANK]) {
+                    const uint32_t off = row * 256 + ((piece ^ (row & 7)) << 4);
+#pragma unroll
+                    for (int j = 0; j < FMM_MAX_RANK; ++j)
+                        if (j < p.R) x[j] = ld_cluster128(peer[j >> 1] + off + (j & 1 ? 1 : 2 * h) * C::HALF_BYTES);
+                };
+                auto sum_and_store = [&](int row, const float4 (&x)[FMM_MAX_RANK]) {
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int j = 0; j < FMM_MAX_RANK; ++j) {
+                            const float wj = p.W[j][b];      // zero for j >= R
+                            if (wj != 0.0f) { o.x = fmaf(wj, x[j].x, o.x); o.y = fmaf(wj, x[j].y, o.y); o.z = fmaf(wj, x[j].z, o.z); o.w = fmaf(wj, x[j].w, o.w); }
+                        }
+                        float* dst = c_tile + ((long long)(b >> 1) * p.m + row) * p.ldc + (long long)(b & 1) * p.n + h * 64;
+                        if (FMM_GUARD(p.guard, dst, 16, 1722)) *reinterpret_cast<float4*>(dst) = o;
+                    }
+                };
+                float4 x0[FMM_MAX_RANK], x1[FMM_MAX_RANK];
+                constexpr int STEP = C::EPI_WARPS * 2;
+                int row = r0 + q * 2 + (lane >> 4);
+                if (row < r1) fetch(row, x0);
+#pragma unroll 1
+                for (; row < r1; row += 2 * STEP) {
+                    const bool more1 = row + STEP < r1, more2 = row + 2 * STEP < r1;
+                    if (more1) fetch(row + STEP, x1);
+                    sum_and_store(row, x0);
+                    if (more2) fetch(row + 2 * STEP, x0);
+                    if (more1) sum_and_store(row + STEP, x1);
+                }
+            }
+        } else {
         if constexpr (C::MX) {
             ok = mbar_wait_warp(bar_tfull(0), 0, ctl, 321);
             tc_fence_after();
@@ -343,6 +443,7 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             if (more2) fetch(row + 2 * STEP, v0);
             if (more1) sum_and_store(row + STEP, v1);
         }
+        }
         (void)ok;
     }
 
@@ -362,12 +463,12 @@ fmm_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 }
 
 // The kernel's shared memory limit, raised once per device.
-template <int MODE, int BLK, int BN>
+template <int MODE, int BLK, int BN, int TPC = 1>
 bool prepare_split(int dev)
 {
     static std::atomic<bool> attr_set[64];
     if (dev >= 0 && dev < 64 && attr_set[dev].load(std::memory_order_acquire)) return true;
-    if (cudaFuncSetAttribute(fmm_split_kernel<MODE, BLK, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitCfg<MODE, BLK, BN>::SMEM_BYTES) != cudaSuccess) {
+    if (cudaFuncSetAttribute(fmm_split_kernel<MODE, BLK, BN, TPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SplitCfg<MODE, BLK, BN, TPC>::SMEM_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -401,8 +502,8 @@ bool ctas_per_sm(int dev, int* own, int* runtime)
     if (cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) != cudaSuccess ||
-        cudaFuncGetAttributes(&attr, fmm_split_kernel<MODE, BLK, BN>) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(runtime, fmm_split_kernel<MODE, BLK, BN>, C::THREADS, C::SMEM_BYTES) != cudaSuccess) {
+        cudaFuncGetAttributes(&attr, fmm_split_kernel<MODE, BLK, BN, 1>) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(runtime, fmm_split_kernel<MODE, BLK, BN, 1>, C::THREADS, C::SMEM_BYTES) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
@@ -420,7 +521,7 @@ int resident_clusters(int dev, int S)
     int n = 0, own = 0, runtime = 0;
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = split_config<MODE, BLK, 128>(S, 1, 1, 1, nullptr, attr);
-    if (!prepare_split<MODE, BLK, 128>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK, 128>, &cfg) != cudaSuccess || n <= 0 ||
+    if (!prepare_split<MODE, BLK, 128>(dev) || cudaOccupancyMaxActiveClusters(&n, fmm_split_kernel<MODE, BLK, 128, 1>, &cfg) != cudaSuccess || n <= 0 ||
         !ctas_per_sm<MODE, BLK, 128>(dev, &own, &runtime)) {
         cudaGetLastError();
         return 0;
@@ -430,7 +531,7 @@ int resident_clusters(int dev, int S)
     return n;
 }
 
-template <int MODE, int BLK, int BN>
+template <int MODE, int BLK, int BN, int TPC = 1>
 fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
 {
     using C = SplitCfg<MODE, BLK, BN>;
@@ -446,7 +547,7 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     } else {
         tmSFA = tmA; tmSFB = tmB;       // unused in this mode
     }
-    if (!prepare_split<MODE, BLK, BN>(g.device)) return FMM_ERR_CUDA;
+    if (!prepare_split<MODE, BLK, BN, TPC>(g.device)) return FMM_ERR_CUDA;
     SplitParams p;
     p.sa = static_cast<const uint8_t*>(g.sa); p.sb = static_cast<const uint8_t*>(g.sb);
     p.sa_term = g.sa_term; p.sb_term = g.sb_term;
@@ -457,7 +558,7 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     if (g.nq == 4) for (int r = 0; r < g.R; ++r) for (int b = 0; b < 4; ++b) p.W[r][b] = g.W[r][b] * g.up;
     else for (int j = 0; j < ksplit; ++j) p.W[j][0] = g.up;
     p.C = g.C; p.ldc = g.Nfull; p.status = g.status; p.guard = g.guard;
-    const int S = g.R * ksplit;
+    const int S = (g.R + TPC - 1) / TPC * ksplit;
 
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = split_config<MODE, BLK, BN>(S, (unsigned)(g.nsub / C::BN), (unsigned)(g.msub / BM), (unsigned)(g.terms / g.R), st, attr);
@@ -465,7 +566,7 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.numAttrs = g.overlap_prev ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, fmm_split_kernel<MODE, BLK, BN>, tmA, tmB, tmSFA, tmSFB, p) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
+    if (cudaLaunchKernelEx(&cfg, fmm_split_kernel<MODE, BLK, BN, TPC>, tmA, tmB, tmSFA, tmSFB, p) != cudaSuccess) { cudaGetLastError(); return FMM_ERR_CUDA; }
     return FMM_OK;
 }
 
@@ -476,11 +577,11 @@ fmm_status_t launch_split(const GemmParams& g, int ksplit, cudaStream_t st)
 // whatever their K: leaves of 128 to 1024, and it takes tiles of 64 or 32 columns as long as about all of them are resident
 // at once.  Rank 7, block 32, one level, 128 columns -> the width chosen: n = 256 8.6 -> 5.1 us, n = 512 10.7 -> 7.2,
 // n = 1024 18.5 -> 14.0, 512 x 4096 x 1024 40.6 -> 19.7, 256 x 8192 x 256 74.7 -> 27.6.
-struct SplitModel { float lat, alone; int widths; float f[3], c[3]; };       // f, c: 128, 64, 32 columns
-constexpr SplitModel SPLIT_MX = {0.65f, 0.67f, 1, {6.6f, 0.f, 0.f}, {0.33f, 0.f, 0.f}};
-constexpr SplitModel SPLIT_B32 = {1.7f, 0.89f, 3, {7.15f, 5.55f, 3.75f}, {2.02f, 1.31f, 0.82f}};
-constexpr SplitModel SPLIT_B128 = {1.55f, 0.85f, 3, {7.5f, 5.9f, 4.25f}, {0.61f, 0.34f, 0.34f}};
-constexpr SplitModel SPLIT_TILE = {1.55f, 0.88f, 3, {6.9f, 4.85f, 3.55f}, {0.47f, 0.37f, 0.33f}};
+struct SplitModel { float lat, alone; int widths; float f[3], c[3], f_two; };       // f, c: 128, 64, 32 columns; f_two: two terms per CTA
+constexpr SplitModel SPLIT_MX = {0.65f, 0.67f, 1, {6.6f, 0.f, 0.f}, {0.33f, 0.f, 0.f}, 10.5f};
+constexpr SplitModel SPLIT_B32 = {1.7f, 0.89f, 3, {7.15f, 5.55f, 3.75f}, {2.02f, 1.31f, 0.82f}, 0.0f};
+constexpr SplitModel SPLIT_B128 = {1.55f, 0.85f, 3, {7.5f, 5.9f, 4.25f}, {0.61f, 0.34f, 0.34f}, 0.0f};
+constexpr SplitModel SPLIT_TILE = {1.55f, 0.88f, 3, {6.9f, 4.85f, 3.55f}, {0.47f, 0.37f, 0.33f}, 0.0f};
 
 template <int MODE, int BLK>
 SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persistent_time)
@@ -488,7 +589,7 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
     const int kst = g.k / BK;
     const long long parents = g.terms / g.R;
     float best_time = persistent_time;
-    SplitChoice best = {0, 0};
+    SplitChoice best = {0, 0, 1};
     for (int ks = 1; g.R * ks <= FMM_MAX_RANK && ks <= kst; ks *= 2) {
         const int cap = resident_clusters<MODE, BLK>(g.device, g.R * ks);
         if (cap <= 0) break;
@@ -497,9 +598,18 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
             const long long tiles = (long long)(g.m / BM) * (g.n / (128 >> w)) * parents;
             const float waves = std::max(1.0f, (float)tiles / places);
             const float time = m.lat + waves * (m.f[w] + ((kst + ks - 1) / ks) * m.c[w]);
-            if (time < best_time) { best_time = time; best = {ks, 128 >> w}; }
+            if (time < best_time) { best_time = time; best = {ks, 128 >> w, 1}; }
         }
         if (g.R > 1) break;
+    }
+    // two terms per CTA (UE8M0): for the products that clusters of R do not hold at once and these do.  f: a longer exchange, as a
+    // CTA sums twice the rows.  n = 2048 32.0 -> 29.9 us a call, 2048 x 512 x 2048 21.7 -> 19.5, 1280 x 3328 x 2816 40.3 -> 38.5, 512 x 4096
+    // x 8192 73.0 -> 68.5, two levels n = 1536 33.8 -> 32.1; where one wave of clusters of R is enough it is slower (n = 1536 19.6, 24.4;
+    // n = 1024 13.2, 15.9), and so it is in more than one wave of its own (n = 2560 52.7, the persistent kernel 45.4).
+    if (m.f_two > 0.0f && g.R > 1) {
+        const int cap = resident_clusters<MODE, BLK>(g.device, (g.R + 1) / 2);
+        const long long tiles = (long long)(g.m / BM) * (g.n / 128) * parents;
+        if (tiles <= cap && m.lat + m.f_two + 2 * kst * m.c[0] < best_time) best = {1, 128, 2};
     }
     return best;
 }
@@ -516,7 +626,7 @@ fmm_status_t launch_fp32(const GemmParams& g, int blk, int ksplit, cudaStream_t 
 
 SplitChoice fmm_split_choice(const GemmParams& g, int blk, int mode)
 {
-    if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0};     // grid dimensions
+    if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0, 1};     // grid dimensions
     const float t = fmm_gemm_shape(g, blk, mode, g.m, g.n).time;
     if (mode == FMM_SCALE_UE8M0_CEIL) return choose_split<FMM_SCALE_UE8M0_CEIL, 32>(g, SPLIT_MX, t);
     if (blk == 32) return choose_split<MODE_FP32_COLUMN, 32>(g, SPLIT_B32, t);
@@ -526,7 +636,7 @@ SplitChoice fmm_split_choice(const GemmParams& g, int blk, int mode)
 
 fmm_status_t fmm_launch_split(const GemmParams& g, int blk, int mode, SplitChoice c, cudaStream_t st)
 {
-    if (mode == FMM_SCALE_UE8M0_CEIL) return launch_split<FMM_SCALE_UE8M0_CEIL, 32, 128>(g, c.ksplit, st);
+    if (mode == FMM_SCALE_UE8M0_CEIL) return c.terms == 2 ? launch_split<FMM_SCALE_UE8M0_CEIL, 32, 128, 2>(g, c.ksplit, st) : launch_split<FMM_SCALE_UE8M0_CEIL, 32, 128>(g, c.ksplit, st);
     if (c.bn == 32) return launch_fp32<32>(g, blk, c.ksplit, st);
     if (c.bn == 64) return launch_fp32<64>(g, blk, c.ksplit, st);
     return launch_fp32<128>(g, blk, c.ksplit, st);
