@@ -303,6 +303,21 @@ __global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_k
 // is two 64-byte row segments per warp; each thread writes 16 contiguous code bytes and the two
 // lanes of a block fill one 32-byte sector.
 
+// The same place of the block p.cpt blocks further on in the grid, into L2: ROWS rows of 16 columns, one row of every input
+// block per thread.
+template <int ROWS>
+__device__ __forceinline__ void prefetch_block(const EncodeParams& p, int block_row)
+{
+    if (p.cpt == 0) return;
+    const uint32_t next = (uint32_t)block_row * gridDim.x + blockIdx.x + (uint32_t)p.cpt;
+    const uint32_t y = next / gridDim.x, x = next - y * gridDim.x;
+    if (y >= (uint32_t)p.rows / ROWS) return;
+    const float* at = p.in + (int64_t)blockIdx.z * p.in_batch_stride + (int64_t)(y * ROWS + threadIdx.x) * p.ld + x * 16;
+#pragma unroll
+    for (int jq = 0; jq < 4; ++jq)
+        if (jq < p.nq) asm volatile("prefetch.global.L2 [%0];" ::"l"(at + p.qoff[jq]));
+}
+
 // B side, block 32, one 32-k block of 16 columns per warp (thread = 16 k of one column, lanes l and l+16 the two
 // halves of a block), so every thread issues all its loads at once.  A thread block is a single warp: the warps
 // share nothing, and one-warp blocks let the scheduler replace each finished warp on its own (2 % faster than four
@@ -330,6 +345,7 @@ __device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
             for (int kk = 0; kk < 16; ++kk)
                 raw[jq][kk] = __ldg(base + p.qoff[jq] + (int64_t)(k0 + kk) * p.ld);
         }
+    prefetch_block<32>(p, kb);
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
         if (row_used<NZ>(r, p.R)) {
@@ -437,6 +453,7 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
             for (int kk = 0; kk < 16; ++kk)
                 raw[jq][kk] = __ldg(base + p.qoff[jq] + (int64_t)(k0 + kk) * p.ld);
         }
+    prefetch_block<128>(p, kc);
     auto combine = [&](int r, float (&v)[16]) {
         bool set = false;
 #pragma unroll
@@ -983,8 +1000,17 @@ fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
-fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaStream_t st)
+fmm_status_t fmm_launch_encode_b(EncodeParams p, int blk, int mode, cudaStream_t st)
 {
+    // A block loads everything first and then computes: the operand's next blocks come into L2 meanwhile, half of the resident ones
+    // ahead (block 128, n = 8192: a quarter 141.6 us for both sides, half 133.9, three quarters 134.6, all 136.8, none 142.6; weight
+    // tiles 177 -> 168, n = 4096 47.3 -> 44.1, block 128 37.4 -> 34.9, block 32 36.0 -> 34.5).  Only for an operand that is not in L2 already:
+    // up to 51 MB it is 0 to 4 % slower (n = 3072 19.2, 20.0).  Panels of a plain pass, with less to compute, gain from twice that
+    // on (n = 4096 28.5, 28.9; n = 8192 108.9, 108.1, weight tiles 137.1, 127.5).  The A side, whose warps keep loads in flight
+    // while they compute, loses 3 % by it.
+    const int64_t bytes = (int64_t)p.rows * p.cols * p.nq * 4;
+    p.cpt = bytes >= (int64_t)(p.R > 4 ? 56 : 112) << 20 && p.batch == 1 ? fmm_sm_count() * (blk == 32 ? 8 : 2) : 0;
+
     dim3 grid((unsigned)(p.cols / 16), (unsigned)(p.rows / blk), (unsigned)p.batch);
     if (mode != FMM_SCALE_FP32_AMAX_DIV_448) launch_b32<FMM_SCALE_UE8M0_CEIL>(p, grid, st);
     else if (blk == 32) launch_b32<FMM_SCALE_FP32_AMAX_DIV_448>(p, grid, st);

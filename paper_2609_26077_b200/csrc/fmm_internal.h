@@ -132,7 +132,7 @@ struct EncodeParams {
     int s_step;               // rows (A side) / columns (B side) by which combination r is shifted inside a shared scale array
     int s_ld;                 // fp32 scales: columns of B / rows of A that the shared scale array covers
     int sf_blocks;            // UE8M0: number of 128-row blocks of the scale-tile array
-    int cpt;                  // A side: 128-k chunks per task (set by the launcher)
+    int cpt;                  // A side: 128-k chunks per task; B side: blocks that it prefetches ahead, 0: none (set by the launcher)
     float amax_floor;
     short b_tile;             // B side: 128 = one fp32 scale per 128 x 128 tile (blk 128 only), 0 = per column
     short preround_bf16;      // B side: round each combination to bfloat16 before the maximum and the cast
@@ -168,7 +168,7 @@ fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, cudaStrea
 fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st);
 // both sides of a small call in one launch: false if it is not one, or has coefficients without kernels of their own
 bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int mode, cudaStream_t st, fmm_status_t* status);
-fmm_status_t fmm_launch_encode_b(const EncodeParams& p, int blk, int mode, cudaStream_t st);
+fmm_status_t fmm_launch_encode_b(EncodeParams p, int blk, int mode, cudaStream_t st);
 // last two recursion levels in one pass (p.rows x p.cols = leaf dimensions, inputs 4*rows x 4*cols)
 bool fmm_encode2_supported(bool b_side, int blk, int b_tile, int preround_bf16);
 fmm_status_t fmm_launch_encode2_a(const EncodeParams& p, int blk, int mode, cudaStream_t st);
