@@ -111,8 +111,7 @@ fmm_status_t fmm_workspace_bytes(const fmm_plan_t* plan, int64_t M, int64_t N, i
  *   the same holds for every call that takes a plan and touches the device.
  * Asynchronous on cuda_stream.  Calls sharing a workspace must be stream-ordered; a plan may be shared by host
  * threads (it is read-only during a call, apart from the launch counter below).  Towards other work on the stream a
- * call is ordinary stream-ordered work: its first kernel, which is set up under the tail of what is enqueued before it, touches
- * nothing until all of that has completed, and
+ * call is ordinary stream-ordered work: its first kernel starts after everything enqueued before it has completed, and
  * whatever is enqueued after it starts after all of its kernels have completed.  Between themselves the kernels of one
  * call overlap where they do not depend on each other (programmatic dependent launch: the B-side encoder starts under
  * the A-side encoder's last wave, the product kernel is set up under the B-side encoder's last blocks). */

@@ -204,7 +204,7 @@ fmm_status_t encode_outer(const fmm_plan* plan, const FmmLayout& L, char* ws, co
             s.out = reinterpret_cast<float*>(ws + inter[level]);
             s.guard = fmm_make_guard(s.out, (size_t)s.batch * s.R * (size_t)(s.rows * (int64_t)s.cols) * 4, nullptr, 0, plan->d_status + FMM_GUARD_WORD);
         }
-        const fmm_status_t s = fmm_launch_comb(c[0], c[1], st);
+        const fmm_status_t s = fmm_launch_comb(c[0], c[1], level > 1, st);
         if (s != FMM_OK) return s;
         ++*launches;
     }
@@ -305,14 +305,14 @@ fmm_status_t encode_all(const fmm_plan* plan, const FmmLayout& L, char* ws, cons
 {
     if (plan->levels <= 1) {
         fmm_status_t s;
-        if (fmm_launch_encode_both(encode_params(plan, L, ws, A, M, K, false, 0, L.m, true), encode_params(plan, L, ws, B, K, N, true, 0, L.n, true),
+        if (fmm_launch_encode_both(encode_params(plan, L, ws, A, M, K, false, 0, L.m, false), encode_params(plan, L, ws, B, K, N, true, 0, L.n, false),
                                    plan->qp.block_k, (int)plan->qp.scale_mode, st, &s)) {
             if (s == FMM_OK) ++*launches;
             return s;
         }
     }
     fmm_status_t s = encode_outer(plan, L, ws, A, B, M, N, K, st, launches);
-    if (s == FMM_OK) s = encode_side(plan, L, ws, A, M, K, false, 0, L.m, true, st, launches);
+    if (s == FMM_OK) s = encode_side(plan, L, ws, A, M, K, false, 0, L.m, *launches > 0, st, launches);     // behind combinations
     if (s == FMM_OK) s = encode_side(plan, L, ws, B, K, N, true, 0, L.n, true, st, launches);
     return s;
 }

@@ -291,8 +291,10 @@ __device__ __forceinline__ void encode_a_tasks(const EncodeParams& p, uint32_t w
 template <int BLK, int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(256, BLK == 128 && NZ != 0 ? 4 : 3) encode_a_kernel(const EncodeParams p)
 {
-    fmmptx::griddep_wait();                        // whatever is before this launch on the stream (launch_encoder)
-    fmmptx::griddep_launch_dependents();           // the B-side encoder of the same call reads nothing written here
+    // The combinations of this call, when this launch overlaps their tail.  Always ahead of the signal: the B-side encoder that it
+    // releases reads nothing written here and does not wait at its start, so what this kernel is behind has to be complete by then.
+    fmmptx::griddep_wait();
+    fmmptx::griddep_launch_dependents();
     encode_a_tasks<BLK, MODE, NZ>(p, blockIdx.x * 8 + fmmptx::warp_uniform(threadIdx.x >> 5), gridDim.x * 8);
 }
 
@@ -551,7 +553,6 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
 template <int BLK, int MODE, uint32_t NZA, uint32_t NZB, bool TILE, bool PRE>
 __global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) encode_both_kernel(const __grid_constant__ EncodeParams pa, const __grid_constant__ EncodeParams pb)
 {
-    fmmptx::griddep_wait();                        // whatever is before this launch on the stream
     const uint32_t b_rows = (uint32_t)pb.rows / BLK;
     const bool b_side = blockIdx.y < b_rows;
     if (b_side) {
@@ -562,7 +563,7 @@ __global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) enco
         encode_a_tasks<BLK, MODE, NZA>(pa, ((blockIdx.y - b_rows) * gridDim.x + blockIdx.x) * WARPS + fmmptx::warp_uniform(threadIdx.x >> 5),
                                        (gridDim.y - b_rows) * gridDim.x * WARPS);
     }
-    fmmptx::griddep_launch_dependents();           // as end_of_b_side
+    fmmptx::griddep_launch_dependents();           // as end_of_b_side (nothing to wait for: an ordinary launch)
     if (TILE && b_side) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
 }
 
@@ -577,7 +578,7 @@ __global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) enco
 template <int BLK, int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(256) encode2_a_kernel(const EncodeParams p)
 {
-    fmmptx::griddep_wait();                        // as encode_a_kernel
+    fmmptx::griddep_wait();                        // as encode_a_kernel, ahead of the signal
     fmmptx::griddep_launch_dependents();
     constexpr int GROUP = BLK / 4;
     const int lane = threadIdx.x & 31;
@@ -716,7 +717,7 @@ __device__ __forceinline__ void axpy(float4& acc, float w, const float4& x)
 // terms FMAs, zero coefficients skipped.  Both sides of a level in one launch (blockIdx.y).
 __global__ void __launch_bounds__(256) comb_kernel(const CombParams pa, const CombParams pb)
 {
-    fmmptx::griddep_wait();                        // the level above, or whatever is before the call on the stream
+    fmmptx::griddep_wait();                        // the level above, when this launch overlaps its tail
     const CombParams& p = blockIdx.y ? pb : pa;
     if (blockIdx.x * 8u >= (uint32_t)p.rows * ((uint32_t)p.cols / 128) || (int)blockIdx.z >= p.batch) return;
     const OuterIndex at = outer_index(p.cols);
@@ -833,10 +834,10 @@ __global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
 }  // namespace
 
 namespace {
-// Launch that may begin under the tail of what is before it on the stream (the kernel waits for that before its first load),
-// so that its launch latency and set-up are hidden.
+// Launch that may begin under the tail of the kernel before it on the stream, one of the same call (which wrote what this one
+// reads: it waits for it before its first load), so that its launch latency and set-up are hidden.
 template <typename K, typename... A>
-fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, const A&... args)
+fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, bool overlap, const A&... args)
 {
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
@@ -844,7 +845,7 @@ fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, con
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    cfg.attrs = at; cfg.numAttrs = overlap ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, args...);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
@@ -853,14 +854,14 @@ fmm_status_t launch_behind(K kernel, dim3 grid, dim3 block, cudaStream_t st, con
 fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st)
 {
     const unsigned tiles = (unsigned)(p.cols / 128);
-    if (steps == 2) return launch_behind(decode2_kernel, dim3((unsigned)(p.rows / 4) * tiles), dim3(32, 4), st, p);
-    return launch_behind(decode_kernel, dim3((unsigned)(p.rows / 8) * tiles, 1, (unsigned)p.batch), dim3(32, 8), st, p);
+    if (steps == 2) return launch_behind(decode2_kernel, dim3((unsigned)(p.rows / 4) * tiles), dim3(32, 4), st, true, p);
+    return launch_behind(decode_kernel, dim3((unsigned)(p.rows / 8) * tiles, 1, (unsigned)p.batch), dim3(32, 8), st, true, p);
 }
 
-fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, cudaStream_t st)
+fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, bool overlap, cudaStream_t st)
 {
     const unsigned ga = (unsigned)(a.rows / 8) * (unsigned)(a.cols / 128), gb = (unsigned)(b.rows / 8) * (unsigned)(b.cols / 128);
-    return launch_behind(comb_kernel, dim3(ga > gb ? ga : gb, 2, (unsigned)(a.batch > b.batch ? a.batch : b.batch)), dim3(32, 8), st, a, b);
+    return launch_behind(comb_kernel, dim3(ga > gb ? ga : gb, 2, (unsigned)(a.batch > b.batch ? a.batch : b.batch)), dim3(32, 8), st, overlap, a, b);
 }
 
 namespace {
@@ -883,11 +884,10 @@ uint32_t coef_mask(const EncodeParams& p)
 // Launch of an encoder.  With `overlap` it carries the programmatic-serialization attribute.  B side: the kernel
 // before it on the stream (the A-side encoder, which signals at its start) need not have drained when this one
 // begins, so its blocks fill the SMs that the other's last wave leaves idle (6 % of the encode phase at n = 8192); what it
-// reads, the caller's matrix or combinations of a kernel before the A-side one, is complete.  A side: its launch latency falls
-// under the tail of whatever is before it, the caller's kernels or the previous call, whose operands and workspace it touches
-// only behind its wait (2 us of a call at every size: n = 256 10.3 -> 7.9 us of device time, 1024 block 128 16.4 -> 14.2,
-// 1280 x 3328 x 2816 UE8M0 42.0 -> 40.0).  The product kernels do not signal early for it: its blocks would take the
-// places of their last CTAs' successors (Winograd, block 128, n = 4096 127 -> 137).
+// reads, the caller's matrix or combinations of a kernel before the A-side one, is complete (encode_a_kernel).  A side: set up
+// under the tail of the combinations of the same call.  The first kernel of a call is launched without: its wait would be
+// for the caller's last kernel, which stands for the work before it only if it waited for that itself, and a caller's kernel that
+// has the attribute need not (2 us of a call that follows another at every size).
 template <typename K, typename... P>
 void launch_encoder(K kernel, dim3 grid, unsigned threads, cudaStream_t st, unsigned cluster, bool overlap, const P&... p)
 {
@@ -964,7 +964,7 @@ bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps,
     const unsigned gx = (unsigned)b.cols / 16, a_blocks = (a_warps + THREADS / 32 - 1) / (THREADS / 32);
     const dim3 grid(gx, (unsigned)b.rows / BLK + (a_blocks + gx - 1) / gx);
     const uint32_t ma = coef_mask(a), mb = coef_mask(b);
-#define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE>, grid, THREADS, st, TILE ? 8 : 1, true, a, b); return true; }
+#define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE>, grid, THREADS, st, TILE ? 8 : 1, false, a, b); return true; }
     FMM_KNOWN_MASK_PAIRS(X)
 #undef X
     return false;

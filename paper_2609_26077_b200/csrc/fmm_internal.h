@@ -137,8 +137,8 @@ struct EncodeParams {
     short b_tile;             // B side: 128 = one fp32 scale per 128 x 128 tile (blk 128 only), 0 = per column
     short preround_bf16;      // B side: round each combination to bfloat16 before the maximum and the cast
     int overlap_prev;         // B side: the kernel launched just before on the stream is the A-side encoder of the same
-                              // call (nothing this kernel reads): it may start while that one drains.  A side: it may be set up
-                              // while whatever is before it on the stream drains, which it waits for
+                              // call (nothing this kernel reads): it may start while that one drains.  A side: that kernel is
+                              // combinations of the same call: it may be set up while that one drains
     FmmGuard guard;           // codes and scales of this side
 };
 // a launch with more parameter bytes takes the host 0.35 us longer (n = 256: 10.2 -> 10.5 us a call)
@@ -163,8 +163,8 @@ struct DecodeParams {
 };
 // steps: 1, or 2 outward steps at once (batch 1; rows x cols and W as for the inner step)
 fmm_status_t fmm_launch_decode(const DecodeParams& p, int steps, cudaStream_t st);
-// one level of combinations of the two sides (a side with rows == 0 has none)
-fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, cudaStream_t st);
+// one level of combinations of the two sides (a side with rows == 0 has none); overlap: behind another such launch
+fmm_status_t fmm_launch_comb(const CombParams& a, const CombParams& b, bool overlap, cudaStream_t st);
 fmm_status_t fmm_launch_encode_a(EncodeParams p, int blk, int mode, cudaStream_t st);
 // both sides of a small call in one launch: false if it is not one, or has coefficients without kernels of their own
 bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int mode, cudaStream_t st, fmm_status_t* status);

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(STAT_THREADS) error_partial_kernel(const float
 {
     __shared__ double sm[3 * (STAT_THREADS / 32)];
     double sd = 0.0, sr = 0.0, mx = 0.0;
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // what is before this launch on the stream (launch_behind)
     // each thread takes pairs: one 8-byte load of C, one 16-byte load of Cref (count is even); four pairs per
     // trip with all loads issued first, so that every thread keeps 96 bytes in flight
     const int64_t pairs = count >> 1;
@@ -98,25 +97,18 @@ __global__ void __launch_bounds__(STAT_THREADS) error_final_kernel(const double*
     if (threadIdx.x == 0 && FMM_GUARD(guard, out3, 24, 1602)) { out3[0] = sd; out3[1] = sr; out3[2] = mx; }
 }
 
-// Launch with the programmatic-serialization attribute: the kernel is set up under the tail of what is before it on the stream
-// and waits for that before its first access (statistics at n = 4096: 2 us for each of the two stages).
-template <typename K, typename... A>
-void launch_behind(K kernel, dim3 grid, unsigned threads, cudaStream_t st, const A&... args)
+// Both stages.  The second is launched with the programmatic-serialization attribute, so that its launch latency falls
+// under the first (2 us of 38 at n = 4096).
+fmm_status_t launch_stats(const float* C, const double* Cref, int64_t count, double* partial, double* out3, const FmmGuard& guard, cudaStream_t st)
 {
+    error_partial_kernel<<<STAT_BLOCKS, STAT_THREADS, 0, st>>>(C, Cref, count, partial, guard);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.stream = st;
+    cfg.gridDim = dim3(1); cfg.blockDim = dim3(STAT_THREADS); cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
-// Both stages.
-fmm_status_t launch_stats(const float* C, const double* Cref, int64_t count, double* partial, double* out3, const FmmGuard& guard, cudaStream_t st)
-{
-    launch_behind(error_partial_kernel, dim3(STAT_BLOCKS), STAT_THREADS, st, C, Cref, count, partial, guard);
-    launch_behind(error_final_kernel, dim3(1), STAT_THREADS, st, static_cast<const double*>(partial), STAT_BLOCKS, out3, guard);
+    cudaLaunchKernelEx(&cfg, error_final_kernel, static_cast<const double*>(partial), STAT_BLOCKS, out3, guard);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
@@ -177,7 +169,6 @@ ref_gemm_fp64_kernel(const float* __restrict__ A, const float* __restrict__ B, d
 #pragma unroll
             for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
     const int steps = (int)(K / REF_BK);
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // what is before this launch on the stream (launch_behind)
 #pragma unroll
     for (int s = 0; s < REF_STAGES - 1; ++s) {
         if (s < steps) load(s, (int64_t)s * REF_BK);
@@ -219,8 +210,8 @@ template <int T>
 void launch_ref(const float* A, const float* B, double* C, int64_t M, int64_t N, int64_t K, const FmmGuard& guard, cudaStream_t st)
 {
     const dim3 grid((unsigned)(N / T), (unsigned)(M / T));
-    if ((((uintptr_t)A | (uintptr_t)B) & 15) == 0) launch_behind(ref_gemm_fp64_kernel<T, true>, grid, 128, st, A, B, C, M, N, K, guard);
-    else launch_behind(ref_gemm_fp64_kernel<T, false>, grid, 128, st, A, B, C, M, N, K, guard);
+    if ((((uintptr_t)A | (uintptr_t)B) & 15) == 0) ref_gemm_fp64_kernel<T, true><<<grid, 128, 0, st>>>(A, B, C, M, N, K, guard);
+    else ref_gemm_fp64_kernel<T, false><<<grid, 128, 0, st>>>(A, B, C, M, N, K, guard);
 }
 
 // Device address of g_stats_guard_code on the current device (FMM_DEBUG build; the release build passes no word and
