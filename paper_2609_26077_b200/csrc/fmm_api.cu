@@ -343,7 +343,7 @@ fmm_status_t multiply(const fmm_plan* plan, const FmmLayout& L, char* ws, float*
     g.sa = ws + L.sa + (e8 ? strip.m0 / 128 * 512 : strip.m0 * 4 * (128 / plan->qp.block_k));
     g.sb = ws + L.sb_down + (e8 ? strip.n0 / 128 * 512 : strip.n0 * 4);
     g.sa_term = (int64_t)L.sa_term; g.sb_term = (int64_t)L.sb_term;
-    g.up = fmm_scale_up(plan->qp);
+    g.up = fmm_scale_up(plan->qp); g.small_weights = plan->small_weights;
     // The product kernel applies the innermost decoder only: leaf products of parent p land in the four
     // blocks of parent p's (2m x 2n) matrix.  For one level that matrix is C itself; for more levels the
     // parents' matrices are stacked in the workspace and decoded outwards level by level (the same
@@ -484,6 +484,7 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
             for (int q = 0; q < (levels ? 4 : 1); ++q) {
                 const float w = !levels ? 1.0f : s + 1 < rank ? fmm_emitted_weight(p->W[r][q], carry[s + 1], p->W[order[s + 1]][q]) : p->W[r][q];
                 if (w == 0.0f) continue;
+                if (carried && levels && fabsf(w) < 1.0f) p->small_weights |= 1u << s;
                 FmmOutEntry e;
                 e.row_off = parent * 2 + (q >> 1); e.col_off = q & 1;
                 e.w = w;

@@ -149,7 +149,8 @@ struct KParams {
     int positions, tiles_n, terms_per_group, items;      // tiles_n: tile positions per row of positions
     const FmmWalkEntry* walk; const FmmOutEntry* out;  // FP32 scales
     const int* pair_start; const FmmPairEntry* pair;   // pair-fused decoder (UE8M0): steps of two products, see FmmPairEntry
-    int order[FMM_MAX_RANK]; short steps, R;           // walk order of the R products of a parent; steps = ceil(R / 2)
+    int order[FMM_MAX_RANK]; short steps;     // walk order of the R products of a parent; steps = ceil(R / 2)
+    unsigned char R, small_weights;           // output warps, bit s: step s of a parent has weights below 1
     float up;                                 // factor of the sums (GemmParams)
     int* status;
     const float* c_base; long long ldc;       // the output matrix as plain memory: used by the FMM_DEBUG store guard only
@@ -181,6 +182,8 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     auto bar_dempty = [&](int i) { return bar_dfull(i) + 16u; };
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + C::OFF_BAR + C::NUM_BARS * 8);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    // DUMP: factor that a half of the accumulator copy is written with, for the step that it is free for
+    volatile float* dump_up = reinterpret_cast<volatile float*>(tmem_slot + 2);
     const Ctl ctl{abort_flag, p.status};
 
     auto uniform = [](uint32_t v) { return C::UNIFORM ? warp_uniform(v) : v; };
@@ -198,6 +201,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         for (int b = 0; b < 4; ++b) mbar_init(bar_tempty(b), NCTA * EPI_WARPS);
         for (int i = 0; i < 2; ++i) { mbar_init(bar_dfull(i), EPI_WARPS / 2); mbar_init(bar_dempty(i), 1); }
         *abort_flag = 0;
+        if (C::DUMP) dump_up[0] = dump_up[1] = p.small_weights & 1 ? 1.0f : p.up;
         fence_barrier_init();
     }
     if (warp == 1) {
@@ -319,6 +323,9 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const uint32_t dump = base + C::OFF_DUMP + half * CHS * 4096, stg = base + C::OFF_STG + half * BUFS * 4096;
         const uint64_t pol_c = policy_evict_last();                         // see the note on the C tiles' L2 policy below
         uint32_t dphase = 0, cnt = 0;
+        // A sum above the range may have a weighted value in it: where a step has a weight below 1 its sum comes without the factor,
+        // which goes with the weights, and its chunks of weight 1 through registers as well (one of T*'s twelve updates).
+        int step = 0;                                                        // of the parent
         bool ok = true;
         for (int w = unit; w < p.items && ok; w += units) {
             const int grp = w / p.positions, pos = w - grp * p.positions;
@@ -329,13 +336,16 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const int o0 = p.walk[s].out0, o1 = rows ? p.walk[s].out1 : o0;
                 if (!mbar_wait_warp(bar_dfull(half), dphase, ctl, 401)) { ok = false; break; }
                 dphase ^= 1u;
+                const bool small = p.small_weights >> step & 1;
+                step = step + 1 == p.R ? 0 : step + 1;
                 bool any_direct = false;
                 for (int o = o0; o < o1; ++o) {
                     const FmmOutEntry ent = p.out[o];
                     const int row0 = ent.row_off * p.m + (tm * NCTA + cta_rank) * BM + half * 64, col0 = ent.col_off * p.n + tn * BN;
                     // A weight of exactly 1 needs no copy: the promoting warps stored the chunks in the swizzled layout the
                     // tensor map expects (and made them visible to the TMA engine), so they go out as they are.
-                    const bool direct = (ent.w == 1.0f);
+                    const bool direct = !small && ent.w == 1.0f;
+                    const float w = small ? ent.w * p.up : ent.w;
                     any_direct |= direct;
                     // this warp's previous update of the same block, `gap` updates of CHS bulk groups ago, has landed
                     if (lane == 0) {
@@ -356,7 +366,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             for (int i4 = 0; i4 < 8; ++i4) v[i4] = lds128(from + lane * 128 + ((i4 ^ (lane & 7)) << 4));
 #pragma unroll
                             for (int i4 = 0; i4 < 8; ++i4) {
-                                v[i4].x *= ent.w; v[i4].y *= ent.w; v[i4].z *= ent.w; v[i4].w *= ent.w;
+                                v[i4].x *= w; v[i4].y *= w; v[i4].z *= w; v[i4].w *= w;
                                 sts128(to + lane * 128 + ((i4 ^ (lane & 7)) << 4), v[i4]);
                             }
                             fence_proxy_async();
@@ -377,7 +387,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 // the TMA engine has read the copy for the last time (chunks sent as they are), and so has every lane
                 if (lane == 0 && any_direct) bulk_wait_read<0>();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(bar_dempty(half));
+                if (lane == 0) {
+                    dump_up[half] = p.small_weights >> step & 1 ? 1.0f : p.up;
+                    mbar_arrive(bar_dempty(half));
+                }
             }
         }
         if (lane == 0) bulk_wait<0>();
@@ -732,9 +745,10 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                     // as 32 x 32 chunks in the 128-byte-swizzled layout of the output tensor map
                     if (!mbar_wait_warp(bar_dempty(q >> 1), dphase ^ 1u, ctl, 304)) { ok = false; break; }
                     dphase ^= 1u;
+                    const float up = dump_up[q >> 1];
                     // thread: rows lane/4 + 8k of the warp's 32-row chunk, column pairs 8j + 2(lane%4) of its columns
                     const uint32_t dchunk = base + C::OFF_DUMP + (q * (BN / 32) + h * (C::CW / 32)) * 4096 + (lane & 1) * 8;
-                    const unsigned long long up2 = pack2(p.up, p.up);
+                    const unsigned long long up2 = pack2(up, up);
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const int rr = (lane >> 2) + 8 * k;
@@ -896,8 +910,8 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
     kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = (short)g.steps;
     for (int r = 0; r < FMM_MAX_RANK; ++r) kp.order[r] = g.order[r];
-    kp.R = (short)(g.terms_per_group > 0 ? g.terms_per_group : 1);       // products per parent (1 for the cubic product)
-    kp.up = g.up;
+    kp.R = (unsigned char)(g.terms_per_group > 0 ? g.terms_per_group : 1);       // products per parent (1 for the cubic product)
+    kp.up = g.up; kp.small_weights = (unsigned char)(separate ? 0 : g.small_weights);
     kp.c_base = g.C; kp.ldc = g.Nfull; kp.guard = g.guard;
 
     cudaLaunchConfig_t cfg;

@@ -102,6 +102,7 @@ struct fmm_plan {
     // device tables
     int* d_status;            // [64] status words (word 0: first bounded wait that gave up)
     FmmWalkEntry* d_walk;     // [2 * terms]: with carried sums, and without
+    unsigned small_weights;   // carried sums: bit s = a weight of step s of a parent is below 1 in magnitude
     FmmOutEntry* d_out;       // [total entries], block offsets in units of leaf blocks (scaled at launch)
     int order[FMM_MAX_RANK];  // pair-fused decoder: walk order of the R products of a parent
     int steps;                // pair-fused decoder: steps per parent, ceil(R / 2)
@@ -179,6 +180,7 @@ struct GemmParams {
     const void* sa; const void* sb;         // sb, one fp32 scale per column: times fmm_scale_down
     int64_t sa_term, sb_term;               // bytes per term
     float up;                               // fmm_scale_up
+    unsigned small_weights;                 // fmm_plan::small_weights
     float* C; int64_t ldc;                  // full output
     int64_t Mfull, Nfull;
     int m, n, k, terms;

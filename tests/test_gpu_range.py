@@ -42,3 +42,25 @@ def test_small_clamp_keeps_small_products(blk):
     # the sums' last places are far above the smallest subnormal number: nothing is lost but where a sum passes through zero
     assert torch.isfinite(got).all()
     assert (got - want).abs().max() <= 2.0 ** -23 * want.abs().max()
+
+
+@pytest.mark.parametrize("K", [512, 1024, 3840])
+def test_products_above_the_range_whose_weighted_sums_are_in_it(K):
+    # U times 8 and W times 1/8: the same C from products that are 8 times larger.  Every kernel that carries sums or exchanges
+    # products weights them before they leave the scaled-down range.  2, 4 and 15 K stages of a term
+    U, V, W = coeffs("phi_optimal")
+    U, W = np.float32(8) * np.asarray(U, np.float32), np.asarray(W, np.float32) / np.float32(8)
+    M, N = 256, 512
+    A, B = Wl.gaussian(M, K, N, seed=8)
+    a, b = dev(A), dev(B)
+    # elements of C up to 2^(e + 2) sqrt(K), products up to 2^(e + 5.5) sqrt(K)
+    e = 124 - int(np.ceil(np.log2(K) / 2))
+    sa, sb = 2.0 ** (e // 2), 2.0 ** (e - e // 2)
+    plan = fmm.Plan(U, V, W, levels=1, block_k=32, scale_mode="fp32")
+    for form in [f for f in SHAPES[(32, "fp32", 0)] if f[4] == 0]:
+        plan.force_product_shape(*form)
+        want = plan.matmul(a, b).double() * 2.0 ** e
+        got = plan.matmul(a * sa, b * sb)
+        assert plan.device_status() == (0, 0)
+        assert torch.isfinite(got).all(), f"{form}"
+        assert torch.equal(got.double(), want), f"{form}"
