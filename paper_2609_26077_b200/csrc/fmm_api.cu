@@ -772,8 +772,11 @@ static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L,
     if (!sig(lane.up[strips], st, lane.comp)) return join(FMM_ERR_CUDA);
     fmm_status_t s = by_rows ? encode_side(plan, L, ws, dB, K, N, true, 0, L.n, false, lane.comp, &launches)
                              : encode_side(plan, L, ws, dA, M, K, false, 0, L.m, false, lane.comp, &launches);
-    // A strip of C goes down behind its product and the next strip's upload, that is with the upload after that one: a copy
-    // that starts while the other direction is busy takes some 45 us to get going, two that start together do not.
+    // Where the uploads are the longer part, a strip of C goes down behind its product and the next strip's upload, that is with the
+    // upload after that one: a copy that starts while the other direction is busy takes some 45 us to get going, two that start
+    // together do not.  Where the downloads are, each one goes as soon as it can (8192 x 2048 x 4096 3.40 ms,
+    // behind the next upload 3.46; 16384 x 512 x 2048 2.68, 2.70; 4096 x 1024 x 4096 1.75, 1.76 to 1.80).
+    const bool with_upload = (M + N) * K > M * N;
     int last = -1;                             // the strip whose product was enqueued last
     int64_t c_lo = 0, c_hi = 0;
     auto send_down = [&]() {
@@ -785,13 +788,14 @@ static fmm_status_t matmul_host_strips(const fmm_plan* plan, const FmmLayout& L,
         Strip part = {0, L.m, 0, L.n};
         if (by_rows) { part.m0 = lo; part.m1 = hi; } else { part.n0 = lo; part.n1 = hi; }
         if (!copy_strip(by_rows ? dA : dB, by_rows ? A : B, by_rows ? M : K, by_rows ? K : N, blocks, by_rows, lo, hi, up, st) ||
-            !sig(lane.up[i], st, lane.comp) || !send_down()) return join(FMM_ERR_CUDA);
+            !sig(lane.up[i], st, lane.comp) || (with_upload && !send_down())) return join(FMM_ERR_CUDA);
         s = by_rows ? encode_side(plan, L, ws, dA, M, K, false, lo, hi, false, lane.comp, &launches)
                     : encode_side(plan, L, ws, dB, K, N, true, lo, hi, false, lane.comp, &launches);
         if (s == FMM_OK) s = multiply(plan, L, ws, dC, M, N, part, lane.comp, &launches, false);
         last = i; c_lo = lo; c_hi = hi;
+        if (s == FMM_OK && !with_upload && !send_down()) s = FMM_ERR_CUDA;
     }
-    if (s == FMM_OK && !send_down()) s = FMM_ERR_CUDA;
+    if (s == FMM_OK && with_upload && !send_down()) s = FMM_ERR_CUDA;
     plan->last_launches.store(launches, std::memory_order_relaxed);
     return join(s);
 }

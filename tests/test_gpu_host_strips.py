@@ -10,7 +10,7 @@ from gpu_common import coeffs, dev
 pytestmark = pytest.mark.gpu
 
 # (realization, levels, M, K, N): rows in strips while M >= N, columns otherwise
-CASES = [("phi_optimal", 1, 2560, 2048, 512), ("strassen", 1, 512, 2304, 2816), ("phi_optimal", 1, 4096, 1024, 4096),
+CASES = [("phi_optimal", 1, 2560, 2048, 512), ("strassen", 1, 512, 2304, 2816), ("phi_optimal", 1, 4096, 1024, 4096), ("strassen", 1, 2048, 1024, 4096),
          ("cubic", 0, 3456, 1024, 256), ("cubic", 0, 256, 1152, 3968), ("phi_optimal", 2, 1024, 4096, 1024)]
 
 
