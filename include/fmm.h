@@ -146,7 +146,9 @@ typedef struct {
     int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; cluster: 1 */
     int columns;                 /* columns of a tile */
     int k_shares;                /* cluster, one term: CTAs that share K (1, 2, 4, 8); otherwise 1 */
-    int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = every product is summed on its own and written by warps of its own; 0 = sums are carried from product to product */
+    int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = every product is summed on its own; 0 = sums are carried
+                                    from product to product.  Warps of their own write the sums out with 1 at every K, with 0 where
+                                    K / 2^levels is 512 or more (below that the warps that sum them do); otherwise 0 */
 } fmm_product_shape_t;
 /* The shape that fmm_matmul and fmm_multiply_only take for this problem size (host call; errors as fmm_matmul). */
 fmm_status_t fmm_product_shape(const fmm_plan_t* plan, int64_t M, int64_t N, int64_t K, fmm_product_shape_t* shape);

@@ -1021,11 +1021,12 @@ fmm_status_t fmm_launch_encode_b(EncodeParams p, int blk, int mode, cudaStream_t
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
 }
 
-// One launch for both sides where the call's cost is its launches (2.6 us of host time, 0.4 to 1.3 us of the device's): up to so
-// many warps per SM.  Above that the A side is better off with the registers and blocks of its own kernel.  Both ways, in us,
-// Phi-optimal, n = 512 / 1024 / 2048 / 3072: UE8M0 10.2, 9.7 / 14.0, 13.1 / 32.0, 32.5 / 57.9, 61.1; weight tiles 11.3, 10.0 /
-// 15.3, 14.4 / 38.9, 37.7 / 76.9, 80.1; block 128 9.3, 8.8 / 13.9, 13.5 / 39.4, 38.2 / 69.1, 72.1; block 32 15.2, 13.0 / 17.2, 17.7 /
-// 64.8, 64.8 / 107, 111 (768: 12.3, 12.9).  The B side's blocks come first: they take longer (the other way round nothing is gained).
+// One launch for both sides where the call's cost is its launches (2.6 us of host time, up to 2 us of the device's): up to so
+// many warps per SM.  Above that the A side is better off with the registers and blocks of its own kernel.  Calls with a launch a
+// side and with one, in us, Phi-optimal, n = 256 / 512 / 1024 / 2048 / 3072: UE8M0 12.3, 10.8 / 12.3, 12.3 / 16.4, 14.4 / 31.2, 31.3 / 60.0,
+// 63.5; weight tiles 10.8, 10.3 / 12.3, 10.7 / 16.4, 16.4 / 39.9, 38.6 / 78.0, 80.6; block 128 10.3, 8.2 / 10.6, 10.3 / 16.1, 15.3 /
+// 41.0, 39.7 / 71.5, 74.1; block 32 10.3, 10.3 / 12.3, 12.3 / 18.5, 20.1 / 66.9, 67.2 / 111, 114.  The B side's blocks come first: they take
+// longer (the other way round nothing is gained).
 bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int mode, cudaStream_t st, fmm_status_t* status)
 {
     if (a.nq != 4 || b.nq != 4 || a.batch != 1 || b.batch != 1) return false;

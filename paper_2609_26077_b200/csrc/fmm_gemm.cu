@@ -902,10 +902,11 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
     kp.m = g.m; kp.n = g.n; kp.k = g.k; kp.msub = g.msub; kp.nsub = g.nsub; kp.terms = g.terms;
     kp.positions = positions; kp.tiles_n = tiles_n; kp.terms_per_group = tpg;
     kp.items = slots;
-    // In the second half of the table every product is summed on its own: with 64 and more K blocks a term the updates that
-    // carried sums save are hidden behind the next product (n = 8192: Phi-optimal 0.9 % of the call, Winograd at 6144 0.4 %;
-    // Strassen at 4096 is 1.6 % faster without, Phi-optimal 2.3 % slower), and they cost the most accuracy: 1.19 times the
-    // error for Winograd, 1.20 for Phi-optimal (n = 4096)
+    // In the second half of the table every product is summed on its own: from SEPARATE_STAGES on the updates that carried sums
+    // save are hidden behind the next product (product kernel, us, carried and separate: Phi-optimal n = 8192 1372, 1374, two levels
+    // 1425, 1445; n = 4096 215.0, 215.8, Winograd 206.1, 208.3, Strassen 211.6, 210.8; with 12 stages a term 173.3, 176.9 / 160.8, 162.1 /
+    // 163.4, 163.5, with 8 121.8, 135.7 / 113.4, 115.4 / 115.0, 114.1), and they cost the most accuracy: 1.19 times the error for
+    // Winograd, 1.20 for Phi-optimal (n = 4096)
     kp.walk = separate ? g.walk + g.terms : g.walk;
     kp.out = g.out; kp.status = g.status;
     kp.pair_start = g.pair_start; kp.pair = g.pair; kp.steps = (short)g.steps;
@@ -924,7 +925,7 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = NCTA; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     // right behind the encoders of the same call: the CTAs may be set up (barriers, TMEM, tensor maps) while the B-side
-    // encoder drains; the two producer warps wait for it before their first load
+    // encoder drains; the producer warps wait for it before their first load
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = g.overlap_prev ? 2 : 1;
@@ -939,9 +940,11 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 // hangs over the edge is multiplied and not stored, so a leaf of an odd number of 128-row or 128-column blocks may take the
 // wide tiles as well, at the price of a part of its last row or column of tiles.  Fitted, together with the cluster kernel's
 // model (fmm_split.cu), to the times of every shape over leaves of 128 to 8192 in every direction and zero to three levels.
-// Over 60 random problems per kind (leaves of 128 to 5000) the choice is the fastest shape for 41 to 54 of them and costs, in
-// the mean, 1.7 % (block 32), 0.3 % (UE8M0), 1.4 % (block 128) and 1.7 % (weight tiles) more than the fastest; the worst are
-// single products of about 10 us, at up to 1.34 times.  Product kernel
+// Over 60 random problems per kind (leaves of 128 to 5000) the choice is the fastest shape for 39 to 54 of them and costs, in
+// the mean, 3.2 % (block 32), 0.7 % (UE8M0), 2.7 % (block 128) and 2.9 % (weight tiles) more than the fastest; those above 12 us
+// 1.5 %, 0.8 %, 0.1 % and 1.4 %.  The worst are single products of about 8 us, at up to 1.33 times, and at block 32, whose constants and the
+// cluster kernel's stand as fitted to a slower promotion, products of 30 to 74 us that the persistent kernel would take in 0.81 times
+// the cluster kernel's time (2816 x 768 x 3840, 7936 x 512 x 768; with carried sums instead of separate ones).  Product kernel
 // against the rule before, which gave wide tiles only to leaves that are multiples of them: UE8M0 8192 x 8192 x 8448 one
 // level 674 -> 492 us, cubic 4096 x 1024 x 4224 47.6 -> 26.4; block 128 8192 x 8192 x 8448 956 -> 787; weight tiles
 // 888 -> 664.

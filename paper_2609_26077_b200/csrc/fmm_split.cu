@@ -14,7 +14,7 @@
 // columns, so where the narrower tiles still find room at once they are the faster ones (see the time models below).
 //
 // With UE8M0 scales a CTA may multiply two of the terms, one after the other: clusters of ceil(R / 2) fit the GPCs where clusters
-// of 7 leave 86 of 296 places empty, and hold 64 tiles at once instead of 30.  The first product waits in registers until the
+// of 7 leave 86 of 296 places empty, and hold 66 tiles at once instead of 30.  The first product waits in registers until the
 // operand ring is free; three halves of 64 columns fit over the ring, so the exchange goes in two passes.  (With FP32 scales the
 // registers hold the running sums, and neither TMEM nor shared memory has room for another product beside a second CTA.)
 //

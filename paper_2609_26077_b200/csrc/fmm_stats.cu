@@ -6,6 +6,7 @@
 //                       single-block second stage, hence bit-reproducible.
 #include <mutex>
 #include "fmm_internal.h"
+#include "fmm_ptx.cuh"
 
 // Scratch of fmm_error_stats_noalloc: one partial triple per reduction block.  It lives in the
 // library image, so every GPU that loads the library carries these 24 KB until the process exits.
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(STAT_THREADS) error_final_kernel(const double*
 {
     __shared__ double sm[3 * (STAT_THREADS / 32)];
     double sd = 0.0, sr = 0.0, mx = 0.0;
-    asm volatile("griddepcontrol.wait;" ::: "memory");       // launched under the first kernel's tail: its partials are complete now
+    fmmptx::griddep_wait();                                  // launched under the first kernel's tail: its partials are complete now
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
         sd += partial[i * 3]; sr += partial[i * 3 + 1]; mx = fmax(mx, partial[i * 3 + 2]);
     }

@@ -38,7 +38,9 @@ def test_matches_one_term_per_cta_and_the_oracle(name, levels, shape):
 
 def test_choice():
     plan = make_plan("phi_optimal", 1, 32, "ue8m0")
-    assert plan.product_shape(2048, 2048, 2048).kernel == TWO          # 64 tiles
+    # 55 and 56 tiles: between what one wave of clusters of seven and of four holds, with room on both sides
+    assert plan.product_shape(1792, 2048, 2048).kernel == TWO
+    assert plan.product_shape(1280, 2816, 3328).kernel == TWO
     assert plan.product_shape(1024, 1024, 1024).kernel == fmm.KERNEL_CLUSTER
     assert plan.product_shape(4096, 4096, 4096).kernel == fmm.KERNEL_PERSISTENT
 

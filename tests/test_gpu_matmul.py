@@ -39,7 +39,7 @@ CASES = [
     ("strassen", 1, (5120, 512, 4096), 32, "ue8m0", "gaussian"),
     ("phi_optimal", 1, (4864, 256, 4096), 32, "ue8m0", "uniform"),
     ("strassen", 1, (5120, 512, 4096), 128, "fp32", "gaussian"),
-    # 16 or more K stages per term: fp32 / block-32 products take the kernel variant with the output warp
+    # 16 or more K stages per term: fp32 / block-32 products are summed on their own (output warps write from 4 stages on)
     ("cubic", 0, (256, 3072, 384), 32, "fp32", "gaussian"),
     ("phi_optimal", 1, (512, 6144, 768), 32, "fp32", "llm"),
     ("winograd", 1, (768, 8192, 256), 32, "fp32", "uniform"),
@@ -83,8 +83,8 @@ def test_repeat_calls_are_bit_reproducible_and_overwrite_c():
 
 
 def test_output_warp_variant_is_bit_reproducible():
-    # 48 K stages per term: the fp32 / block-32 product runs the kernel variant whose post-addition is issued by a
-    # dedicated warp while the next term is being promoted; the order of the add-reductions per tile is still fixed
+    # 48 K stages per term: the fp32 / block-32 product runs the kernel variant whose post-addition is issued by two
+    # dedicated warps while the next term is being promoted; the order of the add-reductions per tile is still fixed
     A, B = Wl.llm_shaped(512, 12288, 512, 2)
     plan = make_plan("phi_optimal", 1, 32, "fp32")
     a, b = dev(A), dev(B)

@@ -57,11 +57,13 @@ def test_every_shape_matches_oracle(name, levels, shape, quantizer):
 
 @pytest.mark.parametrize("quantizer", list(SHAPES))
 def test_shapes_that_do_not_exist_are_refused(quantizer):
-    known = set(SHAPES[quantizer])
     for levels, name in ((0, "cubic"), (1, "strassen")):
+        known = set(SHAPES[quantizer])
+        if quantizer[1] == "ue8m0" and levels:
+            known.add((fmm.KERNEL_CLUSTER_TWO_TERMS, 1, 128, 1, 0))
         plan = make(name, levels, quantizer)
         chosen = tuple(plan.product_shape(256, 256, 256))
-        for form in [(k, c, n, s, w) for k in (1, 2, 3) for c in (1, 2) for n in (32, 64, 128, 256) for s in (1, 2, 3) for w in (0, 1)]:
+        for form in [(k, c, n, s, w) for k in (1, 2, 3, 4) for c in (1, 2) for n in (32, 64, 128, 256) for s in (1, 2, 3) for w in (0, 1)]:
             base = (*form[:3], 1, form[4])
             if base in known and (form[3] == 1 or (form[3] == 2 and form[0] == CL and levels == 0)):
                 plan.force_product_shape(*form)
@@ -84,3 +86,24 @@ def test_more_k_shares_than_chunks_is_a_shape_error():
     plan.force_product_shape()
     plan.matmul(a, a.t().contiguous())
     assert plan.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("K", [768, 1024])
+@pytest.mark.parametrize("name", ["strassen", "phi_optimal"])
+def test_block_32_around_the_output_warps_boundary(name, K):
+    # terms of three and four K stages, more tiles than CTAs (182) and pairs (91 of an odd number of rows of tiles): sums carried,
+    # written by the promoting warps and by the output warps, and separate ones
+    M, N = 3328, 3584
+    A, B = Wl.gaussian(M, K, N, seed=32)
+    a, b = dev(A), dev(B)
+    plan = make(name, 1, (32, "fp32", 0))
+    want = O.fused_fmm(A, B, *coeffs(name), levels=1, blk=32, mode=O.SCALE_FP32)
+    carried = []
+    for form in SHAPES[(32, "fp32", 0)][:4]:
+        plan.force_product_shape(*form)
+        c = plan.matmul(a, b, out=torch.full((M, N), float("nan"), device="cuda"))
+        assert plan.device_status() == (0, 0)
+        assert np.linalg.norm(c.cpu().numpy() - want) <= 1e-5 * np.linalg.norm(want), f"{form}"
+        if form[4] == 0:
+            carried.append(c)
+    assert torch.equal(*carried)
