@@ -603,9 +603,9 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
         if (g.R > 1) break;
     }
     // two terms per CTA (UE8M0): for the products that clusters of R do not hold at once and these do.  f: a longer exchange, as a
-    // CTA sums twice the rows.  n = 2048 32.0 -> 29.9 us a call, 2048 x 512 x 2048 21.7 -> 19.5, 1280 x 3328 x 2816 40.3 -> 38.5, 512 x 4096
-    // x 8192 73.0 -> 68.5, two levels n = 1536 33.8 -> 32.1; where one wave of clusters of R is enough it is slower (n = 1536 19.6, 24.4;
-    // n = 1024 13.2, 15.9), and so it is in more than one wave of its own (n = 2560 52.7, the persistent kernel 45.4).
+    // CTA sums twice the rows.  n = 2048 33.4 -> 30.9 us a call, 2048 x 512 x 2048 23.0 -> 20.6, 1280 x 3328 x 2816 42.3 -> 40.7, 512 x 4096
+    // x 8192 76.0 -> 71.1, two levels n = 1536 35.4 -> 34.3; where one wave of clusters of R is enough it is slower (n = 1536 20.8, 26.6;
+    // n = 1024 14.4, 17.9), and so it is in more than one wave of its own (n = 2560 54.4, the persistent kernel 47.3).
     if (m.f_two > 0.0f && g.R > 1) {
         const int cap = resident_clusters<MODE, BLK>(g.device, (g.R + 1) / 2);
         const long long tiles = (long long)(g.m / BM) * (g.n / 128) * parents;
