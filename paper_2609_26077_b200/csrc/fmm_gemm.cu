@@ -482,7 +482,7 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         // chunks of 16 rows x 32 columns of TMEM with two register sets, the next chunk's load - of the next K block, stage or
         // term as well - in flight while this one is added.  A stage's scales arrive on the barrier that says its first K
         // blocks are multiplied: every wait costs a warp some 40 cycles that nothing hides with two warps to a scheduler.
-        // Block 32: 480 -> 440 cycles per 128 x 128 K block against 256 of arithmetic (cubic n = 4096 251 -> 234.5 us, n = 8192
+        // Block 32: 480 -> 440 cycles per 128 x 128 K block against 256 of arithmetic (cubic n = 4096 253 -> 240 us, n = 8192
         // 1685 -> 1550 in bursts); block 128, n = 4096: 141.5 -> 129 in bursts.  The arithmetic alone runs at 293, with the
         // TMEM loads and no barriers at 328, and the tensor cores' traffic costs another 40.  Measured around it: chunks of
         // 64 columns 5 % slower; 16 promoting warps of a quarter of the columns 3 to 10 %; the next barrier tested ahead of
