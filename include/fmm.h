@@ -142,8 +142,10 @@ fmm_status_t fmm_matmul_host(const fmm_plan_t* plan, const float* A, const float
 typedef struct {
     int kernel;                  /* 1: persistent kernel, a CTA or CTA pair walks the terms of a tile position;
                                     2: cluster kernel, one CTA per term and tile (or per share of K, where there is one term);
-                                    4: the same, UE8M0, one CTA per two terms and tile */
-    int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; cluster: 1 */
+                                    4: the same, UE8M0, one CTA per two terms and tile;
+                                    8: a CTA walks the terms of a tile position of one parent and keeps the position's tiles of
+                                    the parent's output blocks on chip (plans with products to combine: one CTA, 64 columns) */
+    int ctas;                    /* persistent: CTAs that share a tile (1, 2), its rows being 128 times that; others: 1 */
     int columns;                 /* columns of a tile */
     int k_shares;                /* cluster, one term: CTAs that share K (1, 2, 4, 8); otherwise 1 */
     int output_warp;             /* persistent, FP32 scales, block_k 32: 1 = every product is summed on its own; 0 = sums are carried

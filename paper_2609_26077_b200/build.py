@@ -7,7 +7,7 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfmm_b200.so")
-SOURCES = ["fmm_api.cu", "fmm_encode.cu", "fmm_gemm.cu", "fmm_split.cu", "fmm_stats.cu"]
+SOURCES = ["fmm_api.cu", "fmm_encode.cu", "fmm_gemm.cu", "fmm_keep.cu", "fmm_split.cu", "fmm_stats.cu"]
 HEADERS = [os.path.join(CSRC, h) for h in sorted(os.listdir(CSRC)) if h.endswith((".h", ".cuh"))] + [
     os.path.join(HERE, "..", "include", "fmm.h")]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -327,7 +327,7 @@ GemmParams product_params(const fmm_plan* plan, const FmmLayout& L, const Strip&
     g.terms_per_group = plan->levels >= 2 ? plan->rank : (int)L.terms;
     g.device = plan->device; g.sms = plan->sms;
     g.R = plan->levels >= 1 ? plan->rank : 1; g.nq = plan->levels >= 1 ? 4 : 1; g.W = plan->W;
-    g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0;
+    g.sb_tile = plan->qp.b_tile_n == 128 ? 1 : 0; g.updates = plan->updates;
     g.forced = plan->forced;
     return g;
 }
@@ -559,6 +559,8 @@ fmm_status_t fmm_plan_create(fmm_plan_t** out, int rank, const float* U, const f
         pentries.push_back(e);
     }
     pstart.push_back((int)pentries.size());
+
+    p->updates = qp->scale_mode == FMM_SCALE_UE8M0_CEIL ? (int)(pentries.size() / parents) : walk[levels ? rank - 1 : 0].out1;
 
     p->lanes = new (std::nothrow) FmmHostLanes;
     if (!p->lanes) { delete p; return FMM_ERR_ALLOC; }

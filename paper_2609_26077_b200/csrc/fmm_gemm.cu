@@ -961,12 +961,12 @@ constexpr float BASE_MX = 3.3f, BASE_B32 = 2.4f, BASE_B128 = 3.85f, BASE_TILE = 
 template <int N>
 GemmShape best_shape(const GemmParams& g, int m, int n, const ShapeModel (&models)[N], float base)
 {
-    GemmShape best = {0, 0, 0.0f};
+    GemmShape best = {0, 0, 0.0f, 0};
     for (const ShapeModel& s : models) {
         const int positions = tile_positions(m, n, s.ncta, s.bn), units = g.sms / s.ncta, tpg = terms_per_item(g, positions, units);
         const long long longest = ((long long)positions * (g.terms / tpg) + units - 1) / units * tpg;
         const float time = base + (float)longest * ((float)(g.k / BK) * s.c + (g.R > 1 ? s.o : s.o_cubic));
-        if (best.ncta == 0 || time < best.time) best = {s.ncta, s.bn, time};
+        if (best.ncta == 0 || time < best.time) best = {s.ncta, s.bn, time, longest};
     }
     return best;
 }
@@ -1008,6 +1008,7 @@ fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
 {
     if (g.forced.kernel) return g.forced;
     const SplitChoice split = fmm_split_choice(g, blk, mode);
+    if (g.R > 1 && fmm_keep_faster(g, blk, mode, split, fmm_gemm_shape(g, blk, mode, g.m, g.n))) return {8, 1, 64, 1, 0};
     if (split.ksplit > 0) return {split.terms == 2 ? 4 : 2, 1, split.bn, split.ksplit, 0};
     const GemmShape s = fmm_gemm_shape(g, blk, mode, g.msub, g.nsub);
     return {1, s.ncta, s.bn, 1, mode != FMM_SCALE_UE8M0_CEIL && blk == 32 && g.k / BK >= SEPARATE_STAGES};
@@ -1016,6 +1017,7 @@ fmm_product_shape_t fmm_choose_product(const GemmParams& g, int blk, int mode)
 bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R)
 {
     const bool mx = mode == FMM_SCALE_UE8M0_CEIL;
+    if (s.kernel == 8) return R > 1 && s.ctas == 1 && s.columns == 64 && s.k_shares == 1 && !s.output_warp;
     if (s.kernel == 4) return mx && R > 1 && s.ctas == 1 && s.columns == 128 && s.k_shares == 1 && !s.output_warp;
     if (s.kernel == 2) {
         const bool width = s.columns == 128 || (!mx && (s.columns == 64 || s.columns == 32));
@@ -1040,8 +1042,9 @@ fmm_status_t fmm_launch_gemm(const GemmParams& g, int blk, int mode, cudaStream_
 {
     fmm_status_t s;
     const fmm_product_shape_t shape = fmm_choose_product(g, blk, mode);
-    if (shape.kernel == 2 || shape.kernel == 4)
-        s = shape.k_shares <= g.k / BK ? fmm_launch_split(g, blk, mode, {shape.k_shares, shape.columns, shape.kernel / 2}, st) : FMM_ERR_SHAPE;
+    if (shape.kernel == 8) s = fmm_launch_keep(g, blk, mode, st);
+    else if (shape.kernel == 2 || shape.kernel == 4)
+        s = shape.k_shares <= g.k / BK ? fmm_launch_split(g, blk, mode, {shape.k_shares, shape.columns, shape.kernel / 2, 0}, st) : FMM_ERR_SHAPE;
     else if (mode == FMM_SCALE_UE8M0_CEIL) s = launch_shape<FMM_SCALE_UE8M0_CEIL, 32>(g, shape, st);
     else if (blk == 128 && g.sb_tile) s = launch_shape<MODE_FP32_SB_TILE, 128>(g, shape, st);
     else if (blk == 32) s = launch_shape<FMM_SCALE_FP32_AMAX_DIV_448, 32>(g, shape, st);

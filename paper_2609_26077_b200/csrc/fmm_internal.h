@@ -106,6 +106,7 @@ struct fmm_plan {
     FmmOutEntry* d_out;       // [total entries], block offsets in units of leaf blocks (scaled at launch)
     int order[FMM_MAX_RANK];  // pair-fused decoder: walk order of the R products of a parent
     int steps;                // pair-fused decoder: steps per parent, ceil(R / 2)
+    int updates;              // of a parent's output blocks, by the walk with carried sums or by the pair-fused decoder
     int* d_pair_start;        // [parents * steps + 1]
     FmmPairEntry* d_pair;     // entries of all steps
     // kernels launched by the most recent call on this plan; written once, at the end of a call (calls take the
@@ -191,6 +192,7 @@ struct GemmParams {
     int order[FMM_MAX_RANK]; int steps;
     int device, sms;                        // the plan's device and its SM count
     int R, nq;                              // products per parent; blocks of a parent's matrix (4, or 1 for the cubic product)
+    int updates;                            // fmm_plan::updates
     const float (*W)[4];                    // innermost decoder, R x 4 (host pointer; unused when nq == 1)
     int* status;
     int terms_per_group;                    // consecutive terms that feed the same output blocks (R at levels >= 2, else all)
@@ -204,19 +206,24 @@ struct GemmParams {
 fmm_status_t fmm_stats_guard_read(int* code);
 fmm_status_t fmm_launch_bounded_wait_selftest(int* status, unsigned long long limit_ns, cudaStream_t st);
 fmm_status_t fmm_launch_guard_selftest(int* status, cudaStream_t st);
-// Tile shape (CTAs per tile, columns) with which the persistent kernel takes a leaf of m x n, and its time in microseconds by the
-// model the choice is made with
-struct GemmShape { int ncta, bn; float time; };
+// Tile shape (CTAs per tile, columns) with which the persistent kernel takes a leaf of m x n, its time in microseconds by the
+// model the choice is made with, and the terms that its busiest CTA (pair) walks
+struct GemmShape { int ncta, bn; float time; long long longest; };
 GemmShape fmm_gemm_shape(const GemmParams& p, int blk, int mode, int m, int n);
 // How the cluster kernel (fmm_split.cu) takes this product: K shares per term and columns per tile; 0 shares: the persistent
 // kernel is faster
-struct SplitChoice { int ksplit, bn, terms; };        // terms: of a CTA
+struct SplitChoice { int ksplit, bn, terms, places; };        // terms: of a CTA; places: clusters that the device holds at once
 SplitChoice fmm_split_choice(const GemmParams& p, int blk, int mode);
 // The forced shape, or the one that is expected to be fastest.  The kernel is chosen for the whole problem (m, n), also when
 // a launch covers a strip of it (msub, nsub): the strips' results do not depend on the cut
 fmm_product_shape_t fmm_choose_product(const GemmParams& p, int blk, int mode);
 bool fmm_product_shape_exists(const fmm_product_shape_t& s, int blk, int mode, int sb_tile, int R);
 fmm_status_t fmm_launch_split(const GemmParams& p, int blk, int mode, SplitChoice c, cudaStream_t st);
+// The kernel that keeps a parent's output blocks on chip (fmm_keep.cu), for R > 1, and whether it is expected to take the problem in
+// less time than the cluster kernel (`split`, where that has K shares) or else the persistent kernel with the tile shape `tile`, whose
+// busiest CTA (pair) walks `longest` terms
+bool fmm_keep_faster(const GemmParams& p, int blk, int mode, const SplitChoice& split, const GemmShape& tile);
+fmm_status_t fmm_launch_keep(const GemmParams& p, int blk, int mode, cudaStream_t st);
 fmm_status_t fmm_launch_gemm(const GemmParams& p, int blk, int mode, cudaStream_t st, int* launches);
 
 // SMs of the current device (a cached host-side attribute: cheap); 1 where it cannot be read

@@ -589,7 +589,7 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
     const int kst = g.k / BK;
     const long long parents = g.terms / g.R;
     float best_time = persistent_time;
-    SplitChoice best = {0, 0, 1};
+    SplitChoice best = {0, 0, 1, 0};
     for (int ks = 1; g.R * ks <= FMM_MAX_RANK && ks <= kst; ks *= 2) {
         const int cap = resident_clusters<MODE, BLK>(g.device, g.R * ks);
         if (cap <= 0) break;
@@ -598,7 +598,7 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
             const long long tiles = (long long)(g.m / BM) * (g.n / (128 >> w)) * parents;
             const float waves = std::max(1.0f, (float)tiles / places);
             const float time = m.lat + waves * (m.f[w] + ((kst + ks - 1) / ks) * m.c[w]);
-            if (time < best_time) { best_time = time; best = {ks, 128 >> w, 1}; }
+            if (time < best_time) { best_time = time; best = {ks, 128 >> w, 1, cap}; }
         }
         if (g.R > 1) break;
     }
@@ -609,7 +609,7 @@ SplitChoice choose_split(const GemmParams& g, const SplitModel& m, float persist
     if (m.f_two > 0.0f && g.R > 1) {
         const int cap = resident_clusters<MODE, BLK>(g.device, (g.R + 1) / 2);
         const long long tiles = (long long)(g.m / BM) * (g.n / 128) * parents;
-        if (tiles <= cap && m.lat + m.f_two + 2 * kst * m.c[0] < best_time) best = {1, 128, 2};
+        if (tiles <= cap && m.lat + m.f_two + 2 * kst * m.c[0] < best_time) best = {1, 128, 2, cap};
     }
     return best;
 }
@@ -626,7 +626,7 @@ fmm_status_t launch_fp32(const GemmParams& g, int blk, int ksplit, cudaStream_t 
 
 SplitChoice fmm_split_choice(const GemmParams& g, int blk, int mode)
 {
-    if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0, 1};     // grid dimensions
+    if (g.m / BM > 65535 || g.terms / g.R > 65535) return {0, 0, 1, 0};     // grid dimensions
     const float t = fmm_gemm_shape(g, blk, mode, g.m, g.n).time;
     if (mode == FMM_SCALE_UE8M0_CEIL) return choose_split<FMM_SCALE_UE8M0_CEIL, 32>(g, SPLIT_MX, t);
     if (blk == 32) return choose_split<MODE_FP32_COLUMN, 32>(g, SPLIT_B32, t);

@@ -40,7 +40,7 @@ class ProductShape(C.Structure):
         return iter((self.kernel, self.ctas, self.columns, self.k_shares, self.output_warp))
 
 
-KERNEL_PERSISTENT, KERNEL_CLUSTER, KERNEL_CLUSTER_TWO_TERMS = 1, 2, 4
+KERNEL_PERSISTENT, KERNEL_CLUSTER, KERNEL_CLUSTER_TWO_TERMS, KERNEL_BLOCKS_ON_CHIP = 1, 2, 4, 8
 
 
 class FmmError(RuntimeError):
