@@ -57,13 +57,16 @@ struct Cfg {
     // they can (accumulators, two TMEM chunks, scales).  Block 32 with output warps needs less: with 176 to 200 registers
     // ptxas finds a promotion loop that is 3 % faster than with 208 or more, with 168 it is 3 % slower (cubic n = 4096 233.4,
     // 240.9, 247.5 us; block 128 is 2 to 7 % slower with fewer than 224).  Every split is one that ptxas spills nothing with.
-    static constexpr int REGS_CTRL = !ROWS4 || DUMP ? 88 : BLK == 32 ? 72 : 56, REGS_EPI = !ROWS4 ? 208 : DUMP ? 192 : BLK == 32 ? 216 : 224;
+    // The weight-tile kernel needs 216 for two TMEM loads in flight beside 128 sums a thread.
+    static constexpr bool TILE = MODE == MODE_FP32_SB_TILE;
+    static constexpr int REGS_CTRL = MX || DUMP ? 88 : TILE || BLK == 32 ? 72 : 56, REGS_EPI = MX ? 208 : DUMP ? 192 : TILE || BLK == 32 ? 216 : 224;
     static_assert(EPI_WARP0 * 32 * REGS_CTRL + EPI_WARPS * 32 * REGS_EPI <= NUM_THREADS * REGS_AT_LAUNCH, "register pool");
     // Warp index, CTA rank and TMEM base as values the compiler knows to be warp-uniform (see warp_uniform): 3 % of the
     // block-32 kernel at n = 8192 and 4096, 7 % of the single-CTA UE8M0 kernel at 1280 x 2816 x 3328.  Not for the UE8M0
-    // pair kernel, whose 256-column instructions hide their issue (2 % slower), nor for the weight-tile kernel, which
-    // then spills in the promotion loop (10 % slower at n = 4096).
-    static constexpr bool UNIFORM = !(MX && NCTA == 2) && MODE != MODE_FP32_SB_TILE;
+    // pair kernel, whose 256-column instructions hide their issue (2 % slower), nor for the weight-tile pair kernel, which
+    // then spills in the promotion loop (10 % slower at n = 4096); the weight-tile kernel of single CTAs, whose 128-column
+    // instructions do not hide it, gains 19 % (n = 4096 Winograd 105 -> 84.5 us, Phi-optimal 117 -> 99, cubic 98 -> 76).
+    static constexpr bool UNIFORM = !(MX && NCTA == 2) && !(TILE && BN == 256);
     static constexpr int BROWS = BN / NCTA;                  // T_r rows this CTA loads per stage
     static constexpr int A_BYTES = BM * BK;
     static constexpr int B_BYTES = BROWS * BK;
@@ -718,20 +721,24 @@ fmm_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         tc_fence_after();
                         const float s = lds32f(sa_row + ss * C::SB_STAGE_BYTES) * lds32f(base + C::OFF_SB + h * C::CW * 4 + ss * C::SB_STAGE_BYTES);
                         const unsigned long long s2 = pack2(s, s);
+                        // 64 columns at a time, both loads in flight: an accumulator is handed back earlier and waited for less often
+                        // than with 32 (pairs, n = 4096: Phi-optimal 91 -> 88 us, Winograd 77.3 -> 74.6, cubic 75.5 -> 72.4; 16 columns
+                        // with the next load under the arithmetic 1 to 2 % slower)
 #pragma unroll
-                        for (int c = 0; c < C::CW / 32; ++c) {
-                            // (the next chunk's load under this one's arithmetic, as above: 1.5 to 2 % slower)
-                            uint32_t tmp[32];
-                            tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * BN + h * C::CW + c * 32, tmp);
+                        for (int c = 0; c < C::CW / 64; ++c) {
+                            uint32_t tmp[64];
+                            const uint32_t taddr = lane_taddr + buf * BN + c * 64;
+                            tmem_ld32(taddr, tmp);
+                            tmem_ld32(taddr + 32, tmp + 32);
                             tmem_ld_wait();
-                            if (c + 1 == C::CW / 32) {
+                            if (c + 1 == C::CW / 64) {
                                 // the last chunk is in registers: hand the TMEM buffer back before the arithmetic
                                 tc_fence_before();
                                 __syncwarp();
                                 if (lane == 0) release_acc(buf);
                             }
 #pragma unroll
-                            for (int j = 0; j < 16; ++j) acc2[c * 16 + j] = fma2(pack2u(tmp[2 * j], tmp[2 * j + 1]), s2, acc2[c * 16 + j]);
+                            for (int j = 0; j < 32; ++j) acc2[c * 32 + j] = fma2(pack2u(tmp[2 * j], tmp[2 * j + 1]), s2, acc2[c * 32 + j]);
                         }
                         if (++buf == C::ACC_BUFS) buf = 0;
                         __syncwarp();
@@ -951,11 +958,13 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 // Block 128: with the faster promotion the single CTAs have gained more than the pairs, whose constants are fitted again, to 666
 // problems (5 % faster on the 7 % of them that change; cubic n = 4096 122.3 -> 115.7 us a call, two levels 270 -> 257; the pairs stay at
 // n = 8192, 739 against 781, cubic 718 against 893).
+// Weight tiles: the same once more since the single CTAs' issuing warp knows its values to be uniform: the pairs' constants are scaled to
+// them (of 330 problems the choice between the two is 0.1 % off the faster one in the mean, 0.6 % with the constants before).
 struct ShapeModel { int ncta, bn; float c, o, o_cubic; };
 constexpr ShapeModel MODEL_MX[] = {{2, 256, 0.26f, 3.9f, 3.6f}, {1, 256, 0.35f, 3.4f, 2.7f}, {1, 128, 0.22f, 1.7f, 1.2f}};
 constexpr ShapeModel MODEL_B32[] = {{2, 128, 0.71f, 3.6f, 2.2f}, {1, 128, 0.67f, 3.55f, 1.85f}};
 constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 6.0f, 5.1f}, {1, 128, 0.28f, 2.5f, 1.8f}};
-constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.34f, 4.8f, 2.35f}, {1, 128, 0.26f, 2.4f, 1.15f}};
+constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.37f, 5.4f, 3.4f}, {1, 128, 0.26f, 2.4f, 1.15f}};
 constexpr float BASE_MX = 3.3f, BASE_B32 = 2.4f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
 
 template <int N>

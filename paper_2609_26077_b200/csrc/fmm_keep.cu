@@ -490,7 +490,7 @@ constexpr KeepModel KEEP_MX = {{4.72f, 2.94f, 0.1965f, 0.0341f}, {4.91f, 5.86f, 
 constexpr KeepModel KEEP_B128 = {{5.71f, 2.94f, 0.3177f, 0.0311f}, {5.9f, 6.16f, 0.677f, 0.034f}, {},
     {{1, 128, 5.73f, 2.43f, 0.309f, 0.992f, 0.00355f}, {2, 256, 7.17f, 3.2f, 0.59f, 2.088f, 0.00354f}, {}}};
 constexpr KeepModel KEEP_TILE = {{5.68f, 2.655f, 0.2362f, 0.0316f}, {6.01f, 6.06f, 0.592f, 0.0335f}, {},
-    {{1, 128, 5.32f, 2.345f, 0.381f, 0.78f, 0.00362f}, {2, 256, 5.25f, 0.744f, 0.494f, 2.283f, 0.00356f}, {}}};
+    {{1, 128, 5.1f, 1.92f, 0.272f, 0.985f, 0.00355f}, {2, 256, 7.0f, 0.66f, 0.449f, 2.153f, 0.00372f}, {}}};
 
 }  // namespace
 
