@@ -778,8 +778,10 @@ __global__ void __launch_bounds__(256) decode_kernel(const DecodeParams p)
 
 // Two outward steps at once (three levels): the R x R matrices of the second level go to the 16 blocks of the result with the
 // first-level matrices in registers, in the order of two single steps.  The first-level matrices are neither written nor read
-// back (n = 2048: 14 + 10 us as two launches).  The next R loads are in flight while R are combined.
-__global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
+// back (n = 2048: 14 + 10 us as two launches).  Bound by memory latency: R loads in flight per thread and four blocks per SM (109 registers)
+// keep more of it busy than the next R loads under the arithmetic and three (product kernel and decoder, n = 2048 39.1 -> 35.0 us, 4096 x 1024 x
+// 4096 100.7 -> 97.7, 8192 x 1024 x 8192 377 -> 364); 8 bytes per load and up to eight blocks are slower.
+__global__ void __launch_bounds__(128, 4) decode2_kernel(const DecodeParams p)
 {
     fmmptx::griddep_wait();
     const uint32_t tiles = (uint32_t)p.cols / 128, by = blockIdx.x / tiles, bx = blockIdx.x - by * tiles;
@@ -810,16 +812,11 @@ __global__ void __launch_bounds__(128) decode2_kernel(const DecodeParams p)
             }
         }
     };
-    float4 xa[FMM_MAX_RANK], xb[FMM_MAX_RANK];
-    load(0, xa);
+    float4 x[FMM_MAX_RANK];
 #pragma unroll 1
-    for (int r1 = 0; r1 < p.R; r1 += 2) {
-        if (r1 + 1 < p.R) load(r1 + 1, xb);
-        add(r1, xa);
-        if (r1 + 1 < p.R) {
-            if (r1 + 2 < p.R) load(r1 + 2, xa);
-            add(r1 + 1, xb);
-        }
+    for (int r1 = 0; r1 < p.R; ++r1) {
+        load(r1, x);
+        add(r1, x);
     }
 #pragma unroll
     for (int q1 = 0; q1 < 4; ++q1)
