@@ -239,7 +239,7 @@ fmm_keep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         // ROWS4: see the promotion loop of fmm_gemm.cu
         uint32_t set0[C::ROWS4 ? 16 : 1], set1[C::ROWS4 ? 16 : 1];
         unsigned long long sb2[4];
-        float sa1[4];
+        float sa[KB == 4 ? 4 : 1][4];                               // A-side scales of the thread's rows: of a stage's K blocks [row][block], or [0][row]
         const uint32_t sa_lane = base + C::OFF_S + C::SB_BYTES + (q * 32 + (lane >> 2)) * (KB * 4);
         const uint32_t sb_lane = base + C::OFF_S + (h * CW + 2 * (lane & 3)) * 4;
         auto wait_full = [&](int slot, uint32_t phase) {
@@ -249,17 +249,20 @@ fmm_keep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         auto load_chunk = [&](uint32_t* r, int b, int gi, int i) {
             tmem_ld_16x256b_x4(tq + (b * C::GPB + gi) * BN + ((uint32_t)(16 * i) << 16), r);
         };
-        auto load_scales = [&](unsigned long long (&b)[4], float (&a)[4], int s, int g) {
+        auto load_sb = [&](unsigned long long (&d)[4], int s, int g) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = lds64(sb_lane + s * C::S_BYTES + (g * BN + 8 * j) * 4);
+            for (int j = 0; j < 4; ++j) d[j] = lds64(sb_lane + s * C::S_BYTES + (g * BN + 8 * j) * 4);
+        };
+        auto load_sa1 = [&](float (&d)[4], int s) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) a[k] = lds32f(sa_lane + s * C::S_BYTES + (8 * k * KB + g) * 4);
+            for (int k = 0; k < 4; ++k) d[k] = lds32f(sa_lane + s * C::S_BYTES + 8 * k * 4);
         };
         if constexpr (C::ROWS4) {
             ok = wait_full(0, 0);
             tc_fence_after();
             load_chunk(set0, 0, 0, 0);
-            load_scales(sb2, sa1, 0, 0);
+            load_sb(sb2, 0, 0);
+            if constexpr (KB == 1) load_sa1(sa[0], 0);
             tmem_ld_wait16(set0);
         }
         for (int w = blockIdx.x; w < p.items && ok; w += gridDim.x) {
@@ -287,13 +290,21 @@ fmm_keep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                         const bool wrap = ss + 1 == C::S_STAGES;
                         const int sn = wrap ? 0 : ss + 1;
                         const uint32_t pn = wrap ? sphase ^ 1u : sphase;
+                        if constexpr (KB == 4) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const float4 v4 = lds128(sa_lane + ss * C::S_BYTES + 8 * k * 16);
+                                sa[k][0] = v4.x; sa[k][1] = v4.y; sa[k][2] = v4.z; sa[k][3] = v4.w;
+                            }
+                        }
 #pragma unroll
                         for (int g = 0; g < KB; ++g) {
                             // acc += (P * sB) * sA, 16 rows at a time
                             auto promote = [&](const uint32_t* cur, int k0) {
 #pragma unroll
                                 for (int k = k0; k < k0 + 2; ++k) {
-                                    const unsigned long long s2 = pack2(sa1[k], sa1[k]);
+                                    const float s = KB == 4 ? sa[KB == 4 ? k : 0][g] : sa[0][k];
+                                    const unsigned long long s2 = pack2(s, s);
 #pragma unroll
                                     for (int j = 0; j < 4; ++j)
                                         acc[k * 4 + j] = fma2(mul2(pack2u(cur[4 * j + 2 * (k - k0)], cur[4 * j + 2 * (k - k0) + 1]), sb2[j]), s2, acc[k * 4 + j]);
@@ -314,10 +325,11 @@ fmm_keep_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                             unsigned long long sbn[4];
                             float san[4];
                             load_chunk(set0, nb, (g + 1) % KB, 0);
-                            load_scales(sbn, san, g + 1 < KB ? ss : sn, (g + 1) % KB);
+                            load_sb(sbn, g + 1 < KB ? ss : sn, (g + 1) % KB);
+                            if constexpr (KB == 1) load_sa1(san, sn);
                             promote(set1, 2);
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) { sb2[j] = sbn[j]; sa1[j] = san[j]; }
+                            for (int j = 0; j < 4; ++j) { sb2[j] = sbn[j]; if (KB == 1) sa[0][j] = san[j]; }
                             tmem_ld_wait16(set0);
                             buf = nb;
                         }
