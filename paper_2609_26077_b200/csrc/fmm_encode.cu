@@ -325,8 +325,9 @@ __device__ __forceinline__ void prefetch_block(const EncodeParams& p, int block_
 // share nothing, and one-warp blocks let the scheduler replace each finished warp on its own (2 % faster than four
 // warps of one 128-k chunk per block; blocks of two to eight warps side by side, covering 128- to 512-byte row
 // segments, are within 1 %).  Grid: (cols / 16, rows / 32, batch), 32 threads.
+// `only` >= 0: nothing but that combination (a grid with one block for each, see encode_both_kernel).
 template <int MODE, uint32_t NZ>
-__device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
+__device__ __forceinline__ void encode_b32_block(const EncodeParams& p, int b, int only = -1)
 {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x;
@@ -334,7 +335,6 @@ __device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
     const int j = blockIdx.x * 16 + col;
     const int kb = blockIdx.y;                      // this warp's quantization block
     const int kc = kb >> 2;                         // its chunk of 128 k
-    const int b = blockIdx.z;
     const int k0 = kb * 32 + khalf * 16;
     const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
     const int64_t term_codes = p.q_term;
@@ -342,7 +342,7 @@ __device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
     float raw[4][16];
 #pragma unroll
     for (int jq = 0; jq < 4; ++jq)
-        if (jq < p.nq) {
+        if (jq < p.nq && (only < 0 || p.coef[only][jq] != 0.0f)) {
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk)
                 raw[jq][kk] = __ldg(base + p.qoff[jq] + (int64_t)(k0 + kk) * p.ld);
@@ -350,7 +350,7 @@ __device__ __forceinline__ void encode_b32_block(const EncodeParams& p)
     prefetch_block<32>(p, kb);
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
-        if (row_used<NZ>(r, p.R)) {
+        if (row_used<NZ>(r, p.R) && (only < 0 || r == only)) {
             float v[16];
             bool set = false;
 #pragma unroll
@@ -416,7 +416,7 @@ __device__ __forceinline__ void end_of_b_side()
 template <int MODE, uint32_t NZ>
 __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p)
 {
-    encode_b32_block<MODE, NZ>(p);
+    encode_b32_block<MODE, NZ>(p, blockIdx.z);
     end_of_b_side();
 }
 
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(32, 16) encode_b32_kernel(const EncodeParams p
 // operand); every column stores the tile's scale, so the scale array keeps its per-column shape.  PRE rounds each encoded
 // combination to bfloat16 (nearest even) before the maximum and the cast, as the paper's real kernel does.
 template <uint32_t NZ, bool TILE, bool PRE>
-__device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
+__device__ __forceinline__ void encode_b128_block(const EncodeParams& p, int b, int only = -1)
 {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int MODE = FMM_SCALE_FP32_AMAX_DIV_448;
@@ -442,7 +442,6 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
     const int col = lane & 15, khalf = lane >> 4;
     const int j = blockIdx.x * 16 + col;
     const int kc = blockIdx.y;                      // chunk of 128 k = one quantization block
-    const int b = blockIdx.z;
     const int k0 = kc * 128 + warp * 32 + khalf * 16;
     const float* base = p.in + (int64_t)b * p.in_batch_stride + j;
     const int64_t term_codes = p.q_term;
@@ -450,7 +449,7 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
     float raw[4][16];
 #pragma unroll
     for (int jq = 0; jq < 4; ++jq)
-        if (jq < p.nq) {
+        if (jq < p.nq && (only < 0 || p.coef[only][jq] != 0.0f)) {
 #pragma unroll
             for (int kk = 0; kk < 16; ++kk)
                 raw[jq][kk] = __ldg(base + p.qoff[jq] + (int64_t)(k0 + kk) * p.ld);
@@ -483,7 +482,7 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
     };
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
-        if (row_used<NZ>(r, p.R)) {
+        if (row_used<NZ>(r, p.R) && (only < 0 || r == only)) {
             float v[16];
             combine(r, v);
             float amax = 0.0f;
@@ -516,7 +515,7 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
     }
 #pragma unroll
     for (int r = 0; r < FMM_MAX_RANK; ++r) {
-        if (row_used<NZ>(r, p.R)) {
+        if (row_used<NZ>(r, p.R) && (only < 0 || r == only)) {
             const float amax = TILE ? tile_amax[r]
                                     : fmaxf(fmaxf(sub_amax[0][r][col], sub_amax[1][r][col]), fmaxf(sub_amax[2][r][col], sub_amax[3][r][col]));
             float sc; uint32_t e8;
@@ -543,25 +542,26 @@ __device__ __forceinline__ void encode_b128_block(const EncodeParams& p)
 template <uint32_t NZ, bool TILE, bool PRE>
 __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams p)
 {
-    encode_b128_block<NZ, TILE, PRE>(p);
+    encode_b128_block<NZ, TILE, PRE>(p, blockIdx.z);
     end_of_b_side();
     if (TILE) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");           // its own maxima are no longer read either
 }
 
-// Both sides of a call in one launch, for calls whose cost is their launches: the blocks of the B-side encoder, and behind
-// them (gridDim.y - pb.rows / BLK rows of blocks) warps for the A side's tasks.
+// Both sides of a call in one launch, for calls whose cost is their launches: the blocks of the B-side encoder (gridDim.z of them for each
+// place, one per combination, or one for all), and behind them (gridDim.y - pb.rows / BLK rows of blocks) warps for the A side's tasks.
 template <int BLK, int MODE, uint32_t NZA, uint32_t NZB, bool TILE, bool PRE>
 __global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) encode_both_kernel(const __grid_constant__ EncodeParams pa, const __grid_constant__ EncodeParams pb)
 {
     const uint32_t b_rows = (uint32_t)pb.rows / BLK;
     const bool b_side = blockIdx.y < b_rows;
     if (b_side) {
-        if constexpr (BLK == 32) encode_b32_block<MODE, NZB>(pb);
-        else encode_b128_block<NZB, TILE, PRE>(pb);
+        const int only = gridDim.z > 1 ? (int)blockIdx.z : -1;
+        if constexpr (BLK == 32) encode_b32_block<MODE, NZB>(pb, 0, only);
+        else encode_b128_block<NZB, TILE, PRE>(pb, 0, only);
     } else {
         constexpr uint32_t WARPS = BLK / 32;
-        encode_a_tasks<BLK, MODE, NZA>(pa, ((blockIdx.y - b_rows) * gridDim.x + blockIdx.x) * WARPS + fmmptx::warp_uniform(threadIdx.x >> 5),
-                                       (gridDim.y - b_rows) * gridDim.x * WARPS);
+        encode_a_tasks<BLK, MODE, NZA>(pa, ((blockIdx.z * (gridDim.y - b_rows) + blockIdx.y - b_rows) * gridDim.x + blockIdx.x) * WARPS + fmmptx::warp_uniform(threadIdx.x >> 5),
+                                       gridDim.z * (gridDim.y - b_rows) * gridDim.x * WARPS);
     }
     fmmptx::griddep_launch_dependents();           // as end_of_b_side (nothing to wait for: an ordinary launch)
     if (TILE && b_side) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
@@ -955,11 +955,12 @@ void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
     }
 }
 template <int BLK, int MODE, bool TILE, bool PRE>
-bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, cudaStream_t st)
+bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, bool split, cudaStream_t st)
 {
     constexpr unsigned THREADS = BLK == 32 ? 32 : 128;
     const unsigned gx = (unsigned)b.cols / 16, a_blocks = (a_warps + THREADS / 32 - 1) / (THREADS / 32);
-    const dim3 grid(gx, (unsigned)b.rows / BLK + (a_blocks + gx - 1) / gx);
+    const unsigned gz = split ? (unsigned)b.R : 1u;
+    const dim3 grid(gx, (unsigned)b.rows / BLK + (a_blocks + gx * gz - 1) / (gx * gz), gz);
     const uint32_t ma = coef_mask(a), mb = coef_mask(b);
 #define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE>, grid, THREADS, st, TILE ? 8 : 1, false, a, b); return true; }
     FMM_KNOWN_MASK_PAIRS(X)
@@ -1031,13 +1032,19 @@ bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int 
     const int64_t b_warps = (int64_t)(b.cols / 16) * (b.rows / 32);
     if (warps + b_warps > (int64_t)fmm_sm_count() * (blk == 128 ? 32 : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? 16 : 4)) return false;
     const unsigned w = (unsigned)warps;
+    // One combination per B-side block where that still leaves an SM few warps: a block of all R is a chain of 1250 instructions with a
+    // warp or two per scheduler to hide it.  us a call, all combinations and one per block: n = 256 Strassen block 32 10.25 -> 9.72, T* UE8M0
+    // 11.28 -> 10.26, block 128 10.25 -> 9.23; n = 512 T* UE8M0 12.31 -> 11.27, block 128 11.29 -> 10.27, weight tiles 12.29 -> 11.73.  Above
+    // these numbers of warps (half warps per SM) the operand, read by R / 2 blocks, costs more: block 32 n = 512 12.44 against 13.27, UE8M0
+    // 512 x 1024 x 512 12.82 against 13.33, n = 1024 block 128 16.39 against 17.43, UE8M0 15.52 against 18.44.
+    const bool split = 2 * b_warps * b.R <= (int64_t)fmm_sm_count() * (blk == 128 ? 49 : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? 13 : 8);
     bool known;
-    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) known = launch_both<32, FMM_SCALE_UE8M0_CEIL, false, false>(a, b, w, st);
-    else if (blk == 32) known = launch_both<32, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, st);
-    else if (b.b_tile && b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, true>(a, b, w, st);
-    else if (b.b_tile) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, false>(a, b, w, st);
-    else if (b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, true>(a, b, w, st);
-    else known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, st);
+    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) known = launch_both<32, FMM_SCALE_UE8M0_CEIL, false, false>(a, b, w, split, st);
+    else if (blk == 32) known = launch_both<32, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, split, st);
+    else if (b.b_tile && b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, true>(a, b, w, split, st);
+    else if (b.b_tile) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, false>(a, b, w, split, st);
+    else if (b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, true>(a, b, w, split, st);
+    else known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, split, st);
     if (known) *status = cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
     return known;
 }
