@@ -778,7 +778,7 @@ __global__ void __launch_bounds__(256) decode_kernel(const DecodeParams p)
 
 // Two outward steps at once (three levels): the R x R matrices of the second level go to the 16 blocks of the result with the
 // first-level matrices in registers, in the order of two single steps.  The first-level matrices are neither written nor read
-// back (n = 2048: 14 + 10 us as two launches).  Bound by memory latency: R loads in flight per thread and four blocks per SM (109 registers)
+// back (n = 2048: 14 + 10 us as two launches).  Bound by memory latency: R loads in flight per thread and four blocks per SM (128 registers)
 // keep more of it busy than the next R loads under the arithmetic and three (product kernel and decoder, n = 2048 39.1 -> 35.0 us, 4096 x 1024 x
 // 4096 100.7 -> 97.7, 8192 x 1024 x 8192 377 -> 364); 8 bytes per load and up to eight blocks are slower.
 __global__ void __launch_bounds__(128, 4) decode2_kernel(const DecodeParams p)
