@@ -547,15 +547,18 @@ __global__ void __launch_bounds__(128, 4) encode_b128_kernel(const EncodeParams 
     if (TILE) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");           // its own maxima are no longer read either
 }
 
-// Both sides of a call in one launch, for calls whose cost is their launches: the blocks of the B-side encoder (gridDim.z of them for each
-// place, one per combination, or one for all), and behind them (gridDim.y - pb.rows / BLK rows of blocks) warps for the A side's tasks.
-template <int BLK, int MODE, uint32_t NZA, uint32_t NZB, bool TILE, bool PRE>
-__global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : 4) encode_both_kernel(const __grid_constant__ EncodeParams pa, const __grid_constant__ EncodeParams pb)
+// Both sides of a call in one launch, for calls whose cost is their launches: the blocks of the B-side encoder (with ONE gridDim.z of them
+// for each place, one per combination, otherwise one for all), and behind them (gridDim.y - pb.rows / BLK rows of blocks) warps for the A
+// side's tasks.  ONE is a template argument: a combination chosen at run time keeps the compiler from interleaving the
+// combinations of a block that makes all of them (encode, block 128, T*: 256 x 2048 x 2560 8.27 -> 7.48 us, 2048 x 512 x 3072 5.01 -> 4.57).  The
+// panels of a plain pass have no combinations to interleave and take the registers that leave room for five blocks of 128 threads on an SM.
+template <int BLK, int MODE, uint32_t NZA, uint32_t NZB, bool TILE, bool PRE, bool ONE>
+__global__ void __launch_bounds__(BLK == 32 ? 32 : 128, BLK == 32 ? 16 : NZB == 0x00008421u ? 5 : 4) encode_both_kernel(const __grid_constant__ EncodeParams pa, const __grid_constant__ EncodeParams pb)
 {
     const uint32_t b_rows = (uint32_t)pb.rows / BLK;
     const bool b_side = blockIdx.y < b_rows;
     if (b_side) {
-        const int only = gridDim.z > 1 ? (int)blockIdx.z : -1;
+        const int only = ONE ? (int)blockIdx.z : -1;
         if constexpr (BLK == 32) encode_b32_block<MODE, NZB>(pb, 0, only);
         else encode_b128_block<NZB, TILE, PRE>(pb, 0, only);
     } else {
@@ -954,18 +957,23 @@ void launch_b2(const EncodeParams& p, dim3 grid, cudaStream_t st)
         default: launch_encoder(encode2_b_kernel<MODE, 0u>, grid, 256, st, 1, p.overlap_prev, p); return;
     }
 }
-template <int BLK, int MODE, bool TILE, bool PRE>
-bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, bool split, cudaStream_t st)
+template <int BLK, int MODE, bool TILE, bool PRE, bool ONE>
+bool launch_both_as(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, cudaStream_t st)
 {
     constexpr unsigned THREADS = BLK == 32 ? 32 : 128;
     const unsigned gx = (unsigned)b.cols / 16, a_blocks = (a_warps + THREADS / 32 - 1) / (THREADS / 32);
-    const unsigned gz = split ? (unsigned)b.R : 1u;
+    const unsigned gz = ONE ? (unsigned)b.R : 1u;
     const dim3 grid(gx, (unsigned)b.rows / BLK + (a_blocks + gx * gz - 1) / (gx * gz), gz);
     const uint32_t ma = coef_mask(a), mb = coef_mask(b);
-#define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE>, grid, THREADS, st, TILE ? 8 : 1, false, a, b); return true; }
+#define X(U, V) if (ma == U && mb == V) { launch_encoder(encode_both_kernel<BLK, MODE, U, V, TILE, PRE, ONE>, grid, THREADS, st, TILE ? 8 : 1, false, a, b); return true; }
     FMM_KNOWN_MASK_PAIRS(X)
 #undef X
     return false;
+}
+template <int BLK, int MODE, bool TILE, bool PRE>
+bool launch_both(const EncodeParams& a, const EncodeParams& b, unsigned a_warps, bool one, cudaStream_t st)
+{
+    return one ? launch_both_as<BLK, MODE, TILE, PRE, true>(a, b, a_warps, st) : launch_both_as<BLK, MODE, TILE, PRE, false>(a, b, a_warps, st);
 }
 
 // Tasks of the A-side encoder, one per warp; sets their length.  Long tasks keep two steps of loads in flight, but a problem has
