@@ -1041,18 +1041,25 @@ bool fmm_launch_encode_both(EncodeParams a, const EncodeParams& b, int blk, int 
     if (warps + b_warps > (int64_t)fmm_sm_count() * (blk == 128 ? 32 : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? 16 : 4)) return false;
     const unsigned w = (unsigned)warps;
     // One combination per B-side block where that still leaves an SM few warps: a block of all R is a chain of 1250 instructions with a
-    // warp or two per scheduler to hide it.  us a call, all combinations and one per block: n = 256 Strassen block 32 10.25 -> 9.72, T* UE8M0
-    // 11.28 -> 10.26, block 128 10.25 -> 9.23; n = 512 T* UE8M0 12.31 -> 11.27, block 128 11.29 -> 10.27, weight tiles 12.29 -> 11.73.  Above
-    // these numbers of warps (half warps per SM) the operand, read by R / 2 blocks, costs more: block 32 n = 512 12.44 against 13.27, UE8M0
-    // 512 x 1024 x 512 12.82 against 13.33, n = 1024 block 128 16.39 against 17.43, UE8M0 15.52 against 18.44.
-    const bool split = 2 * b_warps * b.R <= (int64_t)fmm_sm_count() * (blk == 128 ? 49 : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? 13 : 8);
+    // warp or two per scheduler to hide it, but with a block for each the operand is read R / 2 times (by the four panels of a plain pass
+    // once) and every warp's start and end are paid for.  What decides is all warps of that launch, the A side's included: the B side's alone misjudge
+    // operands with many rows of A.  The bf16 pre-round lengthens the chain.  Of 973 problems (leaves of 64 to 1536, operands in L2 and not) the
+    // other form would be faster by more than 2 % for 13.  us a call in a graph, Phi-optimal, all combinations and one per block (warps per SM): block
+    // 32 n = 256 7.80, 7.46 (2); 512 x 256 x 512 9.33, 9.26 (3.9); n = 512 10.45, 11.06 (7).  UE8M0 n = 256 9.40, 8.26 (2); n = 512 9.99, 9.75 (7.8);
+    // 512 x 1024 x 512 10.68, 11.70 (16); n = 1024 13.53, 16.21 (31).  Block 128 n = 256 7.54, 6.83 (2.4); 512 x 1536 x 256 9.36, 9.20 (14.3); n = 768 11.19,
+    // 11.53 (18.8); n = 1024 13.76, 14.79 (31).  Weight tiles n = 256 8.46, 7.50; 512 x 1536 x 256 10.31, 10.13; 512 x 1024 x 512 10.73, 11.20 (15.6); n = 1024
+    // 14.27, 16.53.  bf16 pre-round n = 256 8.31, 7.12; 512 x 1024 x 512 10.90, 10.49; n = 1024 14.46, 15.39.
+    const bool panels = b.R == 4;
+    const float most = blk == 128 ? (b.b_tile ? panels : b.preround_bf16 != 0) ? 18.5f : 15.5f
+                     : mode != FMM_SCALE_FP32_AMAX_DIV_448 ? (panels ? 8.0f : 10.0f) : 4.0f;
+    const bool one = (float)(warps + b_warps * b.R) < (float)fmm_sm_count() * most;
     bool known;
-    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) known = launch_both<32, FMM_SCALE_UE8M0_CEIL, false, false>(a, b, w, split, st);
-    else if (blk == 32) known = launch_both<32, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, split, st);
-    else if (b.b_tile && b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, true>(a, b, w, split, st);
-    else if (b.b_tile) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, false>(a, b, w, split, st);
-    else if (b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, true>(a, b, w, split, st);
-    else known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, split, st);
+    if (mode != FMM_SCALE_FP32_AMAX_DIV_448) known = launch_both<32, FMM_SCALE_UE8M0_CEIL, false, false>(a, b, w, one, st);
+    else if (blk == 32) known = launch_both<32, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, one, st);
+    else if (b.b_tile && b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, true>(a, b, w, one, st);
+    else if (b.b_tile) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, true, false>(a, b, w, one, st);
+    else if (b.preround_bf16) known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, true>(a, b, w, one, st);
+    else known = launch_both<128, FMM_SCALE_FP32_AMAX_DIV_448, false, false>(a, b, w, one, st);
     if (known) *status = cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
     return known;
 }
