@@ -958,13 +958,16 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 // Block 128: with the faster promotion the single CTAs have gained more than the pairs, whose constants are fitted again, to 666
 // problems (5 % faster on the 7 % of them that change; cubic n = 4096 122.3 -> 115.7 us a call, two levels 270 -> 257; the pairs stay at
 // n = 8192, 739 against 781, cubic 718 against 893).
-// Weight tiles: the same once more since the single CTAs' issuing warp knows its values to be uniform: the pairs' constants are scaled to
-// them (of 330 problems the choice between the two is 0.1 % off the faster one in the mean, 0.6 % with the constants before).
+// Weight tiles: the same once more since the single CTAs' issuing warp knows its values to be uniform (of 330 problems the choice between the
+// two is 0.1 % off the faster one in the mean, 0.6 % with the constants before).  The pairs' constants are higher than before in that ratio, but nothing
+// has become slower, so both are scaled by 0.87 for the comparison with the cluster kernel: of 160 problems (cubic, rank 7) the choice is 1.9 % off
+// the fastest of these kernels in the mean and without that 3.6 %, at worst 1.66 times (cubic 4480 x 4608 x 640 22.8, 34.5 us; 2816 x 5760 x 1024 51 and
+// 64 a call); 0.8 to 0.9 are within 0.5 %.
 struct ShapeModel { int ncta, bn; float c, o, o_cubic; };
 constexpr ShapeModel MODEL_MX[] = {{2, 256, 0.26f, 3.9f, 3.6f}, {1, 256, 0.35f, 3.4f, 2.7f}, {1, 128, 0.22f, 1.7f, 1.2f}};
 constexpr ShapeModel MODEL_B32[] = {{2, 128, 0.71f, 3.6f, 2.2f}, {1, 128, 0.67f, 3.55f, 1.85f}};
 constexpr ShapeModel MODEL_B128[] = {{2, 256, 0.43f, 6.0f, 5.1f}, {1, 128, 0.28f, 2.5f, 1.8f}};
-constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.37f, 5.4f, 3.4f}, {1, 128, 0.26f, 2.4f, 1.15f}};
+constexpr ShapeModel MODEL_TILE[] = {{2, 256, 0.322f, 4.7f, 2.96f}, {1, 128, 0.226f, 2.09f, 1.0f}};
 constexpr float BASE_MX = 3.3f, BASE_B32 = 2.4f, BASE_B128 = 3.85f, BASE_TILE = 3.65f;
 
 template <int N>

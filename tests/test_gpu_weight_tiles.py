@@ -75,3 +75,11 @@ def test_options_are_validated():
             fmm.Plan(U, V, W, levels=1, b_tile_n=128, **kw)
     with pytest.raises(fmm.FmmError):
         fmm.Plan(U, V, W, levels=1, block_k=128, b_tile_n=64)
+
+
+@pytest.mark.parametrize("shape", [(2816, 5760, 1024), (2560, 4992, 1152), (4480, 4608, 640)])
+def test_cubic_products_of_many_tiles_are_not_left_to_the_cluster_kernel(shape):
+    # which would share each tile's K and take 1.2 to 1.5 times as long
+    M, K, N = shape
+    plan = fmm.Plan(None, None, None, levels=0, block_k=128, scale_mode="fp32", b_tile_n=128)
+    assert plan.product_shape(M, N, K).kernel != fmm.KERNEL_CLUSTER
