@@ -40,7 +40,16 @@ def allowed(kernel):
     return 4 if mode == 1 and mask == 0 else 0
 
 
-@pytest.mark.parametrize("source,kernels", [("fmm_split.cu", 10), ("fmm_encode.cu", 60), ("fmm_stats.cu", 5)])
+OTHERS = [("fmm_split.cu", 10), ("fmm_keep.cu", 4), ("fmm_encode.cu", 60), ("fmm_stats.cu", 5)]
+
+
+def test_every_source_file_is_compiled():
+    # fmm_api.cu has no kernels
+    assert sorted(["fmm_api.cu", "fmm_gemm.cu"] + [source for source, _ in OTHERS]) == sorted(B.SOURCES)
+    assert "__global__" not in open(os.path.join(B.CSRC, "fmm_api.cu")).read()
+
+
+@pytest.mark.parametrize("source,kernels", OTHERS)
 @pytest.mark.skipif(shutil.which(B.NVCC) is None and not os.path.exists(B.NVCC), reason="nvcc not available")
 def test_other_kernels_have_no_register_spills(source, kernels):
     with tempfile.TemporaryDirectory() as tmp:

@@ -47,6 +47,20 @@ for mode, omode, blk in (("fp32", O.SCALE_FP32, 32), ("fp32", O.SCALE_FP32, 128)
         out["cases"].append({"mode": mode, "blk": blk, "levels": levels, "rel": rel, "violation": violation(plan),
                              "status": plan.device_status()})
         plan.close()
+# the product kernel that keeps a parent's blocks on chip, which is chosen for more tiles than the sizes above have
+for mode, omode, blk, tile in (("fp32", O.SCALE_FP32, 32, 0), ("ue8m0", O.SCALE_UE8M0, 32, 0), ("fp32", O.SCALE_FP32, 128, 0), ("fp32", O.SCALE_FP32, 128, 128)):
+    for levels in (1, 2):
+        d = 1 << levels
+        M, K, N = 256 * d, 128 * d, 384 * d
+        A, B = Wl.gaussian(M, K, N, seed=25 + levels)
+        U, V, W = P.get("phi_optimal")
+        plan = fmm.Plan(U, V, W, levels=levels, block_k=blk, scale_mode=mode, b_tile_n=tile)
+        plan.force_product_shape(fmm.KERNEL_BLOCKS_ON_CHIP, 1, 64, 1, 0)
+        got = plan.matmul(torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()).cpu().numpy().astype(np.float64)
+        want = O.fused_fmm(A, B, U, V, W, levels=levels, blk=blk, mode=omode, b_tile=tile)
+        out["cases"].append({"mode": mode, "blk": blk, "levels": levels, "rel": float(np.linalg.norm(got - want) / np.linalg.norm(want)),
+                             "violation": violation(plan), "status": plan.device_status()})
+        plan.close()
 # statistics kernels (no plan)
 Cm = torch.randn(192, 320, device="cuda"); Cr = Cm.double() + 1e-3
 stats = fmm.fmm_error_stats(Cm, Cr).cpu().numpy().tolist()
@@ -70,7 +84,7 @@ def test_whole_path_under_the_range_checked_build():
     assert r.returncode == 0, r.stderr[-3000:]
     line = [ln for ln in r.stdout.splitlines() if ln.startswith("RESULT ")][-1]
     out = json.loads(line[len("RESULT "):])
-    assert len(out["cases"]) == 12
+    assert len(out["cases"]) == 20
     for c in out["cases"]:
         assert c["violation"] == 0, c
         assert c["status"] == [0, 0], c

@@ -54,18 +54,25 @@ def test_more_positions_than_ctas(m, n, quantizer):
 
 @pytest.mark.parametrize("quantizer", QUANTIZERS)
 def test_zero_weights_leave_a_block_alone(quantizer):
-    # an infinity in one product reaches the blocks that it feeds and no other, with the running sums of the position before
-    # still in the registers
+    # NaN in some products reaches the blocks that they feed and no other, and not the next position of the CTA, which starts with the
+    # running sums of this one in its registers
     plan = make("strassen", 1, quantizer)
-    M = N = 2048
+    # 8 x 48 tile positions on at most 148 CTAs: a CTA has a position in the first row of tiles first and one in a later row next
+    M, N = 2048, 6144
+    m, n = M // 2, N // 2
     A = torch.randn(M, 256, device="cuda")
-    A[:M // 2, :128] = float("inf")               # A11, which feeds products of all blocks
+    A[:128, :128] = float("nan")                  # the first row of tiles of A11, which feeds products of C11, C12 and C22, none of C21
     B = torch.randn(256, N, device="cuda")
     plan.force_product_shape(*KEEP)
     got = plan.matmul(A, B)
     plan.force_product_shape(fmm.KERNEL_CLUSTER, 1, 128, 1, 0)
     want = plan.matmul(A, B)
-    assert torch.equal(torch.isnan(got), torch.isnan(want)) and torch.equal(got[~torch.isnan(got)], want[~torch.isnan(want)])
+    reached = torch.zeros(M, N, dtype=torch.bool, device="cuda")
+    reached[:128] = True                          # C11, C12
+    reached[m:m + 128, n:] = True                 # C22
+    for c in (got, want):
+        assert torch.equal(torch.isnan(c), reached) and torch.isfinite(c[~reached]).all()
+    assert torch.equal(got[~reached], want[~reached])
 
 
 def test_choice_and_refusals():

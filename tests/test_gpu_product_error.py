@@ -28,7 +28,8 @@ def dequantized(plan, ws, M, N, K, term):
 @pytest.mark.parametrize("blk,tile,form,bound", [
     # every product is summed on its own; what is left is the order of the seven sums
     (32, 0, (fmm.KERNEL_PERSISTENT, 2, 128, 1, 1), 1.03), (32, 0, (fmm.KERNEL_PERSISTENT, 1, 128, 1, 1), 1.03),
-    (32, 0, (fmm.KERNEL_CLUSTER, 1, 64, 1, 0), 1.03),
+    (32, 0, (fmm.KERNEL_CLUSTER, 1, 64, 1, 0), 1.03), (32, 0, (fmm.KERNEL_BLOCKS_ON_CHIP, 1, 64, 1, 0), 1.03),
+    (128, 0, (fmm.KERNEL_BLOCKS_ON_CHIP, 1, 64, 1, 0), 1.03), (128, 128, (fmm.KERNEL_BLOCKS_ON_CHIP, 1, 64, 1, 0), 1.03),
     # the accumulators start from the carried sum: 1.57 times for independent products (see the walk's own test)
     (32, 0, (fmm.KERNEL_PERSISTENT, 2, 128, 1, 0), 1.6), (128, 0, (fmm.KERNEL_PERSISTENT, 2, 256, 1, 0), 1.6),
     (128, 128, (fmm.KERNEL_PERSISTENT, 2, 256, 1, 0), 1.6)])

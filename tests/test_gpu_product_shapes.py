@@ -1,4 +1,4 @@
-"""Every tile shape of both product kernels, forced, at the sizes where its indexing can go wrong: one tile, leaves that are not
+"""Every tile shape of the product kernels, forced, at the sizes where its indexing can go wrong: one tile, leaves that are not
 a multiple of the tile (half of a CTA pair's rows, half of a wide tile's columns hang over the edge), one K stage, more stages
 than operand slots, several parents - against the oracle; what a plan cannot take is refused."""
 import numpy as np
@@ -19,9 +19,15 @@ SHAPES = {
     (128, "fp32", 0): [(P, 2, 256, 1, 0), (P, 1, 128, 1, 0), (CL, 1, 128, 1, 0), (CL, 1, 64, 1, 0), (CL, 1, 32, 1, 0)],
     (128, "fp32", 128): [(P, 2, 256, 1, 0), (P, 1, 128, 1, 0), (CL, 1, 128, 1, 0), (CL, 1, 64, 1, 0), (CL, 1, 32, 1, 0)],
 }
+# for plans with products to combine, every quantizer
+KEEP = (fmm.KERNEL_BLOCKS_ON_CHIP, 1, 64, 1, 0)
 SIZES = [("strassen", 1, (256, 256, 256)), ("winograd", 1, (768, 1536, 768)), ("cubic8", 1, (256, 512, 768)),
          ("orbit_05", 1, (768, 256, 256)), ("phi_optimal", 2, (512, 1024, 1536)), ("strassen", 3, (1024, 1024, 1024)),
          ("cubic", 0, (384, 1024, 128)), ("cubic", 0, (128, 128, 384))]
+
+
+def shapes(name, quantizer):
+    return SHAPES[quantizer] + ([] if name == "cubic" else [KEEP])
 
 
 def make(name, levels, quantizer):
@@ -38,7 +44,7 @@ def test_every_shape_matches_oracle(name, levels, shape, quantizer):
     a, b = dev(A), dev(B)
     want = O.fused_fmm(A, B, *coeffs(name), levels=levels, blk=blk, mode=MODES[mode], b_tile=tile)
     plan = make(name, levels, quantizer)
-    forms = list(SHAPES[quantizer])
+    forms = shapes(name, quantizer)
     if name == "cubic":
         forms += [(CL, 1, c, s, 0) for _, _, c, _, _ in forms[-1:] for s in (2, 4, 8) if s <= K // 128]
     d = 1 << levels
@@ -58,12 +64,12 @@ def test_every_shape_matches_oracle(name, levels, shape, quantizer):
 @pytest.mark.parametrize("quantizer", list(SHAPES))
 def test_shapes_that_do_not_exist_are_refused(quantizer):
     for levels, name in ((0, "cubic"), (1, "strassen")):
-        known = set(SHAPES[quantizer])
+        known = set(shapes(name, quantizer))
         if quantizer[1] == "ue8m0" and levels:
             known.add((fmm.KERNEL_CLUSTER_TWO_TERMS, 1, 128, 1, 0))
         plan = make(name, levels, quantizer)
         chosen = tuple(plan.product_shape(256, 256, 256))
-        for form in [(k, c, n, s, w) for k in (1, 2, 3, 4) for c in (1, 2) for n in (32, 64, 128, 256) for s in (1, 2, 3) for w in (0, 1)]:
+        for form in [(k, c, n, s, w) for k in (1, 2, 3, 4, 5, 8, 16) for c in (1, 2) for n in (32, 64, 128, 256) for s in (1, 2, 3) for w in (0, 1)]:
             base = (*form[:3], 1, form[4])
             if base in known and (form[3] == 1 or (form[3] == 2 and form[0] == CL and levels == 0)):
                 plan.force_product_shape(*form)

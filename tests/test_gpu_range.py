@@ -6,7 +6,7 @@ import torch
 
 from paper_2609_26077_b200 import fmm, workloads as Wl
 from gpu_common import coeffs, dev
-from test_gpu_product_shapes import SHAPES
+from test_gpu_product_shapes import SHAPES, shapes
 
 pytestmark = pytest.mark.gpu
 
@@ -22,7 +22,7 @@ def test_powers_of_two_pass_through(name, levels, quantizer):
     # elements of B up to 2^124, of its partial products with 8-bit codes up to 2^138; the clamp of the scales stays out of it
     for ea, eb in ((-30, 120), (120, -30), (-30, -30), (40, 40)):
         sa, sb = float(np.float32(2.0) ** ea), float(np.float32(2.0) ** eb)
-        for form in SHAPES[quantizer]:
+        for form in shapes(name, quantizer):
             plan.force_product_shape(*form)
             want = plan.matmul(a, b).double() * 2.0 ** (ea + eb)
             got = plan.matmul(a * sa, b * sb)
@@ -57,7 +57,7 @@ def test_products_above_the_range_whose_weighted_sums_are_in_it(K):
     e = 124 - int(np.ceil(np.log2(K) / 2))
     sa, sb = 2.0 ** (e // 2), 2.0 ** (e - e // 2)
     plan = fmm.Plan(U, V, W, levels=1, block_k=32, scale_mode="fp32")
-    for form in [f for f in SHAPES[(32, "fp32", 0)] if f[4] == 0]:
+    for form in [f for f in shapes("phi_optimal", (32, "fp32", 0)) if f[4] == 0]:
         plan.force_product_shape(*form)
         want = plan.matmul(a, b).double() * 2.0 ** e
         got = plan.matmul(a * sa, b * sb)
