@@ -947,11 +947,11 @@ fmm_status_t launch(const GemmParams& g, cudaStream_t st, bool separate = false)
 // hangs over the edge is multiplied and not stored, so a leaf of an odd number of 128-row or 128-column blocks may take the
 // wide tiles as well, at the price of a part of its last row or column of tiles.  Fitted, together with the cluster kernel's
 // model (fmm_split.cu), to the times of every shape over leaves of 128 to 8192 in every direction and zero to three levels.
-// Over 60 random problems per kind (leaves of 128 to 5000) the choice is the fastest shape for 39 to 54 of them and costs, in
-// the mean, 3.2 % (block 32), 0.7 % (UE8M0), 2.7 % (block 128) and 2.9 % (weight tiles) more than the fastest; those above 12 us
-// 1.5 %, 0.8 %, 0.1 % and 1.4 %.  The worst are single products of about 8 us, at up to 1.33 times, and at block 32, whose constants and the
-// cluster kernel's stand as fitted to a slower promotion, products of 30 to 74 us that the persistent kernel would take in 0.81 times
-// the cluster kernel's time (2816 x 768 x 3840, 7936 x 512 x 768; with carried sums instead of separate ones).  Product kernel
+// Over 60 random problems per kind (leaves of 128 to 5000) the choice among all product kernels is the fastest shape for 43 to 54 of them
+// and costs, in the mean, 3.4 % (block 32), 1.4 % (UE8M0), 2.2 % (block 128) and 0.1 % (weight tiles) more than the fastest; those above
+// 12 us 2.7 %, 1.9 %, 2.0 % and 0.2 %.  The worst are single products of about 8 us, at up to 1.32 times, and at block 32, whose constants and the
+// cluster kernel's stand as fitted to a slower promotion, products of 39 to 66 us that the persistent kernel would take in 0.80 times
+// the cluster kernel's time (3328 x 2304 x 1536, 9728 x 1024 x 512; with carried sums instead of separate ones).  Product kernel
 // against the rule before, which gave wide tiles only to leaves that are multiples of them: UE8M0 8192 x 8192 x 8448 one
 // level 674 -> 492 us, cubic 4096 x 1024 x 4224 47.6 -> 26.4; block 128 8192 x 8192 x 8448 956 -> 787; weight tiles
 // 888 -> 664.

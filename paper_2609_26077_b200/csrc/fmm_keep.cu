@@ -489,7 +489,9 @@ fmm_status_t launch_keep(const GemmParams& g, cudaStream_t st)
 // Fitted to 1500 problems of 40 to 5500 items (Strassen, Winograd, Phi-optimal, one to three levels, leaves of up to 2560 in K): 3 to 8 %
 // off.  With the margin of 3 % the kernel is chosen for half of them, takes 0.80 times the time of the fastest other kernel there in
 // the mean (all problems: 0.88 block 32, 0.85 UE8M0, 0.91 block 128, 0.87 weight tiles; the best choice would gain 0.5 % more)
-// and at most 1.02 times.  Phi-optimal, us, block 32 / UE8M0 / block 128 / weight tiles: 2048 x 512 x 2048 29.7 -> 17.1, 18.8 -> 11.5,
+// and at most 1.02 times.  (In another sample, timed in a graph, at most 1.05 times, of 1012 problems that take it; beyond the fit, at 6272 to 25088 items, it is
+// chosen for 45 of 68 problems, in 0.77 times the other kernels' time in the mean and at most 0.98 times, and would be faster by up to 1.17 times
+// for nine more.)  Phi-optimal, us, block 32 / UE8M0 / block 128 / weight tiles: 2048 x 512 x 2048 29.7 -> 17.1, 18.8 -> 11.5,
 // 24.3 -> 14.7, 24.4 -> 12.7; three levels n = 2048 78.5 -> 55.6, 59.5 -> 41.2, 64.0 -> 46.6, 59.9 -> 41.1; not chosen: one level n = 4096
 // (16 stages) 216 against 274, 70 against 110, 110 against 168, 97 against 126.
 struct KeepTime { float base, o, k, mem; };
